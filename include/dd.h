@@ -117,7 +117,8 @@ dd_status dd_set_profiles(dd_plan_t plan, const int32_t* delay, const int32_t* n
  * round trip).  d_w is [ndm][nchan][kmax] fp32; the delay and tap tables are kept and
  * every n_dc must be <= kmax.  A unit-weight plan becomes a weighted one (fp32 sums).
  * Meant for training loops (the autograd binding calls it before each forward and
- * backward).  Errors: DD_ERR_ARG, DD_ERR_OOM, DD_ERR_CUDA. */
+ * backward).  Weights from the device are summed tap by tap (the host cannot see which
+ * trials share them); a plan whose host weights were shared is rebuilt at its first call.  Errors: DD_ERR_ARG, DD_ERR_OOM, DD_ERR_CUDA. */
 dd_status dd_set_weights_device(dd_plan_t plan, const float* d_w, int32_t kmax, void* stream);
 
 /* Plan facts: t_out = nsamp - d_max for the default nsamp, d_max = max(delta + n - 1),
@@ -249,7 +250,10 @@ dd_status dd_backward(dd_plan_t plan, const float* d_in, int64_t in_ld, int64_t 
 
 /* Kernel schedule of the plan: nch time chunks per CTA (the CTA sums 16/nch trials on
  * the fp32 path, 8/nch on the exact integer path, 24/nch on the run-length path) and cs
- * channels per pipeline stage.
+ * channels per pipeline stage.  Plans whose trials share their tap runs (fp32 sums with
+ * weights given from the host: unit weights, or weights that many trials have in common) use
+ * kernels that form each shared run's sums once: there a CTA sums 24/nch or 48/nch trials (by
+ * the size of the plan's block) and cs is the most channels of a stage.
  * dd_plan_create and dd_set_profiles pick a default; dd_plan_set_schedule overrides it
  * (DD_ERR_UNSUPPORTED if it does not fit in shared memory, the old one is then kept). */
 dd_status dd_plan_set_schedule(dd_plan_t plan, int32_t nch, int32_t cs);

@@ -205,8 +205,10 @@ dd_status launch_backward(dd_plan_s* p, const float* in, int64_t ld, int64_t t_o
             if (st != DD_OK) return st;
         }
         dd_plan_s* t = p->adj;
+        const uint64_t gen = t->dev_gen;
         st = upload_tables(t);
         if (st != DD_OK) return st;
+        if (t->dev_gen != gen) p->adj_w_stale = true;  // new tables hold no weights yet
         const int32_t P = p->dmax;
         const int64_t nsamp = t_out + P;
         // padded gradient rows: P zeros, t_out values, zeros up to a 16-byte multiple

@@ -29,7 +29,13 @@ struct dd_batch_s {
     std::vector<uint32_t*> d_prefix;  // run-length beams: each beam's prefix sums
     std::vector<int64_t> ldp;
     std::vector<dd::BatchItem> items;
-    size_t smem = 0;
+    // one launch per kernel: row kernels with 16 and 8 warps per CTA, then the tap kernels
+    struct Group {
+        int warps;  // of the row kernel; 0: tap kernel
+        size_t first, count, smem;
+    };
+    std::vector<Group> groups;
+    std::vector<uint64_t> gen;         // the uploads that the bound arguments point into
     int grid = 0;
     int device = -1;
     int64_t units = 0;  // sum over beams of trials x outputs
@@ -78,6 +84,7 @@ void free_batch_dev(dd_batch_s* b) {
 void build_items(dd_batch_s* b) {
     constexpr int kGroupBlocks = 16;
     struct Beam {
+        int warps;  // of the beam's row kernel, or 0
         double cost;
         int beam;
     };
@@ -87,19 +94,24 @@ void build_items(dd_batch_s* b) {
         const dd_plan_s* p = b->plans[beam];
         const int64_t t_out = plan_t_out(p);
         const int nst = (p->nchan + p->cs - 1) / p->cs;
-        const int64_t tile = (int64_t)dd::chunk_t(p->pair) * p->nch;
+        const int64_t tile = dd::plan_tile_t(p);
         const int64_t ntile = (t_out + tile - 1) / tile;
         double taps = 0;
-        for (int64_t i = 0; i < (int64_t)p->ndm * p->nchan; ++i) taps += p->rl ? 1.0 : p->taps[(size_t)i];
+        for (int64_t i = 0; i < (int64_t)p->ndm * p->nchan; ++i) taps += p->rl || p->rk ? 1.0 : p->taps[(size_t)i];
         b->units += (int64_t)p->ndm * t_out;
-        order.push_back({taps * (double)t_out + 2.0e4 * nst * ntile * p->nblk, beam});
+        order.push_back({p->rk ? p->row_warps : 0, taps * (double)t_out + 2.0e4 * nst * ntile * p->nblk, beam});
     }
-    std::stable_sort(order.begin(), order.end(), [](const Beam& x, const Beam& y) { return x.cost > y.cost; });
+    std::stable_sort(order.begin(), order.end(), [](const Beam& x, const Beam& y) {
+        return x.warps != y.warps ? x.warps > y.warps : x.cost > y.cost;
+    });
     b->items.clear();
+    b->groups.clear();
     for (const Beam& bm : order) {
         const dd_plan_s* p = b->plans[bm.beam];
         const int64_t t_out = plan_t_out(p);
-        const int64_t tile = (int64_t)dd::chunk_t(p->pair) * p->nch;
+        const int64_t tile = dd::plan_tile_t(p);
+        if (b->groups.empty() || b->groups.back().warps != bm.warps)
+            b->groups.push_back({bm.warps, b->items.size(), 0, 0});
         const int ntile = (int)((t_out + tile - 1) / tile);
         for (int g0 = 0; g0 < p->nblk; g0 += kGroupBlocks)
             for (int tx = 0; tx < ntile; ++tx)
@@ -111,8 +123,15 @@ void build_items(dd_batch_s* b) {
                     it.pad = 0;
                     b->items.push_back(it);
                 }
+        // shared memory: the most that any beam of the launch needs
+        dd_batch_s::Group& g = b->groups.back();
+        g.count = b->items.size() - g.first;
+        g.smem = std::max(g.smem, dd::dedisp_smem_for(p));
     }
 }
+
+// The row kernels' kind for the batch's beams.
+int row_kind(const dd_batch_s* b) { return b->pair ? dd::kRowsFir : (b->rl ? dd::kRowsRl : dd::kRowsU8); }
 
 bool aligned16(const void* ptr) { return ((uintptr_t)ptr & 15u) == 0; }
 
@@ -138,7 +157,6 @@ dd_status dd_batch_create(dd_batch_t* out, const dd_plan_t* plans, int32_t nbeam
     b->u8 = plans[0]->band.in_type == DD_U8;
     b->pair = plans[0]->pair;
     b->rl = plans[0]->rl;
-    for (auto* p : b->plans) b->smem = std::max(b->smem, dd::dedisp_smem_for(p));
     build_items(b);
     *out = b;
     return DD_OK;
@@ -162,8 +180,6 @@ dd_status dd_batch_bind(dd_batch_t b, const void* const* d_in, const int64_t* in
         if (st != DD_OK) return st;
     }
     // plans may have been retuned since dd_batch_create: rebuild the work list
-    b->smem = 0;
-    for (auto* p : b->plans) b->smem = std::max(b->smem, dd::dedisp_smem_for(p));
     build_items(b);
     free_batch_dev(b);
     for (int i = 0; i < nb; ++i) {
@@ -191,8 +207,11 @@ dd_status dd_batch_bind(dd_batch_t b, const void* const* d_in, const int64_t* in
     if (e != cudaSuccess) return dd::cuda_status(e);
     b->short_taps = true;
     for (auto* p : b->plans)
-        b->short_taps = b->short_taps && (p->rl ? p->rl_b : p->pair ? p->umax <= dd::kRPair : p->kmax <= dd::kRInt);
-    const int per_sm = dd::dedisp_batched_blocks_per_sm(b->u8, b->pair, b->short_taps, b->smem, b->rl);
+        if (!p->rk) b->short_taps = b->short_taps && (p->rl ? p->rl_b : p->pair ? p->umax <= dd::kRPair : p->kmax <= dd::kRInt);
+    int per_sm = 32;
+    for (const auto& g : b->groups)
+        per_sm = std::min(per_sm, g.warps ? dd::rows_batched_blocks_per_sm(row_kind(b), b->u8, g.warps, g.smem)
+                                          : dd::dedisp_batched_blocks_per_sm(b->u8, b->pair, b->short_taps, g.smem, b->rl));
     if (per_sm < 1) return DD_ERR_UNSUPPORTED;
     if (b->items.size() >= (size_t)INT32_MAX) return DD_ERR_UNSUPPORTED;
     b->grid = (int)b->items.size();  // one CTA per work item
@@ -212,11 +231,36 @@ dd_status dd_batch_bind(dd_batch_t b, const void* const* d_in, const int64_t* in
     b->in_ld.assign(in_ld, in_ld + nb);
     b->out.assign(d_out, d_out + nb);
     b->out_ld.assign(out_ld, out_ld + nb);
+    size_t smem = 0;
+    for (const auto& g : b->groups) smem = std::max(smem, g.smem);
+    b->gen.clear();
+    for (auto* p : b->plans) b->gen.push_back(p->dev_gen);
     b->bound = true;
     b->box_bound = false;
     dd::log_msg(1, "batch of %d beams (%s): %zu work items (one CTA each, %d resident per SM on %d SMs), "
-             "%zu bytes of shared memory", nb, b->rl ? "run-length sums" : (b->pair ? "fp32 pair units" : "exact integer sums"),
-             b->items.size(), per_sm, sms, b->smem);
+             "%zu launches, up to %zu bytes of shared memory", nb, b->rl ? "run-length sums" : (b->pair ? "fp32 pair units" : "exact integer sums"),
+             b->items.size(), per_sm, sms, b->groups.size(), smem);
+    return DD_OK;
+}
+
+// Whether a bound plan's device tables have been replaced since (new profiles or weights).
+static bool batch_stale(const dd_batch_s* b) {
+    for (size_t i = 0; i < b->plans.size(); ++i)
+        if (b->plans[i]->dev_dirty || b->plans[i]->dev_gen != b->gen[i]) return true;
+    return false;
+}
+
+// Binds the same buffers again, keeping the boxcar stage's.
+static dd_status batch_rebind(dd_batch_s* b) {
+    const std::vector<const void*> in = b->in;
+    const std::vector<int64_t> in_ld = b->in_ld, out_ld = b->out_ld;
+    const std::vector<void*> out = b->out;
+    const bool box = b->box_bound;
+    for (auto* p : b->plans)
+        if (plan_t_out(p) < 1) return DD_ERR_ARG;
+    const dd_status st = dd_batch_bind(b, in.data(), in_ld.data(), out.data(), out_ld.data());
+    if (st != DD_OK) return st;
+    b->box_bound = box;
     return DD_OK;
 }
 
@@ -224,6 +268,10 @@ dd_status dd_batch_dedisperse(dd_batch_t b, void* stream) {
     DD_TRACE("dd_batch_dedisperse");
     if (!b) return DD_ERR_ARG;
     if (!b->bound) return DD_ERR_STATE;
+    if (batch_stale(b)) {
+        const dd_status st = batch_rebind(b);
+        if (st != DD_OK) return st;
+    }
     if (b->rl)  // every beam's prefix sums first
         for (size_t i = 0; i < b->plans.size(); ++i) {
             const dd_status st = dd::launch_prefix_into(b->plans[i], b->in[i], b->in_ld[i], 0,
@@ -231,8 +279,15 @@ dd_status dd_batch_dedisperse(dd_batch_t b, void* stream) {
                                                         (cudaStream_t)stream);
             if (st != DD_OK) return st;
         }
-    return dd::launch_dedisperse_batched(b->u8, b->pair, b->short_taps, b->d_args, b->d_items, (int32_t)b->items.size(),
-                                         b->smem, (cudaStream_t)stream, b->rl);
+    for (const auto& g : b->groups) {
+        const dd_status st =
+            g.warps ? dd::launch_rows_batched(row_kind(b), b->u8, g.warps, b->d_args, b->d_items + g.first,
+                                              (int32_t)g.count, g.smem, (cudaStream_t)stream)
+                    : dd::launch_dedisperse_batched(b->u8, b->pair, b->short_taps, b->d_args, b->d_items + g.first,
+                                                    (int32_t)g.count, g.smem, (cudaStream_t)stream, b->rl);
+        if (st != DD_OK) return st;
+    }
+    return DD_OK;
 }
 
 dd_status dd_batch_bind_boxcar(dd_batch_t b, const int32_t* widths, int32_t nw, double* const* d_mean,
@@ -279,22 +334,15 @@ dd_status dd_batch_run(dd_batch_t b, void* stream) {
     return batch_run(b, (cudaStream_t)stream);
 }
 
-dd_status dd_batch_capture(dd_batch_t b, void* stream) {
-    if (!b || !stream) return DD_ERR_ARG;
-    if (!b->bound) return DD_ERR_STATE;
-    cudaStream_t s = (cudaStream_t)stream;
-    // one eager pass first: it creates every plan's workspace, which a capture may not
-    dd_status st = batch_run(b, s);
-    if (st != DD_OK) return st;
-    cudaError_t e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return dd::cuda_status(e);
+// Captures one block on `s` (every workspace exists) into the batch's graph.
+static dd_status capture_run(dd_batch_s* b, cudaStream_t s) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     b->exec = nullptr;
     b->graph = nullptr;
-    e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+    cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return dd::cuda_status(e);
-    st = batch_run(b, s);
+    const dd_status st = batch_run(b, s);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(s, &g);
     if (st != DD_OK) {
@@ -307,10 +355,33 @@ dd_status dd_batch_capture(dd_batch_t b, void* stream) {
     return dd::cuda_status(e);
 }
 
+dd_status dd_batch_capture(dd_batch_t b, void* stream) {
+    if (!b || !stream) return DD_ERR_ARG;
+    if (!b->bound) return DD_ERR_STATE;
+    cudaStream_t s = (cudaStream_t)stream;
+    // one eager pass first: it creates every plan's workspace, which a capture may not
+    dd_status st = batch_run(b, s);
+    if (st != DD_OK) return st;
+    cudaError_t e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return dd::cuda_status(e);
+    return capture_run(b, s);
+}
+
 dd_status dd_batch_replay(dd_batch_t b, void* stream) {
     DD_TRACE("dd_batch_replay");
     if (!b) return DD_ERR_ARG;
     if (!b->exec) return DD_ERR_STATE;
+    if (batch_stale(b)) {
+        // a plan's tables have moved: this block eagerly, and a new graph for the next
+        dd_status st = batch_run(b, (cudaStream_t)stream);
+        if (st != DD_OK) return st;
+        cudaStream_t s = nullptr;
+        const cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return dd::cuda_status(e);
+        st = capture_run(b, s);
+        cudaStreamDestroy(s);
+        return st;
+    }
     return dd::cuda_status(cudaGraphLaunch(b->exec, (cudaStream_t)stream));
 }
 

@@ -222,7 +222,10 @@ void fill_dedisp_args(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_
     a->blen = p->blen;
     a->cs = p->cs;
     a->nch = p->nch;
-    a->kpad = p->pair ? p->kw : 0;
+    a->kpad = p->pair || p->rk ? p->kw : 0;
+    a->rows_max = p->rows_max;
+    a->lo_ld = p->lo_ld;
+    a->nst = p->nst;
     a->status = p->dev.status;
     a->skip_stage = p->debug_skip_stage;
     a->wait_ns = p->wait_ns;
@@ -232,6 +235,7 @@ void fill_dedisp_args(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_
 }
 
 size_t dedisp_smem_for(const dd_plan_s* p) {
+    if (p->rk) return rows_smem_for(p);
     const int kp = p->pair ? p->kw : 0;
     if (p->rl) return smem_for<uint32_t, false, kStagesRl>(p->lcap, 0, p->cs, p->nch, p->nchan, p->rl_b, p->blen);
     if (!p->pair) return smem_for<uint8_t, false, kStagesInt>(p->lcap, kp, p->cs, p->nch, p->nchan);
@@ -244,6 +248,7 @@ dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_
                             int64_t split_ld) {
     DedispArgs a;
     fill_dedisp_args(p, in, ld, t_offset, t_out, out, out_ld, &a);
+    if (p->rk) return nsplit == 1 ? launch_rows(p, a, s) : DD_ERR_UNSUPPORTED;
     a.nsplit = nsplit;
     a.split_ld = split_ld;
     const bool u8 = p->band.in_type == DD_U8;
@@ -295,6 +300,7 @@ dd_status launch_dedisperse_rl(dd_plan_s* p, const void* in, int64_t ld, int64_t
     if (st != DD_OK) return st;
     DedispArgs a;
     fill_dedisp_args(p, p->d_prefix, ldp, 0, nsamp - p->dmax, out, out_ld, &a);
+    if (p->rk) return launch_rows(p, a, s);
     return p->rl_b ? run<uint32_t, false, kStagesRl, 1>(a, s) : run<uint32_t, false, kStagesRl>(a, s);
 }
 

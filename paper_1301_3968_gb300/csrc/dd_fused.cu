@@ -295,13 +295,39 @@ void grouped_parts(int64_t nblk, int tiles, int nseg, int64_t gb, std::vector<in
             for (int64_t b = g0; b < std::min(nblk, g0 + gb); ++b) order->push_back(b * nseg + k);
 }
 
+// Segments per trial block for the row kernels, whose records are small (about 90 kB per
+// block of the CRAFT-like list, in L2 for any order): the cut whose waves of parts take
+// least, a part costing its tiles and about a third of one for its start.
+int row_segments(int64_t nblk, int tiles, int64_t slots) {
+    int best = 1;
+    double least = 1e300;
+    for (int k = 1; k <= tiles; ++k) {
+        const double t = (double)((nblk * k + slots - 1) / slots) * ((tiles + k - 1) / k + 0.35);
+        if (t < least) {
+            least = t;
+            best = k;
+        }
+    }
+    return best;
+}
+
 bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
 constexpr int64_t kFusedGroup = 16;  // trial blocks per group of fp32 fused parts
 
 }  // namespace
 
-size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C) {
+size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C, bool one_row) {
+    if (p->rk) {
+        // a row per trial and the warps' scratch; one_row: a row per warp group and its other
+        // trials' waiting sums, the scratch then in the padding behind the rows
+        const int nt = row_unit_trials(p->rk), nrow = plan_trials(p) / (one_row ? nt : 1);
+        const int scratch = p->row_warps * fused::kChainFloats;
+        const int words = one_row ? nrow * rowlen + std::max(C + 48, scratch) + p->row_warps * (nt - 1) * row_warp_t(p->rk)
+                                  : fused_rows_ints(nrow, rowlen, C) + scratch;
+        const size_t rows = (size_t)words * 4 + 8 + 2 * 4;
+        return (std::max(dedisp_smem_for(p), rows) + 15) & ~(size_t)15;
+    }
     const int nbuf = p->rl ? kStagesRl : (p->pair ? kStagesPair : kStagesInt);
     // fp32 pair units: a row per trial; run-length path: a row per warp group and the
     // group's other trials' sums
@@ -317,6 +343,7 @@ size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C) {
 int pair_passes(const dd_plan_s* p) { return p->umax <= kRPair ? 1 : (p->umax <= 2 * kRPair ? 2 : 0); }
 
 int fused_blocks_per_sm(const dd_plan_s* p, size_t smem) {
+    if (p->rk) return rows_fused_blocks_per_sm(p, smem);
     if (p->rl) return p->rl_b ? fused_bps<uint32_t, false, kStagesRl, 1>(smem) : fused_bps<uint32_t, false, kStagesRl, 0>(smem);
     if (p->pair) {
         const int np = pair_passes(p);
@@ -331,6 +358,7 @@ int fused_blocks_per_sm(const dd_plan_s* p, size_t smem) {
 
 dd_status launch_dedisperse_fused(const dd_plan_s* p, DedispArgs a, const FusedArgs& f, size_t smem,
                                   cudaStream_t s) {
+    if (p->rk) return launch_rows_fused(p, a, f, smem, s);
     if (p->rl)
         return p->rl_b ? run_fused<uint32_t, false, kStagesRl, 1>(a, f, smem, s) : run_fused<uint32_t, false, kStagesRl, 0>(a, f, smem, s);
     if (p->pair) {
@@ -369,10 +397,10 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
     const bool fp = p->pair;  // fp32 sums (fp32 input, or weighted uint8)
     if (!fp && (p->band.in_type != DD_U8 || !p->out_int)) return DD_ERR_UNSUPPORTED;
     if (widths[nw - 1] - widths[0] != nw - 1) return DD_ERR_UNSUPPORTED;  // w_j = w_0 + j only
-    const int L = chunk_t(fp) * p->nch;
+    const int L = plan_tile_t(p);
     // carried outputs: the longest window (integer), or back to its prefix chain's start
     const int C = fp ? widths[nw - 1] + kBoxSeg - 2 : widths[nw - 1] - 1;
-    if (C > L) return DD_ERR_UNSUPPORTED;
+    if (C > chunk_t(fp) * p->nch) return DD_ERR_UNSUPPORTED;  // (a row kernel's tile is longer)
     const int64_t esz = p->band.in_type == DD_U8 ? 1 : 4;
     if (!aligned16(in) || (in_ld * esz) % 16 != 0) return DD_ERR_ARG;
     if (t_out > INT32_MAX - chunk_t(fp) * kWarps || in_ld > (int64_t)1 << 40) return DD_ERR_OVERFLOW;
@@ -391,13 +419,15 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
         fill_dedisp_args(p, in, in_ld, t_offset, t_out, nullptr, 0, &a);
     }
     const int tiles = (int)((t_out + L - 1) / L);
-    const int tpc = kWarps / p->nch * (p->rl ? kRlUnits : 1) * (fp ? 2 : 1);
+    const int tpc = plan_trials(p);
     const int64_t nblk = (p->ndm + tpc - 1) / tpc;
     // row: C carried outputs, the tile and 32 spare (fp32: 48); the last tile's extra
     // starts read up to C + 14 past a row (fp32: 15 past the row's windows), into the
     // next one or the padding behind the last
     const int rowlen = L + C + (fp ? 48 : 32);
-    const size_t smem = fused_smem_for(p, rowlen, C);
+    size_t smem = fused_smem_for(p, rowlen, C);
+    const bool one_row = p->rk && smem > kSmemMax;
+    if (one_row) smem = fused_smem_for(p, rowlen, C, true);
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -434,7 +464,8 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
         // CRAFT-like list), so the CTAs working together must share few blocks: groups of
         // kFusedGroup blocks, each block cut into as many segments as fill the resident CTAs
         const int64_t gb = std::min<int64_t>(nblk, kFusedGroup);
-        const int nseg = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (slots + gb - 1) / gb));
+        int nseg = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (slots + gb - 1) / gb));
+        if (p->rk) nseg = row_segments(nblk, tiles, slots);
         grouped_parts(nblk, tiles, nseg, gb, &starts, &order);
         nparts = (int)(starts.size() - 1);
     } else {
@@ -458,6 +489,7 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
     f.rowlen = rowlen;
     f.nparts = nparts;
     f.tiles = tiles;
+    f.one_row = one_row;
     f.mlim = INT_MAX / widths[nw - 1];
     f.off = p->dev.off;
     int64_t have_starts = (int64_t)p->fstarts.size();

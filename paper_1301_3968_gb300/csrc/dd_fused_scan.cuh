@@ -40,13 +40,12 @@ constexpr int G = 16;  // widths per register window
 // width of the group forms).
 constexpr int kChainFloats = 80;
 
-// S = kRInt starts of one lane segment (x = row + i0) for widths w0g + j, j < G.
+// S starts of one lane segment (x = row + i0) for widths w0g + j, j < G.
 // q = sum_{k < w0g} x[k] on entry.  !FULL: starts outside [i_lo, i_hi) and windows
 // ending past row index e_hi are left out.
-template <bool FULL>
+template <bool FULL, int S>
 __device__ __forceinline__ void scan_segment(const int* x, uint32_t q, int w0g, int i0, int i_lo,
                                              int i_hi, int e_hi, int (&seg)[G]) {
-    constexpr int S = kRInt;
     uint32_t win[G];
     win[0] = q;
 #pragma unroll
@@ -85,28 +84,31 @@ __device__ __forceinline__ int warp_max16(const int (&seg)[G], int lane) {
 
 // Upper bound of every sum the FULL scan of one width group would form:
 // max_{s, j} P[s + w0g + j] - min_s P[s] <= Q + Mrel, with P the prefix of the segment,
-// Q = P[w0g] - min_s P[s] and Mrel = max(0, max_m sum_{k=w0g}^{w0g+m} x[k]), m < cnt + 29.
-// Q is a window sum of at most wmax values and Mrel one of at most 45, so both are exact
-// in int32 when wmax >= 46 (every such sum fits, by the overflow check).
+// Q = P[w0g] - min_s P[s] and Mrel = max(0, max_m sum_{k=w0g}^{w0g+m} x[k]), m < cnt + S - 2.
+// Q is a window sum of at most wmax values and Mrel one of at most S + 14, so both are
+// exact in int32 when wmax >= S + 15 (every such sum fits, by the overflow check).
+template <int S>
 __device__ __forceinline__ long long group_bound(const int* x, uint32_t q, uint32_t pmin, int w0g, int cnt) {
     int r = 0, mrel = 0;
-    for (int m = 0; m < cnt + 29; ++m) {
+    for (int m = 0; m < cnt + S - 2; ++m) {
         r += x[w0g + m];
         mrel = max(mrel, r);
     }
     return (long long)(int)(q - pmin) + mrel;
 }
 
-// Width groups from kPruneW on skip the scan of segments whose group_bound is below
+// Width groups from prune_w on skip the scan of segments whose group_bound is below
 // the smallest merged maximum of the group (strictly: a tie from an earlier start could
 // still win), which on noise-like series is most of them.
-constexpr int kPruneW = 48;
+template <int S>
+__host__ __device__ constexpr int prune_w() { return S + 15 > 48 ? S + 15 : 48; }
 
-// The scan of one row for one trial (warp-uniform arguments; see epilogue).
+// The scan of one row for one trial (warp-uniform arguments; see epilogue), S starts per lane.
+template <int S>
 __device__ __forceinline__ void scan_row(const FusedArgs& f, const int* row, uint32_t* chain,
                                       unsigned long long* keyrow, int64_t T0, int C, int chunk, int nch,
                                       int lane, int i_lo, int i_hi, int e_hi) {
-    constexpr int R = kRInt, TT = 32 * R;
+    constexpr int R = S, TT = 32 * R;
     __builtin_assume(__isShared(row));
     const int ng = (f.nw + G - 1) / G;
     const int jl = lane >> 1;
@@ -120,7 +122,7 @@ __device__ __forceinline__ void scan_row(const FusedArgs& f, const int* row, uin
         uint32_t q = 0, pmin = 0;
         if (any) {
             for (int kk = 0; kk < f.w0; ++kk) q += (uint32_t)x[kk];
-            if (inner) {  // min_s P[s] over the segment's starts (sums of <= 30 values)
+            if (inner) {  // min_s P[s] over the segment's starts (sums of < S values)
                 int r = 0, mn = 0;
                 for (int s = 0; s < R - 1; ++s) {
                     r += x[s];
@@ -138,27 +140,27 @@ __device__ __forceinline__ void scan_row(const FusedArgs& f, const int* row, uin
             const int bt = (int)(0xffffffffu - (uint32_t)bk);
             const bool full = inner && i0 + R - 1 + w0g + cnt - 1 <= e_hi;
             bool scan = any;
-            if (w0g >= kPruneW) {
+            if (w0g >= prune_w<S>()) {
                 // the smallest merged maximum over the group's widths
                 int thr = (!(lane & 1) && jl < cnt) ? bv : INT_MAX;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) thr = min(thr, __shfl_xor_sync(0xffffffffu, thr, o));
-                if (full && group_bound(x, q, pmin, w0g, cnt) < (long long)thr) scan = false;
+                if (full && group_bound<S>(x, q, pmin, w0g, cnt) < (long long)thr) scan = false;
             }
             if (__any_sync(0xffffffffu, scan)) {
                 int seg[G];
 #pragma unroll
                 for (int j = 0; j < G; ++j) seg[j] = INT_MIN;
                 if (scan && full)
-                    scan_segment<true>(x, q, w0g, i0, i_lo, i_hi, e_hi, seg);
+                    scan_segment<true, S>(x, q, w0g, i0, i_lo, i_hi, e_hi, seg);
                 else if (scan)
-                    scan_segment<false>(x, q, w0g, i0, i_lo, i_hi, e_hi, seg);
+                    scan_segment<false, S>(x, q, w0g, i0, i_lo, i_hi, e_hi, seg);
                 const int mx = warp_max16(seg, lane);
                 const bool better = !(lane & 1) && jl < cnt && mx > INT_MIN &&
                                     (mx > bv || (mx == bv && t_lo < bt));
                 // widths whose maximum beats (or ties from an earlier start) the merged one:
                 // the earliest segment holding it writes its prefix values to the warp's
-                // scratch, and the lanes test one start each for every such width that this
+                // scratch, and the lanes test the starts for every such width that this
                 // segment holds first
                 unsigned need = __ballot_sync(0xffffffffu, better);
                 auto holder = [&](int hl) {  // earliest lane whose segment holds width hl / 2's maximum
@@ -173,7 +175,7 @@ __device__ __forceinline__ void scan_row(const FusedArgs& f, const int* row, uin
                     const int h = holder(__ffs(need) - 1);
                     if (lane == h) {
                         uint32_t P = 0;
-                        for (int kk = 0; kk <= w0g + 45; ++kk) {
+                        for (int kk = 0; kk <= w0g + R + G - 2; ++kk) {
                             if (kk < R) chain[kk] = P;
                             if (kk >= w0g) chain[R + kk - w0g] = P;
                             P += (uint32_t)x[kk];
@@ -186,12 +188,17 @@ __device__ __forceinline__ void scan_row(const FusedArgs& f, const int* row, uin
                         if (holder(hl) != h) continue;  // held first by another segment: a later round
                         const int j = hl >> 1;
                         const int mj = __shfl_sync(0xffffffffu, mx, hl);
-                        const int i = ih + lane;
-                        const bool eq = lane < R && i >= i_lo && i < i_hi && i + w0g + j <= e_hi &&
-                                        (int)(chain[R + lane + j] - chain[lane]) == mj;
-                        const unsigned st = __ballot_sync(0xffffffffu, eq);
-                        if (lane == 0 && st)
-                            atomicMax(keyrow + g * G + j, fused_key(mj, (int)(T0 - C) + ih + __ffs(st) - 1));
+                        int at = -1;  // the earliest start of the segment that reaches it
+#pragma unroll
+                        for (int s0 = 0; s0 < R; s0 += 32) {
+                            const int sl = s0 + lane, i = ih + sl;
+                            const bool eq = sl < R && i >= i_lo && i < i_hi && i + w0g + j <= e_hi &&
+                                            (int)(chain[R + sl + j] - chain[sl]) == mj;
+                            const unsigned st = __ballot_sync(0xffffffffu, eq);
+                            if (at < 0 && st) at = s0 + __ffs(st) - 1;
+                        }
+                        if (lane == 0 && at >= 0)
+                            atomicMax(keyrow + g * G + j, fused_key(mj, (int)(T0 - C) + ih + at));
                         need &= ~(1u << hl);
                     }
                     __syncwarp();  // the scratch is rewritten for the next holder
@@ -274,13 +281,12 @@ __device__ __forceinline__ void epilogue(const DedispArgs& a, const FusedArgs& f
             if (last && ft.seam_out)
                 for (int k = lane; k < C; k += 32) ft.seam_out[2 * cb + k] = row[e_hi - C + k];
         }
-        scan_row(f, row, chain, f.key + (int64_t)du * f.nw, T0, C, chunk, a.nch, lane, i_lo, i_hi, e_hi);
+        scan_row<kRInt>(f, row, chain, f.key + (int64_t)du * f.nw, T0, C, chunk, a.nch, lane, i_lo, i_hi, e_hi);
     }
     // the next tile's bulk copies overwrite the rows
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     __syncthreads();
 }
-
 
 // ----------------------------------------------------------------------------- fp32 plans
 //
@@ -436,45 +442,37 @@ __device__ __forceinline__ void scan_row_f32(int w0, int nw, const float* row, f
     }
 }
 
-// Carries, seams and the scan of a warp group's two trial rows (rows[u], trial d + u).
+// Carries, seams and the scan of one trial's row (`sub` of the nsub warps that share it).
 // Not inlined: its registers are then allocated apart from the channel sums', which
-// keep the whole register file (the call comes once per tile).
-__device__ __noinline__ void scan_pair_rows_f32(float* rows, float* chain, int rowlen, int w0, int nw, int C,
-                                                int L, unsigned long long* key, int ndm, int d, int cb0,
-                                                int chunk, int nch, int lane, int64_t base, int64_t m_lo,
-                                                int64_t m_hi, int e_hi, bool first, bool last,
-                                                float* carry, float* seam_in, float* seam_out) {
-    for (int u = 0; u < 2; ++u) {
-        const int du = d + u;
-        if (du >= ndm) break;
-        float* row = rows + u * rowlen;
-        const int64_t cb = (int64_t)(cb0 + u) * C;  // this trial's carry and seam rows
-        if (chunk == 0) {
-            if (!last)
-                for (int k = lane; k < C; k += 32) carry[cb + k] = row[L + k];
-            if (first && seam_in)
-                for (int k = lane; k < C; k += 32) seam_in[2 * cb + C + k] = row[C + k];
-            if (last && seam_out)
-                for (int k = lane; k < C; k += 32) seam_out[2 * cb + k] = row[e_hi - C + k];
-        }
-        scan_row_f32(w0, nw, row, chain, key + (int64_t)du * nw, base, chunk, nch, lane, m_lo, m_hi, e_hi);
+// keep the whole register file (the calls come once per tile and row).
+__device__ __noinline__ void scan_trial_f32(float* row, float* chain, int w0, int nw, int C, int L,
+                                            unsigned long long* keyrow, int64_t cb, int sub, int nsub, int lane,
+                                            int64_t base, int64_t m_lo, int64_t m_hi, int e_hi, bool first,
+                                            bool last, float* carry, float* seam_in, float* seam_out) {
+    if (sub == 0) {
+        if (!last)
+            for (int k = lane; k < C; k += 32) carry[cb + k] = row[L + k];
+        if (first && seam_in)
+            for (int k = lane; k < C; k += 32) seam_in[2 * cb + C + k] = row[C + k];
+        if (last && seam_out)
+            for (int k = lane; k < C; k += 32) seam_out[2 * cb + k] = row[e_hi - C + k];
     }
+    scan_row_f32(w0, nw, row, chain, keyrow, base, sub, nsub, lane, m_lo, m_hi, e_hi);
 }
 
-// The fused epilogue of one fp32 pair tile (every thread of the CTA calls it): the warp
-// group's two trials d, d + 1 (sums acc0, acc1), T0 = the tile's first output; one row
-// per trial.  The tile owns the segments whose first start lies in [T0 - C, T0 + L - C)
-// (the strip's first tile: from T0; its last: up to the strip end S1, windows ending at
-// or before S1).
-template <int R>
+// The fused epilogue of one fp32 tile (every thread of the CTA calls it): the warp group's
+// NT trials d .. d + NT - 1 (sums acc[u]), T0 = the tile's first output; one row per trial.
+// The tile owns the segments whose first start lies in [T0 - C, T0 + L - C) (the strip's
+// first tile: from T0; its last: up to the strip end S1, windows ending at or before S1).
+// NW warps per CTA.  f.one_row: one row per warp group, its other trials' sums wait in
+// shared memory.
+template <int NT, int R, int NW = kWarps>
 __device__ __forceinline__ void epilogue_f32(const DedispArgs& a, const FusedArgs& f, unsigned char* smem,
                                              int wu, int chunk, int lane, int d, int64_t T0,
-                                             const FusedTile& ft, const float (&acc0)[R],
-                                             const float (&acc1)[R]) {
+                                             const FusedTile& ft, const float (&acc)[NT][R]) {
     constexpr int S = kBoxSeg, TT = 32 * R;
     const int L = TT * a.nch;
     const int C = f.C;
-    float* rows = (float*)smem + 2 * wu * f.rowlen;
     const int64_t S1 = ft.s1;
     const bool first = ft.first, last = ft.last;
     const int64_t base = T0 - C;  // output of row index 0
@@ -483,21 +481,52 @@ __device__ __forceinline__ void epilogue_f32(const DedispArgs& a, const FusedArg
     const int64_t m_lo = (t_lo + S - 1) / S, m_hi = (t_hi + S - 1) / S;
     float* carry = (float*)ft.carry;
     const int ib = C + chunk * TT + lane * R;
+    const int warp = threadIdx.x >> 5;
+    // a trial's row behind its carry
+    auto carry_in = [&](int u, float* row) {
+        if (d + u < a.ndm && chunk == 0 && !first)
+            for (int k = lane; k < C; k += 32) row[k] = carry[(int64_t)(wu * NT + u) * C + k];
+    };
+    auto scan = [&](int u, float* row, float* chain) {
+        if (d + u < a.ndm)
+            scan_trial_f32(row, chain, f.w0, f.nw, C, L, f.key + (int64_t)(d + u) * f.nw, (int64_t)(wu * NT + u) * C,
+                           chunk, a.nch, lane, base, m_lo, m_hi, e_hi, first, last, carry, (float*)ft.seam_in,
+                           (float*)ft.seam_out);
+    };
+    auto off = [&](int u) { return d + u < a.ndm ? (float)f.off[d + u] : 0.f; };
+    if (!f.one_row) {
+        float* rows = (float*)smem + NT * wu * f.rowlen;
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const bool live = d + u < a.ndm;
-        const float o = live ? (float)f.off[d + u] : 0.f;
-        float* row = rows + u * f.rowlen;
+        for (int u = 0; u < NT; ++u) {
+            const float o = off(u);
 #pragma unroll
-        for (int r = 0; r < R; ++r) row[ib + r] = (u == 0 ? acc0[r] : acc1[r]) - o;
-        if (live && chunk == 0 && !first)
-            for (int k = lane; k < C; k += 32) row[k] = carry[(int64_t)(wu * 2 + u) * C + k];
+            for (int r = 0; r < R; ++r) rows[u * f.rowlen + ib + r] = acc[u][r] - o;
+            carry_in(u, rows + u * f.rowlen);
+        }
+        __syncthreads();  // the rows and their carries are complete
+        float* chain = (float*)smem + fused_rows_ints(NT * NW / a.nch, f.rowlen, C) + warp * kChainFloats;
+        for (int u = 0; u < NT; ++u) scan(u, rows + u * f.rowlen, chain);
+    } else {
+        float* row = (float*)smem + wu * f.rowlen;
+        float* pad = (float*)smem + NW / a.nch * f.rowlen;
+        float* chain = pad + warp * kChainFloats;
+        float* wait = pad + max(C + 48, NW * kChainFloats) + warp * (NT - 1) * TT + lane * R;
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            const float o = off(u);
+#pragma unroll
+            for (int r = 0; r < R; ++r) *(u == 0 ? row + ib + r : wait + (u - 1) * TT + r) = acc[u][r] - o;
+        }
+        for (int u = 0; u < NT; ++u) {
+            if (u) {
+                __syncthreads();  // the row is free
+                for (int r = 0; r < R; ++r) row[ib + r] = wait[(u - 1) * TT + r];
+            }
+            carry_in(u, row);
+            __syncthreads();
+            scan(u, row, chain);
+        }
     }
-    __syncthreads();  // the rows and their carries are complete
-    // the warp's chain scratch lies behind the rows
-    float* chain = (float*)smem + fused_rows_ints(2 * kWarps / a.nch, f.rowlen, C) + (threadIdx.x >> 5) * kChainFloats;
-    scan_pair_rows_f32(rows, chain, f.rowlen, f.w0, f.nw, C, L, f.key, a.ndm, d, wu * 2, chunk, a.nch, lane,
-                       base, m_lo, m_hi, e_hi, first, last, carry, (float*)ft.seam_in, (float*)ft.seam_out);
     // the next tile's bulk copies overwrite the rows
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     __syncthreads();

@@ -40,6 +40,51 @@ constexpr int kSmemBudget = 110 * 1024;    // dynamic shared memory per CTA (two
 constexpr int kSmemBudgetOne = 220 * 1024; // fallback: one CTA per SM
 constexpr long long kWaitNs = 2000000000;  // bound on any device-side barrier wait
 
+// Row kernels (dd_rows.cuh): tap sums that the trials of a CTA share are formed once per
+// tile in shared memory.  A warp unit sums row_unit_trials trials: lane l owns kRFir
+// consecutive outputs (fp32), or kRPk consecutive words of two outputs kPkHalf apart (packed
+// integer sums).  The odd counts keep lane-strided loads free of bank conflicts.
+enum RowKind { kRowsNone = 0, kRowsFir = 1, kRowsU8 = 2, kRowsRl = 3 };
+constexpr int kRFir = kRPair;
+constexpr int kRPk = 17;
+constexpr int kPkHalf = 32 * kRPk;
+constexpr int kPkMaxTaps = 257;            // 255 n <= 65535: a run's sum fits a half word
+constexpr int kRowWarps = 16;              // warps per CTA (kWarps where 16 leave SMs idle)
+constexpr int kRowCsMax = 28;              // channels per stage (a warp's lanes issue the copies)
+__host__ __device__ constexpr int row_warp_t(int kind) { return kind == kRowsFir ? 32 * kRFir : 2 * kPkHalf; }
+__host__ __device__ constexpr int row_tile_t(int kind, int nch) { return nch * row_warp_t(kind); }
+__host__ __device__ constexpr int row_unit_trials(int kind) { return kind == kRowsFir ? 3 : 2; }
+__host__ __device__ constexpr int row_trials(int kind, int nw, int nch) { return row_unit_trials(kind) * nw / nch; }
+// Words of a row that a trial's sums read from its start on.
+__host__ __device__ constexpr int row_span(int kind, int nch) {
+    return kind == kRowsFir ? row_tile_t(kind, nch) : (nch - 1) * 2 * kPkHalf + kPkHalf;
+}
+// Stage record of a row kernel: a header (rows of the stage; bit ci: packed sums are moved
+// into 32-bit ones after channel ci; the longest row), an entry per unit and channel (each
+// trial's row position in the stage's row area: trials 0 and 1 as the half words of the first
+// word, trial 2 the second), a descriptor per row (offset of its samples in the
+// staged rows, its position in the row area, its length, taps | offset of its weights
+// << 16), and the rows' weights.  The header and entries are copied beside the rows.
+struct RowGeom {
+    int ent_bytes, desc_off, w_off, rec_bytes;
+    __host__ __device__ RowGeom(int cs, int nu, int rows_max, int kw) {
+        ent_bytes = (16 + 8 * nu * cs + 8 + 15) & ~15;  // (one entry is read ahead)
+        desc_off = ent_bytes;
+        w_off = desc_off + 16 * rows_max;
+        rec_bytes = (w_off + 4 * kw + 15) & ~15;
+    }
+};
+// Shared memory of a row launch: the raw buffer and record, the block's table (lo_ld words),
+// two row halves, the barrier; at least the output transpose.
+__host__ __device__ inline size_t row_smem_bytes(const RowGeom& g, int nw, int esz, int lcap, int cs, int lo_ld,
+                                                 int area) {
+    const size_t tail = 8 + 2 * 4;
+    const size_t all = (((size_t)cs * lcap * esz + g.rec_bytes + 127) & ~(size_t)127) +
+                       ((4 * (size_t)lo_ld + 15) & ~(size_t)15) + 2 * ((size_t)area * 4 + g.ent_bytes) + tail;
+    const size_t st = (size_t)nw * 2 * kPkHalf * 4 + tail;
+    return ((all > st ? all : st) + 15) & ~(size_t)15;
+}
+
 // Byte layout of one dedispersion pipeline stage in shared memory: cs staged input
 // rows of lcap elements, then the stage's profile record.  The record holds, for each
 // of the CTA's nu warp units and each of the stage's channels, an entry (window start
@@ -96,6 +141,11 @@ struct DedispArgs {
     int32_t cs;   // channels per stage
     int32_t nch;  // time chunks per CTA (trials per CTA = kWarps / nch)
     int32_t kpad;  // weight pairs per stage record (pair path)
+    int32_t lo_ld;     // row kernels: words per block of blk_lo ([nchan] minimum delays, the
+                       // number of stages, their first channels and the end)
+    int32_t nst;       // row kernels: records per block
+    int32_t rows_max;  // row kernels: row descriptors per stage record (kpad: its weights,
+                       // blen: words of a half's row area)
     int32_t nsplit;    // channel-sum splits (grid z); split z writes out + z * split_ld
     int64_t split_ld;
     int32_t* status;
@@ -126,6 +176,8 @@ struct FusedArgs {
     const int64_t* order;     // [nparts] part taken by CTA i: parts sorted by their first
                               // time tile, so that CTAs resident together read the same
                               // input columns (shared in L2)
+    int32_t one_row;          // fp32 plans: a warp group has one shared-memory row, which its
+                              // trials use one after the other (their rows do not all fit)
     const double* off;        // [ndm] per-trial offsets (integer valued on integer plans)
     unsigned long long* key;  // [ndm][nw]
     int32_t* carry;     // [nparts][trials per CTA][C] (fp32 plans: float bits)
@@ -218,11 +270,12 @@ struct dd_plan_s {
     bool pair = true;                  // fp32 path: each warp sums two adjacent trials
     int32_t kw = 0;                    // weight pairs per stage record (pair path)
     int32_t umax = 0;                  // most taps of a pair unit, max(n0, n1) (pair path)
-    std::vector<unsigned char> rec;    // host copy of the records
-    bool rec_from_dev_w = false;       // records' weights come from dev.w (device weights)
+    std::vector<unsigned char> rec;    // host copy of the records, rec_host bytes of each (all,
+    int32_t rec_host = 0;              // or what precedes weights that the device fills in)
     int32_t debug_skip_stage = -1;     // test hook: a stage whose bulk copies are never issued
     int64_t wait_ns = dd::kWaitNs;
     bool dev_dirty = true;
+    uint64_t dev_gen = 0;              // the upload that made the device tables
     dd::DevTables dev;
     std::vector<int32_t> widths_on_dev;  // widths last copied to dev.widths
     // adjoint workspace, built on the first dd_backward: the transposed plan (output rows
@@ -244,6 +297,12 @@ struct dd_plan_s {
     int32_t blen = 0;                  // their stride (words)
     uint32_t* d_prefix = nullptr;
     int64_t prefix_elems = 0;
+    // row kernels (RowKind): the schedule above is then theirs
+    int32_t rk = 0;
+    int32_t rows_max = 0;
+    int32_t row_warps = 0, lo_ld = 0, nst = 0;
+    bool w_dev = false;                // weights come from the device (host copy is not theirs)
+    bool w_follows = false;            // a device copy of the weights follows every upload
     // fused dedispersion + boxcar scratch: merged maxima, per-CTA carries, strip seams
     unsigned long long* d_fkey = nullptr;
     int64_t fkey_elems = 0;
@@ -274,6 +333,21 @@ int dedisp_batched_blocks_per_sm(bool u8, bool pair, bool short_taps, size_t sme
 dd_status launch_prefix_into(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                              int64_t nsamp, uint32_t* P, int64_t ldp, cudaStream_t s);
 dd_status cuda_status(cudaError_t e);
+// Outputs per CTA tile and trials per CTA of the plan's schedule.
+inline int plan_tile_t(const dd_plan_s* p) {
+    return p->rk ? row_tile_t(p->rk, p->nch) : chunk_t(p->pair) * p->nch;
+}
+inline int plan_trials(const dd_plan_s* p) {
+    return p->rk ? row_trials(p->rk, p->row_warps, p->nch) : kWarps / p->nch * (p->rl ? kRlUnits : 1) * (p->pair ? 2 : 1);
+}
+// row kernels (dd_rows.cu, dd_rows_fused.cu): shared memory, launches, CTAs per SM
+size_t rows_smem_for(const dd_plan_s* p);
+dd_status launch_rows(const dd_plan_s* p, DedispArgs a, cudaStream_t s);
+dd_status launch_rows_batched(int kind, bool in8, int nw, const DedispArgs* d_args, const BatchItem* d_items,
+                              int32_t nitems, size_t smem, cudaStream_t s);
+int rows_batched_blocks_per_sm(int kind, bool in8, int nw, size_t smem);
+dd_status launch_rows_fused(const dd_plan_s* p, DedispArgs a, const FusedArgs& f, size_t smem, cudaStream_t s);
+int rows_fused_blocks_per_sm(const dd_plan_s* p, size_t smem);
 
 // launchers (stream = cudaStream_t)
 dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
@@ -296,7 +370,8 @@ dd_status launch_norm(dd_plan_s* p, const int32_t* widths, int32_t nw, const dou
                       const double* sd, cudaStream_t s);
 // fused dedispersion + boxcar: dynamic shared memory of the launch (stages, or the scan
 // rows plus the pipeline barriers, whichever is larger), its CTAs per SM, and the launch
-size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C);
+size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C, bool one_row = false);
+constexpr size_t kSmemMax = 227 * 1024;    // dynamic shared memory a CTA can have
 int fused_blocks_per_sm(const dd_plan_s* p, size_t smem);
 dd_status launch_dedisperse_fused(const dd_plan_s* p, DedispArgs a, const FusedArgs& f, size_t smem,
                                   cudaStream_t s);

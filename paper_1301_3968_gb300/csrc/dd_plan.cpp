@@ -2,6 +2,7 @@
 // trial-DM rule (eq. trial DMs, Sec. 6.3), argument checking and the dedispersion
 // schedule (trial blocks and staged window lengths).
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <cstdio>
 #include <cstdarg>
@@ -13,6 +14,8 @@
 #include <new>
 #include <sstream>
 #include <string>
+#include <system_error>
+#include <thread>
 
 #include "dd_internal.h"
 #include "dd_trace.h"
@@ -56,14 +59,49 @@ void build_trials(const dd_band& b, double dm0, double eps, int n, double extra2
     }
 }
 
+// Runs fn(b) for the blocks 0 .. n - 1 on a few threads when there is enough work
+// (entries: table entries touched); on this thread alone where threads cannot be had.
+template <typename F>
+void for_blocks(int n, size_t entries, F fn) {
+    // (a thread costs about what 6 x 10^4 entries do)
+    const int nt = (int)std::min<size_t>(std::min<size_t>(8, std::max(1u, std::thread::hardware_concurrency())),
+                                         std::max<size_t>(1, entries >> 16));
+    std::vector<std::thread> th;
+    int started = 1;
+    if (nt > 1) {
+        th.reserve(nt);
+        try {
+            for (; started < nt; ++started)
+                th.emplace_back([&fn, n, nt, started] {
+                    for (int b = started; b < n; b += nt) fn(b);
+                });
+        } catch (const std::system_error&) {
+        }
+    }
+    for (int b = 0; b < n; b += nt) fn(b);
+    for (int k = started; k < nt; ++k)
+        for (int b = k; b < n; b += nt) fn(b);
+    for (auto& t : th) t.join();
+}
+
+// The largest fn(b) over the blocks (at least 0).
+template <typename F>
+int64_t max_blocks(int n, size_t entries, F fn) {
+    std::vector<int64_t> m((size_t)n, 0);
+    for_blocks(n, entries, [&](int b) { m[b] = fn(b); });
+    int64_t r = 0;
+    for (int64_t v : m) r = std::max(r, v);
+    return r;
+}
+
 // Span of the staged window when `db` consecutive trials share a CTA: the largest
 // max(delta + n) - min(delta) over blocks and channels.
 int64_t block_span(const dd_plan_s* p, int db, std::vector<int32_t>* lo_out) {
     const int C = p->nchan;
     const int nblk = (p->ndm + db - 1) / db;
     if (lo_out) lo_out->assign((size_t)nblk * C, 0);
-    int64_t span = 0;
-    for (int b = 0; b < nblk; ++b) {
+    return max_blocks(nblk, (size_t)p->ndm * C, [&](int b) {
+        int64_t span = 0;
         for (int c = 0; c < C; ++c) {
             int64_t lo = INT64_MAX, hi = 0;
             for (int i = 0; i < db; ++i) {
@@ -76,8 +114,8 @@ int64_t block_span(const dd_plan_s* p, int db, std::vector<int32_t>* lo_out) {
             if (lo_out) (*lo_out)[(size_t)b * C + c] = (int32_t)lo;
             span = std::max(span, hi - lo);
         }
-    }
-    return span;
+        return span;
+    });
 }
 
 // Trials per warp unit: two adjacent trials share one register window on the fp32
@@ -123,8 +161,8 @@ int32_t pair_taps(const dd_plan_s* p) {
 int32_t pair_record_pairs(const dd_plan_s* p, int db, int cs) {
     const int C = p->nchan;
     const int nblk = (p->ndm + db - 1) / db;
-    int64_t most = 0;
-    for (int b = 0; b < nblk; ++b)
+    const int64_t most = max_blocks(nblk, (size_t)p->ndm * C, [&](int b) {
+        int64_t top = 0;
         for (int c0 = 0; c0 < C; c0 += cs) {
             int64_t tot = 0;
             for (int d0 = b * db; d0 < std::min(p->ndm, (b + 1) * db); d0 += 2)
@@ -134,8 +172,10 @@ int32_t pair_record_pairs(const dd_plan_s* p, int db, int cs) {
                     if (d0 + 1 < p->ndm) n = std::max<int64_t>(n, p->taps[a + C]);
                     tot += n;
                 }
-            most = std::max(most, tot);
+            top = std::max(top, tot);
         }
+        return top;
+    });
     return (int32_t)std::min<int64_t>((most + 1) & ~(int64_t)1, INT32_MAX);
 }
 
@@ -146,8 +186,8 @@ int32_t pair_record_pairs(const dd_plan_s* p, int db, int cs) {
 int64_t pair_read_span(const dd_plan_s* p, int db) {
     const int C = p->nchan;
     const int nblk = (p->ndm + db - 1) / db;
-    int64_t span = 0;
-    for (int b = 0; b < nblk; ++b)
+    return max_blocks(nblk, (size_t)p->ndm * C, [&](int b) {
+        int64_t span = 0;
         for (int c = 0; c < C; ++c) {
             int64_t lo = INT64_MAX;
             for (int d = b * db; d < std::min(p->ndm, (b + 1) * db); ++d)
@@ -163,7 +203,8 @@ int64_t pair_read_span(const dd_plan_s* p, int db) {
                 span = std::max(span, st + n - lo);
             }
         }
-    return span;
+        return span;
+    });
 }
 
 // Most distinct tap counts among one trial block's trials on any channel (run-length
@@ -235,10 +276,12 @@ void build_records(dd_plan_s* p) {
     const int kw = p->pair ? p->kw : 0;
     const dd::StageGeom g(stage_esz(p), p->pair, p->lcap, kw, p->cs, nu, p->rl_b, p->blen);
     p->rec_bytes = g.rec_bytes;
-    p->rec.assign((size_t)p->nblk * nst * g.rec_bytes, 0);
-    for (int b = 0; b < p->nblk; ++b)
+    // without the weights where a device copy of them follows
+    p->rec_host = p->w_follows ? g.w_off : g.rec_bytes;
+    p->rec.assign((size_t)p->nblk * nst * p->rec_host, 0);
+    for_blocks(p->nblk, (size_t)p->ndm * C, [&](int b) {
         for (int st = 0; st < nst; ++st) {
-            unsigned char* r = p->rec.data() + ((size_t)b * nst + st) * g.rec_bytes;
+            unsigned char* r = p->rec.data() + ((size_t)b * nst + st) * p->rec_host;
             int32_t* ent = (int32_t*)r;
             float* w = (float*)(r + g.w_off);
             // difference rows: (n0, n1, len0, len1) per channel
@@ -278,7 +321,7 @@ void build_records(dd_plan_s* p) {
                         ent[4 * e + 1] = n;
                         ent[4 * e + 2] = two ? p->delay[a1] - p->delay[a0] : 0;
                         ent[4 * e + 3] = woff;
-                        for (int i = 0; i < 2; ++i) {
+                        for (int i = 0; i < 2 && !p->w_follows; ++i) {
                             if (i == 1 && !two) break;
                             const size_t dc = i ? a1 : a0;
                             for (int k = 0; k < p->taps[dc]; ++k)
@@ -299,12 +342,260 @@ void build_records(dd_plan_s* p) {
                     if (p->rl_b) ent[2 * e + 1] = (hi - lo) == nlist[4 * ci] ? 0 : 1;
                 }
         }
+    });
+}
+
+// ----------------------------------------------------------------------- row schedule
+
+// One distinct tap run of a (trial block, channel): its taps and weights are those of
+// `trial`, its furthest start in the block `reach` past the block's minimum delay.
+struct Row {
+    int32_t n, trial, reach;
+};
+
+// The plan's row kind, if its sums can be formed that way: fp32 sums with weights that
+// the host knows.
+int row_kind_of(const dd_plan_s* p) {
+    if (p->pair) return p->w_dev || p->kmax > 0xffff ? dd::kRowsNone : dd::kRowsFir;
+    return dd::kRowsNone;
+}
+
+// Rows pay up to this many distinct runs per (trial, channel).
+constexpr double kRowsMaxShare = 0.5;
+
+// Warps per CTA of the row kernels.  16 (one CTA per SM) form a stage's rows for twice the
+// trials of 8 (two CTAs per SM), which measured 12 % faster on a long launch (CRAFT-like,
+// 512 trials: 1.08 against 1.22 ms), but leave more of a short launch's last wave idle: the
+// share of the waves' slots that the plan's block fills decides, on 152 SMs.
+int row_warps_of(const dd_plan_s* p, int kind, int nch) {
+    const int64_t tile = dd::row_tile_t(kind, nch);
+    const int64_t tiles = (std::max<int64_t>(1, p->band.nsamp - p->dmax) + tile - 1) / tile;
+    auto fill = [&](int nw, int64_t slots) {
+        const int db = dd::row_trials(kind, nw, nch);
+        const int64_t n = tiles * ((p->ndm + db - 1) / db);
+        return (double)p->ndm / db * tiles / (double)((n + slots - 1) / slots * slots);
+    };
+    return 1.12 * fill(dd::kRowWarps, 152) >= fill(dd::kWarps, 304) ? dd::kRowWarps : dd::kWarps;
+}
+
+// The schedule and records of the row kernels (layout: RowGeom) for nch time chunks and at
+// most cs_fixed channels per stage (0: what gives the fewest stages).  Leaves the plan as it
+// is and returns false where rows do not fit or pay.
+bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
+    const int kind = row_kind_of(p);
+    if (kind == dd::kRowsNone) return false;
+    const double units = (double)p->ndm * p->nchan;
+    const int C = p->nchan;
+    const int nw = row_warps_of(p, kind, nch);
+    const int db = dd::row_trials(kind, nw, nch), nt = dd::row_unit_trials(kind), nu = db / nt;
+    const int nblk = (p->ndm + db - 1) / db;
+    const int esz = stage_esz(p), Q = 16 / esz;
+    const int span = dd::row_span(kind, nch);
+    const bool fir = kind == dd::kRowsFir;
+    auto same = [&](size_t a, size_t b) {
+        if (p->taps[a] != p->taps[b]) return false;
+        return p->unit || std::memcmp(&p->w[a * p->kpad], &p->w[b * p->kpad], (size_t)p->taps[a] * sizeof(float)) == 0;
+    };
+    // the distinct runs of every (block, channel), and each trial's
+    std::vector<std::vector<Row>> rows(nblk);
+    std::vector<std::vector<int32_t>> first(nblk);  // [C + 1] into rows[b]
+    std::vector<uint8_t> rid((size_t)p->ndm * C);
+    std::vector<int32_t> lo((size_t)nblk * C);
+    for_blocks(nblk, (size_t)p->ndm * C, [&](int b) {
+        const int d0 = b * db, d1 = std::min(p->ndm, d0 + db);
+        first[b].resize(C + 1);
+        rows[b].reserve((size_t)C * 2);
+        for (int c = 0; c < C; ++c) {
+            const size_t f = rows[b].size();
+            first[b][c] = (int32_t)f;
+            int32_t l = INT32_MAX;
+            for (int d = d0; d < d1; ++d) l = std::min(l, p->delay[(size_t)d * C + c]);
+            lo[(size_t)b * C + c] = l;
+            size_t hint = f;
+            for (int d = d0; d < d1; ++d) {
+                const size_t dc = (size_t)d * C + c;
+                size_t r = hint;
+                if (r >= rows[b].size() || !same(dc, (size_t)rows[b][r].trial * C + c))
+                    for (r = f; r < rows[b].size(); ++r)
+                        if (r != hint && same(dc, (size_t)rows[b][r].trial * C + c)) break;
+                if (r == rows[b].size()) rows[b].push_back({p->taps[dc], d, 0});
+                rows[b][r].reach = std::max(rows[b][r].reach, p->delay[dc] - l);
+                rid[dc] = (uint8_t)(r - f);
+                hint = r;
+            }
+        }
+        first[b][C] = (int32_t)rows[b].size();
+    });
+    auto len_of = [&](const Row& r) { return (int64_t)((Q - 1 + r.reach + span + 3) & ~3); };
+    size_t total = 0;
+    int64_t need = 0;
+    // the fullest single channel: rows, weights (each row's padded to four), row words
+    int64_t one_r = 1, one_w = 0, one_a = 0;
+    for (int b = 0; b < nblk; ++b) {
+        total += rows[b].size();
+        for (int c = 0; c < C; ++c) {
+            int64_t w = 0, ar = 0;
+            for (int r = first[b][c]; r < first[b][c + 1]; ++r) {
+                w += (rows[b][r].n + 3) & ~3;
+                ar += len_of(rows[b][r]);
+                // samples that building the row reads (dd_rows.cuh)
+                need = std::max(need, len_of(rows[b][r]) + (rows[b][r].n & ~3) + 4);
+            }
+            one_r = std::max<int64_t>(one_r, first[b][c + 1] - first[b][c]);
+            one_w = std::max(one_w, w);
+            one_a = std::max(one_a, ar);
+        }
+    }
+    if ((double)total > kRowsMaxShare * units) return false;
+    const int64_t lcap = (need + Q - 1) / Q * Q;
+    if (lcap > (1 << 20) || one_w > 0xffff || !fir) return false;
+    // Stages: channels in order, as many as the limits on channels (cs), rows, weights and
+    // row words allow.
+    struct Cut {
+        int cs = 0, nst = 0;  // nst: most stages of a block
+        int64_t rmax = 1, wmax = 0, area = 0, total = 0;
+        std::vector<std::vector<int32_t>> start;  // per block: first channels, and the end
+    };
+    auto cut = [&](int cs, int64_t rlim, int64_t wlim, int64_t alim, bool keep) {
+        Cut k;
+        k.cs = cs;
+        if (keep) k.start.resize(nblk);
+        for (int b = 0; b < nblk; ++b) {
+            int n = 0;
+            int64_t w = 0, ar = 0, r = 0, ch = 0;
+            for (int c = 0; c < C; ++c) {
+                int64_t cw = 0, ca = 0;
+                const int64_t cr = first[b][c + 1] - first[b][c];
+                for (int i = first[b][c]; i < first[b][c + 1]; ++i) {
+                    cw += (rows[b][i].n + 3) & ~3;
+                    ca += len_of(rows[b][i]);
+                }
+                if (c == 0 || ch == cs || r + cr > rlim || w + cw > wlim || ar + ca > alim) {
+                    if (keep) k.start[b].push_back(c);
+                    ++n;
+                    w = ar = r = ch = 0;
+                }
+                w += cw;
+                ar += ca;
+                r += cr;
+                ++ch;
+                k.rmax = std::max(k.rmax, r);
+                k.wmax = std::max(k.wmax, w);
+                k.area = std::max(k.area, ar);
+            }
+            if (keep) k.start[b].push_back(C);
+            k.nst = std::max(k.nst, n);
+            k.total += n;
+        }
+        return k;
+    };
+    const size_t budget = cs_fixed > 0 || nw == dd::kRowWarps ? dd::kSmemBudgetOne : dd::kSmemBudget;
+    // limits for at most cs channels; false where a single channel does not fit
+    auto limits = [&](int cs, int64_t* rlim, int64_t* wlim, int64_t* alim) {
+        *rlim = std::max<int64_t>(one_r, 2 * cs);
+        *wlim = fir ? std::min<int64_t>(0xffff, std::max<int64_t>(one_w, (int64_t)cs * ((p->kmax + 3) & ~3) * 5 / 4)) : 0;
+        const dd::RowGeom g(cs, nu, (int)*rlim, (int)*wlim);
+        const size_t rest = dd::row_smem_bytes(g, 0, esz, (int)lcap, cs, 2 * C + 2, 16);
+        if (rest >= budget) return false;
+        *alim = (int64_t)((budget - rest) / 8) & ~(int64_t)3;
+        return *alim >= one_a;
+    };
+    Cut best;
+    int64_t rlim = 0, wlim = 0, alim = 0;
+    const int cs_hi = cs_fixed > 0 ? cs_fixed : dd::kRowCsMax, cs_lo = cs_fixed > 0 ? cs_fixed : 1;
+    for (int cs = std::min(cs_hi, dd::kRowCsMax); cs >= cs_lo; --cs) {
+        if (!limits(cs, &rlim, &wlim, &alim)) continue;
+        Cut k = cut(cs, rlim, wlim, alim, false);
+        if (best.cs == 0 || k.total < best.total) best = k;
+        else break;
+    }
+    if (best.cs == 0) return false;
+    const int cs = best.cs;
+    limits(cs, &rlim, &wlim, &alim);
+    best = cut(cs, rlim, wlim, alim, true);
+    const int nst = best.nst, lo_ld = C + nst + 2;
+    const int32_t area = (int32_t)best.area + 16;  // and what the last row's reads run past it
+    const dd::RowGeom g(cs, nu, (int)best.rmax, (int)best.wmax);
+    std::vector<unsigned char> rec((size_t)nblk * nst * g.rec_bytes, 0);
+    std::vector<int32_t> table((size_t)nblk * lo_ld, 0);
+    for_blocks(nblk, (size_t)p->ndm * C, [&](int b) {
+        int32_t* tb = table.data() + (size_t)b * lo_ld;
+        const int ns = (int)best.start[b].size() - 1;
+        std::copy(lo.begin() + (size_t)b * C, lo.begin() + (size_t)(b + 1) * C, tb);
+        tb[C] = ns;
+        std::copy(best.start[b].begin(), best.start[b].end(), tb + C + 1);
+        std::vector<int32_t> at;
+        for (int st = 0; st < ns; ++st) {
+            unsigned char* q = rec.data() + ((size_t)b * nst + st) * g.rec_bytes;
+            int32_t* hdr = (int32_t*)q;
+            int32_t* ent = (int32_t*)(q + 16);
+            int32_t* desc = (int32_t*)(q + g.desc_off);
+            float* w = (float*)(q + g.w_off);
+            const int c0 = best.start[b][st], c1 = best.start[b][st + 1];
+            const int r0 = first[b][c0];
+            hdr[0] = first[b][c1] - r0;
+            int32_t dst = 0, woff = 0;
+            at.assign((size_t)hdr[0], 0);
+            for (int c = c0; c < c1; ++c)
+                for (int r = first[b][c]; r < first[b][c + 1]; ++r) {
+                    const Row& row = rows[b][r];
+                    int32_t* ds = desc + 4 * (size_t)(r - r0);
+                    at[r - r0] = dst;
+                    ds[0] = (c - c0) * (int32_t)lcap;
+                    ds[1] = dst;
+                    ds[2] = Q - 1 + row.reach + span;
+                    ds[3] = (int32_t)((uint32_t)row.n | (uint32_t)woff << 16);
+                    hdr[2] = std::max(hdr[2], ds[2]);
+                    dst += (int32_t)len_of(row);
+                    if (!fir) continue;
+                    const size_t dc = (size_t)row.trial * C + c;
+                    for (int k = 0; k < row.n; ++k) w[woff + k] = p->unit ? 1.0f : p->w[dc * p->kpad + k];
+                    woff += (row.n + 3) & ~3;
+                }
+            for (int j = 0; j < nu; ++j)
+                for (int c = c0; c < c1; ++c) {
+                    int32_t pos[3] = {0, 0, 0};
+                    const int d0 = b * db + j * nt;
+                    if (d0 >= p->ndm) continue;
+                    for (int u = 0; u < nt; ++u) {
+                        // trials past the list's end add what the unit's last one does
+                        const size_t dc = (size_t)std::min(d0 + u, p->ndm - 1) * C + c;
+                        pos[u] = at[first[b][c] - r0 + rid[dc]] + p->delay[dc] - lo[(size_t)b * C + c];
+                    }
+                    int32_t* e = ent + 2 * (size_t)(j * cs + c - c0);
+                    e[0] = (int32_t)((uint32_t)pos[0] | (uint32_t)pos[1] << 16);
+                    e[1] = pos[2];
+                }
+        }
+    });
+    p->rk = kind;
+    p->row_warps = nw;
+    p->nch = nch;
+    p->cs = cs;
+    p->kw = (int32_t)best.wmax;
+    p->rows_max = (int32_t)best.rmax;
+    p->blen = area;
+    p->lcap = (int32_t)lcap;
+    p->nblk = nblk;
+    p->nst = nst;
+    p->lo_ld = lo_ld;
+    p->rec_bytes = p->rec_host = g.rec_bytes;
+    p->blk_lo.swap(table);
+    p->rec.swap(rec);
+    p->dev_dirty = true;
+    dd::log_msg(1, "plan %d trials x %d channels: shared rows (%.3f per trial and channel), %d trials and %d warps per "
+                "CTA, up to %d channels per stage (%.1f stages per block), staged rows of %d elements, row area of "
+                "%d words, record %d bytes, %zu bytes of shared memory", p->ndm, C, (double)total / units, db, nw, cs,
+                (double)best.total / nblk, p->lcap, p->blen, p->rec_bytes, dd::dedisp_smem_for(p));
+    return true;
 }
 
 // Chooses the CTA shape of the dedispersion kernel (warp units x time chunks), the
 // staged window length and the channels per pipeline stage.  The most trials per CTA
-// (the most reuse of each staged sample) whose window still fits is taken.
+// (the most reuse of each staged sample) whose window still fits is taken.  Where shared
+// rows fit that shape and pay, the row kernels take the plan.
 dd_status build_schedule(dd_plan_s* p) {
+    p->rk = dd::kRowsNone;
     const bool u8 = p->band.in_type == DD_U8;
     p->pair = !(u8 && p->unit);
     const double mean_taps = (double)p->ns_total / ((double)p->ndm * p->nchan);
@@ -330,15 +621,18 @@ dd_status build_schedule(dd_plan_s* p) {
             const int64_t need = staged_len(p, nch, span);
             if (need > (1 << 22)) continue;
             p->blen = p->rl_b ? brow_stride(p, db, nch) : 0;
+            auto fits = [&](int cs, int32_t kw) {
+                return dd::dedisp_smem_bytes(dd::StageGeom(esz, p->pair, (int)need, kw, cs, nu, p->rl_b, p->blen),
+                                             nbuf, p->nchan) <= budgets[pass];
+            };
+            if (!fits(min_cs[pass], p->pair ? pair_record_pairs(p, db, min_cs[pass]) : 0)) continue;
+            if (build_rows(p, nch, 0)) return DD_OK;
             int cs = cs_want;
             int32_t kw = p->pair ? pair_record_pairs(p, db, cs) : 0;
-            while (cs >= min_cs[pass] &&
-                   dd::dedisp_smem_bytes(dd::StageGeom(esz, p->pair, (int)need, kw, cs, nu, p->rl_b, p->blen),
-                                         nbuf, p->nchan) > budgets[pass]) {
+            while (cs > min_cs[pass] && !fits(cs, kw)) {
                 --cs;
-                if (p->pair && cs >= 1) kw = pair_record_pairs(p, db, cs);
+                if (p->pair) kw = pair_record_pairs(p, db, cs);
             }
-            if (cs < min_cs[pass]) continue;
             p->nch = nch;
             p->cs = cs;
             p->kw = kw;
@@ -378,8 +672,10 @@ dd_status build_schedule_fixed(dd_plan_s* p, int nch, int cs) {
     if (dd::dedisp_smem_bytes(dd::StageGeom(esz, p->pair, (int)need, kw, cs, nu, rl_b, blen), stages_of(p),
                               p->nchan) > dd::kSmemBudgetOne)
         return DD_ERR_UNSUPPORTED;
-    p->blen = blen;
+    p->rk = dd::kRowsNone;
     p->rl_b = rl_b;
+    if (build_rows(p, nch, cs)) return DD_OK;
+    p->blen = blen;
     p->nch = nch;
     p->cs = cs;
     p->kw = kw;
@@ -466,9 +762,9 @@ dd_status build_adjoint_plan(dd_plan_s* p) {
             t->taps[cd] = p->taps[dc];
         }
     t->unit = false;
+    t->w_dev = t->w_follows = true;  // filled on the device
     t->kpad = p->kpad;
     t->kuser = p->kuser;
-    t->w.assign((size_t)C * D * t->kpad, 0.0f);
     dd_status st = finish_profiles(t);
     if (st != DD_OK) {
         delete t;
@@ -545,20 +841,38 @@ void destroy_plan(dd_plan_s* p) {
     delete p;
 }
 
+// Numbers every upload, so that a batch sees when a plan's tables have moved.
+static std::atomic<uint64_t> g_dev_gen{0};
+
 dd_status upload_tables(dd_plan_s* p) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_status(e);
     if (!p->dev_dirty && p->dev.device == dev) return DD_OK;
+    if (p->rec_host != p->rec_bytes && !p->w_follows) build_records(p);  // with the host's weights
     free_dev(p);
     p->dev.device = dev;
     const size_t n = (size_t)p->ndm * p->nchan;
     dd_status st;
     if ((st = put(&p->dev.delay, p->delay.data(), n)) != DD_OK) return st;
     if ((st = put(&p->dev.taps, p->taps.data(), n)) != DD_OK) return st;
-    if (!p->unit && (st = put(&p->dev.w, p->w.data(), p->w.size())) != DD_OK) return st;
+    if (!p->unit && p->w_follows) {
+        e = cudaMalloc((void**)&p->dev.w, n * p->kpad * sizeof(float));
+        if (e != cudaSuccess) return cuda_status(e);
+    } else if (!p->unit && (st = put(&p->dev.w, p->w.data(), p->w.size())) != DD_OK) {
+        return st;
+    }
     if ((st = put(&p->dev.blk_lo, p->blk_lo.data(), p->blk_lo.size())) != DD_OK) return st;
-    if ((st = put(&p->dev.rec, p->rec.data(), p->rec.size())) != DD_OK) return st;
+    if (p->rec_host == p->rec_bytes) {
+        if ((st = put(&p->dev.rec, p->rec.data(), p->rec.size())) != DD_OK) return st;
+    } else {
+        const size_t nrec = p->rec.size() / p->rec_host;
+        e = cudaMalloc((void**)&p->dev.rec, nrec * p->rec_bytes);
+        if (e == cudaSuccess)
+            e = cudaMemcpy2D(p->dev.rec, p->rec_bytes, p->rec.data(), p->rec_host, p->rec_host, nrec,
+                             cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_status(e);
+    }
     const int32_t zero = 0;
     if ((st = put(&p->dev.status, &zero, 1)) != DD_OK) return st;
     e = cudaMalloc((void**)&p->dev.off, (size_t)p->ndm * sizeof(double));
@@ -567,6 +881,7 @@ dd_status upload_tables(dd_plan_s* p) {
     // that its calls allocate nothing (lazy module loading would do it at its first call)
     if ((st = noalloc_preload()) != DD_OK) return st;
     p->dev_dirty = false;
+    p->dev_gen = ++g_dev_gen;
     return DD_OK;
 }
 
@@ -677,7 +992,7 @@ dd_status dd_set_profiles(dd_plan_t p, const int32_t* delay, const int32_t* ntap
     std::vector<int32_t> old_d = p->delay, old_t = p->taps;
     std::vector<float> old_w = p->w;
     int32_t old_kpad = p->kpad, old_kuser = p->kuser;
-    bool old_unit = p->unit;
+    bool old_unit = p->unit, old_w_dev = p->w_dev;
     if (delay) std::memcpy(p->delay.data(), delay, n * sizeof(int32_t));
     if (ntaps) std::memcpy(p->taps.data(), ntaps, n * sizeof(int32_t));
     if (w) {
@@ -699,8 +1014,10 @@ dd_status dd_set_profiles(dd_plan_t p, const int32_t* delay, const int32_t* ntap
         p->kuser = 0;
         p->unit = true;
     }
+    p->w_dev = false;
     dd_status st = finish_profiles(p);
     if (st != DD_OK) {
+        p->w_dev = old_w_dev;
         p->delay = old_d;
         p->taps = old_t;
         p->w = old_w;
@@ -718,6 +1035,8 @@ dd_status dd_set_weights_device(dd_plan_t p, const float* d_w, int32_t kmax, voi
     if (!p || !d_w || kmax < 1) return DD_ERR_ARG;
     if (p->kmax > kmax) return DD_ERR_ARG;
     const int32_t kpad = (kmax + 3) / 4 * 4;
+    p->w_follows = true;  // tables built or uploaded here need no weights of the host's
+    dd_status st = DD_OK;
     if (p->unit || p->kpad != kpad || p->kuser != kmax) {
         // switch the plan to weighted with this row length; host weights start at zero
         const size_t n = (size_t)p->ndm * p->nchan;
@@ -725,10 +1044,16 @@ dd_status dd_set_weights_device(dd_plan_t p, const float* d_w, int32_t kmax, voi
         p->kpad = kpad;
         p->kuser = kmax;
         p->unit = false;
-        dd_status st = finish_profiles(p);
-        if (st != DD_OK) return st;
+        p->w_dev = true;
+        st = finish_profiles(p);
+    } else if (p->rk == dd::kRowsFir) {
+        // the rows shared weights that the host knew: back to a record of every trial's own
+        p->w_dev = true;
+        st = build_schedule(p);
     }
-    dd_status st = dd::upload_tables(p);
+    p->w_dev = true;
+    if (st == DD_OK) st = dd::upload_tables(p);
+    p->w_follows = false;
     if (st != DD_OK) return st;
     cudaError_t e = cudaMemcpy2DAsync(p->dev.w, (size_t)kpad * sizeof(float), d_w,
                                       (size_t)kmax * sizeof(float), (size_t)kmax * sizeof(float),
@@ -842,7 +1167,7 @@ dd_status dd_plan_get_schedule(dd_plan_t p, int32_t* nch, int32_t* cs, int32_t* 
     if (!p) return DD_ERR_ARG;
     if (nch) *nch = p->nch;
     if (cs) *cs = p->cs;
-    if (trials_per_cta) *trials_per_cta = trials_per_unit(p) * units_per_warp(p) * dd::kWarps / p->nch;
+    if (trials_per_cta) *trials_per_cta = dd::plan_trials(p);
     return DD_OK;
 }
 
@@ -878,7 +1203,7 @@ std::string tune_key(const dd_plan_s* p) {
     const int kb = (int)std::floor(std::log2((double)p->kmax + 1.0));
     std::ostringstream o;
     o << "C" << p->nchan << "_" << (p->band.in_type == DD_U8 ? "u8" : "f32") << "_"
-      << (p->pair ? "pair" : (p->rl ? "rl" : "int")) << "_s" << sb << "_k" << kb;
+      << (p->rk ? "rows" : "") << (p->pair ? "pair" : (p->rl ? "rl" : "int")) << "_s" << sb << "_k" << kb;
     return o.str();
 }
 
@@ -910,12 +1235,12 @@ dd_status dd_plan_autotune(dd_plan_t p, const void* d_in, int64_t in_ld, void* d
                  hit->second.first, hit->second.second);
         return DD_OK;
     }
-    const bool u8 = stage_esz(p) == 1;
+    const bool u8 = p->rk ? p->rk == dd::kRowsU8 : stage_esz(p) == 1;
     const int cs_list_f[] = {2, 3, 4, 6, 8};
     const int cs_list_u[] = {4, 8, 12, 16};
     const int* cs_list = u8 ? cs_list_u : cs_list_f;
     const int ncs = u8 ? 4 : 5;
-    const int orig_nch = p->nch, orig_cs = p->cs;
+    const int orig_nch = p->nch, orig_cs = p->cs, orig_rk = p->rk;
     int best_nch = orig_nch, best_cs = orig_cs;
     float best = 1e30f;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -926,6 +1251,7 @@ dd_status dd_plan_autotune(dd_plan_t p, const void* d_in, int64_t in_ld, void* d
     for (int nch = 1; nch <= 2 && st == DD_OK; nch *= 2) {
         for (int i = 0; i < ncs; ++i) {
             if (build_schedule_fixed(p, nch, cs_list[i]) != DD_OK) continue;
+            if (p->rk != orig_rk) continue;  // the same sums in every candidate
             st = dd_dedisperse(p, d_in, in_ld, 0, p->band.nsamp, d_out, out_ld, stream);
             if (st != DD_OK) break;
             float t = 1e30f;

@@ -613,10 +613,10 @@ __device__ __forceinline__ bool dedisp_tile(const DedispArgs a, unsigned char* s
 
     if constexpr (FUSED) {
         if constexpr (PAIR) {
-            float f0[R], f1[R];
+            float f[2][R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) unpk(accp[r], f0[r], f1[r]);
-            fused::epilogue_f32<R>(a, *fa, smem, wu, chunk, lane, d, t0, *ft, f0, f1);
+            for (int r = 0; r < R; ++r) unpk(accp[r], f[0][r], f[1][r]);
+            fused::epilogue_f32<2, R>(a, *fa, smem, wu, chunk, lane, d, t0, *ft, f);
         } else {
             fused::epilogue<UPW, RL ? UPW - 1 : 1>(a, *fa, smem, wu, chunk, lane, d, t0, *ft, acc0, accr);
         }
