@@ -250,10 +250,11 @@ dd_status dd_backward(dd_plan_t plan, const float* d_in, int64_t in_ld, int64_t 
 
 /* Kernel schedule of the plan: nch time chunks per CTA (the CTA sums 16/nch trials on
  * the fp32 path, 8/nch on the exact integer path, 24/nch on the run-length path) and cs
- * channels per pipeline stage.  Plans whose trials share their tap runs (fp32 sums with
- * weights given from the host: unit weights, or weights that many trials have in common) use
- * kernels that form each shared run's sums once: there a CTA sums 24/nch or 48/nch trials (by
- * the size of the plan's block) and cs is the most channels of a stage.
+ * channels per pipeline stage.  Plans whose trials share their tap runs (integer sums of runs
+ * up to 257 taps; fp32 sums with unit weights, or with weights given from the host that many
+ * trials have in common) use kernels that form each shared run's sums once: there a CTA sums
+ * 24/nch or 48/nch trials (fp32), 16/nch or 32/nch (integer), by the size of the plan's block,
+ * and cs is the most channels of a stage.
  * dd_plan_create and dd_set_profiles pick a default; dd_plan_set_schedule overrides it
  * (DD_ERR_UNSUPPORTED if it does not fit in shared memory, the old one is then kept). */
 dd_status dd_plan_set_schedule(dd_plan_t plan, int32_t nch, int32_t cs);

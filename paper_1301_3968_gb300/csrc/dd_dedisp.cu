@@ -193,6 +193,73 @@ __global__ void __launch_bounds__(256) k_prefix(const uint8_t* in, int64_t ld, i
         for (int64_t i = end > n ? end : n; i < ldp; ++i) prow[i] = i == n ? carry : 0u;
 }
 
+// The packed form for the row kernels: PW[c][i] = P[c][i] + (P[c][i + kPkHalf] << 16) modulo
+// 2^32, with P constant past n.  As k_prefix; the block's P values and the kPkHalf before them
+// stay in shared memory, so that a block writes the words that end in it.
+__global__ void __launch_bounds__(256) k_prefix_packed(const uint8_t* in, int64_t ld, int64_t t_offset,
+                                                       int64_t n, uint32_t* PW, int64_t ldp) {
+    constexpr int H = kPkHalf, B = 4096;
+    __shared__ __align__(16) uint32_t win[H + B];  // P[base - H .. base + B)
+    __shared__ uint32_t wsum[8];
+    const int c = blockIdx.x;
+    const uint8_t* row = in + (int64_t)c * ld + t_offset;
+    uint32_t* prow = PW + (int64_t)c * ldp;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool vec = (((uintptr_t)row) & 15) == 0;
+    uint32_t carry = 0;
+    for (int64_t base = 0; base < ldp + H; base += B) {
+        const int64_t i0 = base + 16 * tid;
+        uint32_t v[16];
+        if (vec && i0 + 16 <= n) {
+            const uint4 q = *(const uint4*)(row + i0);
+            const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = (w4[k >> 2] >> (8 * (k & 3))) & 0xffu;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = i0 + k < n ? (uint32_t)row[i0 + k] : 0u;
+        }
+        uint32_t sum = 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const uint32_t x = v[k];
+            v[k] = sum;  // exclusive within the thread
+            sum += x;
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const uint32_t x = wsum[w];
+            before += w < warp ? x : 0u;
+            total += x;
+        }
+        const uint32_t off = carry + before + incl - sum;
+#pragma unroll
+        for (int k = 0; k < 16; k += 4)
+            *(uint4*)(win + H + 16 * tid + k) = make_uint4(off + v[k], off + v[k + 1], off + v[k + 2], off + v[k + 3]);
+        carry += total;
+        __syncthreads();
+        // words base - H .. base + B - H (ldp is a multiple of four)
+        for (int k = 4 * tid; k < B; k += 4 * 256) {
+            const int64_t i = base - H + k;
+            if (i < 0 || i >= ldp) continue;
+            const uint4 lo = *(const uint4*)(win + k), hi = *(const uint4*)(win + H + k);
+            *(uint4*)(prow + i) = make_uint4(lo.x + (hi.x << 16), lo.y + (hi.y << 16), lo.z + (hi.z << 16), lo.w + (hi.w << 16));
+        }
+        __syncthreads();
+        for (int k = tid; k < H; k += 256) win[k] = win[B + k];
+        __syncthreads();
+    }
+}
+
 }  // namespace
 
 
@@ -270,7 +337,10 @@ dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_
 // [nchan][ldp] (ldp >= nsamp + 1).
 dd_status launch_prefix_into(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                              int64_t nsamp, uint32_t* P, int64_t ldp, cudaStream_t s) {
-    k_prefix<<<p->nchan, 256, 0, s>>>((const uint8_t*)in, ld, t_offset, nsamp, P, ldp);
+    if (p->rk == kRowsRl)
+        k_prefix_packed<<<p->nchan, 256, 0, s>>>((const uint8_t*)in, ld, t_offset, nsamp, P, ldp);
+    else
+        k_prefix<<<p->nchan, 256, 0, s>>>((const uint8_t*)in, ld, t_offset, nsamp, P, ldp);
     return cuda_status(cudaGetLastError());
 }
 
@@ -289,8 +359,7 @@ dd_status launch_prefix(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offs
         if (e != cudaSuccess) return cuda_status(e);
         p->prefix_elems = need;
     }
-    k_prefix<<<p->nchan, 256, 0, s>>>((const uint8_t*)in, ld, t_offset, nsamp, p->d_prefix, ldp);
-    return cuda_status(cudaGetLastError());
+    return launch_prefix_into(p, in, ld, t_offset, nsamp, p->d_prefix, ldp, s);
 }
 
 dd_status launch_dedisperse_rl(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,

@@ -37,8 +37,9 @@ constexpr int G = 16;  // widths per register window
 
 // A warp's shared scratch for the earliest-start search (4-byte words): the prefix values
 // P_0 .. P_30 of one segment, then P_{w0g} .. P_{w0g+45} (every P_s and P_{s+w} that a
-// width of the group forms).
-constexpr int kChainFloats = 80;
+// width of the group forms).  Segments of up to 35 starts (the packed row kernels' tiles).
+constexpr int kSegPk = 35;
+constexpr int kChainFloats = 2 * kSegPk + G - 1;
 
 // S starts of one lane segment (x = row + i0) for widths w0g + j, j < G.
 // q = sum_{k < w0g} x[k] on entry.  !FULL: starts outside [i_lo, i_hi) and windows
@@ -99,7 +100,8 @@ __device__ __forceinline__ long long group_bound(const int* x, uint32_t q, uint3
 
 // Width groups from prune_w on skip the scan of segments whose group_bound is below
 // the smallest merged maximum of the group (strictly: a tie from an earlier start could
-// still win), which on noise-like series is most of them.
+// still win), which on noise-like series is most of them.  (Groups of 35-start segments
+// from 50 on.)
 template <int S>
 __host__ __device__ constexpr int prune_w() { return S + 15 > 48 ? S + 15 : 48; }
 
@@ -282,6 +284,67 @@ __device__ __forceinline__ void epilogue(const DedispArgs& a, const FusedArgs& f
                 for (int k = lane; k < C; k += 32) ft.seam_out[2 * cb + k] = row[e_hi - C + k];
         }
         scan_row<kRInt>(f, row, chain, f.key + (int64_t)du * f.nw, T0, C, chunk, a.nch, lane, i_lo, i_hi, e_hi);
+    }
+    // the next tile's bulk copies overwrite the rows
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncthreads();
+}
+
+// The fused epilogue of one packed integer tile (dd_rows.cuh; every thread of the CTA
+// calls it): the unit's two trials d, d + 1, one row each, s[u] = the lane's low sums
+// (outputs lane * R + r of the warp's chunk), then its high ones (kPkHalf later).
+// Segments of 35 starts, so that 32 lanes cover the 1088-output tile in one pass.
+template <int R, int NW>
+__device__ __forceinline__ void epilogue_pk(const DedispArgs& a, const FusedArgs& f, unsigned char* smem,
+                                            int wu, int chunk, int lane, int d, int64_t T0,
+                                            const FusedTile& ft, const int (&s)[2][2 * R]) {
+    constexpr int TT = 2 * kPkHalf;
+    const int L = TT * a.nch;
+    const int C = f.C;
+    int* rows = (int*)smem + 2 * wu * f.rowlen;
+    const int64_t S1 = ft.s1;
+    const bool first = ft.first, last = ft.last;
+    const int i_lo = first ? C : 0;
+    const int e_hi = (int)(S1 - T0) + C;
+    const int i_hi = last ? e_hi - f.w0 + 1 : L;
+    uint32_t* chain = (uint32_t*)smem + fused_rows_ints(2 * NW / a.nch, f.rowlen, C) +
+                      (threadIdx.x >> 5) * kChainFloats;
+    const int ib = C + chunk * TT + lane * R;
+    const int64_t tb = T0 + chunk * TT + lane * R;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const bool live = d + u < a.ndm;
+        const int o = live ? (int)f.off[d + u] : 0;
+        int* row = rows + u * f.rowlen;
+        int m = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int v0 = s[u][r] - o, v1 = s[u][R + r] - o;
+            row[ib + r] = v0;
+            row[ib + kPkHalf + r] = v1;
+            if (tb + r < S1) m = max(m, abs(v0));
+            if (tb + kPkHalf + r < S1) m = max(m, abs(v1));
+        }
+        if (live && m > f.mlim) atomicExch(a.status, (int)DD_ERR_OVERFLOW);
+        const int64_t cb = (int64_t)(wu * 2 + u) * C;
+        if (live && chunk == 0 && !first)
+            for (int k = lane; k < C; k += 32) row[k] = ft.carry[cb + k];
+    }
+    __syncthreads();  // the rows and their carries are complete
+#pragma unroll 1
+    for (int u = 0; u < 2; ++u) {
+        if (d + u >= a.ndm) break;
+        const int* row = rows + u * f.rowlen;
+        const int64_t cb = (int64_t)(wu * 2 + u) * C;
+        if (chunk == 0) {
+            if (!last)
+                for (int k = lane; k < C; k += 32) ft.carry[cb + k] = row[L + k];
+            if (first && ft.seam_in)
+                for (int k = lane; k < C; k += 32) ft.seam_in[2 * cb + C + k] = row[C + k];
+            if (last && ft.seam_out)
+                for (int k = lane; k < C; k += 32) ft.seam_out[2 * cb + k] = row[e_hi - C + k];
+        }
+        scan_row<kSegPk>(f, row, chain, f.key + (int64_t)(d + u) * f.nw, T0, C, chunk, a.nch, lane, i_lo, i_hi, e_hi);
     }
     // the next tile's bulk copies overwrite the rows
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");

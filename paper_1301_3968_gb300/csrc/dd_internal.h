@@ -59,16 +59,23 @@ __host__ __device__ constexpr int row_trials(int kind, int nw, int nch) { return
 __host__ __device__ constexpr int row_span(int kind, int nch) {
     return kind == kRowsFir ? row_tile_t(kind, nch) : (nch - 1) * 2 * kPkHalf + kPkHalf;
 }
-// Stage record of a row kernel: a header (rows of the stage; bit ci: packed sums are moved
-// into 32-bit ones after channel ci; the longest row), an entry per unit and channel (each
-// trial's row position in the stage's row area: trials 0 and 1 as the half words of the first
-// word, trial 2 the second), a descriptor per row (offset of its samples in the
+// Words of zeros at the start of a packed row area, read for the channels that fill a stage's
+// last four.
+__host__ __device__ constexpr int row_zero_words(int kind, int nch) {
+    return kind == kRowsFir ? 0 : (row_span(kind, nch) + 3) & ~3;
+}
+// Stage record of a row kernel: a header (rows of the stage; packed kinds: per four channels two
+// bits, 0: the four words may be added in 16-bit halves, 1: two and two, 2: none; the longest
+// row), entries with each trial's row position in the stage's row area (fp32: per unit and
+// channel, trials 0 and 1 as the half words of the first word, trial 2 the second; packed: per
+// unit and four channels, their positions as half words, trial 0's two words then trial 1's), a descriptor per row (offset of its samples in the
 // staged rows, its position in the row area, its length, taps | offset of its weights
 // << 16), and the rows' weights.  The header and entries are copied beside the rows.
 struct RowGeom {
     int ent_bytes, desc_off, w_off, rec_bytes;
-    __host__ __device__ RowGeom(int cs, int nu, int rows_max, int kw) {
-        ent_bytes = (16 + 8 * nu * cs + 8 + 15) & ~15;  // (one entry is read ahead)
+    __host__ __device__ RowGeom(int kind, int cs, int nu, int rows_max, int kw) {
+        // (fp32: one entry is read ahead; packed: cs is a multiple of four)
+        ent_bytes = (16 + (kind == kRowsFir ? 8 * nu * cs + 8 : 4 * nu * cs) + 15) & ~15;
         desc_off = ent_bytes;
         w_off = desc_off + 16 * rows_max;
         rec_bytes = (w_off + 4 * kw + 15) & ~15;

@@ -353,11 +353,12 @@ struct Row {
     int32_t n, trial, reach;
 };
 
-// The plan's row kind, if its sums can be formed that way: fp32 sums with weights that
-// the host knows.
+// The plan's row kind, if its sums can be formed that way: fp32 sums with weights that the
+// host knows, integer sums of runs that fit a half word.
 int row_kind_of(const dd_plan_s* p) {
     if (p->pair) return p->w_dev || p->kmax > 0xffff ? dd::kRowsNone : dd::kRowsFir;
-    return dd::kRowsNone;
+    if (p->kmax > dd::kPkMaxTaps) return dd::kRowsNone;
+    return p->rl ? dd::kRowsRl : dd::kRowsU8;
 }
 
 // Rows pay up to this many distinct runs per (trial, channel).
@@ -370,9 +371,14 @@ constexpr double kRowsMaxShare = 0.5;
 int row_warps_of(const dd_plan_s* p, int kind, int nch) {
     const int64_t tile = dd::row_tile_t(kind, nch);
     const int64_t tiles = (std::max<int64_t>(1, p->band.nsamp - p->dmax) + tile - 1) / tile;
+    auto ctas = [&](int nw) {
+        const int db = dd::row_trials(kind, nw, nch);
+        return tiles * ((p->ndm + db - 1) / db);
+    };
+    if (ctas(dd::kWarps) <= 304) return dd::kWarps;  // one wave: a CTA's own time counts
     auto fill = [&](int nw, int64_t slots) {
         const int db = dd::row_trials(kind, nw, nch);
-        const int64_t n = tiles * ((p->ndm + db - 1) / db);
+        const int64_t n = ctas(nw);
         return (double)p->ndm / db * tiles / (double)((n + slots - 1) / slots * slots);
     };
     return 1.12 * fill(dd::kRowWarps, 152) >= fill(dd::kWarps, 304) ? dd::kRowWarps : dd::kWarps;
@@ -429,26 +435,41 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     auto len_of = [&](const Row& r) { return (int64_t)((Q - 1 + r.reach + span + 3) & ~3); };
     size_t total = 0;
     int64_t need = 0;
-    // the fullest single channel: rows, weights (each row's padded to four), row words
-    int64_t one_r = 1, one_w = 0, one_a = 0;
+    // Stages are cut at multiples of `grain` channels.  Of a grain from channel c of block b:
+    // rows, weights (each row's padded to four) and row words, and the most of each.
+    const int grain = fir ? 1 : 4;
+    struct Need {
+        int64_t r = 0, w = 0, a = 0;
+    };
+    auto grain_need = [&](int b, int c) {
+        Need k;
+        const int r0 = first[b][c], r1 = first[b][std::min(C, c + grain)];
+        k.r = r1 - r0;
+        for (int r = r0; r < r1; ++r) {
+            if (fir) k.w += (rows[b][r].n + 3) & ~3;
+            k.a += len_of(rows[b][r]);
+        }
+        return k;
+    };
+    Need one;
     for (int b = 0; b < nblk; ++b) {
         total += rows[b].size();
-        for (int c = 0; c < C; ++c) {
-            int64_t w = 0, ar = 0;
-            for (int r = first[b][c]; r < first[b][c + 1]; ++r) {
-                w += (rows[b][r].n + 3) & ~3;
-                ar += len_of(rows[b][r]);
-                // samples that building the row reads (dd_rows.cuh)
-                need = std::max(need, len_of(rows[b][r]) + (rows[b][r].n & ~3) + 4);
-            }
-            one_r = std::max<int64_t>(one_r, first[b][c + 1] - first[b][c]);
-            one_w = std::max(one_w, w);
-            one_a = std::max(one_a, ar);
+        for (const Row& r : rows[b]) {
+            // samples that building the row reads (dd_rows.cuh)
+            const int64_t past = fir ? (r.n & ~3) + 4 : kind == dd::kRowsU8 ? dd::kPkHalf + (r.n & ~3) + 4 : r.n;
+            need = std::max(need, len_of(r) + past);
+        }
+        for (int c = 0; c < C; c += grain) {
+            const Need k = grain_need(b, c);
+            one.r = std::max(one.r, k.r);
+            one.w = std::max(one.w, k.w);
+            one.a = std::max(one.a, k.a);
         }
     }
     if ((double)total > kRowsMaxShare * units) return false;
     const int64_t lcap = (need + Q - 1) / Q * Q;
-    if (lcap > (1 << 20) || one_w > 0xffff || !fir) return false;
+    if (lcap > (1 << 20) || one.w > 0xffff) return false;
+    const int64_t zero = dd::row_zero_words(kind, nch);  // the area begins with a row of zeros
     // Stages: channels in order, as many as the limits on channels (cs), rows, weights and
     // row words allow.
     struct Cut {
@@ -462,26 +483,21 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
         if (keep) k.start.resize(nblk);
         for (int b = 0; b < nblk; ++b) {
             int n = 0;
-            int64_t w = 0, ar = 0, r = 0, ch = 0;
-            for (int c = 0; c < C; ++c) {
-                int64_t cw = 0, ca = 0;
-                const int64_t cr = first[b][c + 1] - first[b][c];
-                for (int i = first[b][c]; i < first[b][c + 1]; ++i) {
-                    cw += (rows[b][i].n + 3) & ~3;
-                    ca += len_of(rows[b][i]);
-                }
-                if (c == 0 || ch == cs || r + cr > rlim || w + cw > wlim || ar + ca > alim) {
+            Need in;
+            for (int c = 0, c0 = 0; c < C; c += grain) {
+                const Need m = grain_need(b, c);
+                if (c == 0 || c - c0 >= cs || in.r + m.r > rlim || in.w + m.w > wlim || in.a + m.a > alim) {
                     if (keep) k.start[b].push_back(c);
                     ++n;
-                    w = ar = r = ch = 0;
+                    c0 = c;
+                    in = Need();
                 }
-                w += cw;
-                ar += ca;
-                r += cr;
-                ++ch;
-                k.rmax = std::max(k.rmax, r);
-                k.wmax = std::max(k.wmax, w);
-                k.area = std::max(k.area, ar);
+                in.r += m.r;
+                in.w += m.w;
+                in.a += m.a;
+                k.rmax = std::max(k.rmax, in.r);
+                k.wmax = std::max(k.wmax, in.w);
+                k.area = std::max(k.area, in.a);
             }
             if (keep) k.start[b].push_back(C);
             k.nst = std::max(k.nst, n);
@@ -492,18 +508,19 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     const size_t budget = cs_fixed > 0 || nw == dd::kRowWarps ? dd::kSmemBudgetOne : dd::kSmemBudget;
     // limits for at most cs channels; false where a single channel does not fit
     auto limits = [&](int cs, int64_t* rlim, int64_t* wlim, int64_t* alim) {
-        *rlim = std::max<int64_t>(one_r, 2 * cs);
-        *wlim = fir ? std::min<int64_t>(0xffff, std::max<int64_t>(one_w, (int64_t)cs * ((p->kmax + 3) & ~3) * 5 / 4)) : 0;
-        const dd::RowGeom g(cs, nu, (int)*rlim, (int)*wlim);
-        const size_t rest = dd::row_smem_bytes(g, 0, esz, (int)lcap, cs, 2 * C + 2, 16);
+        *rlim = std::max<int64_t>(one.r, 2 * cs);
+        *wlim = fir ? std::min<int64_t>(0xffff, std::max<int64_t>(one.w, (int64_t)cs * ((p->kmax + 3) & ~3) * 5 / 4)) : 0;
+        const dd::RowGeom g(kind, cs, nu, (int)*rlim, (int)*wlim);
+        const size_t rest = dd::row_smem_bytes(g, 0, esz, (int)lcap, cs, 2 * C + 2, 16 + (int)zero);
         if (rest >= budget) return false;
         *alim = (int64_t)((budget - rest) / 8) & ~(int64_t)3;
-        return *alim >= one_a;
+        return *alim >= one.a;
     };
     Cut best;
     int64_t rlim = 0, wlim = 0, alim = 0;
-    const int cs_hi = cs_fixed > 0 ? cs_fixed : dd::kRowCsMax, cs_lo = cs_fixed > 0 ? cs_fixed : 1;
-    for (int cs = std::min(cs_hi, dd::kRowCsMax); cs >= cs_lo; --cs) {
+    const int cs_hi = cs_fixed > 0 ? (cs_fixed + grain - 1) / grain * grain : dd::kRowCsMax;
+    const int cs_lo = cs_fixed > 0 ? cs_hi : grain;
+    for (int cs = std::min(cs_hi, dd::kRowCsMax); cs >= cs_lo; cs -= grain) {
         if (!limits(cs, &rlim, &wlim, &alim)) continue;
         Cut k = cut(cs, rlim, wlim, alim, false);
         if (best.cs == 0 || k.total < best.total) best = k;
@@ -514,8 +531,9 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     limits(cs, &rlim, &wlim, &alim);
     best = cut(cs, rlim, wlim, alim, true);
     const int nst = best.nst, lo_ld = C + nst + 2;
-    const int32_t area = (int32_t)best.area + 16;  // and what the last row's reads run past it
-    const dd::RowGeom g(cs, nu, (int)best.rmax, (int)best.wmax);
+    const int32_t area = (int32_t)(zero + best.area) + 16;  // and what the last row's reads run past it
+    if (area > 0xffff) return false;  // positions are half words
+    const dd::RowGeom g(kind, cs, nu, (int)best.rmax, (int)best.wmax);
     std::vector<unsigned char> rec((size_t)nblk * nst * g.rec_bytes, 0);
     std::vector<int32_t> table((size_t)nblk * lo_ld, 0);
     for_blocks(nblk, (size_t)p->ndm * C, [&](int b) {
@@ -528,13 +546,13 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
         for (int st = 0; st < ns; ++st) {
             unsigned char* q = rec.data() + ((size_t)b * nst + st) * g.rec_bytes;
             int32_t* hdr = (int32_t*)q;
-            int32_t* ent = (int32_t*)(q + 16);
+            uint32_t* ent = (uint32_t*)(q + 16);
             int32_t* desc = (int32_t*)(q + g.desc_off);
             float* w = (float*)(q + g.w_off);
             const int c0 = best.start[b][st], c1 = best.start[b][st + 1];
             const int r0 = first[b][c0];
             hdr[0] = first[b][c1] - r0;
-            int32_t dst = 0, woff = 0;
+            int32_t dst = (int32_t)zero, woff = 0;
             at.assign((size_t)hdr[0], 0);
             for (int c = c0; c < c1; ++c)
                 for (int r = first[b][c]; r < first[b][c + 1]; ++r) {
@@ -552,19 +570,39 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
                     for (int k = 0; k < row.n; ++k) w[woff + k] = p->unit ? 1.0f : p->w[dc * p->kpad + k];
                     woff += (row.n + 3) & ~3;
                 }
-            for (int j = 0; j < nu; ++j)
-                for (int c = c0; c < c1; ++c) {
-                    int32_t pos[3] = {0, 0, 0};
-                    const int d0 = b * db + j * nt;
-                    if (d0 >= p->ndm) continue;
-                    for (int u = 0; u < nt; ++u) {
-                        // trials past the list's end add what the unit's last one does
-                        const size_t dc = (size_t)std::min(d0 + u, p->ndm - 1) * C + c;
-                        pos[u] = at[first[b][c] - r0 + rid[dc]] + p->delay[dc] - lo[(size_t)b * C + c];
+            // a trial's position in the row area; trials past the list's end add what the
+            // last one does
+            auto pos = [&](int d, int c) -> uint32_t {
+                if (c >= c1) return 0;  // the zeros
+                const size_t dc = (size_t)std::min(d, p->ndm - 1) * C + c;
+                return (uint32_t)(at[first[b][c] - r0 + rid[dc]] + p->delay[dc] - lo[(size_t)b * C + c]);
+            };
+            for (int j = 0; j < nu && b * db + j * nt < p->ndm; ++j) {
+                const int d0 = b * db + j * nt;
+                if (fir) {
+                    for (int c = c0; c < c1; ++c) {
+                        uint32_t* e = ent + 2 * (size_t)(j * cs + c - c0);
+                        e[0] = pos(d0, c) | pos(d0 + 1, c) << 16;
+                        e[1] = pos(d0 + 2, c);
                     }
-                    int32_t* e = ent + 2 * (size_t)(j * cs + c - c0);
-                    e[0] = (int32_t)((uint32_t)pos[0] | (uint32_t)pos[1] << 16);
-                    e[1] = pos[2];
+                } else {
+                    for (int c = c0; c < c1; c += 4) {
+                        uint32_t* e = ent + (size_t)(j * cs + c - c0);
+                        for (int u = 0; u < 2; ++u) {
+                            e[2 * u] = pos(d0 + u, c) | pos(d0 + u, c + 1) << 16;
+                            e[2 * u + 1] = pos(d0 + u, c + 2) | pos(d0 + u, c + 3) << 16;
+                        }
+                    }
+                }
+            }
+            if (!fir)
+                for (int c = c0; c < c1; c += 4) {
+                    int32_t m[4] = {0, 0, 0, 0};  // longest run of each channel
+                    for (int i = 0; i < 4 && c + i < c1; ++i)
+                        for (int r = first[b][c + i]; r < first[b][c + i + 1]; ++r) m[i] = std::max(m[i], rows[b][r].n);
+                    const int mode = m[0] + m[1] + m[2] + m[3] <= dd::kPkMaxTaps ? 0
+                                     : std::max(m[0] + m[1], m[2] + m[3]) <= dd::kPkMaxTaps ? 1 : 2;
+                    hdr[1] |= mode << ((c - c0) / 2);
                 }
         }
     });
@@ -583,9 +621,10 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     p->blk_lo.swap(table);
     p->rec.swap(rec);
     p->dev_dirty = true;
-    dd::log_msg(1, "plan %d trials x %d channels: shared rows (%.3f per trial and channel), %d trials and %d warps per "
-                "CTA, up to %d channels per stage (%.1f stages per block), staged rows of %d elements, row area of "
-                "%d words, record %d bytes, %zu bytes of shared memory", p->ndm, C, (double)total / units, db, nw, cs,
+    dd::log_msg(1, "plan %d trials x %d channels: %s, shared rows (%.3f per trial and channel), %d trials and %d warps "
+                "per CTA, up to %d channels per stage (%.1f stages per block), staged rows of %d elements, row area of "
+                "%d words, record %d bytes, %zu bytes of shared memory", p->ndm, C,
+                fir ? "fp32 sums" : p->rl ? "run-length sums" : "exact integer sums", (double)total / units, db, nw, cs,
                 (double)best.total / nblk, p->lcap, p->blen, p->rec_bytes, dd::dedisp_smem_for(p));
     return true;
 }

@@ -80,31 +80,32 @@ int blocks_per_sm(size_t smem) {
 }  // namespace
 
 size_t rows_smem_for(const dd_plan_s* p) {
-    const RowGeom g(p->cs, p->row_warps / p->nch, p->rows_max, p->kw);
+    const RowGeom g(p->rk, p->cs, p->row_warps / p->nch, p->rows_max, p->kw);
     return row_smem_bytes(g, p->row_warps, p->rl ? 4 : (p->band.in_type == DD_U8 ? 1 : 4), p->lcap, p->cs, p->lo_ld,
                           p->blen);
 }
 
+// fn<kind, uint8 input, warps per CTA>(args) of a row plan
+#define DD_ROWS_NW(fn, kind, in8, nw, ...) \
+    ((nw) == kRowWarps ? fn<kind, in8, kRowWarps>(__VA_ARGS__) : fn<kind, in8, kWarps>(__VA_ARGS__))
+#define DD_ROWS(fn, kind, in8, nw, ...)                                     \
+    ((kind) == kRowsRl   ? DD_ROWS_NW(fn, kRowsRl, false, nw, __VA_ARGS__)  \
+     : (kind) == kRowsU8 ? DD_ROWS_NW(fn, kRowsU8, true, nw, __VA_ARGS__)   \
+     : (in8)             ? DD_ROWS_NW(fn, kRowsFir, true, nw, __VA_ARGS__)  \
+                         : DD_ROWS_NW(fn, kRowsFir, false, nw, __VA_ARGS__))
+
 dd_status launch_rows(const dd_plan_s* p, DedispArgs a, cudaStream_t s) {
     const size_t smem = rows_smem_for(p);
-    const bool in8 = p->band.in_type == DD_U8;
-    if (p->row_warps == kRowWarps)
-        return in8 ? run<kRowsFir, true, kRowWarps>(a, smem, s) : run<kRowsFir, false, kRowWarps>(a, smem, s);
-    return in8 ? run<kRowsFir, true, kWarps>(a, smem, s) : run<kRowsFir, false, kWarps>(a, smem, s);
+    return DD_ROWS(run, p->rk, p->band.in_type == DD_U8, p->row_warps, a, smem, s);
 }
 
 dd_status launch_rows_batched(int kind, bool in8, int nw, const DedispArgs* d_args, const BatchItem* d_items,
                               int32_t nitems, size_t smem, cudaStream_t s) {
-    if (nw == kRowWarps)
-        return in8 ? run_batched<kRowsFir, true, kRowWarps>(d_args, d_items, nitems, smem, s)
-                   : run_batched<kRowsFir, false, kRowWarps>(d_args, d_items, nitems, smem, s);
-    return in8 ? run_batched<kRowsFir, true, kWarps>(d_args, d_items, nitems, smem, s)
-               : run_batched<kRowsFir, false, kWarps>(d_args, d_items, nitems, smem, s);
+    return DD_ROWS(run_batched, kind, in8, nw, d_args, d_items, nitems, smem, s);
 }
 
 int rows_batched_blocks_per_sm(int kind, bool in8, int nw, size_t smem) {
-    if (nw == kRowWarps) return in8 ? blocks_per_sm<kRowsFir, true, kRowWarps>(smem) : blocks_per_sm<kRowsFir, false, kRowWarps>(smem);
-    return in8 ? blocks_per_sm<kRowsFir, true, kWarps>(smem) : blocks_per_sm<kRowsFir, false, kWarps>(smem);
+    return DD_ROWS(blocks_per_sm, kind, in8, nw, smem);
 }
 
 }  // namespace dd

@@ -8,12 +8,13 @@
 // distinct runs per channel.  A CTA therefore forms each distinct run's sums B_{c,q} once
 // per tile, in shared memory (a "row"), and a trial costs one add per channel and output
 // whatever its tap count, where the tap kernels (dd_tile.cuh) cost one multiply-add per tap.
+// The kinds of rows (RowKind) and their units:
 //
-// A warp unit is three trials x 864 outputs, lane l owning 27 consecutive ones (odd:
+// kRowsFir: fp32 sums.  A warp unit is three trials x 864 outputs, lane l owning 27 consecutive ones (odd:
 // lane-strided loads hit 32 banks).  Where each trial uses the row of the one before, at most
 // two samples later (98 % on that list), each sample is loaded once for all three.
 //
-// What bounds it: shared-memory loads, 0.35 of a word per trial, channel and output where a
+// Bound by shared-memory loads, 0.35 of a word per trial, channel and output where a
 // window is shared (else 1), plus the rows' own building (a quad of outputs loads n / 4 + 1
 // quads and stores one), against 1 + (n - 1) / 27 loads and n multiply-adds of the tap kernel.
 // Measured on 4096 CRAFT-like trials x 336 channels x 60261 outputs: tap kernel 17.62 ms, rows
@@ -21,6 +22,22 @@
 // the building skipped and 0.44 with the summing skipped.  Two trials per warp took 1.19 ms,
 // four trials of 15 outputs with one switch per trial 2.40, 8-warp CTAs with two-trial warps
 // 1.91; scalar instead of packed adds 1.24 (two trials).
+//
+// kRowsU8, kRowsRl: exact sums of uint8 samples with unit weights, for runs of at most 257
+// taps (255 n <= 65535).  A row word holds two outputs, B[i] + (B[i + 544] << 16): one load and
+// one 32-bit addition serve both, whatever the start's parity (consecutive outputs in a word
+// would need a second copy of the row for odd starts).  A unit is two trials x 1088 outputs,
+// lane l owning 17 consecutive words.  The channels go four at a time: their words are added up
+// to the point where a half could pass 65535 (the host says: all four, two and two, or each),
+// and those sums into a 32-bit sum of whole words and one of the high halves; low = whole -
+// (high << 16), exact modulo 2^32.  kRowsU8 forms the rows from the staged samples, kRowsRl from
+// packed prefix sums PW[i] = P[i] + (P[i + 544] << 16) in global memory: B = PW[i + n] - PW[i].
+// Bound by shared-memory loads, half a word per trial, channel and output.  (Sharing a word
+// between trials whose starts are close, as the fp32 units do, would save loads but needs a
+// branch per channel; straight code for four channels keeps 68 loads in flight.)
+// Measured: 1500 trials x 336 channels x 21364 outputs 2.62 -> 0.97 ms (1.11e13
+// trial-channel-samples/s; tap kernel 4.1e12), 8192 low-band trials x 1024 channels x 65536
+// outputs (run-length sums, mean 66 taps) 101 -> 48 ms against the 32-bit difference rows.
 //
 // Pipeline: channels stream in stages, as many channels each as their rows fit in a half of
 // the row area.  All warps sum stage i from one half, then build the rows of stage i + 1 in
@@ -41,7 +58,7 @@ namespace {
 // Staged element type; IN8: uint8 input (weighted uint8 plans).
 template <int KIND, bool IN8>
 struct RowIn {
-    using T = typename std::conditional<IN8, uint8_t, float>::type;
+    using T = typename std::conditional<KIND == kRowsRl, uint32_t, typename std::conditional<IN8, uint8_t, float>::type>::type;
 };
 
 // Four consecutive samples from a 16-byte (fp32) or 4-byte (uint8) aligned address.
@@ -191,6 +208,93 @@ __device__ __forceinline__ void fir_channel(const float* rows, int2 e, int lane_
     fir_shared2<-1, 106>(z, a[2], a[2]);
 }
 
+// Packed words of four quads' first sums from uint8 samples, one quad of words per lane: the
+// sums of n samples from byte i and from byte i + kPkHalf, then the next three words by adding
+// the entering and taking off the leaving sample of both halves at once.
+__device__ __forceinline__ void build_u8(const uint8_t* x, int n, int i, int len, uint32_t* dst) {
+    __builtin_assume(__isShared(x));
+    __builtin_assume(__isShared(dst));
+    if (i >= len) return;
+    const int nw = n >> 2, rem = n & 3;
+    const uint32_t mask = (1u << (8 * rem)) - 1u;
+    constexpr uint32_t kOnes = 0x01010101u, kEven = 0x00ff00ffu;
+    const uint32_t* pa = (const uint32_t*)(x + i);
+    const uint32_t* pb = (const uint32_t*)(x + i + kPkHalf);
+    const uint32_t a0 = pa[0], b0 = pb[0];
+    uint32_t a = a0, b = b0, sa = 0, sb = 0;
+    for (int j = 0; j < nw; ++j) {
+        sa = __dp4a(a, kOnes, sa);
+        sb = __dp4a(b, kOnes, sb);
+        a = pa[j + 1];
+        b = pb[j + 1];
+    }
+    sa = __dp4a(a & mask, kOnes, sa);
+    sb = __dp4a(b & mask, kOnes, sb);
+    // the samples entering with the next three words: bytes n .. n + 2
+    const uint32_t ea = __funnelshift_r(a, pa[nw + 1], 8 * rem), eb = __funnelshift_r(b, pb[nw + 1], 8 * rem);
+    const uint32_t xe = a0 & kEven, ye = b0 & kEven, xo = (a0 >> 8) & kEven, yo = (b0 >> 8) & kEven;
+    const uint32_t fe = ea & kEven, ge = eb & kEven, fo = (ea >> 8) & kEven, go = (eb >> 8) & kEven;
+    uint4 o;
+    o.x = sa + (sb << 16);
+    o.y = o.x + __byte_perm(fe, ge, 0x5410) - __byte_perm(xe, ye, 0x5410);
+    o.z = o.y + __byte_perm(fo, go, 0x5410) - __byte_perm(xo, yo, 0x5410);
+    o.w = o.z + __byte_perm(fe, ge, 0x7632) - __byte_perm(xe, ye, 0x7632);
+    *(uint4*)(dst + i) = o;
+}
+
+// 256 packed words from packed prefix sums, eight per lane.
+__device__ __forceinline__ void build_rl(const uint32_t* x, int n, int i, int len, uint32_t* dst) {
+    __builtin_assume(__isShared(x));
+    __builtin_assume(__isShared(dst));
+    const uint32_t* y = x + n;
+    if (i - (i & 31) + 256 <= len) {
+#pragma unroll
+        for (int k = 0; k < 256; k += 32) dst[i + k] = y[i + k] - x[i + k];
+    } else {
+        for (int k = 0; k < 256 && i + k < len; k += 32) dst[i + k] = y[i + k] - x[i + k];
+    }
+}
+
+// A trial's packed integer sums: whole words, and their high halves.
+struct PkAcc {
+    uint32_t whole[kRPk], hi[kRPk];
+};
+
+// Four channels of one trial: pos holds its four row positions as half words.  MODE: how many
+// of the four words may be added before a half could pass 65535.
+template <int MODE>
+__device__ __forceinline__ void pk_channels(const uint32_t* rows, uint2 pos, PkAcc& a) {
+    const uint32_t* p0 = rows + (pos.x & 0xffffu);
+    const uint32_t* p1 = rows + (pos.x >> 16);
+    const uint32_t* p2 = rows + (pos.y & 0xffffu);
+    const uint32_t* p3 = rows + (pos.y >> 16);
+    __builtin_assume(__isShared(p0));
+    __builtin_assume(__isShared(p1));
+    __builtin_assume(__isShared(p2));
+    __builtin_assume(__isShared(p3));
+#pragma unroll
+    for (int r = 0; r < kRPk; ++r) {
+        const uint32_t v0 = p0[r], v1 = p1[r], v2 = p2[r], v3 = p3[r];
+        if constexpr (MODE == 4) {
+            const uint32_t s = v0 + v1 + v2 + v3;
+            a.whole[r] += s;
+            a.hi[r] += s >> 16;
+        } else if constexpr (MODE == 2) {
+            const uint32_t s = v0 + v1, t = v2 + v3;
+            a.whole[r] += s + t;
+            a.hi[r] += s >> 16;
+            a.hi[r] += t >> 16;
+        } else {
+            a.whole[r] += v0 + v1;
+            a.whole[r] += v2 + v3;
+            a.hi[r] += v0 >> 16;
+            a.hi[r] += v1 >> 16;
+            a.hi[r] += v2 >> 16;
+            a.hi[r] += v3 >> 16;
+        }
+    }
+}
+
 struct RowSmem {
     unsigned char* raw;
     int* lo;         // the block's per-channel minimum delays, then its stages' first channels
@@ -248,7 +352,7 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
     const int cs = a.cs;
     const int wpg = a.nch;  // warps along time
     const int nu = NW / wpg;
-    const RowGeom rg(cs, nu, a.rows_max, a.kpad);
+    const RowGeom rg(KIND, cs, nu, a.rows_max, a.kpad);
     const int rec_off = cs * a.lcap * (int)sizeof(TIN);
     const int half_words = a.blen + rg.ent_bytes / 4;
     RowSmem sm;
@@ -271,6 +375,8 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
         sm.lo[c] = lo;
         if (c < a.nchan) past_end |= (((base + lo) & ~(int64_t)(Q - 1)) + a.lcap > a.ld) ? 1 : 0;
     }
+    if constexpr (!FIR)  // the row of zeros that channels past a stage's last read
+        for (int k = tid; k < row_zero_words(KIND, a.nch); k += NW * 32) sm.half[k] = sm.half[half_words + k] = 0u;
     const bool tail = __syncthreads_or(past_end) != 0;
     const int nst = sm.lo[a.nchan];  // stages of this block
     if (warp == 0) issue_rows<TIN>(a, sm, rg, rec_off, blk, 0, base, tail, lane);
@@ -278,12 +384,17 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
     const int bq = (int)(base & (Q - 1));
     const int lane_off = chunk * TW + lane * R;
     bool ok = true;
-    FirAcc sum[NT];
+    typename std::conditional<FIR, FirAcc, PkAcc>::type sum[NT];
 #pragma unroll
     for (int u = 0; u < NT; ++u) {
+        if constexpr (FIR) {
 #pragma unroll
-        for (int j = 0; j < R / 2; ++j) sum[u].v[j] = 0ull;
-        sum[u].t = 0.f;
+            for (int j = 0; j < R / 2; ++j) sum[u].v[j] = 0ull;
+            sum[u].t = 0.f;
+        } else {
+#pragma unroll
+            for (int j = 0; j < R; ++j) sum[u].whole[j] = sum[u].hi[j] = 0u;
+        }
     }
 
     auto build = [&](int i) {  // the rows of stage i, from the raw buffer
@@ -294,19 +405,33 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
         const int c0 = sm.lo[a.nchan + 1 + i], csn = sm.lo[a.nchan + 2 + i] - c0;
         const int4 hdr = *(const int4*)rec;
         int* ed = (int*)(half + a.blen);
-        const int2* es = (const int2*)(rec + 16);
         if (tid == 0) *(int4*)ed = hdr;
-        for (int e = tid; e < nu * cs; e += NW * 32) {
-            const int ci = e % cs;
-            if (ci >= csn) continue;
-            const int sh = (bq + sm.lo[c0 + ci]) & (Q - 1);
-            const int2 v = es[e];
-            ((int2*)(ed + 4))[e] = make_int2(v.x + sh + (sh << 16), v.y + sh);
+        auto shift = [&](int ci) { return ci < csn ? (bq + sm.lo[c0 + ci]) & (Q - 1) : 0; };
+        if constexpr (FIR) {
+            const int2* es = (const int2*)(rec + 16);
+            for (int e = tid; e < nu * cs; e += NW * 32) {
+                const int ci = e % cs;
+                if (ci >= csn) continue;
+                const int sh = shift(ci);
+                const int2 v = es[e];
+                ((int2*)(ed + 4))[e] = make_int2(v.x + sh + (sh << 16), v.y + sh);
+            }
+        } else {
+            const int4* es = (const int4*)(rec + 16);
+            const int ng = cs / 4;
+            for (int e = tid; e < nu * ng; e += NW * 32) {
+                const int c = e % ng * 4;
+                if (c >= csn) continue;
+                const int s01 = shift(c) + (shift(c + 1) << 16), s23 = shift(c + 2) + (shift(c + 3) << 16);
+                const int4 v = es[e];
+                ((int4*)(ed + 4))[e] = make_int4(v.x + s01, v.y + s23, v.z + s01, v.w + s23);
+            }
         }
         const int nrows = hdr.x;
         const int4* desc = (const int4*)(rec + rg.desc_off);
-        // tasks of 64 quads (fp32 rows), one warp each
-        const int per = (hdr.z + 255) >> 8;
+        // tasks of 256 outputs or words (128 words from uint8 samples), one warp each
+        constexpr int kTask = KIND == kRowsU8 ? 128 : 256;
+        const int per = (hdr.z + kTask - 1) / kTask;
         const int dr = NW / per, dp = NW - dr * per;
         int r = warp / per, part = warp - r * per;
         for (; r < nrows; r += dr, part += dp, r += part >= per, part -= part >= per ? per : 0) {
@@ -316,8 +441,13 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
                             q.x + q.z + n <= cs * a.lcap,
                         a.status))
                 continue;
-            build_fir<TIN>(raw + q.x, (const float*)(rec + rg.w_off) + ((uint32_t)q.w >> 16), n, part * 256 + 4 * lane, q.z,
-                           (float*)half + q.y);
+            if constexpr (FIR)
+                build_fir<TIN>(raw + q.x, (const float*)(rec + rg.w_off) + ((uint32_t)q.w >> 16), n,
+                               part * kTask + 4 * lane, q.z, (float*)half + q.y);
+            else if constexpr (KIND == kRowsU8)
+                build_u8(raw + q.x, n, part * kTask + 4 * lane, q.z, half + q.y);
+            else
+                build_rl(raw + q.x, n, part * kTask + lane, q.z, half + q.y);
         }
     };
     auto parity_of = [&](int i) { return (uint32_t)(((MULTI ? ts.uses[0] : 0) + i) & 1); };
@@ -333,16 +463,43 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
         const uint32_t* half = sm.half + (i & 1) * half_words;
         if (d < a.ndm) {
             const int csn = sm.lo[a.nchan + 2 + i] - sm.lo[a.nchan + 1 + i];
-            const int2* ent = (const int2*)(half + a.blen + 4) + wu * cs;
-            __builtin_assume(__isShared(ent));
-            int2 next = ent[0];
+            if constexpr (FIR) {
+                const int2* ent = (const int2*)(half + a.blen + 4) + wu * cs;
+                __builtin_assume(__isShared(ent));
+                int2 next = ent[0];
 #pragma unroll 1
-            for (int ci = 0; ci < csn; ++ci) {
-                const int2 e = next;
-                next = ent[ci + 1];
-                if (!dbg_ok(max(max(e.x & 0xffff, (int)((uint32_t)e.x >> 16)), e.y) + lane_off + R + 4 <= a.blen, a.status))
-                    continue;
-                fir_channel((const float*)half, e, lane_off, sum);
+                for (int ci = 0; ci < csn; ++ci) {
+                    const int2 e = next;
+                    next = ent[ci + 1];
+                    if (!dbg_ok(max(max(e.x & 0xffff, (int)((uint32_t)e.x >> 16)), e.y) + lane_off + R + 4 <= a.blen,
+                                a.status))
+                        continue;
+                    fir_channel((const float*)half, e, lane_off, sum);
+                }
+            } else {
+                const uint4* ent = (const uint4*)(half + a.blen + 4) + wu * (cs / 4);
+                __builtin_assume(__isShared(ent));
+                const uint32_t* rows = half + lane_off;
+                int modes = ((const int4*)(half + a.blen))->y;
+#pragma unroll 1
+                for (int ci = 0; ci < csn; ci += 4, modes >>= 2) {
+                    const uint4 e = ent[ci / 4];
+                    if (!dbg_ok((int)max(max(max(e.x & 0xffffu, e.x >> 16), max(e.y & 0xffffu, e.y >> 16)),
+                                         max(max(e.z & 0xffffu, e.z >> 16), max(e.w & 0xffffu, e.w >> 16))) +
+                                        lane_off + R <= a.blen,
+                                a.status))
+                        continue;
+                    if ((modes & 3) == 0) {
+                        pk_channels<4>(rows, make_uint2(e.x, e.y), sum[0]);
+                        pk_channels<4>(rows, make_uint2(e.z, e.w), sum[1]);
+                    } else if ((modes & 3) == 1) {
+                        pk_channels<2>(rows, make_uint2(e.x, e.y), sum[0]);
+                        pk_channels<2>(rows, make_uint2(e.z, e.w), sum[1]);
+                    } else {
+                        pk_channels<1>(rows, make_uint2(e.x, e.y), sum[0]);
+                        pk_channels<1>(rows, make_uint2(e.z, e.w), sum[1]);
+                    }
+                }
             }
         }
         if (i + 1 < nst) {
@@ -365,22 +522,56 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
     if (!__syncthreads_and(ok)) return false;
     if (MULTI && tid == 0) ts.uses[0] += nst;
 
-    float f[NT][R];
+    if constexpr (FIR) {
+        float f[NT][R];
 #pragma unroll
-    for (int u = 0; u < NT; ++u) {
+        for (int u = 0; u < NT; ++u) {
 #pragma unroll
-        for (int j = 0; j < R / 2; ++j) unpk(sum[u].v[j], f[u][2 * j], f[u][2 * j + 1]);
-        f[u][R - 1] = sum[u].t;
+            for (int j = 0; j < R / 2; ++j) unpk(sum[u].v[j], f[u][2 * j], f[u][2 * j + 1]);
+            f[u][R - 1] = sum[u].t;
+        }
+        if constexpr (FUSED) {
+            fused::epilogue_f32<NT, R, NW>(a, *fa, smem, wu, chunk, lane, d, t0, *ft, f);
+            return true;
+        }
+        float* out = (float*)a.out;
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            store_row<float, R>(smem, f[u], warp, lane, tw, a.t_out,
+                                d + u < a.ndm ? out + (int64_t)(d + u) * a.out_ld : nullptr, a.out_ld, a.status);
+    } else {
+        // low and high sums: outputs tw + lane * R + r and kPkHalf later
+        int s[NT][2 * R];
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                s[u][r] = (int)(sum[u].whole[r] - (sum[u].hi[r] << 16));
+                s[u][R + r] = (int)sum[u].hi[r];
+            }
+        if constexpr (FUSED) {
+            fused::epilogue_pk<R, NW>(a, *fa, smem, wu, chunk, lane, d, t0, *ft, s);
+            return true;
+        }
+        int* st = (int*)smem + warp * TW;
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            if (d + u >= a.ndm) break;
+            int* out = (int*)a.out + (int64_t)(d + u) * a.out_ld;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                st[lane * R + r] = s[u][r];
+                st[kPkHalf + lane * R + r] = s[u][R + r];
+            }
+            __syncwarp();
+#pragma unroll 4
+            for (int j = 0; j < TW / 32; ++j) {
+                const int64_t t = tw + j * 32 + lane;
+                if (t < a.t_out && dbg_ok(t >= 0 && t < a.out_ld, a.status)) out[t] = st[j * 32 + lane];
+            }
+            __syncwarp();
+        }
     }
-    if constexpr (FUSED) {
-        fused::epilogue_f32<NT, R, NW>(a, *fa, smem, wu, chunk, lane, d, t0, *ft, f);
-        return true;
-    }
-    float* out = (float*)a.out;
-#pragma unroll
-    for (int u = 0; u < NT; ++u)
-        store_row<float, R>(smem, f[u], warp, lane, tw, a.t_out,
-                            d + u < a.ndm ? out + (int64_t)(d + u) * a.out_ld : nullptr, a.out_ld, a.status);
     if (MULTI) __syncthreads();  // the staging area is the next tile's stage buffers
     return true;
 }

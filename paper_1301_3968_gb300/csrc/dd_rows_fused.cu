@@ -54,18 +54,18 @@ int fused_bps(size_t smem) {
 
 }  // namespace
 
+#define DD_ROWS_NW(fn, kind, in8, nw, ...) \
+    ((nw) == kRowWarps ? fn<kind, in8, kRowWarps>(__VA_ARGS__) : fn<kind, in8, kWarps>(__VA_ARGS__))
+#define DD_ROWS(fn, p, ...)                                                                 \
+    ((p)->rk == kRowsRl            ? DD_ROWS_NW(fn, kRowsRl, false, (p)->row_warps, __VA_ARGS__)  \
+     : (p)->rk == kRowsU8          ? DD_ROWS_NW(fn, kRowsU8, true, (p)->row_warps, __VA_ARGS__)   \
+     : (p)->band.in_type == DD_U8 ? DD_ROWS_NW(fn, kRowsFir, true, (p)->row_warps, __VA_ARGS__)  \
+                                  : DD_ROWS_NW(fn, kRowsFir, false, (p)->row_warps, __VA_ARGS__))
+
 dd_status launch_rows_fused(const dd_plan_s* p, DedispArgs a, const FusedArgs& f, size_t smem, cudaStream_t s) {
-    const bool in8 = p->band.in_type == DD_U8;
-    if (p->row_warps == kRowWarps)
-        return in8 ? run_fused<kRowsFir, true, kRowWarps>(a, f, smem, s) : run_fused<kRowsFir, false, kRowWarps>(a, f, smem, s);
-    return in8 ? run_fused<kRowsFir, true, kWarps>(a, f, smem, s) : run_fused<kRowsFir, false, kWarps>(a, f, smem, s);
+    return DD_ROWS(run_fused, p, a, f, smem, s);
 }
 
-int rows_fused_blocks_per_sm(const dd_plan_s* p, size_t smem) {
-    const bool in8 = p->band.in_type == DD_U8;
-    if (p->row_warps == kRowWarps)
-        return in8 ? fused_bps<kRowsFir, true, kRowWarps>(smem) : fused_bps<kRowsFir, false, kRowWarps>(smem);
-    return in8 ? fused_bps<kRowsFir, true, kWarps>(smem) : fused_bps<kRowsFir, false, kWarps>(smem);
-}
+int rows_fused_blocks_per_sm(const dd_plan_s* p, size_t smem) { return DD_ROWS(fused_bps, p, smem); }
 
 }  // namespace dd

@@ -158,3 +158,101 @@ def test_fused_weighted_rows(dd, seed, D, steps, w0, w1, parts):
     p1, a1, _ = plan.dedisperse_boxcar(x, widths, mean, sd, nsamp=T)
     assert plan.device_status() == 0
     assert torch.equal(p0.view(torch.int32), p1.view(torch.int32)) and torch.equal(a0, a1)
+
+
+@pytest.mark.parametrize("method", ["direct", "runlength"])
+@pytest.mark.parametrize("seed,C,D,t_out,t_off,steps,tap_sets,group,nch", [
+    (51, 8, 32, 1088, 0, [0, 1, 2], [1, 2, 3, 4], 32, 1),          # one full tile and block
+    (52, 7, 33, 1089, 3, [0, 1, 9], [5, 6, 7, 8], 16, 1),          # one past both
+    (53, 3, 31, 1087, 17, [0, 40], [64, 65], 31, 1),               # one short of both
+    (54, 70, 100, 3000, 5, [0, 1, 2], [63, 64, 65, 66], 25, 1),    # four words' sums just fit, or two and two
+    (55, 41, 40, 2500, 1, [0, 3], [128, 129], 20, 1),              # two and two, or none
+    (56, 30, 37, 2200, 2, [0, 1], [254, 257], 37, 1),              # the longest runs
+    (57, 9, 20, 600, 0, [0, 1], [258], 20, 1),                     # one past: the tap kernels
+    (58, 21, 40, 4500, 0, [0, 2], [3, 200], 20, 2),                # two time chunks per CTA
+    (59, 5, 1, 40, 9, [1], [2], 1, 1),                             # one trial: no sharing
+    (60, 6, 6000, 1800, 0, [0, 1], [2, 6], 400, 1),                # 16 warps per CTA
+])
+@pytest.mark.parametrize("data", ["noise", "saturated"])
+def test_packed_rows_bit_exact(dd, method, seed, C, D, t_out, t_off, steps, tap_sets, group, nch, data):
+    """uint8 sums equal the oracle's, with every sample at 255 too (the largest half words)."""
+    import torch
+    rng = np.random.default_rng(seed)
+    delay, taps = _tables(rng, D, C, steps, tap_sets, group)
+    T = t_out + int((delay + taps - 1).max())
+    ld = (T + t_off + 15) // 16 * 16
+    I = _input(rng, "u8", C, ld) if data == "noise" else np.full((C, ld), 255, np.uint8)
+    plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, T, "u8"), np.zeros(D))
+    plan.set_profiles(delay=delay, taps=taps)
+    plan.set_method(method)
+    if nch > 1:
+        plan.set_schedule(nch, 3)
+        assert plan.schedule()["nch"] == nch
+    got = plan.dedisperse(torch.from_numpy(I).cuda(), t_offset=t_off, nsamp=T).cpu().numpy()
+    assert plan.device_status() == 0
+    rows = sorted(set(rng.integers(0, D, size=12).tolist() + [0, D - 1]))
+    want = oracle.c_dedisperse(I, delay, taps, t_offset=t_off, nsamp=T, rows=rows)
+    np.testing.assert_array_equal(got[rows].astype(np.int64), want)
+
+
+@pytest.mark.parametrize("method", ["direct", "runlength"])
+@pytest.mark.parametrize("seed,D,steps,w0,w1,parts,nch", [
+    (71, 100, [0, 1, 2], 1, 32, 0, 1),
+    (72, 49, [0, 1, 4], 5, 90, 7, 1),     # pruned width groups
+    (73, 2400, [0, 1], 1, 256, 0, 1),     # 16 warps per CTA
+    (74, 60, [0, 1], 960, 993, 5, 1),     # the longest carry a plan takes
+    (75, 40, [0, 2], 1, 70, 4, 2),        # two time chunks per CTA
+])
+def test_fused_packed_rows(dd, method, seed, D, steps, w0, w1, parts, nch):
+    """Fused = unfused, bit for bit, ties (constant channels) included."""
+    import torch
+    rng = np.random.default_rng(seed)
+    C, t_out = 10, 6500
+    delay, taps = _tables(rng, D, C, steps, [2, 3, 7], (D + 1) // 2)
+    T = t_out + int((delay + taps - 1).max())
+    plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, T, "u8"), np.zeros(D))
+    plan.set_profiles(delay=delay, taps=taps)
+    plan.set_method(method)
+    if nch > 1:
+        plan.set_schedule(nch, 4)
+    I = np.clip(rng.normal(128, 3, size=(C, (T + 15) // 16 * 16)), 0, 255).astype(np.uint8)
+    I[:, 2000:3500] = 128
+    x = torch.from_numpy(I).cuda()
+    mean, sd = plan.channel_stats(x, nsamp=T)
+    widths = np.arange(w0, w1 + 1, dtype=np.int32)
+    plan.test_set_fused_parts(parts)
+    p0, a0, _ = plan.boxcar_snr(plan.dedisperse(x, nsamp=T), widths, mean, sd)
+    p1, a1, _ = plan.dedisperse_boxcar(x, widths, mean, sd, nsamp=T)
+    assert plan.device_status() == 0
+    assert torch.equal(p0.view(torch.int32), p1.view(torch.int32)) and torch.equal(a0, a1)
+
+
+def test_batch_of_rows_and_taps(dd):
+    """Beams of the row kernels (8 and 16 warps per CTA) and of the tap kernel in one batch, and
+    the graph of it, equal the beams' own launches."""
+    import torch
+    rng = np.random.default_rng(81)
+    C = 16
+    plans, xs, outs = [], [], []
+    for D, T, group in ((40, 2500, 40), (5000, 2600, 500), (30, 2300, 1)):
+        delay, taps = _tables(rng, D, C, [0, 1], list(range(1, 20)), group)
+        delay %= 60
+        p = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, T, "u8"), np.zeros(D))
+        p.set_profiles(delay=delay, taps=taps)
+        p.set_method("direct")
+        plans.append(p)
+        xs.append(torch.from_numpy(_input(rng, "u8", C, (T + 15) // 16 * 16)).cuda())
+        outs.append(torch.zeros((D, T - p.d_max), dtype=torch.int32, device="cuda"))
+    assert len({p.schedule()["trials_per_cta"] for p in plans}) == 3
+    batch = dd.Batch(plans)
+    batch.bind(xs, outs)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    batch.capture(s)
+    for o in outs:
+        o.zero_()
+    torch.cuda.synchronize()
+    batch.replay(s)
+    s.synchronize()
+    for p, x, o in zip(plans, xs, outs):
+        assert torch.equal(p.dedisperse(x, nsamp=p.band.nsamp), o)
