@@ -6,6 +6,8 @@
 //   sigma_dw^2 = sum_c sigma_c^2 Q_dc(w),  Q_dc(w) = || w_dc (*) 1_w ||^2
 //
 // All reductions run in a fixed order, so results are deterministic.
+#include <cooperative_groups.h>
+
 #include <cfloat>
 #include <type_traits>
 #include <climits>
@@ -42,36 +44,90 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float a) {
     hi = s;
 }
 
+// The kernel waits for memory, so a channel's row is spread over a cluster of CTAs, as many as
+// the device holds at once (stat_split); CTA 0 adds their sums in rank order.  fp32: 336 x 65536
+// samples in 126 us with one CTA of 256 threads per channel, 84 with 1024 (336 CTAs are two
+// waves), 75 with two of 256; uint8: 1024 x 200516 samples in 85 us with single bytes, 42 with
+// 16-byte loads.
+constexpr int kStatThreads = 256;
+constexpr int kStatSplitMax = 8;  // portable cluster size
+
 template <typename TIN>
-__global__ void __launch_bounds__(256) k_chan_stats(const TIN* in, int64_t ld, int64_t t_offset,
-                                                    int64_t n, double* mean, double* sd) {
-    const int c = blockIdx.x;
+__global__ void __launch_bounds__(kStatThreads) k_chan_stats(const TIN* in, int64_t ld, int64_t t_offset,
+                                                               int64_t n, double* mean, double* sd) {
+    constexpr int NT = kStatThreads, NWP = NT / 32;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int c = blockIdx.y, rank = (int)cluster.block_rank(), nr = (int)cluster.num_blocks();
     const TIN* row = in + (int64_t)c * ld + t_offset;
-    __shared__ double sh1[8], sh2[8];
-    __shared__ long long si1[8], si2[8];
+    using Sum = typename std::conditional<sizeof(TIN) == 1, long long, double>::type;
+    __shared__ Sum wsum[2][NWP], part[2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (sizeof(TIN) == 1) {
-        long long s1 = 0, s2 = 0;
-        for (int64_t t = threadIdx.x; t < n; t += blockDim.x) {
-            long long v = (long long)row[t];
-            s1 += v;
-            s2 += v * v;
-        }
+    // the cluster's sums, in thread 0 of rank 0 (fixed order: warps, then ranks)
+    auto sums = [&](Sum& s1, Sum& s2) {
         s1 = warp_sum(s1);
         s2 = warp_sum(s2);
         if (lane == 0) {
-            si1[warp] = s1;
-            si2[warp] = s2;
+            wsum[0][warp] = s1;
+            wsum[1][warp] = s2;
         }
         __syncthreads();
         if (threadIdx.x == 0) {
-            long long a = 0, b = 0;
-            for (int i = 0; i < 8; ++i) {
-                a += si1[i];
-                b += si2[i];
+            s1 = s2 = 0;
+            for (int i = 0; i < NWP; ++i) {
+                s1 += wsum[0][i];
+                s2 += wsum[1][i];
             }
-            const double m = (double)a / (double)n;
-            double var = (double)b / (double)n - m * m;
+            part[0] = s1;
+            part[1] = s2;
+        }
+        cluster.sync();
+        if (rank == 0 && threadIdx.x == 0)
+            for (int r = 1; r < nr; ++r) {
+                const Sum* q = cluster.map_shared_rank(part, r);
+                s1 += q[0];
+                s2 += q[1];
+            }
+        cluster.sync();  // the other CTAs' shared memory has been read
+    };
+    if constexpr (sizeof(TIN) == 1) {
+        // single bytes up to a 16-byte boundary and after the last, 16 at a time between; a
+        // word's sum and sum of squares by byte dot products, 32-bit partial sums of 64 words
+        long long s1 = 0, s2 = 0;
+        const int64_t head = min(n, (int64_t)((16 - ((uintptr_t)row & 15)) & 15));
+        const int64_t nvec = (n - head) / 16;
+        const uint4* v = (const uint4*)(row + head);
+        auto byte = [&](int64_t t) {
+            const long long x = (long long)row[t];
+            s1 += x;
+            s2 += x * x;
+        };
+        const int64_t step = (int64_t)NT * nr, me = (int64_t)rank * NT + threadIdx.x;
+        if (me < head) byte(me);
+        for (int64_t t = head + 16 * nvec + me; t < n; t += step) byte(t);
+        for (int64_t i0 = me; i0 < nvec; i0 += step * 16) {
+            uint32_t a1 = 0, a2 = 0;
+#pragma unroll 4
+            for (int k = 0; k < 16; ++k) {
+                const int64_t i = i0 + k * step;
+                if (i >= nvec) break;
+                const uint4 q = v[i];
+                a1 = __dp4a(q.x, 0x01010101u, a1);
+                a2 = __dp4a(q.x, q.x, a2);
+                a1 = __dp4a(q.y, 0x01010101u, a1);
+                a2 = __dp4a(q.y, q.y, a2);
+                a1 = __dp4a(q.z, 0x01010101u, a1);
+                a2 = __dp4a(q.z, q.z, a2);
+                a1 = __dp4a(q.w, 0x01010101u, a1);
+                a2 = __dp4a(q.w, q.w, a2);
+            }
+            s1 += a1;
+            s2 += a2;
+        }
+        sums(s1, s2);
+        if (rank == 0 && threadIdx.x == 0) {
+            const double m = (double)s1 / (double)n;
+            double var = (double)s2 / (double)n - m * m;
             mean[c] = m;
             sd[c] = sqrt(var > 0 ? var : 0.0);
         }
@@ -87,11 +143,12 @@ __global__ void __launch_bounds__(256) k_chan_stats(const TIN* in, int64_t ld, i
         __syncthreads();
         const float x0 = sx0;
         double s1 = 0, s2 = 0;
-        for (int64_t t0 = threadIdx.x; t0 < n; t0 += (int64_t)blockDim.x * 32) {
+        const int64_t step = (int64_t)NT * nr;
+        for (int64_t t0 = (int64_t)rank * NT + threadIdx.x; t0 < n; t0 += step * 32) {
             float h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
 #pragma unroll 8
             for (int k = 0; k < 32; ++k) {
-                const int64_t t = t0 + (int64_t)k * blockDim.x;
+                const int64_t t = t0 + k * step;
                 const float x = t < n ? (float)row[t] : x0;
                 // x - x0 = vh + vl exactly (TwoSum)
                 const float vh = x - x0;
@@ -107,21 +164,10 @@ __global__ void __launch_bounds__(256) k_chan_stats(const TIN* in, int64_t ld, i
             s1 += (double)h1 + (double)l1;
             s2 += (double)h2 + (double)l2;
         }
-        s1 = warp_sum(s1);
-        s2 = warp_sum(s2);
-        if (lane == 0) {
-            sh1[warp] = s1;
-            sh2[warp] = s2;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double a = 0, b = 0;
-            for (int i = 0; i < 8; ++i) {
-                a += sh1[i];
-                b += sh2[i];
-            }
-            const double m = a / (double)n;
-            double var = b / (double)n - m * m;
+        sums(s1, s2);
+        if (rank == 0 && threadIdx.x == 0) {
+            const double m = s1 / (double)n;
+            double var = s2 / (double)n - m * m;
             mean[c] = (double)x0 + m;
             sd[c] = sqrt(var > 0 ? var : 0.0);
         }
@@ -284,7 +330,8 @@ struct BoxArgs {
     const uint8_t* narrow;
     int32_t narrow_sel;
     int32_t* status;  // the plan's device status word (debug-build bounds checks)
-    int32_t gpc;      // k_boxcar_run: width groups per CTA (1, 2, 4 or 8)
+    int32_t gpc;      // contiguous widths: width groups per CTA (1, 2, 4 or 8)
+    int32_t pre;      // k_boxcar_run on integers: segments' first sums from prefix sums
 };
 
 template <typename T>
@@ -295,6 +342,19 @@ template <>
 __device__ __forceinline__ int lowest<int>() { return INT_MIN; }
 template <>
 __device__ __forceinline__ long long lowest<long long>() { return LLONG_MIN; }
+
+// The warp's largest value (every lane returns it).
+__device__ __forceinline__ int warp_top(int v) { return __reduce_max_sync(0xffffffffu, v); }
+__device__ __forceinline__ float warp_top(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+__device__ __forceinline__ long long warp_top(long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
 
 constexpr int kBoxS = kBoxSeg;  // samples per thread segment
 constexpr int kBoxG = 16;  // widths per CTA
@@ -449,14 +509,13 @@ __device__ __forceinline__ typename Acc<TB>::U to_acc(TX v) {
 
 // xl: the thread's staged samples (raw series values); o: the trial's offset, taken
 // off each sample as it is read.
+// q: the sum of the first w0 of them.
 template <typename TX, typename TB, bool FULL>
-__device__ __forceinline__ void run_segment(const TX* xl, TX o, int w0, int t0, int t_len,
+__device__ __forceinline__ void run_segment(const TX* xl, TX o, typename Acc<TB>::U q, int w0, int t0, int t_len,
                                             TB (&seg)[kBoxG]) {
     constexpr int S = kBoxS, G = kBoxG;
     using U = typename Acc<TB>::U;
     U p = U(0);
-    U q = U(0);
-    for (int k = 0; k < w0; ++k) q += to_acc<TX, TB>((TX)(xl[k] - o));
     U win[G];
     win[0] = q;
 #pragma unroll
@@ -494,6 +553,9 @@ __device__ __forceinline__ void run_segment(const TX* xl, TX o, int w0, int t0, 
 // segments still start at multiples of S (chunks are whole segments).  fp32: three CTAs
 // per SM (80 registers, 72 bytes spilled), 8 % faster than two with no spills on the
 // CRAFT-like series (1.283 -> 1.185 ms with the normaliser).
+// Bound by instruction issue: about 2.8 per (start, width), 1.5 of them the subtraction and half
+// the three-input maximum.  Packed subtractions (two widths per add.rn.f32x2) or the offset taken
+// off the staged chunk once did not pay (943 and 826 us against 777 on 4096 x 60261 x 32).
 template <typename TX, typename TB>
 __global__ void __launch_bounds__(256, std::is_same<TB, float>::value ? 3 : 2) k_boxcar_run(BoxArgs a) {
     constexpr int S = kBoxS, G = kBoxG;
@@ -502,6 +564,7 @@ __global__ void __launch_bounds__(256, std::is_same<TB, float>::value ? 3 : 2) k
     __shared__ TB rb[8][G];
     __shared__ int rc[8][G];
     __shared__ int rt[8][G];
+    __shared__ uint32_t psum[8];
     const int d = blockIdx.y;
     if (a.narrow && (int)a.narrow[d] != a.narrow_sel) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -522,6 +585,10 @@ __global__ void __launch_bounds__(256, std::is_same<TB, float>::value ? 3 : 2) k
     const int bufl = (chunk + w0_last + G + 4 + 3) & ~3;
     TX* const xs0 = (TX*)smem_raw;
     TX* const xs1 = xs0 + bufl;
+    // integers, many width groups: prefix sums of the chunk, so that a segment's first sum of
+    // w0 samples is one difference instead of w0 additions per group (exact modulo 2^32)
+    constexpr bool INT32 = std::is_same<TB, int>::value;
+    uint32_t* const pre = (uint32_t*)(xs1 + bufl);
     const int wlast = w0 + cnt - 1;
     const TX o = (TX)a.off[d];
     const TX* xrow = (const TX*)a.x + (int64_t)d * a.ld;
@@ -569,13 +636,54 @@ __global__ void __launch_bounds__(256, std::is_same<TB, float>::value ? 3 : 2) k
             cp_async_wait<0>();
         }
         __syncthreads();
+        if constexpr (INT32) {
+            if (a.pre) {  // consecutive quads per thread, their sums scanned over the CTA
+                const int n16 = (stage + mis + 3) >> 2, per = (n16 + 255) >> 8;
+                const int q0 = min(n16, tid * per), q1 = min(n16, q0 + per);
+                uint32_t sum = 0;
+                for (int i = q0; i < q1; ++i) {
+                    const int4 v = ((const int4*)xs)[i];
+                    sum += (uint32_t)v.x + (uint32_t)v.y + (uint32_t)v.z + (uint32_t)v.w - 4u * (uint32_t)o;
+                }
+                uint32_t incl = sum;
+#pragma unroll
+                for (int ofs = 1; ofs < 32; ofs <<= 1) {
+                    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, ofs);
+                    if (lane >= ofs) incl += v;
+                }
+                if (lane == 31) psum[warp] = incl;
+                __syncthreads();
+                uint32_t run = incl - sum;
+#pragma unroll
+                for (int w = 0; w < 8; ++w) run += w < warp ? psum[w] : 0u;
+                for (int i = q0; i < q1; ++i) {
+                    const int4 v = ((const int4*)xs)[i];
+                    uint4 r;
+                    r.x = run;
+                    r.y = r.x + (uint32_t)(v.x - o);
+                    r.z = r.y + (uint32_t)(v.y - o);
+                    r.w = r.z + (uint32_t)(v.z - o);
+                    run = r.w + (uint32_t)(v.w - o);
+                    ((uint4*)pre)[i] = r;
+                }
+                __syncthreads();
+            }
+        }
         TB seg[G];
 #pragma unroll
         for (int j = 0; j < G; ++j) seg[j] = lowest<TB>();
-        if (active && tc + chunk - 1 + wlast <= a.t_len)
-            run_segment<TX, TB, true>(xs + mis + ls, o, w0, tc + ls, a.t_len, seg);
-        else if (active && tc + ls < tvalid)
-            run_segment<TX, TB, false>(xs + mis + ls, o, w0, tc + ls, a.t_len, seg);
+        if (active && tc + ls < tvalid) {
+            const TX* xl = xs + mis + ls;
+            U q = U(0);
+            if (INT32 && a.pre)
+                q = (U)(pre[mis + ls + w0] - pre[mis + ls]);
+            else
+                for (int k = 0; k < w0; ++k) q += to_acc<TX, TB>((TX)(xl[k] - o));
+            if (tc + chunk - 1 + wlast <= a.t_len)
+                run_segment<TX, TB, true>(xl, o, q, w0, tc + ls, a.t_len, seg);
+            else
+                run_segment<TX, TB, false>(xl, o, q, w0, tc + ls, a.t_len, seg);
+        }
 #pragma unroll
         for (int j = 0; j < G; ++j) {
             if (seg[j] > best[j]) {
@@ -588,24 +696,15 @@ __global__ void __launch_bounds__(256, std::is_same<TB, float>::value ? 3 : 2) k
     // (max, earliest chunk, earliest thread) over each group's warps
 #pragma unroll
     for (int j = 0; j < G; ++j) {
-        TB b = best[j];
-        int c = bch[j];
-        int t = gt;
-#pragma unroll
-        for (int ofs = 16; ofs > 0; ofs >>= 1) {
-            const TB ob = __shfl_xor_sync(0xffffffffu, b, ofs);
-            const int oc = __shfl_xor_sync(0xffffffffu, c, ofs);
-            const int ot = __shfl_xor_sync(0xffffffffu, t, ofs);
-            if (oc >= 0 && (c < 0 || ob > b || (ob == b && (oc < c || (oc == c && ot < t))))) {
-                b = ob;
-                c = oc;
-                t = ot;
-            }
-        }
+        const TB b = warp_top(best[j]);
+        // the lanes that hold it, by chunk, then by thread (in lane order)
+        const uint32_t c = best[j] == b ? (uint32_t)bch[j] : 0xffffffffu;  // (-1: none)
+        const uint32_t cm = __reduce_min_sync(0xffffffffu, c);
+        const uint32_t who = __ballot_sync(0xffffffffu, c == cm);
         if (lane == 0) {
             rb[warp][j] = b;
-            rc[warp][j] = c;
-            rt[warp][j] = t;
+            rc[warp][j] = (int)cm;
+            rt[warp][j] = gt + __ffs(who) - 1;
         }
     }
     __syncthreads();
@@ -669,8 +768,11 @@ dd_status run_boxcar_contig(const BoxArgs& a0, int w0_last, cudaStream_t s) {
     BoxArgs a = a0;
     const int ng = (a.nw + kBoxG - 1) / kBoxG;
     a.gpc = ng >= 8 ? 8 : (ng >= 4 ? 4 : (ng >= 2 ? 2 : 1));
+    // (w0 additions per segment and group against some 60 instructions for the prefix sums:
+    // widths 1-256 on 8192 x 65536 12.86 -> 12.0 ms; wider lists keep their two buffers)
+    a.pre = std::is_same<TB, int>::value && w0_last > 48 && w0_last <= 8192;
     const int chunk = 32 * (8 / a.gpc) * kBoxS;
-    const size_t smem = (size_t)2 * ((chunk + w0_last + kBoxG + 4 + 3) & ~3) * sizeof(TX);
+    const size_t smem = (size_t)(a.pre ? 3 : 2) * ((chunk + w0_last + kBoxG + 4 + 3) & ~3) * sizeof(TX);
     auto kern = k_boxcar_run<TX, TB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e);
@@ -718,8 +820,10 @@ __global__ void __launch_bounds__(256) k_row_narrow(const int* x, int64_t ld, in
     }
 }
 
-static dd_status dispatch_boxcar(const dd_plan_s* p, const BoxArgs& a, const int32_t* widths,
+static dd_status dispatch_boxcar(const dd_plan_s* p, const BoxArgs& a0, const int32_t* widths,
                                  int32_t nw, cudaStream_t s, bool split_rows) {
+    BoxArgs a = a0;
+    a.pre = 0;
     const int wmax = widths[nw - 1];
     bool contig = true;
     for (int j = 1; j < nw; ++j) contig = contig && widths[j] == widths[0] + j;
@@ -749,11 +853,27 @@ static dd_status dispatch_boxcar(const dd_plan_s* p, const BoxArgs& a, const int
 
 dd_status launch_channel_stats(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                                int64_t nsamp, double* mean, double* sd, cudaStream_t s) {
+    // CTAs per channel: a power of two that 152 SMs hold at once (eight CTAs each), and no more
+    // than leave every thread a load of 16 bytes
+    const int64_t bytes = nsamp * (p->band.in_type == DD_U8 ? 1 : 4);
+    int split = 1;
+    while (split < kStatSplitMax && 2 * split * p->nchan <= 152 * 8 && bytes >= 2 * split * kStatThreads * 16) split *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.gridDim = dim3((unsigned)split, (unsigned)p->nchan);
+    cfg.blockDim = dim3(kStatThreads);
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)split;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaError_t e;
     if (p->band.in_type == DD_U8)
-        k_chan_stats<uint8_t><<<p->nchan, 256, 0, s>>>((const uint8_t*)in, ld, t_offset, nsamp, mean, sd);
+        e = cudaLaunchKernelEx(&cfg, k_chan_stats<uint8_t>, (const uint8_t*)in, ld, t_offset, nsamp, mean, sd);
     else
-        k_chan_stats<float><<<p->nchan, 256, 0, s>>>((const float*)in, ld, t_offset, nsamp, mean, sd);
-    return cuda_status(cudaGetLastError());
+        e = cudaLaunchKernelEx(&cfg, k_chan_stats<float>, (const float*)in, ld, t_offset, nsamp, mean, sd);
+    return cuda_status(e);
 }
 
 static dd_status ensure_norm_ws(dd_plan_s* p, int nw) {
