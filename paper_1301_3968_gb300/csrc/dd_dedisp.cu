@@ -32,6 +32,17 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_dedisp(DedispArgs a) {
     }
 }
 
+// Small launches (see run_unit): grid (time tiles of 8 x 32 kRSmall outputs, trial blocks, pair
+// units of a block).
+template <typename TIN, int NBUF>
+__global__ void __launch_bounds__(kWarps * 32, 2) k_dedisp_unit(DedispArgs a) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ TileState ts;
+    if (threadIdx.x == 0) init_pipeline<NBUF>(pipeline_area(smem, a.smem_bytes, NBUF), ts);
+    __syncthreads();
+    dedisp_tile<TIN, true, NBUF, false, 0, false, true>(a, smem, blockIdx.y, blockIdx.x, ts);
+}
+
 // Batched form: one CTA per work item (beam, trial block, time tile) of the list, in list
 // order (beams by decreasing cost, each in the plain grid's tile order); the hardware
 // starts CTAs in index order as earlier ones finish, which balances uneven beams.
@@ -70,6 +81,28 @@ dd_status run(DedispArgs a, cudaStream_t s) {
     dim3 grid(blk_x ? nblk : ntile, blk_x ? ntile : nblk, (unsigned)a.nsplit);
     if (grid.y > 65535 || a.nsplit < 1 || a.nsplit > 64) return DD_ERR_UNSUPPORTED;
     if ((int64_t)grid.x * grid.y >= INT32_MAX) return DD_ERR_UNSUPPORTED;  // the tile index is int
+    kern<<<grid, kWarps * 32, smem, s>>>(a);
+    return cuda_status(cudaGetLastError());
+}
+
+// A tap launch of at most kUnitCtas CTAs: one CTA per pair unit and 768 outputs instead of per
+// eight units and 864.  A trial's outputs then run on eight warps of one SM, and the blocks'
+// units on SMs of their own; each CTA stages the rows for itself, which costs more copies than
+// it saves once the SMs are full.  One trial x 64 channels x 841 outputs x 32 taps: 36 us
+// against 119.
+constexpr int64_t kUnitCtas = 76;  // half the SMs
+
+template <typename TIN, int NBUF>
+dd_status run_unit(DedispArgs a, cudaStream_t s) {
+    const size_t smem = smem_for<TIN, true, NBUF>(a.lcap, a.kpad, a.cs, a.nch, a.nchan);
+    a.smem_bytes = (uint32_t)smem;
+    auto kern = k_dedisp_unit<TIN, NBUF>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_status(e);
+    const int nu = kWarps / a.nch, tile = kWarps * 32 * kRSmall;
+    const int nblk = (a.ndm + 2 * nu - 1) / (2 * nu);
+    // (the last block's units past the trial list leave at once)
+    dim3 grid((unsigned)((a.t_out + tile - 1) / tile), (unsigned)nblk, (unsigned)std::min(nu, (a.ndm + 1) / 2));
     kern<<<grid, kWarps * 32, smem, s>>>(a);
     return cuda_status(cudaGetLastError());
 }
@@ -321,6 +354,9 @@ dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_
     const bool u8 = p->band.in_type == DD_U8;
     if (!p->pair)
         return p->kmax <= kRInt ? run<uint8_t, false, kStagesInt, 1>(a, s) : run<uint8_t, false, kStagesInt>(a, s);
+    const int64_t tile = (int64_t)chunk_t(true) * a.nch, db = 2 * (kWarps / a.nch);
+    if (nsplit == 1 && (t_out + tile - 1) / tile * ((p->ndm + db - 1) / db) <= kUnitCtas)
+        return u8 ? run_unit<uint8_t, kStagesPair>(a, s) : run_unit<float, kStagesPair>(a, s);
     // union windows of at most R taps: one unrolled pass; at most 2R: two; longer: a loop
     const int passes = p->umax <= kRPair ? 1 : (p->umax <= 2 * kRPair ? 2 : 0);
     if (u8) {

@@ -19,6 +19,7 @@ namespace dd {
 constexpr int kWarps = 8;
 constexpr int kRPair = 27;
 constexpr int kRInt = 31;
+constexpr int kRSmall = 3;                 // small fp32 launches (dd_tile.cuh, UNIT)
 constexpr int kRMax = 31;
 __host__ __device__ constexpr int lane_r(bool pair) { return pair ? kRPair : kRInt; }
 __host__ __device__ constexpr int chunk_t(bool pair) { return 32 * lane_r(pair); }

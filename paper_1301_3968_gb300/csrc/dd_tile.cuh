@@ -221,6 +221,42 @@ __device__ void issue_stage(const DedispArgs& a, const StageGeom& g, const Smem&
     sm.issued[b] += 1;
 }
 
+// issue_stage by a whole warp, one lane per channel (UNIT): a small launch's windows mostly run
+// past the end of the rows, and zeroing them is then a good part of a stage's time.
+template <typename TIN, int NBUF>
+__device__ void issue_stage_warp(const DedispArgs& a, const StageGeom& g, const Smem& sm, int blk, int stage, int b,
+                                 int64_t base, int lane) {
+    constexpr int Q = Elem<TIN>::Q;
+    if (stage == a.skip_stage) return;  // test hook: this stage is never filled
+    unsigned char* buf = sm.stages + b * g.bytes;
+    const int c0 = stage * a.cs;
+    const int csn = min(a.cs, a.nchan - c0);
+    const int nst = (a.nchan + a.cs - 1) / a.cs;
+    int nin = 0;  // (at most 32 channels per stage)
+    int64_t a0 = 0;
+    if (lane < csn) {
+        a0 = (base + sm.lo_all[c0 + lane]) & ~(int64_t)(Q - 1);
+        nin = (int)max((int64_t)0, min((int64_t)a.lcap, a.ld - a0));
+        if (!dbg_ok(a0 >= 0 && (int64_t)csn * a.lcap * sizeof(TIN) <= g.rows_bytes, a.status)) nin = 0;
+        uint4* z = (uint4*)(buf + ((int64_t)lane * a.lcap + nin) * sizeof(TIN));
+        for (int k = 0; k < (int)((a.lcap - nin) * sizeof(TIN) / 16); ++k) z[k] = make_uint4(0, 0, 0, 0);
+        fence_proxy_async();
+    }
+    int bytes = nin * (int)sizeof(TIN);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) bytes += __shfl_xor_sync(0xffffffffu, bytes, o);
+    if (lane == 0) {
+        mbar_expect_tx(&sm.full[b], (uint32_t)(bytes + g.rec_bytes));
+        sm.issued[b] += 1;
+    }
+    __syncwarp();
+    if (nin > 0)
+        bulk_g2s(buf + (int64_t)lane * a.lcap * sizeof(TIN), (const TIN*)a.in + (int64_t)(c0 + lane) * a.ld + a0,
+                 (uint32_t)(nin * sizeof(TIN)), &sm.full[b]);
+    if (lane == 0)
+        bulk_g2s(buf + g.rec_off, a.rec + ((int64_t)blk * nst + stage) * g.rec_bytes, (uint32_t)g.rec_bytes, &sm.full[b]);
+}
+
 // One stage of one warp unit, exact integer sums of uint8 samples with unit weights:
 // for each of the stage's channels a register window of R samples slides along the
 // taps.  At tap k output r reads window sample r + k, held in register (r + k) mod R;
@@ -314,10 +350,9 @@ __device__ __forceinline__ void stage_rl_rows(const uint32_t* brows, const int2*
 // taps, in a fixed order (deterministic); single-precision accumulation of the
 // ~10^3-10^4 terms of an output stays orders of magnitude inside the 1e-5 scale-aware
 // bound.
-template <typename TIN, int SHORT, bool SHIFT>
+template <typename TIN, int SHORT, bool SHIFT, int R>
 __device__ __forceinline__ void pair_channel(const TIN* p, int s, int n, const uint64_t* wk,
-                                             uint64_t (&acc)[kRPair]) {
-    constexpr int R = kRPair;
+                                             uint64_t (&acc)[R]) {
     const TIN* p2 = p + s;  // trial 1's run
     auto ld = [&](int j) -> uint64_t {
         if constexpr (SHIFT) return pk2((float)p[j], (float)p2[j]);
@@ -361,19 +396,57 @@ __device__ __forceinline__ void pair_channel(const TIN* p, int s, int n, const u
     }
 }
 
+// pair_channel for a few outputs per lane (UNIT): the weights and samples of 16 taps are loaded
+// before their multiply-adds, whose chains alone are too short to hide the loads.
+template <typename TIN, bool SHIFT, int R>
+__device__ __forceinline__ void pair_channel_few(const TIN* p, int s, int n, const uint64_t* wk, uint64_t (&acc)[R]) {
+    constexpr int B = 16;
+    const TIN* p2 = p + s;
+    auto ld = [&](int j) -> uint64_t {
+        if constexpr (SHIFT) return pk2((float)p[j], (float)p2[j]);
+        else return pk_dup((float)p[j]);
+    };
+    int k = 0;
+#pragma unroll 1
+    for (; k + B <= n; k += B) {
+        uint64_t w[B], x[B + R - 1];
+#pragma unroll
+        for (int i = 0; i < B; ++i) w[i] = wk[k + i];
+#pragma unroll
+        for (int i = 0; i < B + R - 1; ++i) x[i] = ld(k + i);
+#pragma unroll
+        for (int i = 0; i < B; ++i)
+#pragma unroll
+            for (int r = 0; r < R; ++r) fma2(acc[r], w[i], x[i + r]);
+    }
+    if (k < n) {  // the last taps (loads stay inside the run)
+        uint64_t w[B], x[B + R - 1];
+        const int last = n - 1;
+#pragma unroll
+        for (int i = 0; i < B; ++i) w[i] = wk[min(k + i, last)];
+#pragma unroll
+        for (int i = 0; i < B + R - 1; ++i) x[i] = ld(min(k + i, last + R - 1));
+#pragma unroll
+        for (int i = 0; i < B; ++i)
+            if (k + i < n)
+#pragma unroll
+                for (int r = 0; r < R; ++r) fma2(acc[r], w[i], x[i + r]);
+    }
+}
+
 // One stage of one pair unit: its entries are (trial 0's start - block minimum,
 // max(n0, n1), trial 1's start - trial 0's, offset of the entry's weight pairs in the
 // record's weight list).
-template <typename TIN, int SHORT>
+template <typename TIN, int SHORT, int R>
 __device__ __forceinline__ void stage_pair(const TIN* rows, const int4* ent, const float2* wts,
                                            const int* lo, int csn, int lcap, int bq,
-                                           int lane_off, uint64_t (&acc)[kRPair], int wpairs,
+                                           int lane_off, uint64_t (&acc)[R], int wpairs,
                                            int32_t* status) {
     constexpr int Q = Elem<TIN>::Q;
     for (int ci = 0; ci < csn; ++ci) {
         const int4 q = ent[ci];
         const int i0 = ((bq + lo[ci]) & (Q - 1)) + q.x + lane_off;
-        if (!dbg_ok(q.x >= 0 && q.y >= 1 && i0 + min(q.z, 0) >= 0 && i0 + max(q.z, 0) + kRPair + q.y <= lcap &&
+        if (!dbg_ok(q.x >= 0 && q.y >= 1 && i0 + min(q.z, 0) >= 0 && i0 + max(q.z, 0) + R + q.y <= lcap &&
                         q.w >= 0 && q.w + q.y <= wpairs,
                     status))
             continue;
@@ -381,10 +454,13 @@ __device__ __forceinline__ void stage_pair(const TIN* rows, const int4* ent, con
         const uint64_t* wk = (const uint64_t*)(wts + q.w);
         __builtin_assume(__isShared(p));
         __builtin_assume(__isShared(wk));
-        if (q.z == 0)
-            pair_channel<TIN, SHORT, false>(p, 0, q.y, wk, acc);
+        if constexpr (R < 8) {
+            if (q.z == 0) pair_channel_few<TIN, false, R>(p, 0, q.y, wk, acc);
+            else pair_channel_few<TIN, true, R>(p, q.z, q.y, wk, acc);
+        } else if (q.z == 0)
+            pair_channel<TIN, SHORT, false, R>(p, 0, q.y, wk, acc);
         else
-            pair_channel<TIN, SHORT, true>(p, q.z, q.y, wk, acc);
+            pair_channel<TIN, SHORT, true, R>(p, q.z, q.y, wk, acc);
     }
 }
 
@@ -420,11 +496,15 @@ struct TileState {
 // FUSED: instead of storing the tile, scan it for boxcar maxima (fa: the scan's
 // arguments, ft: the strip the tile belongs to); exact sums on the integer paths, the
 // unfused fp32 scan's prefix chains on the pair path.
-template <typename TIN, bool PAIR, int NBUF, bool MULTI, int SHORT, bool FUSED = false>
+// UNIT: the CTA's warps all sum one pair unit (blockIdx.z) of the trial block, kRSmall outputs
+// per lane, for launches whose blocks and full tiles would leave most SMs idle; the same sums in
+// the same order.
+template <typename TIN, bool PAIR, int NBUF, bool MULTI, int SHORT, bool FUSED = false, bool UNIT = false>
 __device__ __forceinline__ bool dedisp_tile(const DedispArgs a, unsigned char* smem, int blk,
                                             int tx, TileState& ts, const FusedArgs* fa = nullptr,
                                             const fused::FusedTile* ft = nullptr) {
-    constexpr int R = lane_r(PAIR);
+    static_assert(!UNIT || (PAIR && !MULTI && !FUSED), "UNIT is a form of the plain pair launch");
+    constexpr int R = UNIT ? kRSmall : lane_r(PAIR);
     constexpr int TT = 32 * R;          // outputs per warp time chunk
     constexpr int Q = Elem<TIN>::Q;
     constexpr int TPW = PAIR ? 2 : 1;   // trials per warp unit
@@ -439,16 +519,17 @@ __device__ __forceinline__ bool dedisp_tile(const DedispArgs a, unsigned char* s
     const Smem sm = carve<NBUF>(smem, g, a.smem_bytes, a.nchan);
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int wu = warp / a.nch, chunk = warp - wu * a.nch;
+    const int nch = UNIT ? kWarps : a.nch;                    // warps along time
+    const int wu = UNIT ? (int)blockIdx.z : warp / nch, chunk = UNIT ? warp : warp - wu * nch;
     const int dmi = wu * UPW;                                 // first unit of the warp
     const int d = blk * (TPW * nu) + dmi * TPW;               // its first trial
-    const int64_t t0 = (int64_t)tx * TT * a.nch;              // CTA time start
+    const int64_t t0 = (int64_t)tx * TT * nch;                // CTA time start
     const int64_t tw = t0 + (int64_t)chunk * TT;               // warp time start
     const int64_t base = a.t_offset + t0;
     const int nst = (a.nchan + cs - 1) / cs;
     // the CTA's stages: a contiguous share of the channel sum when the launch splits it
     // (blockIdx.z = split, partial sums to separate outputs), else all of them
-    const int split = (int)blockIdx.z;
+    const int split = UNIT ? 0 : (int)blockIdx.z;
     const int s_lo = (int)((int64_t)split * nst / a.nsplit);
     const int nloc = (int)((int64_t)(split + 1) * nst / a.nsplit) - s_lo;
 
@@ -460,8 +541,12 @@ __device__ __forceinline__ bool dedisp_tile(const DedispArgs a, unsigned char* s
         past_end |= (((base + lo) & ~(int64_t)(Q - 1)) + a.lcap > a.ld) ? 1 : 0;
     }
     const bool tail = __syncthreads_or(past_end) != 0;
-    if (tid == 0)
+    if constexpr (UNIT) {
+        if (warp == 0)
+            for (int i = 0; i < NBUF && i < nloc; ++i) issue_stage_warp<TIN, NBUF>(a, g, sm, blk, i, i, base, lane);
+    } else if (tid == 0) {
         for (int i = 0; i < NBUF && i < nloc; ++i) issue_stage<TIN, NBUF>(a, g, sm, blk, s_lo + i, i, base, tail);
+    }
 
     TACC acc0[R];
     uint64_t accp[PAIR ? R : 1];    // packed (trial 0, trial 1) sums of a pair unit
@@ -583,14 +668,25 @@ __device__ __forceinline__ bool dedisp_tile(const DedispArgs a, unsigned char* s
             if constexpr (PAIR) {
                 const int4* ent4 = (const int4*)(buf + g.rec_off) + dmi * cs;
                 const float2* wts = (const float2*)(buf + g.rec_off + g.w_off);
-                stage_pair<TIN, SHORT>(rows, ent4, wts, lo_all + c0, csn, a.lcap, bq, lane_off, accp,
+                stage_pair<TIN, SHORT, R>(rows, ent4, wts, lo_all + c0, csn, a.lcap, bq, lane_off, accp,
                                        a.kpad, a.status);
             } else {
                 stage_int<TIN, SHORT>(rows, ent, lo_all + c0, csn, a.lcap, bq, lane_off, acc0, a.status);
             }
         }
         __syncwarp();
-        if (lane == 0) {
+        if constexpr (UNIT) {
+            int old = 0;
+            if (lane == 0) {
+                __threadfence_block();
+                old = atomicAdd(&sm.cnt[b], 1);
+                if (old == kWarps - 1) sm.cnt[b] = 0;
+            }
+            if (__shfl_sync(0xffffffffu, old, 0) == kWarps - 1 && i + NBUF < nloc) {  // last warp out
+                __threadfence_block();
+                issue_stage_warp<TIN, NBUF>(a, g, sm, blk, s + NBUF, b, base, lane);
+            }
+        } else if (lane == 0) {
             __threadfence_block();
             const int old = atomicAdd(&sm.cnt[b], 1);
             if (old == kWarps - 1) {  // last warp out refills the buffer
