@@ -34,17 +34,26 @@ class Band:
                        DD_U8 if self.in_type == "u8" else DD_F32, float(self.k_dm))
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+# Pointers are passed as plain integers (the declared argument types convert them): a small
+# block's step is bound by this marshalling, not by its kernels.
+def _ptr(t) -> int | None:
+    return None if t is None else t.data_ptr()
 
 
-def _np_ptr(a) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if a is None else a.ctypes.data)
+def _np_ptr(a) -> int | None:
+    return None if a is None else a.ctypes.data
 
 
-def _stream(stream=None) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream(stream=None) -> int:
+    """cudaStream_t of `stream`, or of the current device's current stream."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def alu_peak(kind: str = "fma", stream=None) -> float:
@@ -161,6 +170,7 @@ class Plan:
                                        self.ndm), "dd_plan_create")
         self._h = h
         self._kw = 0
+        self._wver = 0      # counts the profile and weight changes made through this object
 
     # ------------------------------------------------------------------ profiles
     def set_profiles(self, delay=None, taps=None, weights=None) -> None:
@@ -176,6 +186,7 @@ class Plan:
             if w.ndim != 3 or w.shape[:2] != (self.ndm, self.band.nchan):
                 raise ValueError(f"weights shape {w.shape}")
             k = w.shape[2]
+        self._wver += 1
         check(self._lib.dd_set_profiles(self._h, _np_ptr(d), _np_ptr(t), _np_ptr(w), k),
               "dd_set_profiles")
         self._kw = k
@@ -184,25 +195,25 @@ class Plan:
         """Device weights [D][C][K] fp32 (contiguous), copied in stream order."""
         if not (w.is_cuda and w.dtype == torch.float32 and w.is_contiguous() and w.dim() == 3):
             raise ValueError("weights must be a contiguous CUDA float32 [D][C][K] tensor")
+        self._wver += 1
         check(self._lib.dd_set_weights_device(self._h, _ptr(w), int(w.shape[2]), _stream(stream)),
               "dd_set_weights_device")
         self._kw = int(w.shape[2])
 
+    def _facts(self):
+        """(t_out, d_max, kmax, ns_total, out_is_int) of dd_plan_info."""
+        b = (ctypes.c_int64 * 5)()   # one zeroed 8-byte slot each (little endian)
+        at = ctypes.addressof(b)
+        check(self._lib.dd_plan_info(self._h, at, at + 8, at + 16, at + 24, at + 32), "dd_plan_info")
+        return b
+
     def info(self) -> dict:
-        t_out = ctypes.c_int64()
-        d_max = ctypes.c_int32()
-        kmax = ctypes.c_int32()
-        ns = ctypes.c_int64()
-        oi = ctypes.c_int32()
-        check(self._lib.dd_plan_info(self._h, *(ctypes.cast(ctypes.byref(v), ctypes.c_void_p)
-                                                for v in (t_out, d_max, kmax, ns, oi))),
-              "dd_plan_info")
-        return dict(t_out=t_out.value, d_max=d_max.value, kmax=kmax.value, ns_total=ns.value,
-                    out_is_int=bool(oi.value))
+        b = self._facts()
+        return dict(t_out=b[0], d_max=b[1], kmax=b[2], ns_total=b[3], out_is_int=bool(b[4]))
 
     @property
     def d_max(self) -> int:
-        return self.info()["d_max"]
+        return self._facts()[1]
 
     def tables(self):
         d = np.zeros((self.ndm, self.band.nchan), np.int32)
@@ -220,16 +231,17 @@ class Plan:
         return x.stride(0)
 
     def out_dtype(self):
-        return torch.int32 if self.info()["out_is_int"] else torch.float32
+        return torch.int32 if self._facts()[4] else torch.float32
 
     def dedisperse(self, x: torch.Tensor, t_offset: int = 0, nsamp: int | None = None,
                    out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
         """eq. p_dedisp for every trial: returns [D][nsamp - d_max]."""
         ld = self._check_input(x)
         nsamp = (x.shape[1] - t_offset) if nsamp is None else nsamp
-        t_out = nsamp - self.d_max
         if out is None:
-            out = torch.empty((self.ndm, max(t_out, 0)), dtype=self.out_dtype(), device=x.device)
+            f = self._facts()
+            out = torch.empty((self.ndm, max(nsamp - f[1], 0)), dtype=torch.int32 if f[4] else torch.float32,
+                              device=x.device)
         check(self._lib.dd_dedisperse(self._h, _ptr(x), ld, t_offset, nsamp, _ptr(out),
                                       out.stride(0), _stream(stream)), "dd_dedisperse")
         return out
@@ -478,15 +490,17 @@ class DDFunction(torch.autograd.Function):
         out = plan.dedisperse(x.detach(), t_offset=t_offset, nsamp=nsamp)
         ctx.save_for_backward(x, w)
         ctx.plan = plan
+        ctx.wver = plan._wver
         ctx.t_offset = t_offset
         ctx.nsamp = nsamp
         return out
 
     @staticmethod
     def backward(ctx, gout):
-        x, w = ctx.saved_tensors
+        x, w = ctx.saved_tensors    # (raises if w was changed in place since)
         plan = ctx.plan
-        plan.set_weights(w.detach().contiguous())
+        if plan._wver != ctx.wver:  # another forward has given the plan other weights
+            plan.set_weights(w.detach().contiguous())
         gw, gin = plan.backward(x.detach(), gout.contiguous(), t_offset=ctx.t_offset,
                                 nsamp=ctx.nsamp, want_gw=ctx.needs_input_grad[1],
                                 want_gin=ctx.needs_input_grad[0])
