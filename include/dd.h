@@ -31,8 +31,10 @@
  *     size, row lengths, shared memory), autotuner results, batch bindings; 2 = also every
  *     device call with its sizes.
  *   - No call here allocates device memory except dd_plan_create / dd_set_profiles /
- *     the first device call on a plan (tables; on a device's first plan also the 8 MiB
- *     array of dd_boxcar_snr_noalloc), dd_boxcar_snr when the width count
+ *     the first device call on a plan (tables; on an integer plan whose direct sums read
+ *     prefix sums, 4 bytes per channel and sample of the band's block, at most 2 GiB unless
+ *     the longest delay needs more; on a device's first plan also the 8 MiB array of
+ *     dd_boxcar_snr_noalloc), dd_boxcar_snr when the width count
  *     grows (normaliser workspace), dd_dedisperse on a run-length plan when nsamp
  *     grows (prefix scratch), dd_dedisperse_boxcar when its scratch grows, and the
  *     first dd_backward (adjoint workspace).
@@ -261,7 +263,9 @@ dd_status dd_plan_set_schedule(dd_plan_t plan, int32_t nch, int32_t cs);
 dd_status dd_plan_get_schedule(dd_plan_t plan, int32_t* nch, int32_t* cs, int32_t* trials_per_cta);
 
 /* How a plan forms the tap sums of eq. p_dedisp.
- *   DD_METHOD_DIRECT:    every tap is one multiply-add (any weights).
+ *   DD_METHOD_DIRECT:    every tap is one multiply-add (any weights), or, for integer plans
+ *     whose trials share their tap runs (see dd_plan_set_schedule), the shared runs' sums from
+ *     prefix sums in a scratch of fixed size, longer calls in pieces (the same exact sums).
  *   DD_METHOD_RUNLENGTH: uint8 unit-weight plans only.  A run of n unit taps is a
  *     difference of per-channel prefix sums, sum_{k<n} I[c][s+k] = P_c[s+n] - P_c[s]
  *     with P_c[i] = sum_{j<i} I[c][t_offset+j], so each (trial, channel) costs two

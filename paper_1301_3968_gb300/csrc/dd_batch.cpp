@@ -26,7 +26,7 @@ struct dd_batch_s {
     bool rl = false;         // run-length beams (per-channel prefix sums, then differences)
     bool short_taps = true;  // every plan's tap runs fit one register window (run-length
                              // beams: every plan shares difference rows in the CTA)
-    std::vector<uint32_t*> d_prefix;  // run-length beams: each beam's prefix sums
+    std::vector<uint32_t*> d_prefix;  // beams that read prefix sums: theirs (else null)
     std::vector<int64_t> ldp;
     std::vector<dd::BatchItem> items;
     // one launch per kernel: row kernels with 16 and 8 warps per CTA, then the tap kernels
@@ -131,7 +131,7 @@ void build_items(dd_batch_s* b) {
 }
 
 // The row kernels' kind for the batch's beams.
-int row_kind(const dd_batch_s* b) { return b->pair ? dd::kRowsFir : (b->rl ? dd::kRowsRl : dd::kRowsU8); }
+int row_kind(const dd_batch_s* b) { return b->pair ? dd::kRowsFir : dd::kRowsPk; }
 
 bool aligned16(const void* ptr) { return ((uintptr_t)ptr & 15u) == 0; }
 
@@ -185,11 +185,13 @@ dd_status dd_batch_bind(dd_batch_t b, const void* const* d_in, const int64_t* in
     for (int i = 0; i < nb; ++i) {
         dd_plan_s* p = b->plans[i];
         const int64_t t_out = plan_t_out(p);
-        if (!b->rl) {
+        if (!dd::reads_prefix(p)) {
             dd::fill_dedisp_args(p, d_in[i], in_ld[i], 0, t_out, d_out[i], out_ld[i], &args[i]);
+            b->d_prefix.push_back(nullptr);
+            b->ldp.push_back(0);
             continue;
         }
-        // run-length beams read their own prefix sums, which the batch owns
+        // beams that read prefix sums have their own, which the batch owns
         const int64_t ldp = (p->band.nsamp + 1 + 3) & ~(int64_t)3;
         uint32_t* q = nullptr;
         const cudaError_t e = cudaMalloc((void**)&q, (size_t)ldp * p->nchan * sizeof(uint32_t));
@@ -272,8 +274,8 @@ dd_status dd_batch_dedisperse(dd_batch_t b, void* stream) {
         const dd_status st = batch_rebind(b);
         if (st != DD_OK) return st;
     }
-    if (b->rl)  // every beam's prefix sums first
-        for (size_t i = 0; i < b->plans.size(); ++i) {
+    for (size_t i = 0; i < b->plans.size(); ++i)  // the prefix sums of the beams that read them
+        if (b->d_prefix[i]) {
             const dd_status st = dd::launch_prefix_into(b->plans[i], b->in[i], b->in_ld[i], 0,
                                                         b->plans[i]->band.nsamp, b->d_prefix[i], b->ldp[i],
                                                         (cudaStream_t)stream);

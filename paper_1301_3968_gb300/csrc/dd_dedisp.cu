@@ -373,7 +373,7 @@ dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_
 // [nchan][ldp] (ldp >= nsamp + 1).
 dd_status launch_prefix_into(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                              int64_t nsamp, uint32_t* P, int64_t ldp, cudaStream_t s) {
-    if (p->rk == kRowsRl)
+    if (p->rk == kRowsPk)
         k_prefix_packed<<<p->nchan, 256, 0, s>>>((const uint8_t*)in, ld, t_offset, nsamp, P, ldp);
     else
         k_prefix<<<p->nchan, 256, 0, s>>>((const uint8_t*)in, ld, t_offset, nsamp, P, ldp);
@@ -388,12 +388,14 @@ dd_status launch_prefix(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offs
     *ldp_out = ldp;
     const int64_t need = ldp * p->nchan;
     if (need > p->prefix_elems) {
-        cudaFree(p->d_prefix);
+        if (p->prefix_own) cudaFree(p->d_prefix);
         p->d_prefix = nullptr;
         p->prefix_elems = 0;
+        p->prefix_own = false;
         cudaError_t e = cudaMalloc((void**)&p->d_prefix, (size_t)need * sizeof(uint32_t));
         if (e != cudaSuccess) return cuda_status(e);
         p->prefix_elems = need;
+        p->prefix_own = true;
     }
     return launch_prefix_into(p, in, ld, t_offset, nsamp, p->d_prefix, ldp, s);
 }
@@ -407,6 +409,25 @@ dd_status launch_dedisperse_rl(dd_plan_s* p, const void* in, int64_t ld, int64_t
     fill_dedisp_args(p, p->d_prefix, ldp, 0, nsamp - p->dmax, out, out_ld, &a);
     if (p->rk) return launch_rows(p, a, s);
     return p->rl_b ? run<uint32_t, false, kStagesRl, 1>(a, s) : run<uint32_t, false, kStagesRl>(a, s);
+}
+
+dd_status launch_dedisperse_pk(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
+                               int64_t nsamp, void* out, int64_t out_ld, cudaStream_t s) {
+    // outputs per piece: whole tiles, as many as the scratch holds with the delays behind them
+    const int64_t tile = row_tile_t(kRowsPk, p->nch), t_out = nsamp - p->dmax;
+    const int64_t cols = p->prefix_elems / p->nchan;
+    int64_t piece = std::min(cols - 4 - p->dmax, 65535 * tile);  // (grid y)
+    if (piece < t_out) piece = piece / tile * tile;
+    if (piece < 1) return DD_ERR_OOM;
+    for (int64_t t0 = 0; t0 < t_out; t0 += piece) {
+        const int64_t n = std::min(piece, t_out - t0) + p->dmax, ldp = (n + 1 + 3) & ~(int64_t)3;
+        dd_status st = launch_prefix_into(p, in, ld, t_offset + t0, n, p->d_prefix, ldp, s);
+        if (st != DD_OK) return st;
+        DedispArgs a;
+        fill_dedisp_args(p, p->d_prefix, ldp, 0, n - p->dmax, (int32_t*)out + t0, out_ld, &a);
+        if ((st = launch_rows(p, a, s)) != DD_OK) return st;
+    }
+    return DD_OK;
 }
 
 dd_status launch_dedisperse_batched(bool u8, bool pair, bool short_taps, const DedispArgs* d_args,

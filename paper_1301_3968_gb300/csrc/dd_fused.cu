@@ -411,7 +411,7 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
     if ((st = launch_norm(p, widths, nw, mean, sd, s)) != DD_OK) return st;
 
     DedispArgs a;
-    if (p->rl) {
+    if (reads_prefix(p)) {
         int64_t ldp = 0;
         if ((st = launch_prefix(p, in, in_ld, t_offset, nsamp, &ldp, s)) != DD_OK) return st;
         fill_dedisp_args(p, p->d_prefix, ldp, 0, t_out, nullptr, 0, &a);

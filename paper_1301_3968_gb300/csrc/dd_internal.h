@@ -45,7 +45,7 @@ constexpr long long kWaitNs = 2000000000;  // bound on any device-side barrier w
 // tile in shared memory.  A warp unit sums row_unit_trials trials: lane l owns kRFir
 // consecutive outputs (fp32), or kRPk consecutive words of two outputs kPkHalf apart (packed
 // integer sums).  The odd counts keep lane-strided loads free of bank conflicts.
-enum RowKind { kRowsNone = 0, kRowsFir = 1, kRowsU8 = 2, kRowsRl = 3 };
+enum RowKind { kRowsNone = 0, kRowsFir = 1, kRowsPk = 2 };
 constexpr int kRFir = kRPair;
 constexpr int kRPk = 17;
 constexpr int kPkHalf = 32 * kRPk;
@@ -65,30 +65,38 @@ __host__ __device__ constexpr int row_span(int kind, int nch) {
 __host__ __device__ constexpr int row_zero_words(int kind, int nch) {
     return kind == kRowsFir ? 0 : (row_span(kind, nch) + 3) & ~3;
 }
-// Stage record of a row kernel: a header (rows of the stage; packed kinds: per four channels two
-// bits, 0: the four words may be added in 16-bit halves, 1: two and two, 2: none; the longest
-// row), entries with each trial's row position in the stage's row area (fp32: per unit and
-// channel, trials 0 and 1 as the half words of the first word, trial 2 the second; packed: per
-// unit and four channels, their positions as half words, trial 0's two words then trial 1's), a descriptor per row (offset of its samples in the
-// staged rows, its position in the row area, its length, taps | offset of its weights
-// << 16), and the rows' weights.  The header and entries are copied beside the rows.
+// Stage record of a row kernel.  The stage's channels are items: single channels, or (packed)
+// pairs of adjacent ones whose sums one row holds per pattern, a pattern being both runs and the
+// relative delay.
+//   header   rows; packed: per four items two bits, 0: their four words may be added in 16-bit
+//            halves, 1: two and two, 2: none; the longest row; items
+//   entries  each trial's position in the stage's row area (fp32: per unit and item, trials 0 and 1
+//            as the half words of the first word, trial 2 the second; packed: per unit and four
+//            items, their positions as half words, trial 0's two words then trial 1's)
+//   rows     source in the raw samples (and a pattern's second channel's) as half words; position |
+//            length << 16; taps (n0 | n1 << 16; n1 = 0: a single channel's); offset of the weights
+//   weights  of the rows
+// The header and the entries are copied beside the rows.
 struct RowGeom {
-    int ent_bytes, desc_off, w_off, rec_bytes;
+    int ent_off, ent_bytes, desc_off, w_off, rec_bytes;
     __host__ __device__ RowGeom(int kind, int cs, int nu, int rows_max, int kw) {
+        ent_off = 16;
         // (fp32: one entry is read ahead; packed: cs is a multiple of four)
-        ent_bytes = (16 + (kind == kRowsFir ? 8 * nu * cs + 8 : 4 * nu * cs) + 15) & ~15;
-        desc_off = ent_bytes;
+        ent_bytes = ((kind == kRowsFir ? 8 * nu * cs + 8 : 4 * nu * cs) + 15) & ~15;
+        desc_off = ent_off + ent_bytes;
         w_off = desc_off + 16 * rows_max;
         rec_bytes = (w_off + 4 * kw + 15) & ~15;
     }
+    // words of a row half: the area, the header and the entries
+    __host__ __device__ int half_words(int area) const { return area + (ent_off + ent_bytes) / 4; }
 };
-// Shared memory of a row launch: the raw buffer and record, the block's table (lo_ld words),
-// two row halves, the barrier; at least the output transpose.
+// Shared memory of a row launch: the raw buffer and record, the block's table (lo_ld words), two
+// row halves, the barrier; at least the output transpose.
 __host__ __device__ inline size_t row_smem_bytes(const RowGeom& g, int nw, int esz, int lcap, int cs, int lo_ld,
                                                  int area) {
     const size_t tail = 8 + 2 * 4;
     const size_t all = (((size_t)cs * lcap * esz + g.rec_bytes + 127) & ~(size_t)127) +
-                       ((4 * (size_t)lo_ld + 15) & ~(size_t)15) + 2 * ((size_t)area * 4 + g.ent_bytes) + tail;
+                       ((4 * (size_t)lo_ld + 15) & ~(size_t)15) + 2 * (size_t)g.half_words(area) * 4 + tail;
     const size_t st = (size_t)nw * 2 * kPkHalf * 4 + tail;
     return ((all > st ? all : st) + 15) & ~(size_t)15;
 }
@@ -238,6 +246,7 @@ struct BatchItem {
 
 struct DevTables {
     int device = -1;
+    unsigned char* slab = nullptr;  // the allocation that the tables down to `off` lie in
     int32_t* delay = nullptr;   // [ndm][nchan]
     int32_t* taps = nullptr;    // [ndm][nchan]
     float* w = nullptr;         // [ndm][nchan][kpad]  (weighted plans)
@@ -305,6 +314,7 @@ struct dd_plan_s {
     int32_t blen = 0;                  // their stride (words)
     uint32_t* d_prefix = nullptr;
     int64_t prefix_elems = 0;
+    bool prefix_own = false;           // d_prefix is an allocation of its own (else in the slab)
     // row kernels (RowKind): the schedule above is then theirs
     int32_t rk = 0;
     int32_t rows_max = 0;
@@ -340,6 +350,11 @@ dd_status launch_dedisperse_batched(bool u8, bool pair, bool short_taps, const D
 int dedisp_batched_blocks_per_sm(bool u8, bool pair, bool short_taps, size_t smem, bool rl = false);
 dd_status launch_prefix_into(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                              int64_t nsamp, uint32_t* P, int64_t ldp, cudaStream_t s);
+// direct plans on packed rows: prefix sums into the plan's scratch and the launch, in pieces that fit
+dd_status launch_dedisperse_pk(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
+                               int64_t nsamp, void* out, int64_t out_ld, cudaStream_t s);
+// the plan's sums read prefix sums instead of samples
+inline bool reads_prefix(const dd_plan_s* p) { return p->rl || p->rk == kRowsPk; }
 dd_status cuda_status(cudaError_t e);
 // Outputs per CTA tile and trials per CTA of the plan's schedule.
 inline int plan_tile_t(const dd_plan_s* p) {

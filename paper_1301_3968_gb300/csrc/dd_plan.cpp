@@ -348,9 +348,15 @@ void build_records(dd_plan_s* p) {
 // ----------------------------------------------------------------------- row schedule
 
 // One distinct tap run of a (trial block, channel): its taps and weights are those of
-// `trial`, its furthest start in the block `reach` past the block's minimum delay.
+// `trial`; its trials start beg .. end samples past the block's minimum delay.
 struct Row {
-    int32_t n, trial, reach;
+    int32_t n, trial, beg, end;
+};
+// A pair of adjacent channels of a block whose trials share (run, run, relative delay): a row
+// per pattern holds both channels' sums.  a, b: the runs' rows (indexes in the block's rows);
+// beg, end, beg1: the starts on the first channel, and of the earliest trial on the second.
+struct Pattern {
+    int32_t a, b, rel, beg, end, beg1;
 };
 
 // The plan's row kind, if its sums can be formed that way: fp32 sums with weights that the
@@ -358,7 +364,8 @@ struct Row {
 int row_kind_of(const dd_plan_s* p) {
     if (p->pair) return p->w_dev || p->kmax > 0xffff ? dd::kRowsNone : dd::kRowsFir;
     if (p->kmax > dd::kPkMaxTaps) return dd::kRowsNone;
-    return p->rl ? dd::kRowsRl : dd::kRowsU8;
+    // (the prefix sums of a direct plan live in a scratch that holds its longest delay)
+    return p->rl || (double)p->nchan * (p->dmax + 16.0 * 2 * dd::kPkHalf) * 4.0 <= 16e9 ? dd::kRowsPk : dd::kRowsNone;
 }
 
 // Rows pay up to this many distinct runs per (trial, channel).
@@ -368,14 +375,16 @@ constexpr double kRowsMaxShare = 0.5;
 // trials of 8 (two CTAs per SM), which measured 12 % faster on a long launch (CRAFT-like,
 // 512 trials: 1.08 against 1.22 ms), but leave more of a short launch's last wave idle: the
 // share of the waves' slots that the plan's block fills decides, on 152 SMs.
-int row_warps_of(const dd_plan_s* p, int kind, int nch) {
+int row_warps_of(const dd_plan_s* p, int kind, int nch, bool* one_wave) {
     const int64_t tile = dd::row_tile_t(kind, nch);
     const int64_t tiles = (std::max<int64_t>(1, p->band.nsamp - p->dmax) + tile - 1) / tile;
     auto ctas = [&](int nw) {
         const int db = dd::row_trials(kind, nw, nch);
         return tiles * ((p->ndm + db - 1) / db);
     };
-    if (ctas(dd::kWarps) <= 304) return dd::kWarps;  // one wave: a CTA's own time counts
+    // one CTA per SM or fewer: its own time counts, and it may have the SM's shared memory
+    *one_wave = ctas(dd::kWarps) <= 152;
+    if (ctas(dd::kWarps) <= 304) return dd::kWarps;
     auto fill = [&](int nw, int64_t slots) {
         const int db = dd::row_trials(kind, nw, nch);
         const int64_t n = ctas(nw);
@@ -392,10 +401,11 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     if (kind == dd::kRowsNone) return false;
     const double units = (double)p->ndm * p->nchan;
     const int C = p->nchan;
-    const int nw = row_warps_of(p, kind, nch);
+    bool one_wave = false;
+    const int nw = row_warps_of(p, kind, nch, &one_wave);
     const int db = dd::row_trials(kind, nw, nch), nt = dd::row_unit_trials(kind), nu = db / nt;
     const int nblk = (p->ndm + db - 1) / db;
-    const int esz = stage_esz(p), Q = 16 / esz;
+    const int esz = kind == dd::kRowsFir && p->band.in_type == DD_U8 ? 1 : 4, Q = 16 / esz;  // samples or prefix sums
     const int span = dd::row_span(kind, nch);
     const bool fir = kind == dd::kRowsFir;
     auto same = [&](size_t a, size_t b) {
@@ -405,8 +415,14 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     // the distinct runs of every (block, channel), and each trial's
     std::vector<std::vector<Row>> rows(nblk);
     std::vector<std::vector<int32_t>> first(nblk);  // [C + 1] into rows[b]
-    std::vector<uint8_t> rid((size_t)p->ndm * C);
+    std::vector<uint8_t> rid((size_t)p->ndm * C);   // in its channel's rows, or pair's patterns
     std::vector<int32_t> lo((size_t)nblk * C);
+    // the block's channels as items, each one channel or a pair (patterns i0 .. i1 of pats[b])
+    struct Item {
+        int32_t c, nc, i0, i1;
+    };
+    std::vector<std::vector<Item>> items(nblk);
+    std::vector<std::vector<Pattern>> pats(nblk);
     for_blocks(nblk, (size_t)p->ndm * C, [&](int b) {
         const int d0 = b * db, d1 = std::min(p->ndm, d0 + db);
         first[b].resize(C + 1);
@@ -424,116 +440,195 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
                 if (r >= rows[b].size() || !same(dc, (size_t)rows[b][r].trial * C + c))
                     for (r = f; r < rows[b].size(); ++r)
                         if (r != hint && same(dc, (size_t)rows[b][r].trial * C + c)) break;
-                if (r == rows[b].size()) rows[b].push_back({p->taps[dc], d, 0});
-                rows[b][r].reach = std::max(rows[b][r].reach, p->delay[dc] - l);
+                const int32_t at = p->delay[dc] - l;
+                if (r == rows[b].size()) rows[b].push_back({p->taps[dc], d, at, at});
+                rows[b][r].beg = std::min(rows[b][r].beg, at);
+                rows[b][r].end = std::max(rows[b][r].end, at);
                 rid[dc] = (uint8_t)(r - f);
                 hint = r;
             }
         }
         first[b][C] = (int32_t)rows[b].size();
+        // Integer sums: pairs of channels whose trials share their patterns.  In shared-memory
+        // words per trial-block tile a run's row of L words costs 3 L to build (two loads and a
+        // store) and a pattern's 5 L; a trial reads `span` words per channel, or per pair.
+        std::vector<Pattern> ps;
+        std::vector<uint8_t> id((size_t)(d1 - d0));
+        for (int c = 0; c < C;) {
+            bool pair = !fir && c + 1 < C;
+            if (pair) {
+                ps.clear();
+                int n0 = 0, n1 = 0;
+                double single = 2.0 * (d1 - d0) * span, both = (double)(d1 - d0) * span;
+                for (int k = c; k < c + 2; ++k)
+                    for (int r = first[b][k]; r < first[b][k + 1]; ++r) {
+                        const double L = rows[b][r].end - rows[b][r].beg + span;
+                        single += 3.0 * L;
+                        (k == c ? n0 : n1) = std::max(k == c ? n0 : n1, rows[b][r].n);
+                    }
+                pair = n0 + n1 <= dd::kPkMaxTaps;
+                for (int d = d0; d < d1 && pair; ++d) {
+                    const size_t dc = (size_t)d * C + c;
+                    const int32_t ra = first[b][c] + rid[dc], rb1 = first[b][c + 1] + rid[dc + 1];
+                    const int32_t at = p->delay[dc] - lo[(size_t)b * C + c], at1 = p->delay[dc + 1] - lo[(size_t)b * C + c + 1];
+                    size_t i = 0;
+                    while (i < ps.size() && !(ps[i].a == ra && ps[i].b == rb1 && ps[i].rel == at1 - at)) ++i;
+                    if (i == ps.size()) ps.push_back({ra, rb1, at1 - at, at, at, at1});
+                    if (at < ps[i].beg) {
+                        ps[i].beg = at;
+                        ps[i].beg1 = at1;
+                    }
+                    ps[i].end = std::max(ps[i].end, at);
+                    id[d - d0] = (uint8_t)i;
+                }
+                for (const Pattern& q : ps) both += 5.0 * (q.end - q.beg + span);
+                pair = pair && both < single;
+            }
+            const int32_t i0 = (int32_t)pats[b].size();
+            if (pair) {
+                pats[b].insert(pats[b].end(), ps.begin(), ps.end());
+                for (int d = d0; d < d1; ++d) rid[(size_t)d * C + c] = id[d - d0];
+            }
+            items[b].push_back({c, pair ? 2 : 1, i0, (int32_t)pats[b].size()});
+            c += pair ? 2 : 1;
+        }
     });
-    auto len_of = [&](const Row& r) { return (int64_t)((Q - 1 + r.reach + span + 3) & ~3); };
+    // Words of a row: fp32, a run's whole staged window (its start is aligned to the raw buffer's
+    // quads); packed, what its own trials read.
+    auto whole_len = [&](const Row& r) { return (int64_t)((Q - 1 + r.end + span + 3) & ~3); };
+    auto own_len = [&](int32_t beg, int32_t end) { return (int64_t)((end - beg + span + 3) & ~3); };
+    auto low_bits = [&](int b, int c) { return lo[(size_t)b * C + c] & (Q - 1); };
     size_t total = 0;
     int64_t need = 0;
-    // Stages are cut at multiples of `grain` channels.  Of a grain from channel c of block b:
-    // rows, weights (each row's padded to four) and row words, and the most of each.
+    // Stages are cut at multiples of `grain` items.  Of the grain from item v of block b:
+    // channels, rows, weights (each row's padded to four) and words of the row area, and the most
+    // of each.
     const int grain = fir ? 1 : 4;
     struct Need {
-        int64_t r = 0, w = 0, a = 0;
+        int64_t c = 0, r = 0, w = 0, a = 0;
+        void add(const Need& o) {
+            c += o.c;
+            r += o.r;
+            w += o.w;
+            a += o.a;
+        }
+        void top(const Need& o) {
+            c = std::max(c, o.c);
+            r = std::max(r, o.r);
+            w = std::max(w, o.w);
+            a = std::max(a, o.a);
+        }
     };
-    auto grain_need = [&](int b, int c) {
+    std::vector<std::vector<Need>> grains(nblk);  // of the items v, v + grain, ...
+    auto count_grain = [&](int b, size_t v) {
         Need k;
-        const int r0 = first[b][c], r1 = first[b][std::min(C, c + grain)];
-        k.r = r1 - r0;
-        for (int r = r0; r < r1; ++r) {
-            if (fir) k.w += (rows[b][r].n + 3) & ~3;
-            k.a += len_of(rows[b][r]);
+        for (size_t i = v; i < std::min(items[b].size(), v + grain); ++i) {
+            const Item& it = items[b][i];
+            k.c += it.nc;
+            if (it.nc == 2) {
+                for (int q = it.i0; q < it.i1; ++q) k.a += own_len(pats[b][q].beg, pats[b][q].end);
+                k.r += it.i1 - it.i0;
+                continue;
+            }
+            for (int r = first[b][it.c]; r < first[b][it.c + 1]; ++r) {
+                const Row& row = rows[b][r];
+                k.r += 1;
+                if (fir) k.w += (row.n + 3) & ~3;
+                k.a += fir ? whole_len(row) : own_len(row.beg, row.end);
+            }
         }
         return k;
     };
     Need one;
     for (int b = 0; b < nblk; ++b) {
         total += rows[b].size();
-        for (const Row& r : rows[b]) {
-            // samples that building the row reads (dd_rows.cuh)
-            const int64_t past = fir ? (r.n & ~3) + 4 : kind == dd::kRowsU8 ? dd::kPkHalf + (r.n & ~3) + 4 : r.n;
-            need = std::max(need, len_of(r) + past);
-        }
-        for (int c = 0; c < C; c += grain) {
-            const Need k = grain_need(b, c);
-            one.r = std::max(one.r, k.r);
-            one.w = std::max(one.w, k.w);
-            one.a = std::max(one.a, k.a);
+        for (int c = 0; c < C; ++c)
+            for (int i = first[b][c]; i < first[b][c + 1]; ++i) {
+                // samples that building the row reads (dd_rows.cuh)
+                const Row& r = rows[b][i];
+                need = std::max(need, fir ? whole_len(r) + (r.n & ~3) + 4
+                                          : low_bits(b, c) + r.end + (int64_t)((span + 3) & ~3) + 3 + r.n);
+            }
+        for (size_t v = 0; v < items[b].size(); v += grain) {
+            const Need k = count_grain(b, v);
+            grains[b].push_back(k);
+            one.top(k);
         }
     }
     if ((double)total > kRowsMaxShare * units) return false;
     const int64_t lcap = (need + Q - 1) / Q * Q;
-    if (lcap > (1 << 20) || one.w > 0xffff) return false;
+    if (lcap > 0xffff || one.w > 0xffff) return false;
     const int64_t zero = dd::row_zero_words(kind, nch);  // the area begins with a row of zeros
-    // Stages: channels in order, as many as the limits on channels (cs), rows, weights and
-    // row words allow.
+    // Stages: items in order, as many as the limits allow.
     struct Cut {
         int cs = 0, nst = 0;  // nst: most stages of a block
-        int64_t rmax = 1, wmax = 0, area = 0, total = 0;
-        std::vector<std::vector<int32_t>> start;  // per block: first channels, and the end
+        int64_t total = 0;
+        Need most;
+        std::vector<std::vector<int32_t>> start;  // per block: first items, and the end
     };
-    auto cut = [&](int cs, int64_t rlim, int64_t wlim, int64_t alim, bool keep) {
+    auto cut = [&](int cs, const Need& lim, bool keep) {
         Cut k;
         k.cs = cs;
         if (keep) k.start.resize(nblk);
         for (int b = 0; b < nblk; ++b) {
             int n = 0;
             Need in;
-            for (int c = 0, c0 = 0; c < C; c += grain) {
-                const Need m = grain_need(b, c);
-                if (c == 0 || c - c0 >= cs || in.r + m.r > rlim || in.w + m.w > wlim || in.a + m.a > alim) {
-                    if (keep) k.start[b].push_back(c);
+            for (size_t v = 0; v < items[b].size(); v += grain) {
+                const Need& m = grains[b][v / grain];
+                if (v == 0 || in.c + m.c > lim.c || in.r + m.r > lim.r || in.w + m.w > lim.w || in.a + m.a > lim.a) {
+                    if (keep) k.start[b].push_back((int32_t)v);
                     ++n;
-                    c0 = c;
                     in = Need();
                 }
-                in.r += m.r;
-                in.w += m.w;
-                in.a += m.a;
-                k.rmax = std::max(k.rmax, in.r);
-                k.wmax = std::max(k.wmax, in.w);
-                k.area = std::max(k.area, in.a);
+                in.add(m);
+                k.most.top(in);
             }
-            if (keep) k.start[b].push_back(C);
+            if (keep) k.start[b].push_back((int32_t)items[b].size());
             k.nst = std::max(k.nst, n);
             k.total += n;
         }
         return k;
     };
-    const size_t budget = cs_fixed > 0 || nw == dd::kRowWarps ? dd::kSmemBudgetOne : dd::kSmemBudget;
-    // limits for at most cs channels; false where a single channel does not fit
-    auto limits = [&](int cs, int64_t* rlim, int64_t* wlim, int64_t* alim) {
-        *rlim = std::max<int64_t>(one.r, 2 * cs);
-        *wlim = fir ? std::min<int64_t>(0xffff, std::max<int64_t>(one.w, (int64_t)cs * ((p->kmax + 3) & ~3) * 5 / 4)) : 0;
-        const dd::RowGeom g(kind, cs, nu, (int)*rlim, (int)*wlim);
-        const size_t rest = dd::row_smem_bytes(g, 0, esz, (int)lcap, cs, 2 * C + 2, 16 + (int)zero);
+    // (a fixed stage size that does not fit beside a second CTA may take the SM's shared memory)
+    size_t budget = nw == dd::kRowWarps || one_wave ? dd::kSmemBudgetOne : dd::kSmemBudget;
+    auto smem_of = [&](int cs, const Need& m, int stages) {
+        const dd::RowGeom g(kind, cs, nu, (int)m.r, (int)m.w);
+        return dd::row_smem_bytes(g, 0, esz, (int)lcap, cs, C + stages + 2, (int)(zero + m.a) + 16);
+    };
+    // limits for at most cs channels; false where a single grain does not fit
+    auto limits = [&](int cs, Need* lim) {
+        lim->c = cs;
+        if (one.c > cs || cs * lcap > 0xffff) return false;
+        lim->r = std::max<int64_t>(one.r, 2 * cs);
+        lim->w = fir ? std::min<int64_t>(0xffff, std::max<int64_t>(one.w, (int64_t)cs * ((p->kmax + 3) & ~3) * 5 / 4)) : 0;
+        lim->a = 0;
+        const size_t rest = smem_of(cs, *lim, C);
         if (rest >= budget) return false;
-        *alim = (int64_t)((budget - rest) / 8) & ~(int64_t)3;
-        return *alim >= one.a;
+        lim->a = (int64_t)((budget - rest) / 8) & ~(int64_t)3;
+        return lim->a >= one.a;
     };
     Cut best;
-    int64_t rlim = 0, wlim = 0, alim = 0;
-    const int cs_hi = cs_fixed > 0 ? (cs_fixed + grain - 1) / grain * grain : dd::kRowCsMax;
+    Need lim;
+    const int cs_hi = std::min(dd::kRowCsMax, cs_fixed > 0 ? (std::max<int>(cs_fixed, (int)one.c) + grain - 1) / grain * grain : dd::kRowCsMax);
     const int cs_lo = cs_fixed > 0 ? cs_hi : grain;
-    for (int cs = std::min(cs_hi, dd::kRowCsMax); cs >= cs_lo; cs -= grain) {
-        if (!limits(cs, &rlim, &wlim, &alim)) continue;
-        Cut k = cut(cs, rlim, wlim, alim, false);
-        if (best.cs == 0 || k.total < best.total) best = k;
-        else break;
+    for (int pass = 0; pass < 2 && best.cs == 0; ++pass) {
+        if (pass == 1 && (cs_fixed == 0 || budget == dd::kSmemBudgetOne)) break;
+        if (pass == 1) budget = dd::kSmemBudgetOne;
+        for (int cs = cs_hi; cs >= cs_lo; cs -= grain) {
+            if (!limits(cs, &lim)) continue;
+            Cut k = cut(cs, lim, false);
+            if (best.cs == 0 || k.total < best.total) best = k;
+        }
     }
     if (best.cs == 0) return false;
     const int cs = best.cs;
-    limits(cs, &rlim, &wlim, &alim);
-    best = cut(cs, rlim, wlim, alim, true);
+    limits(cs, &lim);
+    best = cut(cs, lim, true);
+    const Need& most = best.most;
     const int nst = best.nst, lo_ld = C + nst + 2;
-    const int32_t area = (int32_t)(zero + best.area) + 16;  // and what the last row's reads run past it
+    const int32_t area = (int32_t)(zero + most.a) + 16;  // and what the last row's reads run past it
     if (area > 0xffff) return false;  // positions are half words
-    const dd::RowGeom g(kind, cs, nu, (int)best.rmax, (int)best.wmax);
+    const dd::RowGeom g(kind, cs, nu, (int)most.r, (int)most.w);
     std::vector<unsigned char> rec((size_t)nblk * nst * g.rec_bytes, 0);
     std::vector<int32_t> table((size_t)nblk * lo_ld, 0);
     for_blocks(nblk, (size_t)p->ndm * C, [&](int b) {
@@ -541,68 +636,98 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
         const int ns = (int)best.start[b].size() - 1;
         std::copy(lo.begin() + (size_t)b * C, lo.begin() + (size_t)(b + 1) * C, tb);
         tb[C] = ns;
-        std::copy(best.start[b].begin(), best.start[b].end(), tb + C + 1);
-        std::vector<int32_t> at;
+        for (int st = 0; st <= ns; ++st)  // first channels
+            tb[C + 1 + st] = st < ns ? items[b][best.start[b][st]].c : C;
+        std::vector<int32_t> at_row, at_pat;
         for (int st = 0; st < ns; ++st) {
             unsigned char* q = rec.data() + ((size_t)b * nst + st) * g.rec_bytes;
             int32_t* hdr = (int32_t*)q;
-            uint32_t* ent = (uint32_t*)(q + 16);
-            int32_t* desc = (int32_t*)(q + g.desc_off);
+            uint32_t* ent = (uint32_t*)(q + g.ent_off);
+            uint32_t* desc = (uint32_t*)(q + g.desc_off);
             float* w = (float*)(q + g.w_off);
-            const int c0 = best.start[b][st], c1 = best.start[b][st + 1];
-            const int r0 = first[b][c0];
-            hdr[0] = first[b][c1] - r0;
+            const int v0 = best.start[b][st], v1 = best.start[b][st + 1];
+            const int c0 = tb[C + 1 + st];
+            const int nv = v1 - v0;
+            hdr[3] = nv;
             int32_t dst = (int32_t)zero, woff = 0;
-            at.assign((size_t)hdr[0], 0);
-            for (int c = c0; c < c1; ++c)
-                for (int r = first[b][c]; r < first[b][c + 1]; ++r) {
-                    const Row& row = rows[b][r];
-                    int32_t* ds = desc + 4 * (size_t)(r - r0);
-                    at[r - r0] = dst;
-                    ds[0] = (c - c0) * (int32_t)lcap;
-                    ds[1] = dst;
-                    ds[2] = Q - 1 + row.reach + span;
-                    ds[3] = (int32_t)((uint32_t)row.n | (uint32_t)woff << 16);
-                    hdr[2] = std::max(hdr[2], ds[2]);
-                    dst += (int32_t)len_of(row);
-                    if (!fir) continue;
-                    const size_t dc = (size_t)row.trial * C + c;
-                    for (int k = 0; k < row.n; ++k) w[woff + k] = p->unit ? 1.0f : p->w[dc * p->kpad + k];
-                    woff += (row.n + 3) & ~3;
+            at_row.assign((size_t)(first[b][tb[C + 2 + st]] - first[b][c0]), 0);
+            const int r0 = first[b][c0], q0 = items[b][v0].i0;
+            at_pat.assign((size_t)(items[b][v1 - 1].i1 - q0), 0);
+            auto emit = [&](int32_t src0, int32_t src1, int32_t len, int32_t n0, int32_t n1, int32_t wo) {
+                uint32_t* ds = desc + 4 * (size_t)hdr[0]++;
+                ds[0] = (uint32_t)src0 | (uint32_t)src1 << 16;
+                ds[1] = (uint32_t)dst | (uint32_t)len << 16;
+                ds[2] = (uint32_t)n0 | (uint32_t)n1 << 16;
+                ds[3] = (uint32_t)wo;
+                hdr[2] = std::max(hdr[2], len);
+            };
+            for (int v = v0; v < v1; ++v) {
+                const Item& it = items[b][v];
+                const int32_t raw = (it.c - c0) * (int32_t)lcap;
+                for (int i = it.i0; i < it.i1; ++i) {
+                    const Pattern& t = pats[b][i];
+                    at_pat[i - q0] = dst;
+                    emit(raw + low_bits(b, it.c) + t.beg, raw + (int32_t)lcap + low_bits(b, it.c + 1) + t.beg1,
+                         t.end - t.beg + span, rows[b][t.a].n, rows[b][t.b].n, 0);
+                    dst += (int32_t)own_len(t.beg, t.end);
                 }
-            // a trial's position in the row area; trials past the list's end add what the
-            // last one does
-            auto pos = [&](int d, int c) -> uint32_t {
-                if (c >= c1) return 0;  // the zeros
-                const size_t dc = (size_t)std::min(d, p->ndm - 1) * C + c;
-                return (uint32_t)(at[first[b][c] - r0 + rid[dc]] + p->delay[dc] - lo[(size_t)b * C + c]);
+                if (it.nc == 2) continue;
+                for (int r = first[b][it.c]; r < first[b][it.c + 1]; ++r) {
+                    const Row& row = rows[b][r];
+                    at_row[r - r0] = dst;
+                    if (fir) {
+                        emit(raw, 0, Q - 1 + row.end + span, row.n, 0, woff);
+                        dst += (int32_t)whole_len(row);
+                        const size_t dc = (size_t)row.trial * C + it.c;
+                        for (int k = 0; k < row.n; ++k) w[woff + k] = p->unit ? 1.0f : p->w[dc * p->kpad + k];
+                        woff += (row.n + 3) & ~3;
+                    } else {
+                        emit(raw + low_bits(b, it.c) + row.beg, 0, row.end - row.beg + span, row.n, 0, 0);
+                        dst += (int32_t)own_len(row.beg, row.end);
+                    }
+                }
+            }
+            // a trial's position in the row area (fp32: before its channel's misalignment in the raw
+            // buffer); trials past the list's end add what the last one does
+            auto pos = [&](int d, int v) -> uint32_t {
+                if (v >= v1) return 0;  // the zeros
+                const Item& it = items[b][v];
+                const size_t dc = (size_t)std::min(d, p->ndm - 1) * C + it.c;
+                const int32_t start = p->delay[dc] - lo[(size_t)b * C + it.c];
+                if (it.nc == 2) return (uint32_t)(at_pat[it.i0 - q0 + rid[dc]] + start - pats[b][it.i0 + rid[dc]].beg);
+                const int r = first[b][it.c] + rid[dc];
+                return (uint32_t)(at_row[r - r0] + start - (fir ? 0 : rows[b][r].beg));
             };
             for (int j = 0; j < nu && b * db + j * nt < p->ndm; ++j) {
                 const int d0 = b * db + j * nt;
                 if (fir) {
-                    for (int c = c0; c < c1; ++c) {
-                        uint32_t* e = ent + 2 * (size_t)(j * cs + c - c0);
-                        e[0] = pos(d0, c) | pos(d0 + 1, c) << 16;
-                        e[1] = pos(d0 + 2, c);
+                    for (int v = v0; v < v1; ++v) {
+                        uint32_t* e = ent + 2 * (size_t)(j * cs + v - v0);
+                        e[0] = pos(d0, v) | pos(d0 + 1, v) << 16;
+                        e[1] = pos(d0 + 2, v);
                     }
                 } else {
-                    for (int c = c0; c < c1; c += 4) {
-                        uint32_t* e = ent + (size_t)(j * cs + c - c0);
+                    for (int v = v0; v < v1; v += 4) {
+                        uint32_t* e = ent + (size_t)(j * cs + v - v0);
                         for (int u = 0; u < 2; ++u) {
-                            e[2 * u] = pos(d0 + u, c) | pos(d0 + u, c + 1) << 16;
-                            e[2 * u + 1] = pos(d0 + u, c + 2) | pos(d0 + u, c + 3) << 16;
+                            e[2 * u] = pos(d0 + u, v) | pos(d0 + u, v + 1) << 16;
+                            e[2 * u + 1] = pos(d0 + u, v + 2) | pos(d0 + u, v + 3) << 16;
                         }
                     }
                 }
             }
             if (!fir)
-                for (int c = c0; c < c1; c += 4) {
-                    int32_t m[4] = {0, 0, 0, 0};  // longest run of each channel
-                    for (int i = 0; i < 4 && c + i < c1; ++i)
-                        for (int r = first[b][c + i]; r < first[b][c + i + 1]; ++r) m[i] = std::max(m[i], rows[b][r].n);
+                for (int v = v0; v < v1; v += 4) {
+                    int32_t m[4] = {0, 0, 0, 0};  // most taps in a word of each item
+                    for (int i = 0; i < 4 && v + i < v1; ++i)
+                        for (int c = items[b][v + i].c; c < items[b][v + i].c + items[b][v + i].nc; ++c) {
+                            int32_t n = 0;
+                            for (int r = first[b][c]; r < first[b][c + 1]; ++r) n = std::max(n, rows[b][r].n);
+                            m[i] += n;
+                        }
                     const int mode = m[0] + m[1] + m[2] + m[3] <= dd::kPkMaxTaps ? 0
                                      : std::max(m[0] + m[1], m[2] + m[3]) <= dd::kPkMaxTaps ? 1 : 2;
-                    hdr[1] |= mode << ((c - c0) / 2);
+                    hdr[1] |= mode << ((v - v0) / 2);
                 }
         }
     });
@@ -610,8 +735,8 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     p->row_warps = nw;
     p->nch = nch;
     p->cs = cs;
-    p->kw = (int32_t)best.wmax;
-    p->rows_max = (int32_t)best.rmax;
+    p->kw = (int32_t)most.w;
+    p->rows_max = (int32_t)most.r;
     p->blen = area;
     p->lcap = (int32_t)lcap;
     p->nblk = nblk;
@@ -621,10 +746,15 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     p->blk_lo.swap(table);
     p->rec.swap(rec);
     p->dev_dirty = true;
-    dd::log_msg(1, "plan %d trials x %d channels: %s, shared rows (%.3f per trial and channel), %d trials and %d warps "
-                "per CTA, up to %d channels per stage (%.1f stages per block), staged rows of %d elements, row area of "
+    size_t npairs = 0, npats = 0;
+    for (int b = 0; b < nblk; ++b) {
+        npairs += C - items[b].size();
+        npats += pats[b].size();
+    }
+    dd::log_msg(1, "plan %d trials x %d channels: %s, shared rows (%.3f per trial and channel; %zu channel pairs with "
+                "%zu patterns), %d trials and %d warps per CTA, up to %d channels per stage (%.1f stages per block), staged rows of %d elements, row area of "
                 "%d words, record %d bytes, %zu bytes of shared memory", p->ndm, C,
-                fir ? "fp32 sums" : p->rl ? "run-length sums" : "exact integer sums", (double)total / units, db, nw, cs,
+                fir ? "fp32 sums" : p->rl ? "run-length sums" : "exact integer sums", (double)total / units, npairs, npats, db, nw, cs,
                 (double)best.total / nblk, p->lcap, p->blen, p->rec_bytes, dd::dedisp_smem_for(p));
     return true;
 }
@@ -694,9 +824,11 @@ dd_status build_schedule(dd_plan_s* p) {
     return DD_ERR_UNSUPPORTED;
 }
 
-// Fixed CTA shape (nch time chunks) and stage size (cs channels), if it fits.
-dd_status build_schedule_fixed(dd_plan_s* p, int nch, int cs) {
+// Fixed CTA shape (nch time chunks) and stage size (cs channels), if it fits.  tuned: the
+// autotuner's, which may be a row schedule that the tap kernels have no shared memory for.
+dd_status build_schedule_fixed(dd_plan_s* p, int nch, int cs, bool tuned = false) {
     if (nch < 1 || nch > dd::kWarps || (dd::kWarps % nch) != 0 || cs < 1 || cs > 32) return DD_ERR_ARG;
+    if (tuned && build_rows(p, nch, cs)) return DD_OK;
     const int esz = stage_esz(p);
     const int nu = dd::kWarps / nch * units_per_warp(p);
     const int db = trials_per_unit(p) * nu;
@@ -752,8 +884,8 @@ dd_status finish_profiles(dd_plan_s* p) {
     if (p->out_int && p->max_abs_row > INT32_MAX) return DD_ERR_OVERFLOW;
     p->adj_stale = true;
     p->adj_w_stale = true;
-    int64_t bws = 0;
-    for (int d0 = 0; d0 < p->ndm; d0 += 8)
+    int64_t bws = 0;  // (fp32 input only: the weight gradient's staging)
+    for (int d0 = 0; d0 < (p->band.in_type == DD_F32 ? p->ndm : 0); d0 += 8)
         for (int c = 0; c < p->nchan; ++c) {
             int32_t lo = INT32_MAX, hi = 0;
             for (int d = d0; d < std::min(p->ndm, d0 + 8); ++d) {
@@ -843,13 +975,11 @@ static void free_dev(dd_plan_s* p) {
     int cur = -1;
     cudaGetDevice(&cur);
     if (cur != p->dev.device) cudaSetDevice(p->dev.device);
-    cudaFree(p->dev.delay);
-    cudaFree(p->dev.taps);
-    cudaFree(p->dev.w);
-    cudaFree(p->dev.blk_lo);
-    cudaFree(p->dev.rec);
-    cudaFree(p->dev.status);
-    cudaFree(p->dev.off);
+    if (!p->prefix_own) {  // in the slab
+        p->d_prefix = nullptr;
+        p->prefix_elems = 0;
+    }
+    cudaFree(p->dev.slab);
     cudaFree(p->dev.mu);
     cudaFree(p->dev.isd);
     cudaFree(p->dev.widths);
@@ -859,19 +989,11 @@ static void free_dev(dd_plan_s* p) {
     p->widths_on_dev.clear();
 }
 
-template <typename T>
-static dd_status put(T** dst, const T* src, size_t n) {
-    cudaError_t e = cudaMalloc((void**)dst, std::max<size_t>(n, 1) * sizeof(T));
-    if (e != cudaSuccess) return cuda_status(e);
-    if (n) e = cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice);
-    return cuda_status(e);
-}
-
 void destroy_plan(dd_plan_s* p) {
     if (p->adj) destroy_plan(p->adj);
     if (p->d_gpad) cudaFree(p->d_gpad);
     if (p->d_gsplit) cudaFree(p->d_gsplit);
-    if (p->d_prefix) cudaFree(p->d_prefix);
+    if (p->prefix_own) cudaFree(p->d_prefix);
     if (p->d_fkey) cudaFree(p->d_fkey);
     if (p->d_fcarry) cudaFree(p->d_fcarry);
     if (p->d_fseam) cudaFree(p->d_fseam);
@@ -891,31 +1013,60 @@ dd_status upload_tables(dd_plan_s* p) {
     if (p->rec_host != p->rec_bytes && !p->w_follows) build_records(p);  // with the host's weights
     free_dev(p);
     p->dev.device = dev;
+    // one allocation for all tables
     const size_t n = (size_t)p->ndm * p->nchan;
-    dd_status st;
-    if ((st = put(&p->dev.delay, p->delay.data(), n)) != DD_OK) return st;
-    if ((st = put(&p->dev.taps, p->taps.data(), n)) != DD_OK) return st;
-    if (!p->unit && p->w_follows) {
-        e = cudaMalloc((void**)&p->dev.w, n * p->kpad * sizeof(float));
-        if (e != cudaSuccess) return cuda_status(e);
-    } else if (!p->unit && (st = put(&p->dev.w, p->w.data(), p->w.size())) != DD_OK) {
-        return st;
+    const size_t nrec = p->rec_host ? p->rec.size() / p->rec_host : 0;
+    const size_t wlen = p->unit ? 0 : n * (size_t)p->kpad;
+    size_t total = 0;
+    auto room = [&](size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t at_delay = room(n * 4), at_taps = room(n * 4), at_lo = room(p->blk_lo.size() * 4),
+                 at_rec = room(nrec * p->rec_bytes), at_w = room(wlen * sizeof(float)), at_status = room(4),
+                 at_off = room((size_t)p->ndm * sizeof(double));
+    // direct plans' prefix sums: room for the band's block (or 64 Ki outputs), within 2 GiB or what
+    // the longest delay needs; longer calls go in pieces (launch_dedisperse_pk)
+    int64_t pre = 0;
+    if (p->rk == kRowsPk && !p->rl) {
+        const int64_t want = std::max<int64_t>(p->band.nsamp, (int64_t)p->dmax + 65536);
+        const int64_t least = (int64_t)p->dmax + 2 * row_tile_t(kRowsPk, p->nch);
+        pre = ((std::max(least, std::min(want, ((int64_t)1 << 29) / p->nchan)) + 1 + 3) & ~(int64_t)3) * p->nchan;
+        if (pre <= p->prefix_elems) pre = 0;  // there is as much
     }
-    if ((st = put(&p->dev.blk_lo, p->blk_lo.data(), p->blk_lo.size())) != DD_OK) return st;
-    if (p->rec_host == p->rec_bytes) {
-        if ((st = put(&p->dev.rec, p->rec.data(), p->rec.size())) != DD_OK) return st;
-    } else {
-        const size_t nrec = p->rec.size() / p->rec_host;
-        e = cudaMalloc((void**)&p->dev.rec, nrec * p->rec_bytes);
-        if (e == cudaSuccess)
-            e = cudaMemcpy2D(p->dev.rec, p->rec_bytes, p->rec.data(), p->rec_host, p->rec_host, nrec,
-                             cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return cuda_status(e);
+    const size_t at_pre = room((size_t)pre * 4);
+    e = cudaMalloc((void**)&p->dev.slab, total);
+    if (e != cudaSuccess) return cuda_status(e);
+    unsigned char* slab = p->dev.slab;
+    p->dev.delay = (int32_t*)(slab + at_delay);
+    p->dev.taps = (int32_t*)(slab + at_taps);
+    p->dev.blk_lo = (int32_t*)(slab + at_lo);
+    p->dev.rec = slab + at_rec;
+    p->dev.w = p->unit ? nullptr : (float*)(slab + at_w);
+    p->dev.status = (int32_t*)(slab + at_status);
+    p->dev.off = (double*)(slab + at_off);
+    if (pre) {
+        if (p->prefix_own) cudaFree(p->d_prefix);
+        p->prefix_own = false;
+        p->d_prefix = (uint32_t*)(slab + at_pre);
+        p->prefix_elems = pre;
     }
     const int32_t zero = 0;
-    if ((st = put(&p->dev.status, &zero, 1)) != DD_OK) return st;
-    e = cudaMalloc((void**)&p->dev.off, (size_t)p->ndm * sizeof(double));
+    auto up = [&](void* dst, const void* src, size_t bytes) {
+        if (e == cudaSuccess && bytes) e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    };
+    up(p->dev.delay, p->delay.data(), n * 4);
+    up(p->dev.taps, p->taps.data(), n * 4);
+    up(p->dev.blk_lo, p->blk_lo.data(), p->blk_lo.size() * 4);
+    up(p->dev.status, &zero, 4);
+    if (!p->w_follows) up(p->dev.w, p->w.data(), wlen * sizeof(float));
+    if (p->rec_host == p->rec_bytes)
+        up(p->dev.rec, p->rec.data(), p->rec.size());
+    else if (e == cudaSuccess)
+        e = cudaMemcpy2D(p->dev.rec, p->rec_bytes, p->rec.data(), p->rec_host, p->rec_host, nrec, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_status(e);
+    dd_status st;
     // place dd_boxcar_snr_noalloc's scratch array and kernels on this device now, so
     // that its calls allocate nothing (lazy module loading would do it at its first call)
     if ((st = noalloc_preload()) != DD_OK) return st;
@@ -993,19 +1144,31 @@ dd_status dd_plan_create(dd_plan_t* out, const dd_band* band, const double* dms,
     const double k = kdm_of(*band);
     const double top = band_top_ghz(*band);
     const double dnu = band->df_mhz / 1000.0;
-    for (int d = 0; d < ndm; ++d) {
-        for (int c = 0; c < band->nchan; ++c) {
-            const double nu = chan_top_ghz(*band, c);
-            const double lo = nu - dnu;
-            const double raw_d = k * dms[d] * (1.0 / (nu * nu) - 1.0 / (top * top)) / band->dt_ms;
-            const double raw_n = k * dms[d] * (1.0 / (lo * lo) - 1.0 / (nu * nu)) / band->dt_ms;
-            if (!(raw_d < 2.0e9) || !(raw_n < 2.0e9)) {
-                delete p;
-                return DD_ERR_OVERFLOW;
+    // the channels' factors of DM, then the tables
+    std::vector<double> fd(band->nchan), fn(band->nchan);
+    for (int c = 0; c < band->nchan; ++c) {
+        const double nu = chan_top_ghz(*band, c);
+        const double lo = nu - dnu;
+        fd[c] = 1.0 / (nu * nu) - 1.0 / (top * top);
+        fn[c] = 1.0 / (lo * lo) - 1.0 / (nu * nu);
+    }
+    const int nblk = (ndm + 15) / 16;
+    const int64_t far = max_blocks(nblk, n, [&](int b) -> int64_t {
+        for (int d = 16 * b; d < std::min(ndm, 16 * b + 16); ++d) {
+            const double kdm = k * dms[d];
+            for (int c = 0; c < band->nchan; ++c) {
+                const double raw_d = kdm * fd[c] / band->dt_ms;
+                const double raw_n = kdm * fn[c] / band->dt_ms;
+                if (!(raw_d < 2.0e9) || !(raw_n < 2.0e9)) return 1;
+                p->delay[(size_t)d * band->nchan + c] = (int32_t)std::floor(raw_d);
+                p->taps[(size_t)d * band->nchan + c] = std::max(1, (int32_t)std::ceil(raw_n));
             }
-            p->delay[(size_t)d * band->nchan + c] = (int32_t)std::floor(raw_d);
-            p->taps[(size_t)d * band->nchan + c] = std::max(1, (int32_t)std::ceil(raw_n));
         }
+        return 0;
+    });
+    if (far) {
+        delete p;
+        return DD_ERR_OVERFLOW;
     }
     dd_status st = finish_profiles(p);
     if (st != DD_OK) {
@@ -1140,6 +1303,7 @@ dd_status dd_dedisperse(dd_plan_t p, const void* in, int64_t in_ld, int64_t t_of
     dd_status st = dd::upload_tables(p);
     if (st != DD_OK) return st;
     if (p->rl) return dd::launch_dedisperse_rl(p, in, in_ld, t_offset, nsamp, out, out_ld, (cudaStream_t)stream);
+    if (p->rk == dd::kRowsPk) return dd::launch_dedisperse_pk(p, in, in_ld, t_offset, nsamp, out, out_ld, (cudaStream_t)stream);
     return dd::launch_dedisperse(p, in, in_ld, t_offset, t_out, out, out_ld, (cudaStream_t)stream);
 }
 
@@ -1194,12 +1358,16 @@ dd_status dd_backward(dd_plan_t p, const float* in, int64_t in_ld, int64_t t_off
                                (cudaStream_t)stream);
 }
 
+static dd_status set_schedule(dd_plan_s* p, int nch, int cs, bool tuned) {
+    const int old_nch = p->nch, old_cs = p->cs;
+    dd_status st = build_schedule_fixed(p, nch, cs, tuned);
+    if (st != DD_OK && (p->nch != old_nch || p->cs != old_cs)) build_schedule_fixed(p, old_nch, old_cs, true);
+    return st;
+}
+
 dd_status dd_plan_set_schedule(dd_plan_t p, int32_t nch, int32_t cs) {
     if (!p) return DD_ERR_ARG;
-    const int old_nch = p->nch, old_cs = p->cs;
-    dd_status st = build_schedule_fixed(p, nch, cs);
-    if (st != DD_OK && (p->nch != old_nch || p->cs != old_cs)) build_schedule_fixed(p, old_nch, old_cs);
-    return st;
+    return set_schedule(p, nch, cs, false);
 }
 
 dd_status dd_plan_get_schedule(dd_plan_t p, int32_t* nch, int32_t* cs, int32_t* trials_per_cta) {
@@ -1268,18 +1436,19 @@ dd_status dd_plan_autotune(dd_plan_t p, const void* d_in, int64_t in_ld, void* d
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto cache = read_cache(cache_path);
     auto hit = cache.find(key);
-    if (hit != cache.end() && dd_plan_set_schedule(p, hit->second.first, hit->second.second) == DD_OK) {
+    if (hit != cache.end() && set_schedule(p, hit->second.first, hit->second.second, true) == DD_OK) {
         if (best_ms) *best_ms = -1.0f;
         dd::log_msg(1, "autotune %s: cached schedule (%d time chunks, %d channels per stage)", key.c_str(),
                  hit->second.first, hit->second.second);
         return DD_OK;
     }
-    const bool u8 = p->rk ? p->rk == dd::kRowsU8 : stage_esz(p) == 1;
-    const int cs_list_f[] = {2, 3, 4, 6, 8};
-    const int cs_list_u[] = {4, 8, 12, 16};
-    const int* cs_list = u8 ? cs_list_u : cs_list_f;
-    const int ncs = u8 ? 4 : 5;
     const int orig_nch = p->nch, orig_cs = p->cs, orig_rk = p->rk;
+    std::vector<std::pair<int, int>> cand;  // (time chunks, channels per stage)
+    if (orig_rk) cand.push_back({orig_nch, orig_cs});
+    for (int nch = 1; nch <= 2; nch *= 2)
+        for (int cs : orig_rk ? std::vector<int>{8, 16, 28}
+                              : stage_esz(p) == 1 ? std::vector<int>{4, 8, 12, 16} : std::vector<int>{2, 3, 4, 6, 8})
+            cand.push_back({nch, cs});
     int best_nch = orig_nch, best_cs = orig_cs;
     float best = 1e30f;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1287,38 +1456,37 @@ dd_status dd_plan_autotune(dd_plan_t p, const void* d_in, int64_t in_ld, void* d
     if (ce == cudaSuccess) ce = cudaEventCreate(&e1);
     if (ce != cudaSuccess) return dd::cuda_status(ce);
     dd_status st = DD_OK;
-    for (int nch = 1; nch <= 2 && st == DD_OK; nch *= 2) {
-        for (int i = 0; i < ncs; ++i) {
-            if (build_schedule_fixed(p, nch, cs_list[i]) != DD_OK) continue;
-            if (p->rk != orig_rk) continue;  // the same sums in every candidate
+    for (size_t i = 0; i < cand.size() && st == DD_OK; ++i) {
+        // a row plan's first candidate is its schedule as it stands
+        if (!(orig_rk && i == 0) && build_schedule_fixed(p, cand[i].first, cand[i].second, true) != DD_OK) continue;
+        if (p->rk != orig_rk) continue;  // the same sums in every candidate
+        st = dd_dedisperse(p, d_in, in_ld, 0, p->band.nsamp, d_out, out_ld, stream);
+        if (st != DD_OK) break;
+        float t = 1e30f;
+        for (int rep = 0; rep < 2; ++rep) {
+            cudaEventRecord(e0, s);
             st = dd_dedisperse(p, d_in, in_ld, 0, p->band.nsamp, d_out, out_ld, stream);
+            cudaEventRecord(e1, s);
             if (st != DD_OK) break;
-            float t = 1e30f;
-            for (int rep = 0; rep < 2; ++rep) {
-                cudaEventRecord(e0, s);
-                st = dd_dedisperse(p, d_in, in_ld, 0, p->band.nsamp, d_out, out_ld, stream);
-                cudaEventRecord(e1, s);
-                if (st != DD_OK) break;
-                ce = cudaEventSynchronize(e1);
-                if (ce != cudaSuccess) {
-                    st = dd::cuda_status(ce);
-                    break;
-                }
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                t = std::min(t, ms);
+            ce = cudaEventSynchronize(e1);
+            if (ce != cudaSuccess) {
+                st = dd::cuda_status(ce);
+                break;
             }
-            if (st != DD_OK) break;
-            if (t < best) {
-                best = t;
-                best_nch = nch;
-                best_cs = cs_list[i];
-            }
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            t = std::min(t, ms);
+        }
+        if (st != DD_OK) break;
+        if (t < best) {
+            best = t;
+            best_nch = cand[i].first;
+            best_cs = cand[i].second;
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (build_schedule_fixed(p, best_nch, best_cs) != DD_OK) build_schedule_fixed(p, orig_nch, orig_cs);
+    if (build_schedule_fixed(p, best_nch, best_cs, true) != DD_OK) build_schedule_fixed(p, orig_nch, orig_cs, true);
     if (st != DD_OK) return st;
     if (best_ms) *best_ms = best;
     dd::log_msg(1, "autotune %s: %d time chunks, %d channels per stage, %.3f ms (default %d, %d)", key.c_str(),

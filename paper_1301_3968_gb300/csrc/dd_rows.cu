@@ -4,8 +4,8 @@
 namespace dd {
 namespace {
 
-// Tile order as k_dedisp: run-length rows with trial blocks along x (the resident CTAs share
-// time tiles, whose prefix rows then come from L2), other kinds in groups of 16 blocks.
+// Tile order as k_dedisp: packed rows with trial blocks along x (the resident CTAs share time
+// tiles, whose prefix sums then come from L2), fp32 rows in groups of 16 blocks.
 constexpr int kGroupBlocks = 16;
 
 template <int KIND, bool IN8, int NW>
@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) k_rows(DedispArgs a) {
     __shared__ TileState ts;
     if (threadIdx.x == 0) init_pipeline<1>(pipeline_area(smem, a.smem_bytes, 1), ts);
     __syncthreads();
-    if constexpr (KIND == kRowsRl) {
+    if constexpr (KIND == kRowsPk) {
         row_tile<KIND, IN8, NW, false, false>(a, smem, blockIdx.x, blockIdx.y, ts);
     } else {
         const int ntile = (int)gridDim.x, nblk = (int)gridDim.y;
@@ -50,7 +50,7 @@ dd_status run(DedispArgs a, size_t smem, cudaStream_t s) {
     const int64_t tile = row_tile_t(KIND, a.nch);
     const int db = row_trials(KIND, NW, a.nch);
     const unsigned ntile = (unsigned)((a.t_out + tile - 1) / tile), nblk = (unsigned)((a.ndm + db - 1) / db);
-    const bool blk_x = KIND == kRowsRl;
+    const bool blk_x = KIND == kRowsPk;
     dim3 grid(blk_x ? nblk : ntile, blk_x ? ntile : nblk);
     if (grid.y > 65535 || (int64_t)grid.x * grid.y >= INT32_MAX) return DD_ERR_UNSUPPORTED;
     kern<<<grid, NW * 32, smem, s>>>(a);
@@ -81,18 +81,17 @@ int blocks_per_sm(size_t smem) {
 
 size_t rows_smem_for(const dd_plan_s* p) {
     const RowGeom g(p->rk, p->cs, p->row_warps / p->nch, p->rows_max, p->kw);
-    return row_smem_bytes(g, p->row_warps, p->rl ? 4 : (p->band.in_type == DD_U8 ? 1 : 4), p->lcap, p->cs, p->lo_ld,
-                          p->blen);
+    const int esz = p->rk == kRowsFir && p->band.in_type == DD_U8 ? 1 : 4;  // samples or prefix sums
+    return row_smem_bytes(g, p->row_warps, esz, p->lcap, p->cs, p->lo_ld, p->blen);
 }
 
 // fn<kind, uint8 input, warps per CTA>(args) of a row plan
 #define DD_ROWS_NW(fn, kind, in8, nw, ...) \
     ((nw) == kRowWarps ? fn<kind, in8, kRowWarps>(__VA_ARGS__) : fn<kind, in8, kWarps>(__VA_ARGS__))
 #define DD_ROWS(fn, kind, in8, nw, ...)                                     \
-    ((kind) == kRowsRl   ? DD_ROWS_NW(fn, kRowsRl, false, nw, __VA_ARGS__)  \
-     : (kind) == kRowsU8 ? DD_ROWS_NW(fn, kRowsU8, true, nw, __VA_ARGS__)   \
-     : (in8)             ? DD_ROWS_NW(fn, kRowsFir, true, nw, __VA_ARGS__)  \
-                         : DD_ROWS_NW(fn, kRowsFir, false, nw, __VA_ARGS__))
+    ((kind) == kRowsPk ? DD_ROWS_NW(fn, kRowsPk, false, nw, __VA_ARGS__)    \
+     : (in8)           ? DD_ROWS_NW(fn, kRowsFir, true, nw, __VA_ARGS__)    \
+                       : DD_ROWS_NW(fn, kRowsFir, false, nw, __VA_ARGS__))
 
 dd_status launch_rows(const dd_plan_s* p, DedispArgs a, cudaStream_t s) {
     const size_t smem = rows_smem_for(p);

@@ -23,21 +23,24 @@
 // four trials of 15 outputs with one switch per trial 2.40, 8-warp CTAs with two-trial warps
 // 1.91; scalar instead of packed adds 1.24 (two trials).
 //
-// kRowsU8, kRowsRl: exact sums of uint8 samples with unit weights, for runs of at most 257
-// taps (255 n <= 65535).  A row word holds two outputs, B[i] + (B[i + 544] << 16): one load and
-// one 32-bit addition serve both, whatever the start's parity (consecutive outputs in a word
-// would need a second copy of the row for odd starts).  A unit is two trials x 1088 outputs,
-// lane l owning 17 consecutive words.  The channels go four at a time: their words are added up
-// to the point where a half could pass 65535 (the host says: all four, two and two, or each),
-// and those sums into a 32-bit sum of whole words and one of the high halves; low = whole -
-// (high << 16), exact modulo 2^32.  kRowsU8 forms the rows from the staged samples, kRowsRl from
-// packed prefix sums PW[i] = P[i] + (P[i + 544] << 16) in global memory: B = PW[i + n] - PW[i].
-// Bound by shared-memory loads, half a word per trial, channel and output.  (Sharing a word
-// between trials whose starts are close, as the fp32 units do, would save loads but needs a
-// branch per channel; straight code for four channels keeps 68 loads in flight.)
-// Measured: 1500 trials x 336 channels x 21364 outputs 2.62 -> 0.97 ms (1.11e13
-// trial-channel-samples/s; tap kernel 4.1e12), 8192 low-band trials x 1024 channels x 65536
-// outputs (run-length sums, mean 66 taps) 101 -> 48 ms against the 32-bit difference rows.
+// kRowsPk: exact sums of uint8 samples with unit weights, for runs of at most 257 taps (255 n <=
+// 65535).  A row word holds two outputs, B[i] + (B[i + 544] << 16): one load and one 32-bit addition
+// serve both, whatever the start's parity (consecutive outputs in a word would need a second copy
+// of the row for odd starts).  A unit is two trials x 1088 outputs, lane l owning 17 consecutive
+// words.  Rows come from packed prefix sums PW[i] = P[i] + (P[i + 544] << 16) in global memory
+// (k_prefix_packed): B = PW[i + n] - PW[i], exact modulo 2^32.
+// Where it pays (the host counts shared-memory words), two adjacent channels are one item: their
+// trials share the relative delay and both runs in a few patterns (2.2 per pair and 32-trial block
+// on the CRAFT-like lists, 3.2 on the low-band list), a row per pattern holds both channels' sums,
+// and a trial reads one word for the two.
+// Items go four at a time: their words are added up to the point where a half could pass 65535 (the
+// host says: all four, two and two, or each), and those sums into a 32-bit sum of whole words and
+// one of the high halves; low = whole - (high << 16), exact modulo 2^32.
+// Bound by shared-memory loads: a quarter to half a word per trial, channel and output, and the
+// rows' building.  Measured (trial-channel-samples/s): 1500 trials x 336 channels x 21364 outputs:
+// tap kernel 4.1e12, rows from the staged samples in the CTA 1.11e13 (1.20e13 with patterns), from
+// prefix sums 1.76e13; 2048 low-band trials x 1024 x 65536: 32-bit difference rows 5.5e12, packed
+// rows 1.21e13, with patterns 1.54e13.
 //
 // Pipeline: channels stream in stages, as many channels each as their rows fit in a half of
 // the row area.  All warps sum stage i from one half, then build the rows of stage i + 1 in
@@ -58,7 +61,7 @@ namespace {
 // Staged element type; IN8: uint8 input (weighted uint8 plans).
 template <int KIND, bool IN8>
 struct RowIn {
-    using T = typename std::conditional<KIND == kRowsRl, uint32_t, typename std::conditional<IN8, uint8_t, float>::type>::type;
+    using T = typename std::conditional<KIND == kRowsPk, uint32_t, typename std::conditional<IN8, uint8_t, float>::type>::type;
 };
 
 // Four consecutive samples from a 16-byte (fp32) or 4-byte (uint8) aligned address.
@@ -208,50 +211,27 @@ __device__ __forceinline__ void fir_channel(const float* rows, int2 e, int lane_
     fir_shared2<-1, 106>(z, a[2], a[2]);
 }
 
-// Packed words of four quads' first sums from uint8 samples, one quad of words per lane: the
-// sums of n samples from byte i and from byte i + kPkHalf, then the next three words by adding
-// the entering and taking off the leaving sample of both halves at once.
-__device__ __forceinline__ void build_u8(const uint8_t* x, int n, int i, int len, uint32_t* dst) {
+// 256 packed words from packed prefix sums, eight per lane: of one run (x, n taps), or of two
+// channels' runs at once (z, m taps; m = 0: one run).
+__device__ __forceinline__ void build_rl(const uint32_t* x, int n, const uint32_t* z, int m, int i, int len,
+                                         uint32_t* dst) {
     __builtin_assume(__isShared(x));
+    __builtin_assume(__isShared(z));
     __builtin_assume(__isShared(dst));
-    if (i >= len) return;
-    const int nw = n >> 2, rem = n & 3;
-    const uint32_t mask = (1u << (8 * rem)) - 1u;
-    constexpr uint32_t kOnes = 0x01010101u, kEven = 0x00ff00ffu;
-    const uint32_t* pa = (const uint32_t*)(x + i);
-    const uint32_t* pb = (const uint32_t*)(x + i + kPkHalf);
-    const uint32_t a0 = pa[0], b0 = pb[0];
-    uint32_t a = a0, b = b0, sa = 0, sb = 0;
-    for (int j = 0; j < nw; ++j) {
-        sa = __dp4a(a, kOnes, sa);
-        sb = __dp4a(b, kOnes, sb);
-        a = pa[j + 1];
-        b = pb[j + 1];
-    }
-    sa = __dp4a(a & mask, kOnes, sa);
-    sb = __dp4a(b & mask, kOnes, sb);
-    // the samples entering with the next three words: bytes n .. n + 2
-    const uint32_t ea = __funnelshift_r(a, pa[nw + 1], 8 * rem), eb = __funnelshift_r(b, pb[nw + 1], 8 * rem);
-    const uint32_t xe = a0 & kEven, ye = b0 & kEven, xo = (a0 >> 8) & kEven, yo = (b0 >> 8) & kEven;
-    const uint32_t fe = ea & kEven, ge = eb & kEven, fo = (ea >> 8) & kEven, go = (eb >> 8) & kEven;
-    uint4 o;
-    o.x = sa + (sb << 16);
-    o.y = o.x + __byte_perm(fe, ge, 0x5410) - __byte_perm(xe, ye, 0x5410);
-    o.z = o.y + __byte_perm(fo, go, 0x5410) - __byte_perm(xo, yo, 0x5410);
-    o.w = o.z + __byte_perm(fe, ge, 0x7632) - __byte_perm(xe, ye, 0x7632);
-    *(uint4*)(dst + i) = o;
-}
-
-// 256 packed words from packed prefix sums, eight per lane.
-__device__ __forceinline__ void build_rl(const uint32_t* x, int n, int i, int len, uint32_t* dst) {
-    __builtin_assume(__isShared(x));
-    __builtin_assume(__isShared(dst));
-    const uint32_t* y = x + n;
+    const uint32_t *y = x + n, *u = z + m;
+    __builtin_assume(__isShared(y));
+    __builtin_assume(__isShared(u));
     if (i - (i & 31) + 256 <= len) {
+        if (m) {
 #pragma unroll
-        for (int k = 0; k < 256; k += 32) dst[i + k] = y[i + k] - x[i + k];
+            for (int k = 0; k < 256; k += 32) dst[i + k] = (y[i + k] - x[i + k]) + (u[i + k] - z[i + k]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 256; k += 32) dst[i + k] = y[i + k] - x[i + k];
+        }
     } else {
-        for (int k = 0; k < 256 && i + k < len; k += 32) dst[i + k] = y[i + k] - x[i + k];
+        for (int k = 0; k < 256 && i + k < len; k += 32)
+            dst[i + k] = (y[i + k] - x[i + k]) + (m ? u[i + k] - z[i + k] : 0u);
     }
 }
 
@@ -354,7 +334,7 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
     const int nu = NW / wpg;
     const RowGeom rg(KIND, cs, nu, a.rows_max, a.kpad);
     const int rec_off = cs * a.lcap * (int)sizeof(TIN);
-    const int half_words = a.blen + rg.ent_bytes / 4;
+    const int half_words = rg.half_words(a.blen);
     RowSmem sm;
     sm.raw = smem;
     sm.lo = (int*)(smem + ((rec_off + rg.rec_bytes + 127) & ~127));
@@ -401,53 +381,42 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
         const unsigned char* rec = smem + rec_off;
         const TIN* raw = (const TIN*)smem;
         uint32_t* half = sm.half + (i & 1) * half_words;
-        // the entries, each moved by its channel's misalignment in the raw buffer
-        const int c0 = sm.lo[a.nchan + 1 + i], csn = sm.lo[a.nchan + 2 + i] - c0;
+        const int c0 = sm.lo[a.nchan + 1 + i];
         const int4 hdr = *(const int4*)rec;
+        // the misalignment of channel ci of the stage in the raw buffer
+        auto shift = [&](int ci) { return (bq + sm.lo[c0 + ci]) & (Q - 1); };
+        // the entries; fp32 ones moved by that (packed rows begin at their trials' starts)
         int* ed = (int*)(half + a.blen);
         if (tid == 0) *(int4*)ed = hdr;
-        auto shift = [&](int ci) { return ci < csn ? (bq + sm.lo[c0 + ci]) & (Q - 1) : 0; };
         if constexpr (FIR) {
-            const int2* es = (const int2*)(rec + 16);
+            const int2* es = (const int2*)(rec + rg.ent_off);
             for (int e = tid; e < nu * cs; e += NW * 32) {
-                const int ci = e % cs;
-                if (ci >= csn) continue;
-                const int sh = shift(ci);
-                const int2 v = es[e];
-                ((int2*)(ed + 4))[e] = make_int2(v.x + sh + (sh << 16), v.y + sh);
+                const int v = e % cs;
+                if (v >= hdr.w) continue;
+                const int sh = shift(v);
+                const int2 q = es[e];
+                ((int2*)(ed + 4))[e] = make_int2(q.x + sh + (sh << 16), q.y + sh);
             }
         } else {
-            const int4* es = (const int4*)(rec + 16);
-            const int ng = cs / 4;
-            for (int e = tid; e < nu * ng; e += NW * 32) {
-                const int c = e % ng * 4;
-                if (c >= csn) continue;
-                const int s01 = shift(c) + (shift(c + 1) << 16), s23 = shift(c + 2) + (shift(c + 3) << 16);
-                const int4 v = es[e];
-                ((int4*)(ed + 4))[e] = make_int4(v.x + s01, v.y + s23, v.z + s01, v.w + s23);
-            }
+            const int4* es = (const int4*)(rec + rg.ent_off);
+            for (int e = tid; e < nu * (cs / 4); e += NW * 32) ((int4*)(ed + 4))[e] = es[e];
         }
-        const int nrows = hdr.x;
-        const int4* desc = (const int4*)(rec + rg.desc_off);
-        // tasks of 256 outputs or words (128 words from uint8 samples), one warp each
-        constexpr int kTask = KIND == kRowsU8 ? 128 : 256;
-        const int per = (hdr.z + kTask - 1) / kTask;
-        const int dr = NW / per, dp = NW - dr * per;
+        // tasks of 256 outputs or words of a row, one warp each
+        const uint4* desc = (const uint4*)(rec + rg.desc_off);
+        const int per = (hdr.z + 255) >> 8, dr = NW / per, dp = NW - dr * per;
         int r = warp / per, part = warp - r * per;
-        for (; r < nrows; r += dr, part += dp, r += part >= per, part -= part >= per ? per : 0) {
-            const int4 q = desc[r];  // (source, destination, length, taps | weights << 16)
-            const int n = q.w & 0xffff;
-            if (!dbg_ok(q.x >= 0 && q.y >= 0 && q.z >= 0 && n >= 1 && q.y + ((q.z + 3) & ~3) <= a.blen &&
-                            q.x + q.z + n <= cs * a.lcap,
+        for (; r < hdr.x; r += dr, part += dp, r += part >= per, part -= part >= per ? per : 0) {
+            const uint4 q = desc[r];
+            const int src = (int)(q.x & 0xffff), len = (int)(q.y >> 16), dst = (int)(q.y & 0xffff);
+            const int n = (int)(q.z & 0xffff), m = (int)(q.z >> 16);
+            if (!dbg_ok(n >= 1 && dst + ((len + 3) & ~3) <= a.blen && src + len + n <= cs * a.lcap &&
+                            (int)(q.x >> 16) + (m ? len + m : 0) <= cs * a.lcap,
                         a.status))
                 continue;
             if constexpr (FIR)
-                build_fir<TIN>(raw + q.x, (const float*)(rec + rg.w_off) + ((uint32_t)q.w >> 16), n,
-                               part * kTask + 4 * lane, q.z, (float*)half + q.y);
-            else if constexpr (KIND == kRowsU8)
-                build_u8(raw + q.x, n, part * kTask + 4 * lane, q.z, half + q.y);
+                build_fir<TIN>(raw + src, (const float*)(rec + rg.w_off) + q.w, n, part * 256 + 4 * lane, len, (float*)half + dst);
             else
-                build_rl(raw + q.x, n, part * kTask + lane, q.z, half + q.y);
+                build_rl(raw + src, n, raw + (q.x >> 16), m, part * 256 + lane, len, half + dst);
         }
     };
     auto parity_of = [&](int i) { return (uint32_t)(((MULTI ? ts.uses[0] : 0) + i) & 1); };
@@ -462,13 +431,13 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
     for (int i = 0; ok && i < nst; ++i) {
         const uint32_t* half = sm.half + (i & 1) * half_words;
         if (d < a.ndm) {
-            const int csn = sm.lo[a.nchan + 2 + i] - sm.lo[a.nchan + 1 + i];
+            const int nv = ((const int4*)(half + a.blen))->w;  // items
             if constexpr (FIR) {
                 const int2* ent = (const int2*)(half + a.blen + 4) + wu * cs;
                 __builtin_assume(__isShared(ent));
                 int2 next = ent[0];
 #pragma unroll 1
-                for (int ci = 0; ci < csn; ++ci) {
+                for (int ci = 0; ci < nv; ++ci) {
                     const int2 e = next;
                     next = ent[ci + 1];
                     if (!dbg_ok(max(max(e.x & 0xffff, (int)((uint32_t)e.x >> 16)), e.y) + lane_off + R + 4 <= a.blen,
@@ -482,7 +451,7 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
                 const uint32_t* rows = half + lane_off;
                 int modes = ((const int4*)(half + a.blen))->y;
 #pragma unroll 1
-                for (int ci = 0; ci < csn; ci += 4, modes >>= 2) {
+                for (int ci = 0; ci < nv; ci += 4, modes >>= 2) {
                     const uint4 e = ent[ci / 4];
                     if (!dbg_ok((int)max(max(max(e.x & 0xffffu, e.x >> 16), max(e.y & 0xffffu, e.y >> 16)),
                                          max(max(e.z & 0xffffu, e.z >> 16), max(e.w & 0xffffu, e.w >> 16))) +

@@ -56,9 +56,8 @@ int fused_bps(size_t smem) {
 
 #define DD_ROWS_NW(fn, kind, in8, nw, ...) \
     ((nw) == kRowWarps ? fn<kind, in8, kRowWarps>(__VA_ARGS__) : fn<kind, in8, kWarps>(__VA_ARGS__))
-#define DD_ROWS(fn, p, ...)                                                                 \
-    ((p)->rk == kRowsRl            ? DD_ROWS_NW(fn, kRowsRl, false, (p)->row_warps, __VA_ARGS__)  \
-     : (p)->rk == kRowsU8          ? DD_ROWS_NW(fn, kRowsU8, true, (p)->row_warps, __VA_ARGS__)   \
+#define DD_ROWS(fn, p, ...)                                                                     \
+    ((p)->rk == kRowsPk            ? DD_ROWS_NW(fn, kRowsPk, false, (p)->row_warps, __VA_ARGS__)  \
      : (p)->band.in_type == DD_U8 ? DD_ROWS_NW(fn, kRowsFir, true, (p)->row_warps, __VA_ARGS__)  \
                                   : DD_ROWS_NW(fn, kRowsFir, false, (p)->row_warps, __VA_ARGS__))
 

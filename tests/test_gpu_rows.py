@@ -256,3 +256,20 @@ def test_batch_of_rows_and_taps(dd):
     s.synchronize()
     for p, x, o in zip(plans, xs, outs):
         assert torch.equal(p.dedisperse(x, nsamp=p.band.nsamp), o)
+
+
+def test_direct_calls_longer_than_the_band_go_in_pieces(dd):
+    """A direct plan's prefix sums have room for its band's block; a longer call is summed in
+    pieces, with the same results."""
+    import torch
+    rng = np.random.default_rng(91)
+    C, D, T = 6, 40, 150000
+    delay, taps = _tables(rng, D, C, [0, 1, 2], [2, 9], 20)
+    I = _input(rng, "u8", C, T + 16)
+    plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, 3000, "u8"), np.zeros(D))
+    plan.set_profiles(delay=delay, taps=taps)
+    plan.set_method("direct")
+    got = plan.dedisperse(torch.from_numpy(I).cuda(), t_offset=5, nsamp=T).cpu().numpy()
+    rows = [0, 17, D - 1]
+    want = oracle.c_dedisperse(I, delay, taps, t_offset=5, nsamp=T, rows=rows)
+    np.testing.assert_array_equal(got[rows].astype(np.int64), want)
