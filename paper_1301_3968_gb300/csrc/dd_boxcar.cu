@@ -547,6 +547,46 @@ __device__ __forceinline__ void run_segment(const TX* xl, TX o, typename Acc<TB>
     }
 }
 
+// The earliest of the kBoxS starts from t0 whose width-w sum of x - o is b (a warp; modulo 2^32):
+// the first window's sum over the lanes, then one start per lane from a scan of the differences.
+__device__ __forceinline__ int first_start(const int* xrow, int o, int t_len, int w, int t0, int b, int lane) {
+    uint32_t r = 0;
+#pragma unroll 4
+    for (int k = lane; k < w; k += 32) r += (uint32_t)(xrow[t0 + k] - o);  // (t0 + w <= t_len)
+    r = warp_sum(r);
+    const int t = t0 + lane;
+    const bool in = lane < kBoxS && t + w <= t_len;
+    const uint32_t diff = in && t + w < t_len ? (uint32_t)xrow[t + w] - (uint32_t)xrow[t] : 0u;
+    uint32_t incl = diff;
+#pragma unroll
+    for (int ofs = 1; ofs < 32; ofs <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, ofs);
+        if (lane >= ofs) incl += v;
+    }
+    const unsigned hit = __ballot_sync(0xffffffffu, in && (int)(r + incl - diff) == b);
+    return hit ? t0 + __ffs(hit) - 1 : -1;
+}
+
+// S/N of trial d's width j from the largest sum and its start, and the candidate it may be.
+__device__ __forceinline__ void emit_peak(const BoxArgs& a, int d, int j, double b, int arg) {
+    const int64_t o2 = (int64_t)d * a.nw + j;
+    if (!dbg_ok(d < a.ndm && j < a.nw, a.status)) return;
+    const float snr = (float)((b - (double)a.mu[o2]) * (double)a.isd[o2]);
+    a.peak[o2] = snr;
+    a.arg[o2] = arg;
+    if (a.cands && snr > a.thresh) {
+        const int k = atomicAdd(a.ncands, 1);
+        if (k < a.cap) {
+            dd_candidate cd;
+            cd.dm_index = d;
+            cd.width_index = j;
+            cd.t = arg;
+            cd.snr = snr;
+            a.cands[k] = cd;
+        }
+    }
+}
+
 // grid (CTAs of gpc width groups, trials).  The CTA's warps split into gpc groups of
 // 8 / gpc warps; all of them scan the same staged chunk of 32 * (8 / gpc) * S samples,
 // each group for its own 16 widths, so a row is read once per gpc groups.  Thread
@@ -761,6 +801,156 @@ __global__ void __launch_bounds__(256, std::is_same<TB, float>::value ? 3 : 2) k
     }
 }
 
+// Any increasing width list on integer series whose sums fit int32.  The chunk's prefix sums P of
+// x - o lie in shared memory (modulo 2^32, differences exact), a thread holds P of its kBoxS
+// consecutive starts in registers, and B_w(t) = P[t + w] - P[t] costs one load (odd stride: no
+// conflicts), one subtraction and half a three-input maximum whatever the widths are.  Maxima are
+// kept per segment and chunk as in k_boxcar_run; a warp per width finds the earliest start of the
+// winning segment.  Bound by instruction issue (2.6 per start and width) and the shared loads.
+// k_boxcar's running sums cost two loads, an addition, a comparison and two selects each: octave
+// widths 1-512 on 1500 x 21364 (normaliser included) 291 us with it, 129 with this.
+__host__ __device__ inline int list_buf(int wmax) { return (256 * kBoxS + wmax + 12) & ~3; }
+
+__global__ void __launch_bounds__(256, 3) k_boxcar_list(BoxArgs a) {
+    constexpr int S = kBoxS, G = kBoxG, chunk = 256 * S;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int rb[8][G];
+    __shared__ int rc[8][G];
+    __shared__ int rt[8][G];
+    __shared__ uint32_t psum[8];
+    const int d = blockIdx.y;
+    if (a.narrow && (int)a.narrow[d] != a.narrow_sel) return;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int j0 = blockIdx.x * G;
+    const int cnt = min(G, a.nw - j0);
+    const int wmin = a.widths[j0], wmax = a.widths[j0 + cnt - 1];
+    const int bufl = list_buf(a.widths[a.nw - 1]);
+    int* const raw = (int*)smem_raw;
+    uint32_t* const P = (uint32_t*)(raw + bufl);
+    const int o = (int)a.off[d];
+    const int* xrow = (const int*)a.x + (int64_t)d * a.ld;
+    const int mis = (int)(((uintptr_t)xrow >> 2) & 3);
+    const int n16 = (chunk + wmax + mis + 4) >> 2;  // quads: P[0 .. chunk + wmax] behind the misalignment
+    if (!dbg_ok(4 * n16 <= bufl, a.status)) return;
+    int best[G], bch[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+        best[j] = INT_MIN;
+        bch[j] = -1;
+    }
+    auto load = [&](int tc) {  // as k_boxcar_run's; pieces past the row's end keep older words
+        for (int i = tid; i < n16; i += 256) {
+            const int t = tc - mis + 4 * i;
+            if (t < 0) {
+                for (int k = -t; k < 4; ++k) {
+                    const bool ok = t + k < a.t_len;
+                    cp_async4(raw + 4 * i + k, ok ? xrow + t + k : xrow, ok);
+                }
+            } else if (t < a.t_len) {
+                cp_async16(raw + 4 * i, xrow + t, 4 * min(4, a.t_len - t));
+            }
+        }
+        cp_async_commit();
+    };
+    const int tvalid = a.t_len - wmin + 1;
+    const int per = ((n16 + 255) >> 8) | 1;  // quads per thread in the scan (odd: no conflicts)
+    const int q0 = min(n16, tid * per), q1 = min(n16, q0 + per);
+    const int ls = tid * S;
+    load(0);
+    for (int ci = 0, tc = 0; tc < tvalid; ++ci, tc += chunk) {
+        cp_async_wait<0>();
+        __syncthreads();
+        uint32_t sum = 0;
+        for (int i = q0; i < q1; ++i) {
+            const int4 v = ((const int4*)raw)[i];
+            sum += (uint32_t)v.x + (uint32_t)v.y + (uint32_t)v.z + (uint32_t)v.w - 4u * (uint32_t)o;
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int ofs = 1; ofs < 32; ofs <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, ofs);
+            if (lane >= ofs) incl += v;
+        }
+        if (lane == 31) psum[warp] = incl;
+        __syncthreads();
+        uint32_t run = incl - sum;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) run += w < warp ? psum[w] : 0u;
+        for (int i = q0; i < q1; ++i) {
+            const int4 v = ((const int4*)raw)[i];
+            uint4 r;
+            r.x = run;
+            r.y = r.x + (uint32_t)(v.x - o);
+            r.z = r.y + (uint32_t)(v.y - o);
+            r.w = r.z + (uint32_t)(v.z - o);
+            run = r.w + (uint32_t)(v.w - o);
+            ((uint4*)P)[i] = r;
+        }
+        __syncthreads();  // P is complete, the raw samples are free
+        if (tc + chunk < tvalid) load(tc + chunk);
+        if (tc + ls < tvalid) {
+            const uint32_t* p = P + mis + ls;
+            __builtin_assume(__isShared(p));
+            uint32_t q[S];
+#pragma unroll
+            for (int k = 0; k < S; ++k) q[k] = p[k];
+            const bool full = tc + ls + S - 1 + wmax <= a.t_len;
+#pragma unroll
+            for (int j = 0; j < G; ++j) {
+                if (j < cnt) {
+                    const int w = a.widths[j0 + j];
+                    const uint32_t* y = p + w;
+                    __builtin_assume(__isShared(y));
+                    int m = INT_MIN;
+                    if (full) {
+#pragma unroll
+                        for (int k = 0; k + 1 < S; k += 2)
+                            m = __vimax3_s32(m, (int)(y[k] - q[k]), (int)(y[k + 1] - q[k + 1]));
+                        m = max(m, (int)(y[S - 1] - q[S - 1]));
+                    } else {
+                        const int last = a.t_len - w - tc - ls;  // starts past it run off the series
+#pragma unroll
+                        for (int k = 0; k < S; ++k)
+                            if (k <= last) m = max(m, (int)(y[k] - q[k]));
+                    }
+                    if (m > best[j]) {
+                        best[j] = m;
+                        bch[j] = ci;
+                    }
+                }
+            }
+        }
+        __syncthreads();  // P is rewritten by the next chunk
+    }
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+        const int b = warp_top(best[j]);
+        const uint32_t c = best[j] == b ? (uint32_t)bch[j] : 0xffffffffu;
+        const uint32_t cm = __reduce_min_sync(0xffffffffu, c);
+        const uint32_t who = __ballot_sync(0xffffffffu, c == cm);
+        if (lane == 0) {
+            rb[warp][j] = b;
+            rc[warp][j] = (int)cm;
+            rt[warp][j] = tid + __ffs(who) - 1;
+        }
+    }
+    __syncthreads();
+    for (int j = warp; j < cnt; j += 8) {  // a warp per width
+        int b = rb[0][j], c = rc[0][j], th = rt[0][j];
+        for (int k = 1; k < 8; ++k) {
+            const int ob = rb[k][j], oc = rc[k][j], ot = rt[k][j];
+            if (oc >= 0 && (c < 0 || ob > b || (ob == b && (oc < c || (oc == c && ot < th))))) {
+                b = ob;
+                c = oc;
+                th = ot;
+            }
+        }
+        const int w = a.widths[j0 + j];
+        const int arg = c < 0 ? -1 : first_start(xrow, o, a.t_len, w, c * chunk + th * S, b, lane);
+        if (lane == 0) emit_peak(a, d, j0 + j, (double)b, arg);
+    }
+}
+
 // Width groups per CTA: up to eight (a row is read once per eight groups; measured on the
 // large block's 16 groups: 0.208 s with four per CTA, 0.200 s with eight).
 template <typename TX, typename TB>
@@ -777,6 +967,22 @@ dd_status run_boxcar_contig(const BoxArgs& a0, int w0_last, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e);
     dim3 grid((unsigned)((ng + a.gpc - 1) / a.gpc), (unsigned)a.ndm);
+    if (grid.y > 65535) return DD_ERR_UNSUPPORTED;
+    kern<<<grid, 256, smem, s>>>(a);
+    return cuda_status(cudaGetLastError());
+}
+
+// Lists up to this width leave k_boxcar_list, with its raw and prefix buffers, two CTAs per SM;
+// wider ones keep k_boxcar's single buffer.  (Twelve octaves to 2048: 475 us with k_boxcar, 167
+// with k_boxcar_list; 40 widths in steps of 3 to 118: 791 and 366; two widths: 184 and 90.)
+constexpr int kListWmax = 4096;
+
+dd_status run_boxcar_list(const BoxArgs& a, int wmax_all, cudaStream_t s) {
+    const size_t smem = (size_t)2 * list_buf(wmax_all) * sizeof(int);
+    auto kern = k_boxcar_list;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_status(e);
+    dim3 grid((unsigned)((a.nw + kBoxG - 1) / kBoxG), (unsigned)a.ndm);
     if (grid.y > 65535) return DD_ERR_UNSUPPORTED;
     kern<<<grid, 256, smem, s>>>(a);
     return cuda_status(cudaGetLastError());
@@ -834,7 +1040,8 @@ static dd_status dispatch_boxcar(const dd_plan_s* p, const BoxArgs& a0, const in
     // width-w sum fits int32 when wmax * 255 * max_d N_S(d) < 2^31
     const long long bound = (long long)wmax * p->max_abs_row;
     if (bound < (long long)INT_MAX)
-        return contig ? run_boxcar_contig<int, int>(a, w0_last, s) : run_boxcar<int, int>(a, wmax, s);
+        return contig ? run_boxcar_contig<int, int>(a, w0_last, s)
+               : (wmax <= kListWmax ? run_boxcar_list(a, wmax, s) : run_boxcar<int, int>(a, wmax, s));
     if (!contig || !split_rows || !p->dev.narrow)
         return contig ? run_boxcar_contig<int, long long>(a, w0_last, s) : run_boxcar<int, long long>(a, wmax, s);
     // the plan-wide bound needs int64, but rows of noise-like series rarely do: measure
@@ -950,7 +1157,7 @@ dd_status preload_boxcar_kernels() {
     const void* kerns[] = {
         (const void*)k_norm,
         (const void*)k_boxcar_run<float, float>, (const void*)k_boxcar<float, float>,
-        (const void*)k_boxcar_run<int, int>, (const void*)k_boxcar<int, int>,
+        (const void*)k_boxcar_run<int, int>, (const void*)k_boxcar<int, int>, (const void*)k_boxcar_list,
         (const void*)k_boxcar_run<int, long long>, (const void*)k_boxcar<int, long long>,
     };
     for (const void* k : kerns) {
