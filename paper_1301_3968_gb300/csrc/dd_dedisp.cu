@@ -380,6 +380,38 @@ dd_status launch_prefix_into(const dd_plan_s* p, const void* in, int64_t ld, int
     return cuda_status(cudaGetLastError());
 }
 
+// A stream that is being captured is not ordered here (its events cannot leave the capture).
+// The legacy stream, which outlives every call, is recorded when another stream follows it.
+PrefixUse::PrefixUse(dd_plan_s* plan, cudaStream_t stream) : p(plan), s(stream) {
+    if (!p || p->rl) return;
+    lock = std::unique_lock<std::mutex>(p->prefix_mu);
+    if (s == nullptr || s == cudaStreamLegacy) {
+        id = 1;
+    } else {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return;
+        }
+        err = cudaStreamGetId(s, &id);
+        id += 2;
+    }
+    if (err != cudaSuccess || p->prefix_stream == 0 || p->prefix_stream == id) return;
+    if (p->prefix_stream == 1) err = mark(cudaStreamLegacy);
+    if (err == cudaSuccess) err = cudaStreamWaitEvent(s, p->prefix_done, 0);
+}
+
+cudaError_t PrefixUse::mark(cudaStream_t q) {
+    cudaError_t e = cudaSuccess;
+    if (!p->prefix_done) e = cudaEventCreateWithFlags(&p->prefix_done, cudaEventDisableTiming);
+    return e == cudaSuccess ? cudaEventRecord(p->prefix_done, q) : e;
+}
+
+PrefixUse::~PrefixUse() {
+    if (id == 0 || err != cudaSuccess) return;
+    if (id == 1 || mark(s) == cudaSuccess) p->prefix_stream = id;
+}
+
 // Run-length path: prefix sums of columns t_offset .. t_offset + nsamp - 1 into the
 // plan's scratch, then the run-length sums over them.
 dd_status launch_prefix(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset, int64_t nsamp,
@@ -388,12 +420,17 @@ dd_status launch_prefix(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offs
     *ldp_out = ldp;
     const int64_t need = ldp * p->nchan;
     if (need > p->prefix_elems) {
-        if (p->prefix_own) cudaFree(p->d_prefix);
-        p->d_prefix = nullptr;
-        p->prefix_elems = 0;
-        p->prefix_own = false;
-        cudaError_t e = cudaMalloc((void**)&p->d_prefix, (size_t)need * sizeof(uint32_t));
+        if (p->rl && p->prefix_own) {
+            cudaFree(p->d_prefix);
+            p->d_prefix = nullptr;
+            p->prefix_elems = 0;
+            p->prefix_own = false;
+        }
+        uint32_t* q = nullptr;  // (a direct plan keeps its scratch if there is no more)
+        cudaError_t e = cudaMalloc((void**)&q, (size_t)need * sizeof(uint32_t));
         if (e != cudaSuccess) return cuda_status(e);
+        if (p->prefix_own) cudaFree(p->d_prefix);
+        p->d_prefix = q;
         p->prefix_elems = need;
         p->prefix_own = true;
     }
@@ -419,6 +456,8 @@ dd_status launch_dedisperse_pk(dd_plan_s* p, const void* in, int64_t ld, int64_t
     int64_t piece = std::min(cols - 4 - p->dmax, 65535 * tile);  // (grid y)
     if (piece < t_out) piece = piece / tile * tile;
     if (piece < 1) return DD_ERR_OOM;
+    PrefixUse use(p, s);
+    if (use.err != cudaSuccess) return cuda_status(use.err);
     for (int64_t t0 = 0; t0 < t_out; t0 += piece) {
         const int64_t n = std::min(piece, t_out - t0) + p->dmax, ldp = (n + 1 + 3) & ~(int64_t)3;
         dd_status st = launch_prefix_into(p, in, ld, t_offset + t0, n, p->d_prefix, ldp, s);

@@ -411,6 +411,8 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
     if ((st = launch_norm(p, widths, nw, mean, sd, s)) != DD_OK) return st;
 
     DedispArgs a;
+    PrefixUse use(reads_prefix(p) ? p : nullptr, s);
+    if (use.err != cudaSuccess) return cuda_status(use.err);
     if (reads_prefix(p)) {
         int64_t ldp = 0;
         if ((st = launch_prefix(p, in, in_ld, t_offset, nsamp, &ldp, s)) != DD_OK) return st;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <mutex>
 #include <vector>
 
 #include "dd.h"
@@ -315,6 +316,11 @@ struct dd_plan_s {
     uint32_t* d_prefix = nullptr;
     int64_t prefix_elems = 0;
     bool prefix_own = false;           // d_prefix is an allocation of its own (else in the slab)
+    // direct plans: a call on another stream waits for the last one's reads of the prefix sums
+    // (calls on several streams needed no workspace when the taps were summed one by one)
+    std::mutex prefix_mu;
+    unsigned long long prefix_stream = 0;  // the last call's stream (its id; 0: none, 1: the legacy one)
+    cudaEvent_t prefix_done = nullptr;
     // row kernels (RowKind): the schedule above is then theirs
     int32_t rk = 0;
     int32_t rows_max = 0;
@@ -348,6 +354,23 @@ dd_status launch_dedisperse_batched(bool u8, bool pair, bool short_taps, const D
                                     const BatchItem* d_items, int32_t nitems, size_t smem, cudaStream_t s,
                                     bool rl = false);
 int dedisp_batched_blocks_per_sm(bool u8, bool pair, bool short_taps, size_t smem, bool rl = false);
+// A call's use of its plan's prefix scratch (p null: none), from the prefix pass to the last launch
+// that reads it: on a direct plan it waits for the last use on another stream.
+struct PrefixUse {
+    PrefixUse(dd_plan_s* p, cudaStream_t s);
+    ~PrefixUse();
+    PrefixUse(const PrefixUse&) = delete;
+    PrefixUse& operator=(const PrefixUse&) = delete;
+    cudaError_t err = cudaSuccess;
+
+private:
+    cudaError_t mark(cudaStream_t q);
+    dd_plan_s* p;
+    cudaStream_t s;
+    std::unique_lock<std::mutex> lock;
+    unsigned long long id = 0;
+};
+
 dd_status launch_prefix_into(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                              int64_t nsamp, uint32_t* P, int64_t ldp, cudaStream_t s);
 // direct plans on packed rows: prefix sums into the plan's scratch and the launch, in pieces that fit

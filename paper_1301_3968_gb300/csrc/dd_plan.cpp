@@ -979,6 +979,9 @@ static void free_dev(dd_plan_s* p) {
         p->d_prefix = nullptr;
         p->prefix_elems = 0;
     }
+    if (p->prefix_done) cudaEventDestroy(p->prefix_done);
+    p->prefix_done = nullptr;
+    p->prefix_stream = 0;
     cudaFree(p->dev.slab);
     cudaFree(p->dev.mu);
     cudaFree(p->dev.isd);

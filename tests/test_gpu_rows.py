@@ -273,3 +273,36 @@ def test_direct_calls_longer_than_the_band_go_in_pieces(dd):
     rows = [0, 17, D - 1]
     want = oracle.c_dedisperse(I, delay, taps, t_offset=5, nsamp=T, rows=rows)
     np.testing.assert_array_equal(got[rows].astype(np.int64), want)
+
+
+@pytest.mark.parametrize("fused", [False, True])
+def test_direct_plan_on_alternating_streams(dd, fused):
+    """Two streams take one direct plan's calls in turn, with no synchronisation between them:
+    each reads its own block's prefix sums."""
+    import torch
+    rng = np.random.default_rng(61)
+    C, D, T = 64, 600, 40000
+    delay, taps = _tables(rng, D, C, [0, 1], [2, 3], 48)
+    plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, T, "u8"), np.zeros(D))
+    plan.set_profiles(delay=delay, taps=taps)
+    assert plan.method == "direct"
+    xs = [torch.from_numpy(_input(rng, "u8", C, T)).cuda() for _ in range(4)]
+    m, sd = plan.channel_stats(xs[0])
+    wl = np.arange(1, 9, dtype=np.int32)
+    want = [plan.dedisperse(x) for x in xs]
+    peak = plan.dedisperse_boxcar(xs[3], wl, m, sd)[0] if fused else None
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.default_stream(), torch.cuda.Stream()]
+    for _ in range(3):
+        got = []
+        for x, s in zip(xs, streams):
+            with torch.cuda.stream(s):
+                if fused and s is streams[3]:
+                    p = plan.dedisperse_boxcar(x, wl, m, sd)[0]
+                else:
+                    got.append(plan.dedisperse(x))
+        torch.cuda.synchronize()
+        for g, w in zip(got, want):
+            assert torch.equal(g, w)
+        if fused:
+            assert torch.equal(p, peak)
