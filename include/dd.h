@@ -293,7 +293,9 @@ dd_status dd_plan_get_method(dd_plan_t plan, int32_t* method);
  * and appends
  * it to the text cache at cache_path (may be NULL) under a key of channel count, input
  * type, path, and the powers of two of the trial-block delay spread and the widest tap
- * run.  A cached key is applied without timing (*best_ms = -1).  Synchronises the
+ * run.  A plan whose trials share their tap sums (row kernels; 8, 16, 28 channels) keeps its
+ * own schedule, recorded as 0 channels, unless another is clearly faster.  A cached key is
+ * applied without timing (*best_ms = -1).  Synchronises the
  * stream; overwrites d_out.  Errors: DD_ERR_ARG, DD_ERR_CUDA. */
 dd_status dd_plan_autotune(dd_plan_t plan, const void* d_in, int64_t in_ld, void* d_out,
                            int64_t out_ld, const char* cache_path, float* best_ms, void* stream);
