@@ -37,8 +37,12 @@ constexpr int G = 16;  // widths per register window
 
 // A warp's shared scratch for the earliest-start search (4-byte words): the prefix values
 // P_0 .. P_30 of one segment, then P_{w0g} .. P_{w0g+45} (every P_s and P_{s+w} that a
-// width of the group forms).  Segments of up to 35 starts (the packed row kernels' tiles).
-constexpr int kSegPk = 35;
+// width of the group forms).  The packed row kernels' segments are 34 starts, of which 32 lanes
+// make their 1088-output tile exactly: 35 (odd, so without the two-way bank conflicts) left one
+// lane a partial segment, and its warp the masked scan beside the full one for every group
+// (1500 low-band trials x 1024 channels x 35300 outputs, widths 1-256: 8.01 ms with 35, 5.94 with
+// 34 and two starts per step; widths 1-64: 4.84 and 4.34).
+constexpr int kSegPk = 34;
 constexpr int kChainFloats = 2 * kSegPk + G - 1;
 
 // S starts of one lane segment (x = row + i0) for widths w0g + j, j < G.
@@ -51,17 +55,31 @@ __device__ __forceinline__ void scan_segment(const int* x, uint32_t q, int w0g, 
     win[0] = q;
 #pragma unroll
     for (int j = 1; j < G; ++j) win[j] = win[j - 1] + (uint32_t)x[w0g + j - 1];
+    auto val = [&](uint32_t P, uint32_t p, int s, int j) {
+        return FULL || (i0 + s >= i_lo && i0 + s < i_hi && i0 + s + w0g + j <= e_hi) ? (int)(P - p) : INT_MIN;
+    };
     uint32_t p = 0;
+    if constexpr (S % 2 == 0) {  // two starts per step, merged with one three-input maximum
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
+        for (int s = 0; s < S; s += 2) {
+            const uint32_t p1 = p + (uint32_t)x[s];
+            const uint32_t next = win[(s + G - 1) % G] + (uint32_t)x[s + w0g + G - 1];
 #pragma unroll
-        for (int j = 0; j < G; ++j) {
-            int v = (int)(win[(j + s) % G] - p);
-            if (!FULL) v = (i0 + s >= i_lo && i0 + s < i_hi && i0 + s + w0g + j <= e_hi) ? v : INT_MIN;
-            seg[j] = max(seg[j], v);
+            for (int j = 0; j < G; ++j)
+                seg[j] = __vimax3_s32(seg[j], val(win[(j + s) % G], p, s, j),
+                                      val(j + 1 < G ? win[(j + s + 1) % G] : next, p1, s + 1, j));
+            win[s % G] = next;
+            p = p1 + (uint32_t)x[s + 1];
+            win[(s + 1) % G] = next + (uint32_t)x[s + w0g + G];
         }
-        p += (uint32_t)x[s];
-        win[s % G] = win[(s + G - 1) % G] + (uint32_t)x[s + w0g + G - 1];
+    } else {  // (the tap kernel's epilogue, which would spill more)
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+#pragma unroll
+            for (int j = 0; j < G; ++j) seg[j] = max(seg[j], val(win[(j + s) % G], p, s, j));
+            p += (uint32_t)x[s];
+            win[s % G] = win[(s + G - 1) % G] + (uint32_t)x[s + w0g + G - 1];
+        }
     }
 }
 
@@ -100,10 +118,47 @@ __device__ __forceinline__ long long group_bound(const int* x, uint32_t q, uint3
 
 // Width groups from prune_w on skip the scan of segments whose group_bound is below
 // the smallest merged maximum of the group (strictly: a tie from an earlier start could
-// still win), which on noise-like series is most of them.  (Groups of 35-start segments
-// from 50 on.)
+// still win), which on noise-like series is most of them.  (Groups of 34-start segments
+// from 49 on.)
 template <int S>
 __host__ __device__ constexpr int prune_w() { return S + 15 > 48 ? S + 15 : 48; }
+
+// The search for the earliest start is latency in one warp of a CTA that waits for it at the tile's
+// end, and common in the first tiles of a part: the holders of all widths are found in one pass
+// and the holder's prefix values by warp scans from q (a lane walking from the segment's start,
+// holders found width by width: 9.55 ms where this takes 8.01, widths 1-256 as above).
+
+// In lanes 2 j and 2 j + 1: the earliest lane whose segment holds width j's maximum, which lane
+// 2 j has in mx.
+template <typename T>
+__device__ __forceinline__ int holders(T mx, const T (&seg)[G], bool scan, int jl) {
+    int hold = -1;
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+        const T mj = __shfl_sync(0xffffffffu, mx, 2 * j);
+        const int h = __ffs(__ballot_sync(0xffffffffu, scan && seg[j] == mj)) - 1;
+        if (j == jl) hold = h;
+    }
+    return hold;
+}
+
+// out[k] = base + the first k values of x, k < N (a warp).
+template <int N>
+__device__ __forceinline__ void write_prefix(const int* x, uint32_t base, uint32_t* out, int lane) {
+#pragma unroll
+    for (int b = 0; b < N; b += 32) {
+        const int k = b + lane;
+        const uint32_t v = k < N - 1 ? (uint32_t)x[k] : 0u;
+        uint32_t incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (k < N) out[k] = base + incl - v;
+        base += __shfl_sync(0xffffffffu, incl, 31);
+    }
+}
 
 // The scan of one row for one trial (warp-uniform arguments; see epilogue), S starts per lane.
 template <int S>
@@ -161,49 +216,38 @@ __device__ __forceinline__ void scan_row(const FusedArgs& f, const int* row, uin
                 const bool better = !(lane & 1) && jl < cnt && mx > INT_MIN &&
                                     (mx > bv || (mx == bv && t_lo < bt));
                 // widths whose maximum beats (or ties from an earlier start) the merged one:
-                // the earliest segment holding it writes its prefix values to the warp's
+                // the warp writes the prefix values of the earliest segment holding it to its
                 // scratch, and the lanes test the starts for every such width that this
                 // segment holds first
                 unsigned need = __ballot_sync(0xffffffffu, better);
-                auto holder = [&](int hl) {  // earliest lane whose segment holds width hl / 2's maximum
-                    const int j = hl >> 1;
-                    const int mj = __shfl_sync(0xffffffffu, mx, hl);
-                    int sj = INT_MIN;
+                if (need) {
+                    const int hold = holders(mx, seg, scan, jl);
+                    while (need) {  // warp-uniform
+                        const int h = __shfl_sync(0xffffffffu, hold, __ffs(need) - 1);
+                        const int ih = __shfl_sync(0xffffffffu, i0, h);
+                        write_prefix<R>(row + ih, 0u, chain, lane);
+                        write_prefix<R + G - 1>(row + ih + w0g, __shfl_sync(0xffffffffu, q, h), chain + R, lane);
+                        __syncwarp();
+                        const unsigned same = __ballot_sync(0xffffffffu, hold == h) & need;
+                        for (unsigned rest = same; rest; rest &= rest - 1) {
+                            const int hl = __ffs(rest) - 1;
+                            const int j = hl >> 1;
+                            const int mj = __shfl_sync(0xffffffffu, mx, hl);
+                            int at = -1;  // the earliest start of the segment that reaches it
 #pragma unroll
-                    for (int jj = 0; jj < G; ++jj) sj = jj == j ? seg[jj] : sj;
-                    return __ffs(__ballot_sync(0xffffffffu, scan && sj == mj)) - 1;
-                };
-                while (need) {  // warp-uniform
-                    const int h = holder(__ffs(need) - 1);
-                    if (lane == h) {
-                        uint32_t P = 0;
-                        for (int kk = 0; kk <= w0g + R + G - 2; ++kk) {
-                            if (kk < R) chain[kk] = P;
-                            if (kk >= w0g) chain[R + kk - w0g] = P;
-                            P += (uint32_t)x[kk];
+                            for (int s0 = 0; s0 < R; s0 += 32) {
+                                const int sl = s0 + lane, i = ih + sl;
+                                const bool eq = sl < R && i >= i_lo && i < i_hi && i + w0g + j <= e_hi &&
+                                                (int)(chain[R + sl + j] - chain[sl]) == mj;
+                                const unsigned st = __ballot_sync(0xffffffffu, eq);
+                                if (at < 0 && st) at = s0 + __ffs(st) - 1;
+                            }
+                            if (lane == 0 && at >= 0)
+                                atomicMax(keyrow + g * G + j, fused_key(mj, (int)(T0 - C) + ih + at));
                         }
+                        need &= ~same;
+                        __syncwarp();  // the scratch is rewritten for the next holder
                     }
-                    __syncwarp();
-                    const int ih = __shfl_sync(0xffffffffu, i0, h);
-                    for (unsigned rest = need; rest; rest &= rest - 1) {
-                        const int hl = __ffs(rest) - 1;
-                        if (holder(hl) != h) continue;  // held first by another segment: a later round
-                        const int j = hl >> 1;
-                        const int mj = __shfl_sync(0xffffffffu, mx, hl);
-                        int at = -1;  // the earliest start of the segment that reaches it
-#pragma unroll
-                        for (int s0 = 0; s0 < R; s0 += 32) {
-                            const int sl = s0 + lane, i = ih + sl;
-                            const bool eq = sl < R && i >= i_lo && i < i_hi && i + w0g + j <= e_hi &&
-                                            (int)(chain[R + sl + j] - chain[sl]) == mj;
-                            const unsigned st = __ballot_sync(0xffffffffu, eq);
-                            if (at < 0 && st) at = s0 + __ffs(st) - 1;
-                        }
-                        if (lane == 0 && at >= 0)
-                            atomicMax(keyrow + g * G + j, fused_key(mj, (int)(T0 - C) + ih + at));
-                        need &= ~(1u << hl);
-                    }
-                    __syncwarp();  // the scratch is rewritten for the next holder
                 }
             }
             if (any)
@@ -293,7 +337,7 @@ __device__ __forceinline__ void epilogue(const DedispArgs& a, const FusedArgs& f
 // The fused epilogue of one packed integer tile (dd_rows.cuh; every thread of the CTA
 // calls it): the unit's two trials d, d + 1, one row each, s[u] = the lane's low sums
 // (outputs lane * R + r of the warp's chunk), then its high ones (kPkHalf later).
-// Segments of 35 starts, so that 32 lanes cover the 1088-output tile in one pass.
+// Segments of 34 starts: 32 lanes cover the 1088-output tile.
 template <int R, int NW>
 __device__ __forceinline__ void epilogue_pk(const DedispArgs& a, const FusedArgs& f, unsigned char* smem,
                                             int wu, int chunk, int lane, int d, int64_t T0,
@@ -461,42 +505,48 @@ __device__ __forceinline__ void scan_row_f32(int w0, int nw, const float* row, f
             const float mx = warp_max16_f32(seg, lane);
             const bool better = !(lane & 1) && jl < cnt && mx > -FLT_MAX &&
                                 (mx > bv || (mx == bv && t_first < bt));
-            // widths whose maximum beats the merged one: the earliest segment holding it
-            // writes its chain to the warp's scratch, and the lanes test one start each for
+            // widths whose maximum beats the merged one: the chain of the earliest segment
+            // holding it goes to the warp's scratch, and the lanes test one start each for
             // every such width that this segment holds first
             unsigned need = __ballot_sync(0xffffffffu, better);
-            auto holder = [&](int hl) {  // earliest lane whose segment holds width hl / 2's maximum
-                const int j = hl >> 1;
-                const float mj = __shfl_sync(0xffffffffu, mx, hl);
-                float sj = -FLT_MAX;
+            if (need) {
+                const int hold = holders(mx, seg, any, jl);
+                while (need) {  // warp-uniform
+                    const int h = __shfl_sync(0xffffffffu, hold, __ffs(need) - 1);
+                    const int ih = __shfl_sync(0xffffffffu, i0, h);
+                    const int eh = __shfl_sync(0xffffffffu, e_rel, h);
+                    const int th = __shfl_sync(0xffffffffu, (int)(m * S), h);
+                    const float qh = __shfl_sync(0xffffffffu, q, h);
+                    // one lane writes P_0.., another P_{w0g}.. (the chain's own value, q), each in order
+                    if (lane < 2) {
+                        const int k0 = lane ? w0g : 0, n = lane ? S + G - 1 : S;
+                        const float* xh = row + ih + k0;
+                        float* out = chain + (lane ? S : 0);
+                        float P = lane ? qh : 0.f;
+                        for (int k = 0; k < n; k += 8) {
+                            float v[8];
 #pragma unroll
-                for (int jj = 0; jj < G; ++jj) sj = jj == j ? seg[jj] : sj;
-                return __ffs(__ballot_sync(0xffffffffu, any && sj == mj)) - 1;
-            };
-            while (need) {  // warp-uniform
-                const int h = holder(__ffs(need) - 1);
-                if (lane == h) {
-                    float P = 0.f;
-                    for (int k = 0; k <= w0g + 45; ++k) {
-                        if (k < S) chain[k] = P;
-                        if (k >= w0g) chain[S + k - w0g] = P;
-                        P += k < e_rel ? x[k] : 0.f;
+                            for (int i = 0; i < 8; ++i) v[i] = k + i < n - 1 && k0 + k + i < eh ? xh[k + i] : 0.f;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                if (k + i < n) out[k + i] = P;
+                                P += v[i];
+                            }
+                        }
                     }
+                    __syncwarp();
+                    const unsigned same = __ballot_sync(0xffffffffu, hold == h) & need;
+                    for (unsigned rest = same; rest; rest &= rest - 1) {
+                        const int hl = __ffs(rest) - 1;
+                        const int j = hl >> 1;
+                        const float mj = __shfl_sync(0xffffffffu, mx, hl);
+                        const bool eq = lane < S && lane + w0g + j <= eh && chain[S + lane + j] - chain[lane] == mj;
+                        const unsigned st = __ballot_sync(0xffffffffu, eq);
+                        if (lane == 0 && st) atomicMax(keyrow + g * G + j, fused_key_f32(mj, th + __ffs(st) - 1));
+                    }
+                    need &= ~same;
+                    __syncwarp();  // the scratch is rewritten for the next holder
                 }
-                __syncwarp();
-                const int eh = __shfl_sync(0xffffffffu, e_rel, h);
-                const int th = __shfl_sync(0xffffffffu, (int)(m * S), h);
-                for (unsigned rest = need; rest; rest &= rest - 1) {
-                    const int hl = __ffs(rest) - 1;
-                    if (holder(hl) != h) continue;  // held first by another segment: a later round
-                    const int j = hl >> 1;
-                    const float mj = __shfl_sync(0xffffffffu, mx, hl);
-                    const bool eq = lane < S && lane + w0g + j <= eh && chain[S + lane + j] - chain[lane] == mj;
-                    const unsigned st = __ballot_sync(0xffffffffu, eq);
-                    if (lane == 0 && st) atomicMax(keyrow + g * G + j, fused_key_f32(mj, th + __ffs(st) - 1));
-                    need &= ~(1u << hl);
-                }
-                __syncwarp();  // the scratch is rewritten for the next holder
             }
             if (any)
 #pragma unroll
