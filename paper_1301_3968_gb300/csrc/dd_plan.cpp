@@ -371,6 +371,13 @@ int row_kind_of(const dd_plan_s* p) {
 // Rows pay up to this many distinct runs per (trial, channel).
 constexpr double kRowsMaxShare = 0.5;
 
+// fp32 rows pay where a window often serves the next trial as well: the same run count, at most two
+// samples later.  Elsewhere a trial reads a word per channel and output, which costs what seven or
+// eight packed multiply-adds of the tap kernel do, and a block's spread of starts makes long rows:
+// 92 trials over DM 0-1945 (0.16 of the pairs near) x 336 channels x 4433 samples took 542 us, with
+// taps 178; 400 low-band trials over DM 0-60 (0.36) 2.66 ms, with taps 3.24.
+constexpr double kRowsMinNear = 0.3;
+
 // Warps per CTA of the row kernels.  16 (one CTA per SM) form a stage's rows for twice the
 // trials of 8 (two CTAs per SM), which measured 12 % faster on a long launch (CRAFT-like,
 // 512 trials: 1.08 against 1.22 ms), but leave more of a short launch's last wave idle: the
@@ -412,6 +419,12 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
         if (p->taps[a] != p->taps[b]) return false;
         return p->unit || std::memcmp(&p->w[a * p->kpad], &p->w[b * p->kpad], (size_t)p->taps[a] * sizeof(float)) == 0;
     };
+    if (fir && p->ndm > 1) {  // (over the list's own neighbours: no matter how blocks fall)
+        int64_t near = 0;
+        for (size_t i = (size_t)C; i < (size_t)p->ndm * C; ++i)
+            near += p->taps[i] == p->taps[i - C] && (uint32_t)(p->delay[i] - p->delay[i - C]) <= 2u;
+        if ((double)near < kRowsMinNear * (units - C)) return false;
+    }
     // the distinct runs of every (block, channel), and each trial's
     std::vector<std::vector<Row>> rows(nblk);
     std::vector<std::vector<int32_t>> first(nblk);  // [C + 1] into rows[b]

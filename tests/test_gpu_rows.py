@@ -306,3 +306,30 @@ def test_direct_plan_on_alternating_streams(dd, fused):
             assert torch.equal(g, w)
         if fused:
             assert torch.equal(p, peak)
+
+
+@pytest.mark.parametrize("steps", [[0, 5, 9], [3, 9], [0, 1, 2, 9]])
+@pytest.mark.parametrize("D", [2, 33])
+def test_coarse_lists_against_oracle(dd, steps, D):
+    """Lists whose neighbours share no, few or most windows, on either side of the rule for fp32
+    rows; a list and its halves give the same bits where all are on one side."""
+    import torch
+    rng = np.random.default_rng(71)
+    C, T = 12, 3000
+    delay, taps = _tables(rng, D, C, steps, [2, 3, 7], 48)
+    w = _weights(rng, taps, 48)
+    I = _input(rng, "f32", C, T)
+    x = torch.from_numpy(I).cuda()
+
+    def run(sel):
+        p = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, T, "f32"), np.zeros(len(delay[sel])))
+        p.set_profiles(delay=delay[sel], taps=taps[sel], weights=w[sel])
+        return p.dedisperse(x, nsamp=T)
+
+    got = run(slice(0, D))
+    want = oracle.c_dedisperse(I, delay, taps, w=w, nsamp=T)
+    scale = oracle.c_abs_scale(I, delay, taps, w=w, nsamp=T)
+    assert (np.abs(got.cpu().numpy() - want) <= 1e-5 * scale).all()
+    if steps == [3, 9]:  # no window is shared in any part
+        n = got.shape[1]
+        assert torch.equal(torch.cat([run(slice(0, D // 2))[:, :n], run(slice(D // 2, D))[:, :n]]), got)
