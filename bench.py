@@ -104,8 +104,39 @@ def craft_workload(dd, dev, ndm=None, rank=0, ws=1):
         nsamp_in=cfg["nsamp"],
         ndm=hi - lo, ndm_total=len(dms), shards=shards, dms=dms, wchan=cfg["wchan"], band=band,
         widths=cfg["widths"], delay=delay, taps=taps, w=w, dtype="f32",
-        flops=2.0 * float(taps.astype(np.int64).sum()) * t_out, ns_total=int(info["ns_total"]),
+        flops_direct=2.0 * float(taps.astype(np.int64).sum()) * t_out, ns_total=int(info["ns_total"]),
+        **row_work(delay, taps, t_out, plan.schedule()["trials_per_cta"]),
     )
+
+
+def row_work(delay, taps, t_out, block):
+    """What the fp32 row kernel executes on a list whose weights depend on the channel only: per
+    block of trials, channel and distinct tap count a row of n multiply-adds per position (864
+    outputs per tile and the trials' spread of starts), and one add per trial, channel and output.
+    Shared-memory words: a unit of three trials reads 27 per lane and trial, or only the shift
+    where a trial reads the row of the one before at most two samples later; a row position
+    reads n / 4 + 1 and writes one."""
+    tiles = -(-t_out // 864)
+    fma = build = 0
+    for b in range(0, len(taps), block):
+        n, d = taps[b:b + block], delay[b:b + block].astype(np.int64)
+        for v in np.unique(n):
+            m = n == v
+            has = m.any(axis=0)
+            span = np.where(m, d, -1).max(axis=0) - np.where(m, d, 1 << 40).min(axis=0)
+            pos = int((864 + span[has]).sum()) * tiles
+            fma += int(v) * pos
+            build += (int(v) // 4 + 2) * pos
+    words = 0
+    for j in range(len(taps)):
+        if j % block % 3 == 0:
+            words += 27 * taps.shape[1]
+        else:
+            sh = delay[j] - delay[j - 1]
+            near = (taps[j] == taps[j - 1]) & (sh >= 0) & (sh <= 2)
+            words += int(np.where(near, sh, 27).sum())
+    adds = float(taps.size) * t_out
+    return dict(flops=2.0 * fma + adds, smem_bytes=4.0 * (build + words * 32.0 * tiles))
 
 
 # ----------------------------------------------------------------------------- clocks
@@ -523,20 +554,20 @@ def _batch_case(dd, dev, flush, stream, cfg, reps, tune, widths, graph=True):
             batch.capture(gs)
             res["graph_step_ms"] = _ev_time(lambda: batch.replay(gs), reps, flush, gs)
     info = batch.info()
-    # work: trial x output samples; additions the direct path executes (one per tap,
+    # work: trial x output samples; additions of direct sums (one per tap,
     # trial and output) and the graded exact count (min(n, 2) per trial, channel and
     # output plus one per input sample for a prefix pass)
-    units = executed = graded = 0.0
+    units = direct = graded = 0.0
     for p, o in zip(plans, outs):
         _, taps = p.tables()
         t_out = o.shape[1]
         units += float(p.ndm) * t_out
-        executed += float(taps.astype(np.int64).sum()) * t_out
+        direct += float(taps.astype(np.int64).sum()) * t_out
         graded += float(np.minimum(taps, 2).astype(np.int64).sum()) * t_out + float(b.nchan) * p.band.nsamp
     batch.close()
     for p in plans:
         p.close()
-    res.update(units=units, executed_adds=executed, graded_adds=graded, items=info["items"],
+    res.update(units=units, direct_adds=direct, graded_adds=graded, items=info["items"],
                grid=info["grid"], nbeams=len(plans), samples=sum(x.shape[1] for x in xs),
                trials=sum(o.shape[0] for o in outs))
     return res
@@ -570,7 +601,7 @@ def batched_extra(dd, dev, flush, stream, reps=3, iadd_tops=None):
         "batched_fwd_value": units / (r["batched_fwd_ms"] / 1e3),
         "graph_step_value": units / (r["graph_step_ms"] / 1e3), "unit": UNIT,
         "batched_over_plain_fwd": r["plain_fwd_ms"] / r["batched_fwd_ms"],
-        "executed_adds_per_block": r["executed_adds"], "graded_adds_per_block": r["graded_adds"],
+        "direct_adds_per_block": r["direct_adds"], "graded_adds_per_block": r["graded_adds"],
         "small_beams": {
             "workload": (f"{small['nbeams']} beams, 336 ch, 2^14-2^15 samples and 512-1024 trials each "
                          f"({small['samples']} samples, {small['trials']} trials in all), autotuned"),
@@ -580,9 +611,8 @@ def batched_extra(dd, dev, flush, stream, reps=3, iadd_tops=None):
             "batched_fwd_value": small["units"] / (small["batched_fwd_ms"] / 1e3)},
     }
     if iadd_tops:
-        # the direct integer path: one add per tap (two per three-input add); graded: the
-        # exact minimum of a prefix-difference method
-        res["executed_frac_of_measured_iadd"] = r["executed_adds"] / (r["batched_fwd_ms"] / 1e3) / 1e12 / iadd_tops
+        # graded: the exact minimum of a prefix-difference method (the packed rows share it
+        # between trials, and one 32-bit addition serves two outputs)
         res["graded_frac_of_measured_iadd"] = r["graded_adds"] / (r["batched_fwd_ms"] / 1e3) / 1e12 / iadd_tops
     return res
 
@@ -652,25 +682,25 @@ def large_extra(dd, dev, flush, stream, chunk=1 << 18, nsamp=1 << 20, ndm=8192, 
         "fused_step_ms": fu_ms, "fused_value": units / (fu_ms / 1e3), "fused_over_step": fu_ms / st_ms,
         "fused_status": fu_status,
         "fused_series_bytes_not_stored": plan.ndm * chunk * 4,
-        # the run-length kernel's bound: shared-memory reads, one 4-byte word per (trial,
-        # channel, output) from the CTA's difference rows (two without them), against
-        # the SMs x 128 B/clk at the measured clock
-        "smem_read_bytes_per_block": 4.0 * dct,
-        "smem_read_tbps": 4.0 * dct / (dd_ms / 1e3) / 1e12,
+        # the packed rows' bound: shared-memory reads, at the least one 4-byte word per trial, pair
+        # of channels and pair of outputs (the rows' building and single channels come on top),
+        # against the SMs x 128 B/clk at the measured clock
+        "smem_read_bytes_per_block": dct,
+        "smem_read_tbps": dct / (dd_ms / 1e3) / 1e12,
         "smem_peak_tbps": sms * SMEM_BYTES_PER_CLK_PER_SM * sm_mhz * 1e6 / 1e12,
         "graded_adds_per_block": graded,
         "graded_tops": graded / (dd_ms / 1e3) / 1e12,
-        "bound": "shared-memory reads (1 word per trial, channel and output with the CTA's difference rows; see profiles)",
+        "bound": "shared-memory reads (a quarter of a word per trial, channel and output at the least; see profiles)",
     }
     res["smem_read_frac"] = res["smem_read_tbps"] / res["smem_peak_tbps"]
     res["smem_peak_kind"] = f"derived: {sms} SMs x {SMEM_BYTES_PER_CLK_PER_SM} B/clk x {sm_mhz:.0f} MHz"
-    if iadd_tops:
+    if iadd_tops:  # (one 32-bit addition serves two outputs and up to two channels: may pass 1)
         res["graded_frac_of_measured_iadd"] = res["graded_tops"] / iadd_tops
     plan.close()
     return res
 
 
-TRAFFIC_SOURCES = ["dd_tile.cuh", "dd_dedisp.cu", "dd_internal.h", "dd_packed.cuh", "dd_fused_scan.cuh",
+TRAFFIC_SOURCES = ["dd_rows.cuh", "dd_rows.cu", "dd_tile.cuh", "dd_internal.h", "dd_packed.cuh",
                    "dd_debug.cuh"]
 
 
@@ -690,7 +720,7 @@ def _profile_traffic():
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as f:
-            rec = json.load(f)["k_dedisp_f32_craft"]
+            rec = json.load(f)["k_rows_f32_craft"]
         sha = kernel_source_sha()
     except (OSError, KeyError, ValueError):
         return None
@@ -718,7 +748,9 @@ def _result(args, W, ws, rank, ms, value, k_ms, clocks, e2e, extras=None, live=N
     peak_name = max(cands, key=cands.get)
     peak_tflops = cands[peak_name]
     k_avg = sum(k_ms) / len(k_ms)
-    achieved = W["flops"] / (k_avg / 1e3) / 1e12
+    achieved = W["smem_bytes"] / (k_avg / 1e3) / 1e12
+    smem_peak = sms * SMEM_BYTES_PER_CLK_PER_SM * sm_max * 1e6 / 1e12
+    flop_rate = W["flops"] / (k_avg / 1e3) / 1e12
     res = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
@@ -731,21 +763,27 @@ def _result(args, W, ws, rank, ms, value, k_ms, clocks, e2e, extras=None, live=N
                                    "on the data path")},
         "e2e": e2e,
         "gpu_launches": LAUNCHES_PER_STEP * args.steps * ws,   # every rank launches its own
-        "roofline": {"bound": "alu", "kernel": "k_dedisp<float,float,weighted>",
-                     "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
-                     "frac": achieved / peak_tflops,
+        # the row kernel is bound by its shared-memory reads; flops_per_launch is what it executes,
+        # direct_* what one multiply-add per trial, channel, tap and output would take
+        "roofline": {"bound": "smem", "kernel": "k_rows<kRowsFir>",
+                     "achieved": achieved, "peak": smem_peak, "unit": "TB/s",
+                     "frac": achieved / smem_peak,
                      "traffic": args.traffic if args.traffic is not None else _profile_traffic(),
-                     "peak_kind": (f"{peak_name}: the largest of the derived rate ({sms} SMs x "
-                                   f"{FP32_LANES_PER_SM} FP32 lanes x 2 flop x {sm_max:.0f} MHz, {kind} "
-                                   "sm_max_mhz = %.1f) and the measured scalar and packed FMA rates" % derived),
-                     "peak_candidates": cands,
-                     "kernel_ms": k_avg, "flops_per_launch": W["flops"]},
+                     "peak_kind": (f"derived: {sms} SMs x {SMEM_BYTES_PER_CLK_PER_SM} B/clk x {sm_max:.0f} MHz "
+                                   f"({kind} sm_max_mhz)"),
+                     "kernel_ms": k_avg, "smem_bytes_per_launch": W["smem_bytes"],
+                     "flops_per_launch": W["flops"], "tflops": flop_rate,
+                     "fp32_peak_tflops": peak_tflops,
+                     "fp32_peak_kind": (f"{peak_name}: the largest of the derived rate ({sms} SMs x "
+                                        f"{FP32_LANES_PER_SM} FP32 lanes x 2 flop x {sm_max:.0f} MHz = "
+                                        "%.1f) and the measured scalar and packed FMA rates" % derived),
+                     "fp32_peak_candidates": cands,
+                     "direct_flops_per_launch": W["flops_direct"],
+                     "direct_equivalent_tflops": W["flops_direct"] / (k_avg / 1e3) / 1e12},
         "alu_peaks_measured": live,
         "clocks": clocks,
     }
     if live:
-        res["roofline"]["frac_of_measured_fma"] = achieved / live["fma_tflops"]
-        res["roofline"]["frac_of_measured_fma2"] = achieved / live["fma2_tflops"]
         res["config"]["sms"] = sms
     if shard is not None:
         res["shard"] = shard
