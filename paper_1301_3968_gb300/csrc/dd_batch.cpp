@@ -157,6 +157,16 @@ dd_status dd_batch_create(dd_batch_t* out, const dd_plan_t* plans, int32_t nbeam
     b->u8 = plans[0]->band.in_type == DD_U8;
     b->pair = plans[0]->pair;
     b->rl = plans[0]->rl;
+    // Beams of one wave each have stages for an SM of their own; where their CTAs together are
+    // more than the SMs, two should fit (6 beams of some 110 trials x 336 channels x 7400 outputs,
+    // block with statistics and boxcar: 945 us, with two 827).
+    auto small = [](const dd_plan_s* p) { return p->rk && p->row_warps == dd::kWarps; };
+    int64_t ctas = 0;
+    for (const dd_plan_s* p : b->plans)
+        if (small(p)) ctas += (plan_t_out(p) + dd::plan_tile_t(p) - 1) / dd::plan_tile_t(p) * p->nblk;
+    if (ctas > 152)
+        for (dd_plan_s* p : b->plans)
+            if (small(p)) dd::share_sm(p);
     build_items(b);
     *out = b;
     return DD_OK;

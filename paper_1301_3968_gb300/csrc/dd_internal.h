@@ -325,6 +325,8 @@ struct dd_plan_s {
     int32_t rk = 0;
     int32_t rows_max = 0;
     int32_t row_warps = 0, lo_ld = 0, nst = 0;
+    bool own_schedule = true;          // not one that a caller or the autotuner set
+    bool shares_sm = false;            // rows leave room for two CTAs even where the plan has one wave
     bool w_dev = false;                // weights come from the device (host copy is not theirs)
     bool w_follows = false;            // a device copy of the weights follows every upload
     // fused dedispersion + boxcar scratch: merged maxima, per-CTA carries, strip seams
@@ -354,6 +356,9 @@ dd_status launch_dedisperse_batched(bool u8, bool pair, bool short_taps, const D
                                     const BatchItem* d_items, int32_t nitems, size_t smem, cudaStream_t s,
                                     bool rl = false);
 int dedisp_batched_blocks_per_sm(bool u8, bool pair, bool short_taps, size_t smem, bool rl = false);
+// The plan's own schedule for a launch with other plans' CTAs (dd_plan.cpp).
+void share_sm(dd_plan_s* p);
+
 // A call's use of its plan's prefix scratch (p null: none), from the prefix pass to the last launch
 // that reads it: on a direct plan it waits for the last use on another stream.
 struct PrefixUse {

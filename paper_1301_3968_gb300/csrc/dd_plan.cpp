@@ -603,7 +603,7 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
         return k;
     };
     // (a fixed stage size that does not fit beside a second CTA may take the SM's shared memory)
-    size_t budget = nw == dd::kRowWarps || one_wave ? dd::kSmemBudgetOne : dd::kSmemBudget;
+    size_t budget = nw == dd::kRowWarps || (one_wave && !p->shares_sm) ? dd::kSmemBudgetOne : dd::kSmemBudget;
     auto smem_of = [&](int cs, const Need& m, int stages) {
         const dd::RowGeom g(kind, cs, nu, (int)m.r, (int)m.w);
         return dd::row_smem_bytes(g, 0, esz, (int)lcap, cs, C + stages + 2, (int)(zero + m.a) + 16);
@@ -778,6 +778,7 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
 // rows fit that shape and pay, the row kernels take the plan.
 dd_status build_schedule(dd_plan_s* p) {
     p->rk = dd::kRowsNone;
+    p->own_schedule = true;
     const bool u8 = p->band.in_type == DD_U8;
     p->pair = !(u8 && p->unit);
     const double mean_taps = (double)p->ns_total / ((double)p->ndm * p->nchan);
@@ -841,6 +842,7 @@ dd_status build_schedule(dd_plan_s* p) {
 // autotuner's, which may be a row schedule that the tap kernels have no shared memory for.
 dd_status build_schedule_fixed(dd_plan_s* p, int nch, int cs, bool tuned = false) {
     if (nch < 1 || nch > dd::kWarps || (dd::kWarps % nch) != 0 || cs < 1 || cs > 32) return DD_ERR_ARG;
+    p->own_schedule = false;
     if (tuned && build_rows(p, nch, cs)) return DD_OK;
     const int esz = stage_esz(p);
     const int nu = dd::kWarps / nch * units_per_warp(p);
@@ -1003,6 +1005,14 @@ static void free_dev(dd_plan_s* p) {
     if (cur >= 0 && cur != p->dev.device) cudaSetDevice(cur);
     p->dev = DevTables{};
     p->widths_on_dev.clear();
+}
+
+void share_sm(dd_plan_s* p) {
+    if (p->shares_sm || !p->own_schedule) return;
+    p->shares_sm = true;
+    if (build_schedule(p) == DD_OK) return;
+    p->shares_sm = false;
+    build_schedule(p);
 }
 
 void destroy_plan(dd_plan_s* p) {

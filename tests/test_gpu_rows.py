@@ -333,3 +333,28 @@ def test_coarse_lists_against_oracle(dd, steps, D):
     if steps == [3, 9]:  # no window is shared in any part
         n = got.shape[1]
         assert torch.equal(torch.cat([run(slice(0, D // 2))[:, :n], run(slice(D // 2, D))[:, :n]]), got)
+
+
+def test_batch_of_one_wave_beams(dd):
+    """Beams that alone leave SMs idle and together do not get smaller stages: the same sums, from
+    the batch and from the plans afterwards."""
+    import torch
+    rng = np.random.default_rng(81)
+    C, T, D = 40, 20000, 60
+    plans, xs, outs, want = [], [], [], []
+    for k in range(4):
+        delay, taps = _tables(rng, D, C, [0, 1, 3], [1, 2, 5], 20)
+        p = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, T, "u8"), np.zeros(D))
+        p.set_profiles(delay=delay, taps=taps)
+        plans.append(p)
+        xs.append(torch.from_numpy(_input(rng, "u8", C, T)).cuda())
+        outs.append(torch.zeros((D, T - p.d_max), dtype=torch.int32, device="cuda"))
+        want.append(p.dedisperse(xs[-1], nsamp=T))
+    batch = dd.Batch(plans)
+    batch.bind(xs, outs)
+    batch.dedisperse()
+    torch.cuda.synchronize()
+    for p, x, o, w in zip(plans, xs, outs, want):
+        assert torch.equal(o, w)
+        assert torch.equal(p.dedisperse(x, nsamp=T), w)
+        assert p.device_status() == 0
