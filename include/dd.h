@@ -237,6 +237,13 @@ dd_status dd_dedisperse_boxcar(dd_plan_t plan, const void* d_in, int64_t in_ld, 
  * Errors: DD_ERR_ARG. */
 dd_status dd_test_set_fused_parts(dd_plan_t plan, int32_t nparts);
 
+/* Test hook (host only): the shared memory that the fused launch of a row kernel takes for C
+ * carried outputs: kind 1 = fp32, 2 = packed integer rows; 8 or 16 warps per CTA; nch time chunks.
+ * *one_row = 1 where a warp's trials take turns in one row.  Errors: DD_ERR_ARG,
+ * DD_ERR_UNSUPPORTED (more than a CTA can have). */
+dd_status dd_test_fused_smem(int32_t kind, int32_t warps, int32_t nch, int32_t C, int64_t* bytes,
+                             int32_t* one_row);
+
 /* Adjoint of the weighted map of eq. p_dedisp (no counterpart in the paper): given
  * g = d(loss)/d(out) (d_gout [ndm][gout_ld] fp32, nsamp - d_max valid columns),
  *   d_gw [ndm][nchan][kmax] : gw_dck   = sum_t g[d][t] I[c][t_offset + t + delta + k]

@@ -317,17 +317,28 @@ constexpr int64_t kFusedGroup = 16;  // trial blocks per group of fp32 fused par
 
 }  // namespace
 
-size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C, bool one_row) {
-    if (p->rk) {
-        // a row per trial and the warps' scratch; one_row: a row per warp group and its other
-        // trials' waiting sums, the scratch then in the padding behind the rows
-        const int nt = row_unit_trials(p->rk), nrow = plan_trials(p) / (one_row ? nt : 1);
-        const int scratch = p->row_warps * fused::kChainFloats;
-        const int words = one_row ? nrow * rowlen + std::max(C + 48, scratch) + p->row_warps * (nt - 1) * row_warp_t(p->rk)
-                                  : fused_rows_ints(nrow, rowlen, C) + scratch;
-        const size_t rows = (size_t)words * 4 + 8 + 2 * 4;
-        return (std::max(dedisp_smem_for(p), rows) + 15) & ~(size_t)15;
+// Shared-memory row stride: C carried outputs, the tile and 32 spare (fp32: 48); the last tile's
+// extra starts read up to C + 14 past a row (fp32: 15 past the row's windows), into the next one or
+// the padding behind the last.
+int fused_rowlen(int L, int C, bool fp) { return L + C + (fp ? 48 : 32); }
+
+// Shared memory of a row kernel's fused launch for carries of C outputs, least: what the
+// dedispersion itself takes; *one_row: whether a warp group's trials take turns in one row.
+size_t rows_fused_smem(int kind, int nw, int nch, int C, size_t least, bool* one_row) {
+    const int rowlen = fused_rowlen(row_tile_t(kind, nch), C, kind == kRowsFir);
+    size_t smem = 0;
+    for (int one = 0; one < 2; ++one) {
+        *one_row = one != 0;
+        const size_t rows = (size_t)fused::RowScan(kind, nw, nch, rowlen, C, *one_row).words * 4 + 8 + 2 * 4;
+        smem = (std::max(least, rows) + 15) & ~(size_t)15;
+        if (smem <= kSmemMax) break;
     }
+    return smem;
+}
+
+size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C, bool* one_row) {
+    *one_row = false;
+    if (p->rk) return rows_fused_smem(p->rk, p->row_warps, p->nch, C, dedisp_smem_for(p), one_row);
     const int nbuf = p->rl ? kStagesRl : (p->pair ? kStagesPair : kStagesInt);
     // fp32 pair units: a row per trial; run-length path: a row per warp group and the
     // group's other trials' sums
@@ -423,13 +434,10 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
     const int tiles = (int)((t_out + L - 1) / L);
     const int tpc = plan_trials(p);
     const int64_t nblk = (p->ndm + tpc - 1) / tpc;
-    // row: C carried outputs, the tile and 32 spare (fp32: 48); the last tile's extra
-    // starts read up to C + 14 past a row (fp32: 15 past the row's windows), into the
-    // next one or the padding behind the last
-    const int rowlen = L + C + (fp ? 48 : 32);
-    size_t smem = fused_smem_for(p, rowlen, C);
-    const bool one_row = p->rk && smem > kSmemMax;
-    if (one_row) smem = fused_smem_for(p, rowlen, C, true);
+    const int rowlen = fused_rowlen(L, C, fp);
+    bool one_row = false;
+    const size_t smem = fused_smem_for(p, rowlen, C, &one_row);
+    if (p->rk && smem > kSmemMax) return DD_ERR_UNSUPPORTED;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -537,6 +545,18 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
         k_fused_final<<<nb, 256, 0, s>>>(f.key, p->ndm, nw, p->dev.mu, p->dev.isd, peak, arg, thresh, cands,
                                          cap, ncands);
     return cuda_status(cudaGetLastError());
+}
+
+extern "C" dd_status dd_test_fused_smem(int32_t kind, int32_t warps, int32_t nch, int32_t C, int64_t* bytes,
+                                        int32_t* one_row) {
+    using namespace dd;
+    if ((kind != kRowsFir && kind != kRowsPk) || (warps != kWarps && warps != kRowWarps) || nch < 1 || nch > kWarps ||
+        kWarps % nch || C < 0 || C > chunk_t(kind == kRowsFir) * nch || !bytes || !one_row)
+        return DD_ERR_ARG;
+    bool one = false;
+    *bytes = (int64_t)rows_fused_smem(kind, warps, nch, C, 0, &one);
+    *one_row = one;
+    return *bytes > (int64_t)kSmemMax ? DD_ERR_UNSUPPORTED : DD_OK;
 }
 
 extern "C" dd_status dd_test_set_fused_parts(dd_plan_t p, int32_t nparts) {

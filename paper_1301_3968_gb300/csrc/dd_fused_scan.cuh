@@ -45,6 +45,29 @@ constexpr int G = 16;  // widths per register window
 constexpr int kSegPk = 34;
 constexpr int kChainFloats = 2 * kSegPk + G - 1;
 
+// Where the fused epilogue of a row kernel's tile (epilogue_pk, epilogue_f32) keeps what, in
+// 4-byte words of the CTA's shared memory; the launch sizes it and the epilogues address it by
+// this one table.  A row per trial, C + 48 words that the last row's reads may run into, then the
+// warps' scratch.  one_row, where that is more than a CTA can have: a row per warp group, the
+// scratch, then its other trials' waiting sums; reads past the last row run into those (what they
+// return belongs to no window).  One row fits for every carry the call takes (1088- and 864-output
+// tiles, 8 and 16 warps); it costs a copy and two barriers per further trial of a tile
+// (packed, 1500 low-band trials x 1024 channels x 35300 outputs: widths 602-633 in two rows take 4.63 ms,
+// 604-635 in one 4.63, 700-731 4.72; the tap kernel's scan of the last 21.8).
+struct RowScan {
+    int chain, wait, words;
+    __host__ __device__ RowScan(int kind, int nw, int nch, int rowlen, int C, bool one_row) {
+        const int nt = row_unit_trials(kind), rows = (one_row ? nw / nch : row_trials(kind, nw, nch)) * rowlen;
+        chain = one_row ? rows : rows + C + 48;
+        wait = chain + nw * kChainFloats;
+        words = wait;
+        if (one_row) {
+            words += nw * (nt - 1) * row_warp_t(kind);
+            if (words < rows + C + 48) words = rows + C + 48;
+        }
+    }
+};
+
 // S starts of one lane segment (x = row + i0) for widths w0g + j, j < G.
 // q = sum_{k < w0g} x[k] on entry.  !FULL: starts outside [i_lo, i_hi) and windows
 // ending past row index e_hi are left out.
@@ -337,48 +360,68 @@ __device__ __forceinline__ void epilogue(const DedispArgs& a, const FusedArgs& f
 // The fused epilogue of one packed integer tile (dd_rows.cuh; every thread of the CTA
 // calls it): the unit's two trials d, d + 1, one row each, s[u] = the lane's low sums
 // (outputs lane * R + r of the warp's chunk), then its high ones (kPkHalf later).
+// ONE_ROW: one row per warp group, the second trial's sums wait in shared memory (a kernel of its
+// own: with a run-time switch, narrow lists took 2.5 % longer).
 // Segments of 34 starts: 32 lanes cover the 1088-output tile.
-template <int R, int NW>
+template <int R, int NW, bool ONE_ROW>
 __device__ __forceinline__ void epilogue_pk(const DedispArgs& a, const FusedArgs& f, unsigned char* smem,
                                             int wu, int chunk, int lane, int d, int64_t T0,
                                             const FusedTile& ft, const int (&s)[2][2 * R]) {
     constexpr int TT = 2 * kPkHalf;
     const int L = TT * a.nch;
     const int C = f.C;
-    int* rows = (int*)smem + 2 * wu * f.rowlen;
+    const RowScan lay(kRowsPk, NW, a.nch, f.rowlen, C, ONE_ROW);
+    int* rows = (int*)smem + (ONE_ROW ? 1 : 2) * wu * f.rowlen;
+    int* wait = (int*)smem + lay.wait + (int)(threadIdx.x >> 5) * TT + lane * R;  // (ONE_ROW)
     const int64_t S1 = ft.s1;
     const bool first = ft.first, last = ft.last;
     const int i_lo = first ? C : 0;
     const int e_hi = (int)(S1 - T0) + C;
     const int i_hi = last ? e_hi - f.w0 + 1 : L;
-    uint32_t* chain = (uint32_t*)smem + fused_rows_ints(2 * NW / a.nch, f.rowlen, C) +
-                      (threadIdx.x >> 5) * kChainFloats;
+    uint32_t* chain = (uint32_t*)smem + lay.chain + (threadIdx.x >> 5) * kChainFloats;
     const int ib = C + chunk * TT + lane * R;
     const int64_t tb = T0 + chunk * TT + lane * R;
+    // a trial's row behind its carry
+    auto carry_in = [&](int u, int* row) {
+        if (d + u < a.ndm && chunk == 0 && !first)
+            for (int k = lane; k < C; k += 32) row[k] = ft.carry[(int64_t)(wu * 2 + u) * C + k];
+    };
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        const bool live = d + u < a.ndm;
+        const bool live = d + u < a.ndm, waits = u == 1 && ONE_ROW;
         const int o = live ? (int)f.off[d + u] : 0;
         int* row = rows + u * f.rowlen;
+        int* at = waits ? wait : row + ib;
         int m = 0;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int v0 = s[u][r] - o, v1 = s[u][R + r] - o;
-            row[ib + r] = v0;
-            row[ib + kPkHalf + r] = v1;
+            at[r] = v0;
+            at[kPkHalf + r] = v1;
             if (tb + r < S1) m = max(m, abs(v0));
             if (tb + kPkHalf + r < S1) m = max(m, abs(v1));
         }
         if (live && m > f.mlim) atomicExch(a.status, (int)DD_ERR_OVERFLOW);
-        const int64_t cb = (int64_t)(wu * 2 + u) * C;
-        if (live && chunk == 0 && !first)
-            for (int k = lane; k < C; k += 32) row[k] = ft.carry[cb + k];
+        if (!waits) carry_in(u, row);
     }
     __syncthreads();  // the rows and their carries are complete
 #pragma unroll 1
     for (int u = 0; u < 2; ++u) {
-        if (d + u >= a.ndm) break;
-        const int* row = rows + u * f.rowlen;
+        int* row = rows + (ONE_ROW ? 0 : u * f.rowlen);
+        if (ONE_ROW && u) {
+            __syncthreads();  // the row is free
+#pragma unroll 1
+            for (int r = 0; r < R; ++r) {
+                row[ib + r] = wait[r];
+                row[ib + kPkHalf + r] = wait[kPkHalf + r];
+            }
+            carry_in(u, row);
+            __syncthreads();
+        }
+        if (d + u >= a.ndm) {
+            if (ONE_ROW) continue;  // (every warp meets the barriers above)
+            break;
+        }
         const int64_t cb = (int64_t)(wu * 2 + u) * C;
         if (chunk == 0) {
             if (!last)
@@ -617,13 +660,14 @@ __device__ __forceinline__ void epilogue_f32(const DedispArgs& a, const FusedArg
             carry_in(u, rows + u * f.rowlen);
         }
         __syncthreads();  // the rows and their carries are complete
+        // (the row kernels' layout, RowScan, is this one too)
         float* chain = (float*)smem + fused_rows_ints(NT * NW / a.nch, f.rowlen, C) + warp * kChainFloats;
         for (int u = 0; u < NT; ++u) scan(u, rows + u * f.rowlen, chain);
     } else {
+        const RowScan lay(kRowsFir, NW, a.nch, f.rowlen, C, true);
         float* row = (float*)smem + wu * f.rowlen;
-        float* pad = (float*)smem + NW / a.nch * f.rowlen;
-        float* chain = pad + warp * kChainFloats;
-        float* wait = pad + max(C + 48, NW * kChainFloats) + warp * (NT - 1) * TT + lane * R;
+        float* chain = (float*)smem + lay.chain + warp * kChainFloats;
+        float* wait = (float*)smem + lay.wait + warp * (NT - 1) * TT + lane * R;
 #pragma unroll
         for (int u = 0; u < NT; ++u) {
             const float o = off(u);

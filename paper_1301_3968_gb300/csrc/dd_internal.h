@@ -193,7 +193,7 @@ struct FusedArgs {
     const int64_t* order;     // [nparts] part taken by CTA i: parts sorted by their first
                               // time tile, so that CTAs resident together read the same
                               // input columns (shared in L2)
-    int32_t one_row;          // fp32 plans: a warp group has one shared-memory row, which its
+    int32_t one_row;          // row kernels: a warp group has one shared-memory row, which its
                               // trials use one after the other (their rows do not all fit)
     const double* off;        // [ndm] per-trial offsets (integer valued on integer plans)
     unsigned long long* key;  // [ndm][nw]
@@ -420,9 +420,13 @@ dd_status launch_prefix(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offs
 dd_status launch_norm(dd_plan_s* p, const int32_t* widths, int32_t nw, const double* mean,
                       const double* sd, cudaStream_t s);
 // fused dedispersion + boxcar: dynamic shared memory of the launch (stages, or the scan
-// rows plus the pipeline barriers, whichever is larger), its CTAs per SM, and the launch
-size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C, bool one_row = false);
-constexpr size_t kSmemMax = 227 * 1024;    // dynamic shared memory a CTA can have
+// rows plus the pipeline barriers, whichever is larger; *one_row: FusedArgs::one_row), its
+// CTAs per SM, and the launch
+size_t fused_smem_for(const dd_plan_s* p, int rowlen, int C, bool* one_row);
+// dynamic shared memory of a row kernel's fused launch at most: a CTA's 227 KB less the kernel's
+// static variables (checked beside it)
+constexpr size_t kSmemStatic = 512;
+constexpr size_t kSmemMax = 227 * 1024 - kSmemStatic;
 int fused_blocks_per_sm(const dd_plan_s* p, size_t smem);
 dd_status launch_dedisperse_fused(const dd_plan_s* p, DedispArgs a, const FusedArgs& f, size_t smem,
                                   cudaStream_t s);

@@ -320,8 +320,9 @@ __device__ __forceinline__ void issue_rows(const DedispArgs& a, const RowSmem& s
     if (lane == 31) bulk_g2s(sm.raw + rec_off, rec, (uint32_t)rg.rec_bytes, sm.full);
 }
 
-// One CTA tile: trial block `blk`, time tile `tx`.  MULTI, FUSED as dedisp_tile.
-template <int KIND, bool IN8, int NW, bool MULTI, bool FUSED>
+// One CTA tile: trial block `blk`, time tile `tx`.  MULTI, FUSED as dedisp_tile; ONE_ROW: the
+// fused scan of packed rows in its form for wide lists.
+template <int KIND, bool IN8, int NW, bool MULTI, bool FUSED, bool ONE_ROW = false>
 __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem, int blk, int tx, TileState& ts,
                                          const FusedArgs* fa = nullptr, const fused::FusedTile* ft = nullptr) {
     using TIN = typename RowIn<KIND, IN8>::T;
@@ -519,7 +520,7 @@ __device__ __forceinline__ bool row_tile(const DedispArgs a, unsigned char* smem
                 s[u][R + r] = (int)sum[u].hi[r];
             }
         if constexpr (FUSED) {
-            fused::epilogue_pk<R, NW>(a, *fa, smem, wu, chunk, lane, d, t0, *ft, s);
+            fused::epilogue_pk<R, NW, ONE_ROW>(a, *fa, smem, wu, chunk, lane, d, t0, *ft, s);
             return true;
         }
         int* st = (int*)smem + warp * TW;

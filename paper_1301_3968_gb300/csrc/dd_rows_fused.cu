@@ -5,13 +5,16 @@
 namespace dd {
 namespace {
 
-template <int KIND, bool IN8, int NW>
+// ONE_ROW: packed rows whose trials take turns in one row per warp group (FusedArgs::one_row; the
+// fp32 rows read that at run time).
+template <int KIND, bool IN8, int NW, bool ONE_ROW>
 __global__ void __launch_bounds__(NW * 32, 16 / NW) k_rows_fused(DedispArgs a, const FusedArgs f) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ TileState ts;
     if (threadIdx.x == 0) init_pipeline<1>(pipeline_area(smem, a.smem_bytes, 1), ts);
     __syncthreads();
     __shared__ fused::FusedTile ft;  // the tile's strip (as k_dedisp_fused)
+    static_assert(sizeof(TileState) + sizeof(fused::FusedTile) + 64 <= kSmemStatic, "static shared memory");
     const int s = (int)f.order[blockIdx.x];
     const int i0 = (int)f.starts[s], i1 = (int)f.starts[s + 1];
     for (int it = i0; it < i1; ++it) {
@@ -29,14 +32,20 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) k_rows_fused(DedispArgs a, c
             ft.seam_in = tx0 > 0 ? f.seam + (int64_t)s * tpc * 2 * f.C : nullptr;
             ft.seam_out = tx1 < f.tiles ? f.seam + (int64_t)(s + 1) * tpc * 2 * f.C : nullptr;
         }
-        if (!row_tile<KIND, IN8, NW, true, true>(a, smem, blk, tx, ts, &f, &ft)) break;
+        if (!row_tile<KIND, IN8, NW, true, true, ONE_ROW>(a, smem, blk, tx, ts, &f, &ft)) break;
     }
 }
 
 template <int KIND, bool IN8, int NW>
 dd_status run_fused(DedispArgs a, const FusedArgs& f, size_t smem, cudaStream_t s) {
     a.smem_bytes = (uint32_t)smem;
-    auto kern = k_rows_fused<KIND, IN8, NW>;
+    auto kern = k_rows_fused<KIND, IN8, NW, false>;
+    if constexpr (KIND == kRowsPk) {
+        if (f.one_row) {  // (the rows of eight warps always fit)
+            if constexpr (NW == kRowWarps) kern = k_rows_fused<KIND, IN8, NW, true>;
+            else return DD_ERR_UNSUPPORTED;
+        }
+    }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e);
     kern<<<(unsigned)f.nparts, NW * 32, smem, s>>>(a, f);
@@ -46,7 +55,7 @@ dd_status run_fused(DedispArgs a, const FusedArgs& f, size_t smem, cudaStream_t 
 template <int KIND, bool IN8, int NW>
 int fused_bps(size_t smem) {
     int n = 0;
-    auto kern = k_rows_fused<KIND, IN8, NW>;
+    auto kern = k_rows_fused<KIND, IN8, NW, false>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, NW * 32, smem) != cudaSuccess) return 0;
     return n;

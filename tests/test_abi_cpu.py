@@ -327,3 +327,29 @@ def test_dd_log_reports_plan_decisions(lib):
     env.pop("DD_LOG")
     off = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=120)
     assert off.returncode == 0 and "[dd]" not in off.stderr
+
+
+@pytest.mark.parametrize("kind,unit,tile,spare,chunk", [(1, 3, 864, 48, 864), (2, 2, 1088, 32, 992)])
+@pytest.mark.parametrize("warps", [8, 16])
+@pytest.mark.parametrize("nch", [1, 2, 4, 8])
+def test_fused_scan_of_row_plans_fits_its_launch(lib, kind, unit, tile, spare, chunk, warps, nch):
+    """The fused call takes carries of C <= chunk * nch outputs.  For each of them the launch of a
+    row kernel covers what its epilogue addresses -- a row per trial, or one per warp group and
+    the other trials' waiting sums; the search scratch; what the last row's reads may run into;
+    the copies' barrier -- within what a CTA can have beside a few static variables."""
+    nbytes, one = ctypes.c_int64(), ctypes.c_int32()
+    seen = set()
+    for C in range(0, chunk * nch + 1):
+        assert lib.dd_test_fused_smem(kind, warps, nch, C, ctypes.addressof(nbytes), ctypes.addressof(one)) == 0
+        row = tile * nch + C + spare
+        rows = warps // nch * (1 if one.value else unit) * row
+        scratch = warps * 83
+        if one.value:
+            need = max(rows + scratch + warps * (unit - 1) * tile, rows + C + 48)
+        else:
+            need = rows + C + 48 + scratch
+        assert 4 * need + 16 <= nbytes.value <= 227 * 1024 - 256, C
+        seen.add(one.value)
+    assert 0 in seen and (warps == 8 or seen == {0, 1})
+    assert lib.dd_test_fused_smem(kind, warps, nch, chunk * nch + 1, ctypes.addressof(nbytes),
+                                  ctypes.addressof(one)) == 1

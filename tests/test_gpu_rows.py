@@ -227,6 +227,42 @@ def test_fused_packed_rows(dd, method, seed, D, steps, w0, w1, parts, nch):
     assert torch.equal(p0.view(torch.int32), p1.view(torch.int32)) and torch.equal(a0, a1)
 
 
+@pytest.mark.parametrize("method", ["direct", "runlength"])
+@pytest.mark.parametrize("seed,nch,w0,w1,parts", [
+    (76, 1, 600, 634, 0),       # C = 633: a row per trial no longer leaves room for static variables
+    (77, 1, 630, 635, 0),       # the first widths that take turns in one row per warp
+    (78, 1, 660, 700, 6),
+    (79, 1, 930, 993, 0),       # the longest carry
+    (80, 2, 1240, 1260, 0),     # two time chunks, on either side of their line
+    (81, 2, 1255, 1262, 7),
+    (82, 2, 1970, 1985, 0),
+])
+def test_fused_packed_rows_of_wide_lists(dd, method, seed, nch, w0, w1, parts):
+    """Sixteen warps per CTA and carries whose rows do not all fit its shared memory: fused =
+    unfused, bit for bit."""
+    import torch
+    rng = np.random.default_rng(seed)
+    C, t_out, D = 6, 6500, 2373
+    delay, taps = _tables(rng, D, C, [0, 1], [2, 3, 7], 1184)
+    T = t_out + int((delay + taps - 1).max())
+    plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, T, "u8"), np.zeros(D))
+    plan.set_profiles(delay=delay, taps=taps)
+    plan.set_method(method)
+    if nch > 1:
+        plan.set_schedule(nch, 4)
+    assert plan.schedule()["trials_per_cta"] == 32 // nch
+    I = np.clip(rng.normal(128, 3, size=(C, (T + 15) // 16 * 16)), 0, 255).astype(np.uint8)
+    I[:, 2000:3500] = 128
+    x = torch.from_numpy(I).cuda()
+    mean, sd = plan.channel_stats(x, nsamp=T)
+    widths = np.arange(w0, w1 + 1, dtype=np.int32)
+    plan.test_set_fused_parts(parts)
+    p0, a0, _ = plan.boxcar_snr(plan.dedisperse(x, nsamp=T), widths, mean, sd)
+    p1, a1, _ = plan.dedisperse_boxcar(x, widths, mean, sd, nsamp=T)
+    assert plan.device_status() == 0
+    assert torch.equal(p0.view(torch.int32), p1.view(torch.int32)) and torch.equal(a0, a1)
+
+
 def test_batch_of_rows_and_taps(dd):
     """Beams of the row kernels (8 and 16 warps per CTA) and of the tap kernel in one batch, and
     the graph of it, equal the beams' own launches."""
