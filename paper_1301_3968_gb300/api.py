@@ -170,7 +170,6 @@ class Plan:
                                        self.ndm), "dd_plan_create")
         self._h = h
         self._kw = 0
-        self._wver = 0      # counts the profile and weight changes made through this object
 
     # ------------------------------------------------------------------ profiles
     def set_profiles(self, delay=None, taps=None, weights=None) -> None:
@@ -186,7 +185,6 @@ class Plan:
             if w.ndim != 3 or w.shape[:2] != (self.ndm, self.band.nchan):
                 raise ValueError(f"weights shape {w.shape}")
             k = w.shape[2]
-        self._wver += 1
         check(self._lib.dd_set_profiles(self._h, _np_ptr(d), _np_ptr(t), _np_ptr(w), k),
               "dd_set_profiles")
         self._kw = k
@@ -195,10 +193,15 @@ class Plan:
         """Device weights [D][C][K] fp32 (contiguous), copied in stream order."""
         if not (w.is_cuda and w.dtype == torch.float32 and w.is_contiguous() and w.dim() == 3):
             raise ValueError("weights must be a contiguous CUDA float32 [D][C][K] tensor")
-        self._wver += 1
         check(self._lib.dd_set_weights_device(self._h, _ptr(w), int(w.shape[2]), _stream(stream)),
               "dd_set_weights_device")
         self._kw = int(w.shape[2])
+
+    def weights_id(self) -> int:
+        """Identifies the weights on the device (0: not known); see dd_plan_weights_id."""
+        b = ctypes.c_uint64()
+        check(self._lib.dd_plan_weights_id(self._h, ctypes.addressof(b)), "dd_plan_weights_id")
+        return b.value
 
     def _facts(self):
         """(t_out, d_max, kmax, ns_total, out_is_int) of dd_plan_info."""
@@ -490,7 +493,7 @@ class DDFunction(torch.autograd.Function):
         out = plan.dedisperse(x.detach(), t_offset=t_offset, nsamp=nsamp)
         ctx.save_for_backward(x, w)
         ctx.plan = plan
-        ctx.wver = plan._wver
+        ctx.wid = plan.weights_id()
         ctx.t_offset = t_offset
         ctx.nsamp = nsamp
         return out
@@ -499,7 +502,7 @@ class DDFunction(torch.autograd.Function):
     def backward(ctx, gout):
         x, w = ctx.saved_tensors    # (raises if w was changed in place since)
         plan = ctx.plan
-        if plan._wver != ctx.wver:  # another forward has given the plan other weights
+        if ctx.wid == 0 or plan.weights_id() != ctx.wid:  # the plan may hold others by now
             plan.set_weights(w.detach().contiguous())
         gw, gin = plan.backward(x.detach(), gout.contiguous(), t_offset=ctx.t_offset,
                                 nsamp=ctx.nsamp, want_gw=ctx.needs_input_grad[1],

@@ -329,6 +329,8 @@ struct dd_plan_s {
     bool shares_sm = false;            // rows leave room for two CTAs even where the plan has one wave
     bool w_dev = false;                // weights come from the device (host copy is not theirs)
     bool w_follows = false;            // a device copy of the weights follows every upload
+    uint64_t w_id = 0;                 // the upload or copy that the device's weights come from
+    bool w_captured = false;           // a captured stream sets them too
     // fused dedispersion + boxcar scratch: merged maxima, per-CTA carries, strip seams
     unsigned long long* d_fkey = nullptr;
     int64_t fkey_elems = 0;

@@ -1028,7 +1028,8 @@ void destroy_plan(dd_plan_s* p) {
     delete p;
 }
 
-// Numbers every upload, so that a batch sees when a plan's tables have moved.
+// Numbers every upload and every copy of weights, so that a batch sees when a plan's tables have
+// moved and a caller when its weights are gone.
 static std::atomic<uint64_t> g_dev_gen{0};
 
 dd_status upload_tables(dd_plan_s* p) {
@@ -1097,7 +1098,8 @@ dd_status upload_tables(dd_plan_s* p) {
     // that its calls allocate nothing (lazy module loading would do it at its first call)
     if ((st = noalloc_preload()) != DD_OK) return st;
     p->dev_dirty = false;
-    p->dev_gen = ++g_dev_gen;
+    p->dev_gen = p->w_id = ++g_dev_gen;
+    p->w_captured = false;  // (earlier captures read tables that are gone)
     return DD_OK;
 }
 
@@ -1288,8 +1290,21 @@ dd_status dd_set_weights_device(dd_plan_t p, const float* d_w, int32_t kmax, voi
                                       (size_t)p->ndm * p->nchan, cudaMemcpyDeviceToDevice,
                                       (cudaStream_t)stream);
     if (e != cudaSuccess) return dd::cuda_status(e);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing((cudaStream_t)stream, &cap);
+    if (e != cudaSuccess) return dd::cuda_status(e);
+    if (cap != cudaStreamCaptureStatusNone) p->w_captured = true;
+    p->w_id = ++dd::g_dev_gen;
     p->adj_w_stale = true;
     return dd::launch_repack(p, (cudaStream_t)stream);
+}
+
+dd_status dd_plan_weights_id(dd_plan_t p, uint64_t* id) {
+    if (!p || !id) return DD_ERR_ARG;
+    int dev = -1;
+    const bool here = !p->dev_dirty && !p->w_captured && cudaGetDevice(&dev) == cudaSuccess && p->dev.device == dev;
+    *id = here ? p->w_id : 0;
+    return DD_OK;
 }
 
 dd_status dd_plan_info(dd_plan_t p, int64_t* t_out, int32_t* d_max, int32_t* kmax,
