@@ -123,12 +123,12 @@ dd_status dd_set_profiles(dd_plan_t plan, const int32_t* delay, const int32_t* n
  * trials share them); a plan whose host weights were shared is rebuilt at its first call.  Errors: DD_ERR_ARG, DD_ERR_OOM, DD_ERR_CUDA. */
 dd_status dd_set_weights_device(dd_plan_t plan, const float* d_w, int32_t kmax, void* stream);
 
-/* Identifies the weights on the device: *id changes with every upload of the plan's tables (which
+/* Identifies the weights on the device: the value changes with every upload of the plan's tables (which
  * a new schedule, method, profile or device brings, and which puts the host's weights there) and
  * with every dd_set_weights_device.  0 = not known: the tables are not on the current device as
  * the plan now stands, or a captured stream set weights, which its graph may set again at any
- * time.  Equal ids other than 0 mean the same weights.  Host only.  Errors: DD_ERR_ARG. */
-dd_status dd_plan_weights_id(dd_plan_t plan, uint64_t* id);
+ * time.  Equal values other than 0 mean the same weights.  Host only. */
+uint64_t dd_plan_weights_id(dd_plan_t plan);
 
 /* Plan facts: t_out = nsamp - d_max for the default nsamp, d_max = max(delta + n - 1),
  * kmax = max n_dc, ns_total = sum_{d,c} n_dc, out_is_int = 1 when sums are int32.

@@ -54,7 +54,7 @@ SIGNATURES = {
     "dd_plan_create": (c_i32, [ctypes.POINTER(c_vp), ctypes.POINTER(dd_band), c_vp, c_i32]),
     "dd_set_profiles": (c_i32, [c_vp, c_vp, c_vp, c_vp, c_i32]),
     "dd_set_weights_device": (c_i32, [c_vp, c_vp, c_i32, c_vp]),
-    "dd_plan_weights_id": (c_i32, [c_vp, c_vp]),
+    "dd_plan_weights_id": (ctypes.c_uint64, [c_vp]),
     "dd_plan_info": (c_i32, [c_vp, c_vp, c_vp, c_vp, c_vp, c_vp]),
     "dd_get_tables": (c_i32, [c_vp, c_vp, c_vp]),
     "dd_dedisperse": (c_i32, [c_vp, c_vp, c_i64, c_i64, c_i64, c_vp, c_i64, c_vp]),

@@ -199,9 +199,7 @@ class Plan:
 
     def weights_id(self) -> int:
         """Identifies the weights on the device (0: not known); see dd_plan_weights_id."""
-        b = ctypes.c_uint64()
-        check(self._lib.dd_plan_weights_id(self._h, ctypes.addressof(b)), "dd_plan_weights_id")
-        return b.value
+        return self._lib.dd_plan_weights_id(self._h)
 
     def _facts(self):
         """(t_out, d_max, kmax, ns_total, out_is_int) of dd_plan_info."""

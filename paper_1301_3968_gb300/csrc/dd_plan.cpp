@@ -1299,12 +1299,10 @@ dd_status dd_set_weights_device(dd_plan_t p, const float* d_w, int32_t kmax, voi
     return dd::launch_repack(p, (cudaStream_t)stream);
 }
 
-dd_status dd_plan_weights_id(dd_plan_t p, uint64_t* id) {
-    if (!p || !id) return DD_ERR_ARG;
+uint64_t dd_plan_weights_id(dd_plan_t p) {
     int dev = -1;
-    const bool here = !p->dev_dirty && !p->w_captured && cudaGetDevice(&dev) == cudaSuccess && p->dev.device == dev;
-    *id = here ? p->w_id : 0;
-    return DD_OK;
+    if (!p || p->dev_dirty || p->w_captured || cudaGetDevice(&dev) != cudaSuccess || p->dev.device != dev) return 0;
+    return p->w_id;
 }
 
 dd_status dd_plan_info(dd_plan_t p, int64_t* t_out, int32_t* d_max, int32_t* kmax,
