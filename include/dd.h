@@ -321,8 +321,9 @@ dd_status dd_plan_autotune(dd_plan_t plan, const void* d_in, int64_t in_ld, void
  * batch); a beam's block is the band's nsamp samples from column 0.  The work list has
  * one item per CTA tile (beam, trial block, time tile), and the launch one CTA per item in
  * list order: beams by decreasing estimated cost, each beam's tiles in the order of its
- * own launch (dd_dedisperse).  Plans whose own launch leaves SMs idle may get another of
- * their own schedules (never one set or tuned), with the same results.
+ * own launch (dd_dedisperse).  For plans whose own launch leaves SMs idle the batch may take
+ * another of their schedules (never where one was set or tuned), with the same results; its tables
+ * are the batch's, the plans and what was captured from them stay as they are.
  * Run-length beams first get their per-channel prefix sums (one small launch per beam,
  * into device memory the batch owns: 4 bytes per channel and sample, allocated by
  * dd_batch_bind), then the batched launch sums them. */

@@ -21,7 +21,11 @@
 #include "dd_trace.h"
 
 struct dd_batch_s {
-    std::vector<dd_plan_s*> plans;
+    std::vector<dd_plan_s*> plans;    // the caller's
+    // per beam the plan whose schedule the launch takes: the caller's, or the batch's own of it
+    // (twin, of the profiles and schedule twin_id)
+    std::vector<dd_plan_s*> sched, twin;
+    std::vector<uint64_t> twin_id;
     bool u8 = false, pair = true;
     bool rl = false;         // run-length beams (per-channel prefix sums, then differences)
     bool short_taps = true;  // every plan's tap runs fit one register window (run-length
@@ -91,7 +95,7 @@ void build_items(dd_batch_s* b) {
     std::vector<Beam> order;
     b->units = 0;
     for (int beam = 0; beam < (int)b->plans.size(); ++beam) {
-        const dd_plan_s* p = b->plans[beam];
+        const dd_plan_s* p = b->sched[beam];
         const int64_t t_out = plan_t_out(p);
         const int nst = (p->nchan + p->cs - 1) / p->cs;
         const int64_t tile = dd::plan_tile_t(p);
@@ -107,7 +111,7 @@ void build_items(dd_batch_s* b) {
     b->items.clear();
     b->groups.clear();
     for (const Beam& bm : order) {
-        const dd_plan_s* p = b->plans[bm.beam];
+        const dd_plan_s* p = b->sched[bm.beam];
         const int64_t t_out = plan_t_out(p);
         const int64_t tile = dd::plan_tile_t(p);
         if (b->groups.empty() || b->groups.back().warps != bm.warps)
@@ -127,6 +131,28 @@ void build_items(dd_batch_s* b) {
         dd_batch_s::Group& g = b->groups.back();
         g.count = b->items.size() - g.first;
         g.smem = std::max(g.smem, dd::dedisp_smem_for(p));
+    }
+}
+
+// The schedules of the launch.  Beams of one wave each have stages for an SM of their own; where
+// their CTAs together are more than the SMs, two should fit (6 beams of some 110 trials x 336
+// channels x 7400 outputs, block with statistics and boxcar: 945 us, with two 827).  Those are
+// twins, which the batch keeps: the plans stay as they are.
+void choose_schedules(dd_batch_s* b) {
+    auto small = [](const dd_plan_s* p) { return p->rk && p->row_warps == dd::kWarps && p->own_schedule; };
+    int64_t ctas = 0;
+    for (const dd_plan_s* p : b->plans)
+        if (p->rk && p->row_warps == dd::kWarps)
+            ctas += (plan_t_out(p) + dd::plan_tile_t(p) - 1) / dd::plan_tile_t(p) * p->nblk;
+    for (size_t i = 0; i < b->plans.size(); ++i) {
+        dd_plan_s* p = b->plans[i];
+        const bool want = ctas > 152 && small(p);
+        if (b->twin_id[i] != p->sched_id || !want) {
+            if (b->twin[i]) dd::destroy_plan(b->twin[i]);
+            b->twin[i] = want ? dd::twin_of(p) : nullptr;
+            b->twin_id[i] = want ? p->sched_id : 0;
+        }
+        b->sched[i] = b->twin[i] ? b->twin[i] : p;
     }
 }
 
@@ -157,16 +183,10 @@ dd_status dd_batch_create(dd_batch_t* out, const dd_plan_t* plans, int32_t nbeam
     b->u8 = plans[0]->band.in_type == DD_U8;
     b->pair = plans[0]->pair;
     b->rl = plans[0]->rl;
-    // Beams of one wave each have stages for an SM of their own; where their CTAs together are
-    // more than the SMs, two should fit (6 beams of some 110 trials x 336 channels x 7400 outputs,
-    // block with statistics and boxcar: 945 us, with two 827).
-    auto small = [](const dd_plan_s* p) { return p->rk && p->row_warps == dd::kWarps; };
-    int64_t ctas = 0;
-    for (const dd_plan_s* p : b->plans)
-        if (small(p)) ctas += (plan_t_out(p) + dd::plan_tile_t(p) - 1) / dd::plan_tile_t(p) * p->nblk;
-    if (ctas > 152)
-        for (dd_plan_s* p : b->plans)
-            if (small(p)) dd::share_sm(p);
+    b->sched = b->plans;
+    b->twin.assign(nbeams, nullptr);
+    b->twin_id.assign(nbeams, 0);
+    choose_schedules(b);
     build_items(b);
     *out = b;
     return DD_OK;
@@ -189,11 +209,18 @@ dd_status dd_batch_bind(dd_batch_t b, const void* const* d_in, const int64_t* in
         dd_status st = dd::upload_tables(p);
         if (st != DD_OK) return st;
     }
-    // plans may have been retuned since dd_batch_create: rebuild the work list
-    build_items(b);
+    // plans may have been retuned since dd_batch_create: schedules and work list again
+    b->bound = false;
     free_batch_dev(b);
+    choose_schedules(b);
+    for (int i = 0; i < nb; ++i)
+        if (b->twin[i]) {
+            const dd_status st = dd::upload_tables(b->twin[i]);
+            if (st != DD_OK) return st;
+        }
+    build_items(b);
     for (int i = 0; i < nb; ++i) {
-        dd_plan_s* p = b->plans[i];
+        dd_plan_s* p = b->sched[i];
         const int64_t t_out = plan_t_out(p);
         if (!dd::reads_prefix(p)) {
             dd::fill_dedisp_args(p, d_in[i], in_ld[i], 0, t_out, d_out[i], out_ld[i], &args[i]);
@@ -218,7 +245,7 @@ dd_status dd_batch_bind(dd_batch_t b, const void* const* d_in, const int64_t* in
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return dd::cuda_status(e);
     b->short_taps = true;
-    for (auto* p : b->plans)
+    for (auto* p : b->sched)
         if (!p->rk) b->short_taps = b->short_taps && (p->rl ? p->rl_b : p->pair ? p->umax <= dd::kRPair : p->kmax <= dd::kRInt);
     int per_sm = 32;
     for (const auto& g : b->groups)
@@ -286,8 +313,8 @@ dd_status dd_batch_dedisperse(dd_batch_t b, void* stream) {
     }
     for (size_t i = 0; i < b->plans.size(); ++i)  // the prefix sums of the beams that read them
         if (b->d_prefix[i]) {
-            const dd_status st = dd::launch_prefix_into(b->plans[i], b->in[i], b->in_ld[i], 0,
-                                                        b->plans[i]->band.nsamp, b->d_prefix[i], b->ldp[i],
+            const dd_status st = dd::launch_prefix_into(b->sched[i], b->in[i], b->in_ld[i], 0,
+                                                        b->sched[i]->band.nsamp, b->d_prefix[i], b->ldp[i],
                                                         (cudaStream_t)stream);
             if (st != DD_OK) return st;
         }
@@ -408,6 +435,8 @@ dd_status dd_batch_info(dd_batch_t b, int32_t* nitems, int32_t* grid, int64_t* u
 dd_status dd_batch_destroy(dd_batch_t b) {
     if (!b) return DD_ERR_ARG;
     free_batch_dev(b);
+    for (dd_plan_s* t : b->twin)
+        if (t) dd::destroy_plan(t);
     delete b;
     return DD_OK;
 }

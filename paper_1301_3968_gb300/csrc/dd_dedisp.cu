@@ -326,9 +326,10 @@ void fill_dedisp_args(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_
     a->rows_max = p->rows_max;
     a->lo_ld = p->lo_ld;
     a->nst = p->nst;
-    a->status = p->dev.status;
-    a->skip_stage = p->debug_skip_stage;
-    a->wait_ns = p->wait_ns;
+    const dd_plan_s* own = p->owner ? p->owner : p;
+    a->status = own->dev.status;
+    a->skip_stage = own->debug_skip_stage;
+    a->wait_ns = own->wait_ns;
     a->smem_bytes = (uint32_t)dedisp_smem_for(p);
     a->nsplit = 1;
     a->split_ld = 0;

@@ -327,6 +327,8 @@ struct dd_plan_s {
     int32_t row_warps = 0, lo_ld = 0, nst = 0;
     bool own_schedule = true;          // not one that a caller or the autotuner set
     bool shares_sm = false;            // rows leave room for two CTAs even where the plan has one wave
+    uint64_t sched_id = 0;             // the profiles and schedule as they were last built
+    dd_plan_s* owner = nullptr;        // a twin's plan (twin_of): its status word and test hooks count
     bool w_dev = false;                // weights come from the device (host copy is not theirs)
     bool w_follows = false;            // a device copy of the weights follows every upload
     uint64_t w_id = 0;                 // the upload or copy that the device's weights come from
@@ -358,8 +360,10 @@ dd_status launch_dedisperse_batched(bool u8, bool pair, bool short_taps, const D
                                     const BatchItem* d_items, int32_t nitems, size_t smem, cudaStream_t s,
                                     bool rl = false);
 int dedisp_batched_blocks_per_sm(bool u8, bool pair, bool short_taps, size_t smem, bool rl = false);
-// The plan's own schedule for a launch with other plans' CTAs (dd_plan.cpp).
-void share_sm(dd_plan_s* p);
+// A plan with p's profiles and another of its schedules, which leaves p, its tables and what was
+// captured from it as they are: the stages for a launch with other plans' CTAs (shares_sm).  For p's
+// lifetime, until p->sched_id changes; null where its sums would differ from p's.
+dd_plan_s* twin_of(dd_plan_s* p);
 
 // A call's use of its plan's prefix scratch (p null: none), from the prefix pass to the last launch
 // that reads it: on a direct plan it waits for the last use on another stream.

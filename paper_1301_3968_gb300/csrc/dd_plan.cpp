@@ -772,11 +772,16 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     return true;
 }
 
+// Numbers every built schedule, every upload and every copy of weights, so that a batch sees when a
+// plan has changed or its tables have moved and a caller when its weights are gone.
+std::atomic<uint64_t> g_gen{0};
+
 // Chooses the CTA shape of the dedispersion kernel (warp units x time chunks), the
 // staged window length and the channels per pipeline stage.  The most trials per CTA
 // (the most reuse of each staged sample) whose window still fits is taken.  Where shared
 // rows fit that shape and pay, the row kernels take the plan.
 dd_status build_schedule(dd_plan_s* p) {
+    p->sched_id = ++g_gen;
     p->rk = dd::kRowsNone;
     p->own_schedule = true;
     const bool u8 = p->band.in_type == DD_U8;
@@ -842,6 +847,7 @@ dd_status build_schedule(dd_plan_s* p) {
 // autotuner's, which may be a row schedule that the tap kernels have no shared memory for.
 dd_status build_schedule_fixed(dd_plan_s* p, int nch, int cs, bool tuned = false) {
     if (nch < 1 || nch > dd::kWarps || (dd::kWarps % nch) != 0 || cs < 1 || cs > 32) return DD_ERR_ARG;
+    p->sched_id = ++g_gen;
     p->own_schedule = false;
     if (tuned && build_rows(p, nch, cs)) return DD_OK;
     const int esz = stage_esz(p);
@@ -1007,12 +1013,32 @@ static void free_dev(dd_plan_s* p) {
     p->widths_on_dev.clear();
 }
 
-void share_sm(dd_plan_s* p) {
-    if (p->shares_sm || !p->own_schedule) return;
-    p->shares_sm = true;
-    if (build_schedule(p) == DD_OK) return;
-    p->shares_sm = false;
-    build_schedule(p);
+dd_plan_s* twin_of(dd_plan_s* p) {
+    dd_plan_s* t = new (std::nothrow) dd_plan_s;
+    if (!t) return nullptr;
+    t->band = p->band;
+    t->nchan = p->nchan;
+    t->ndm = p->ndm;
+    t->dms = p->dms;
+    t->delay = p->delay;
+    t->taps = p->taps;
+    t->w = p->w;
+    t->kpad = p->kpad;
+    t->kuser = p->kuser;
+    t->unit = p->unit;
+    t->kmax = p->kmax;
+    t->dmax = p->dmax;
+    t->ns_total = p->ns_total;
+    t->out_int = p->out_int;
+    t->max_abs_row = p->max_abs_row;
+    t->method = p->method;
+    t->w_dev = p->w_dev;
+    t->owner = p;
+    t->shares_sm = true;
+    // (integer sums are the same from the tap kernels, which such a schedule may be; fp32 ones are not)
+    if (build_schedule(t) == DD_OK && (!t->pair || t->rk == p->rk)) return t;
+    delete t;
+    return nullptr;
 }
 
 void destroy_plan(dd_plan_s* p) {
@@ -1027,10 +1053,6 @@ void destroy_plan(dd_plan_s* p) {
     free_dev(p);
     delete p;
 }
-
-// Numbers every upload and every copy of weights, so that a batch sees when a plan's tables have
-// moved and a caller when its weights are gone.
-static std::atomic<uint64_t> g_dev_gen{0};
 
 dd_status upload_tables(dd_plan_s* p) {
     int dev = -1;
@@ -1098,7 +1120,7 @@ dd_status upload_tables(dd_plan_s* p) {
     // that its calls allocate nothing (lazy module loading would do it at its first call)
     if ((st = noalloc_preload()) != DD_OK) return st;
     p->dev_dirty = false;
-    p->dev_gen = p->w_id = ++g_dev_gen;
+    p->dev_gen = p->w_id = ++g_gen;
     p->w_captured = false;  // (earlier captures read tables that are gone)
     return DD_OK;
 }
@@ -1294,7 +1316,7 @@ dd_status dd_set_weights_device(dd_plan_t p, const float* d_w, int32_t kmax, voi
     e = cudaStreamIsCapturing((cudaStream_t)stream, &cap);
     if (e != cudaSuccess) return dd::cuda_status(e);
     if (cap != cudaStreamCaptureStatusNone) p->w_captured = true;
-    p->w_id = ++dd::g_dev_gen;
+    p->w_id = ++g_gen;
     p->adj_w_stale = true;
     return dd::launch_repack(p, (cudaStream_t)stream);
 }

@@ -353,3 +353,15 @@ def test_fused_scan_of_row_plans_fits_its_launch(lib, kind, unit, tile, spare, c
     assert 0 in seen and (warps == 8 or seen == {0, 1})
     assert lib.dd_test_fused_smem(kind, warps, nch, chunk * nch + 1, ctypes.addressof(nbytes),
                                   ctypes.addressof(one)) == 1
+
+
+def test_batch_leaves_its_plans_as_they_are(lib):
+    """Beams of one wave each take other stages in a batch's launch; the plans keep theirs (and so
+    their tables, which captured graphs read)."""
+    import paper_1301_3968_gb300 as dd
+    plans = [dd.Plan(dd.Band(336, 1130.0, 1.0, 1.0, 11000, "u8"), np.linspace(0, 600, 110)) for _ in range(6)]
+    before = [p.schedule() for p in plans]
+    batch = dd.Batch(plans)
+    assert [p.schedule() for p in plans] == before
+    batch.close()
+    assert [p.schedule() for p in plans] == before

@@ -63,3 +63,41 @@ def test_backward_uses_the_weights_of_its_forward(dd, between):
     assert plan.device_status() == 0
     for a, b in zip(want, (y.detach(), xi.grad, wi.grad)):
         assert torch.equal(a, b)
+
+
+def test_graph_of_a_plan_outlives_batches_of_it(dd):
+    """A graph captured from a plan replays after a batch of the plan was made, run and closed, and
+    after the plan's own calls since; the batch follows new profiles of a plan."""
+    import torch
+    rng = np.random.default_rng(5)
+    C, T, D = 336, 9000, 110
+    plans = [dd.Plan(dd.Band(C, 1130.0, 1.0, 1.0, T, "u8"), np.linspace(0, 600, D)) for _ in range(5)]
+    xs = [torch.from_numpy(rng.integers(0, 256, size=(C, T // 16 * 16 + 16)).astype(np.uint8)).cuda() for _ in plans]
+    want = [p.dedisperse(x, nsamp=T) for p, x in zip(plans, xs)]
+    out = torch.empty_like(want[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plans[0].dedisperse(xs[0], nsamp=T, out=out)
+    ids = [p.weights_id() for p in plans]
+    batch = dd.Batch(plans)
+    outs = [torch.zeros_like(w) for w in want]
+    batch.bind(xs, outs)
+    batch.dedisperse()
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, w) for o, w in zip(outs, want))
+    assert torch.equal(plans[0].dedisperse(xs[0], nsamp=T), want[0])
+    assert [p.weights_id() for p in plans] == ids and 0 not in ids   # no table was uploaded anew
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want[0])
+    delay, taps = plans[1].tables()
+    plans[1].set_profiles(delay=delay[::-1], taps=taps[::-1])
+    batch.dedisperse()
+    torch.cuda.synchronize()
+    assert torch.equal(outs[1], want[1].flip(0)) and torch.equal(outs[0], want[0])
+    assert all(p.device_status() == 0 for p in plans)
+    batch.close()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want[0])
