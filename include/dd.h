@@ -31,13 +31,15 @@
  *     size, row lengths, shared memory), autotuner results, batch bindings; 2 = also every
  *     device call with its sizes.
  *   - No call here allocates device memory except dd_plan_create / dd_set_profiles /
- *     the first device call on a plan (tables; on an integer plan whose direct sums read
- *     prefix sums, 4 bytes per channel and sample of the band's block, at most 2 GiB unless
- *     the longest delay needs more; on a device's first plan also the 8 MiB array of
+ *     the first device call on a plan (tables; on a device's first plan also the 8 MiB array of
  *     dd_boxcar_snr_noalloc), dd_boxcar_snr when the width count
- *     grows (normaliser workspace), dd_dedisperse on a run-length plan when nsamp
- *     grows (prefix scratch), dd_dedisperse_boxcar when its scratch grows, and the
- *     first dd_backward (adjoint workspace).
+ *     grows (normaliser workspace), dd_dedisperse when nsamp grows, on a run-length plan or an
+ *     integer plan whose direct sums read prefix sums (prefix scratch, 4 bytes per channel and
+ *     sample; the latter's at most 2 GiB unless the longest delay needs more, and less, with
+ *     the call in pieces, where that is not to be had; its smaller ones of earlier calls are kept
+ *     until the tables change, for captured calls that read them), dd_dedisperse_boxcar when its scratch
+ *     grows (on those plans prefix sums of all its samples, too), dd_batch_bind, and the first
+ *     dd_backward (adjoint workspace).
  */
 #ifndef DD_H
 #define DD_H
@@ -226,8 +228,9 @@ dd_status dd_boxcar_snr_noalloc(dd_plan_t plan, const void* d_series, int64_t ld
  * nsamp <= 2^24 on the run-length path.
  * Other arguments, outputs and errors as dd_dedisperse and dd_boxcar_snr.  Allocates
  * plan-owned device scratch when the sizes grow: the merged maxima (8 bytes per trial
- * and width) and, per part, its carried outputs and seams (12 C bytes per trial of a
- * CTA's block).  A call with a new width list or a new launch geometry copies small
+ * and width), per part its carried outputs and seams (12 C bytes per trial of a
+ * CTA's block) and, on plans that read prefix sums, those of all samples (4 bytes per channel
+ * and sample).  A call with a new width list or a new launch geometry copies small
  * host tables to the device synchronously, so make one such call before capturing the
  * stream in a CUDA graph.  Calls on one plan share its scratch: order them on one
  * stream. */
@@ -279,7 +282,7 @@ dd_status dd_plan_get_schedule(dd_plan_t plan, int32_t* nch, int32_t* cs, int32_
 /* How a plan forms the tap sums of eq. p_dedisp.
  *   DD_METHOD_DIRECT:    every tap is one multiply-add (any weights), or, for integer plans
  *     whose trials share their tap runs (see dd_plan_set_schedule), the shared runs' sums from
- *     prefix sums in a scratch of fixed size, longer calls in pieces (the same exact sums).
+ *     prefix sums in a scratch of at most 2 GiB, longer calls in pieces (the same exact sums).
  *   DD_METHOD_RUNLENGTH: uint8 unit-weight plans only.  A run of n unit taps is a
  *     difference of per-channel prefix sums, sum_{k<n} I[c][s+k] = P_c[s+n] - P_c[s]
  *     with P_c[i] = sum_{j<i} I[c][t_offset+j], so each (trial, channel) costs two
@@ -440,6 +443,10 @@ dd_status dd_detector_profile(const double* pbar, int32_t nchan, int32_t nt, con
  * one warm-up launch, one timed launch (about 0.1 s); synchronises the stream.
  * Errors: DD_ERR_ARG, DD_ERR_OOM, DD_ERR_CUDA. */
 dd_status dd_alu_peak(int32_t kind, double* ops_per_s, void* stream);
+
+/* Test hook: prefix scratch of more than `bytes` is not to be had (0: no limit), as if the device's
+ * memory were full.  Errors: DD_ERR_ARG. */
+dd_status dd_test_set_scratch_limit(dd_plan_t plan, int64_t bytes);
 
 /* Releases the plan's host and device memory (after its work has finished). */
 dd_status dd_plan_destroy(dd_plan_t plan);

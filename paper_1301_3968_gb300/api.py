@@ -396,6 +396,10 @@ class Plan:
         """Test hook: never issue the copies of one channel stage; bound waits by wait_ns."""
         check(self._lib.dd_test_set_wait(self._h, int(skip_stage), int(wait_ns)), "dd_test_set_wait")
 
+    def test_set_scratch_limit(self, nbytes: int = 0) -> None:
+        """Test hook: prefix scratch of more than nbytes is not to be had (0: no limit)."""
+        check(self._lib.dd_test_set_scratch_limit(self._h, int(nbytes)), "dd_test_set_scratch_limit")
+
     def close(self) -> None:
         if getattr(self, "_h", None):
             self._lib.dd_plan_destroy(self._h)

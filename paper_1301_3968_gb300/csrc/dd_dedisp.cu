@@ -413,28 +413,46 @@ PrefixUse::~PrefixUse() {
     if (id == 1 || mark(s) == cudaSuccess) p->prefix_stream = id;
 }
 
+// Room for `need` words of prefix sums (or DD_ERR_OOM, which leaves a direct plan what it has).  A
+// run-length plan gives its old scratch back first.  A direct plan may get its scratch in a captured
+// call, and keeps an old one for earlier captures until its tables change; the new one is twice as
+// large (within `most`, where there is room), so that few are kept.
+dd_status prefix_room(dd_plan_s* p, int64_t need, int64_t most = INT64_MAX) {
+    if (need <= p->prefix_elems) return DD_OK;
+    if (p->rl && p->d_prefix) {
+        cudaFree(p->d_prefix);
+        p->d_prefix = nullptr;
+        p->prefix_elems = 0;
+    }
+    uint32_t* q = nullptr;
+    const int64_t more = std::max(need, std::min(most, 2 * p->prefix_elems));
+    cudaError_t e = cudaErrorMemoryAllocation;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (!p->rl) cudaThreadExchangeStreamCaptureMode(&mode);
+    for (const int64_t n : {more, need}) {
+        if (p->scratch_limit > 0 && n * (int64_t)sizeof(uint32_t) > p->scratch_limit) continue;
+        e = cudaMalloc((void**)&q, (size_t)n * sizeof(uint32_t));
+        if (e == cudaSuccess) {
+            if (p->d_prefix) p->prefix_old.push_back(p->d_prefix);
+            p->d_prefix = q;
+            p->prefix_elems = n;
+            break;
+        }
+        cudaGetLastError();
+        if (e != cudaErrorMemoryAllocation || n == need) break;
+    }
+    if (!p->rl) cudaThreadExchangeStreamCaptureMode(&mode);
+    return cuda_status(e);
+}
+
 // Run-length path: prefix sums of columns t_offset .. t_offset + nsamp - 1 into the
 // plan's scratch, then the run-length sums over them.
 dd_status launch_prefix(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset, int64_t nsamp,
                         int64_t* ldp_out, cudaStream_t s) {
     const int64_t ldp = (nsamp + 1 + 3) & ~(int64_t)3;
     *ldp_out = ldp;
-    const int64_t need = ldp * p->nchan;
-    if (need > p->prefix_elems) {
-        if (p->rl && p->prefix_own) {
-            cudaFree(p->d_prefix);
-            p->d_prefix = nullptr;
-            p->prefix_elems = 0;
-            p->prefix_own = false;
-        }
-        uint32_t* q = nullptr;  // (a direct plan keeps its scratch if there is no more)
-        cudaError_t e = cudaMalloc((void**)&q, (size_t)need * sizeof(uint32_t));
-        if (e != cudaSuccess) return cuda_status(e);
-        if (p->prefix_own) cudaFree(p->d_prefix);
-        p->d_prefix = q;
-        p->prefix_elems = need;
-        p->prefix_own = true;
-    }
+    const dd_status st = prefix_room(p, ldp * p->nchan);
+    if (st != DD_OK) return st;
     return launch_prefix_into(p, in, ld, t_offset, nsamp, p->d_prefix, ldp, s);
 }
 
@@ -451,18 +469,26 @@ dd_status launch_dedisperse_rl(dd_plan_s* p, const void* in, int64_t ld, int64_t
 
 dd_status launch_dedisperse_pk(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                                int64_t nsamp, void* out, int64_t out_ld, cudaStream_t s) {
-    // outputs per piece: whole tiles, as many as the scratch holds with the delays behind them
-    const int64_t tile = row_tile_t(kRowsPk, p->nch), t_out = nsamp - p->dmax;
-    const int64_t cols = p->prefix_elems / p->nchan;
-    int64_t piece = std::min(cols - 4 - p->dmax, 65535 * tile);  // (grid y)
-    if (piece < t_out) piece = piece / tile * tile;
-    if (piece < 1) return DD_ERR_OOM;
     PrefixUse use(p, s);
     if (use.err != cudaSuccess) return cuda_status(use.err);
+    // Columns of scratch: the call's, within 2 GiB or what the longest delay and two tiles need;
+    // what there is, or that least, where no more is to be had.
+    const int64_t tile = row_tile_t(kRowsPk, p->nch), t_out = nsamp - p->dmax;
+    auto round4 = [](int64_t n) { return (n + 3) & ~(int64_t)3; };
+    const int64_t least = round4((int64_t)p->dmax + 2 * tile + 1);
+    const int64_t most = std::max(least, ((int64_t)1 << 29) / p->nchan & ~(int64_t)3);
+    const int64_t want = std::min(round4(nsamp + 1), most);
+    dd_status st = prefix_room(p, want * p->nchan, most * p->nchan);
+    if (st == DD_ERR_OOM) st = prefix_room(p, std::min(want, least) * p->nchan);
+    if (st != DD_OK) return st;
+    // outputs per piece: whole tiles, as many as the scratch holds with the delays behind them
+    const int64_t cols = p->prefix_elems / p->nchan & ~(int64_t)3;
+    int64_t piece = std::min(cols - 1 - p->dmax, 65535 * tile);  // (grid y)
+    if (piece < t_out) piece = piece / tile * tile;
+    if (piece < 1) return DD_ERR_OOM;
     for (int64_t t0 = 0; t0 < t_out; t0 += piece) {
         const int64_t n = std::min(piece, t_out - t0) + p->dmax, ldp = (n + 1 + 3) & ~(int64_t)3;
-        dd_status st = launch_prefix_into(p, in, ld, t_offset + t0, n, p->d_prefix, ldp, s);
-        if (st != DD_OK) return st;
+        if ((st = launch_prefix_into(p, in, ld, t_offset + t0, n, p->d_prefix, ldp, s)) != DD_OK) return st;
         DedispArgs a;
         fill_dedisp_args(p, p->d_prefix, ldp, 0, n - p->dmax, (int32_t*)out + t0, out_ld, &a);
         if ((st = launch_rows(p, a, s)) != DD_OK) return st;

@@ -315,7 +315,8 @@ struct dd_plan_s {
     int32_t blen = 0;                  // their stride (words)
     uint32_t* d_prefix = nullptr;
     int64_t prefix_elems = 0;
-    bool prefix_own = false;           // d_prefix is an allocation of its own (else in the slab)
+    std::vector<uint32_t*> prefix_old; // direct plans: smaller ones before it, which captured calls may read
+    int64_t scratch_limit = 0;         // test hook: larger prefix scratch is not to be had (0: no limit)
     // direct plans: a call on another stream waits for the last one's reads of the prefix sums
     // (calls on several streams needed no workspace when the taps were summed one by one)
     std::mutex prefix_mu;
@@ -384,7 +385,8 @@ private:
 
 dd_status launch_prefix_into(const dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                              int64_t nsamp, uint32_t* P, int64_t ldp, cudaStream_t s);
-// direct plans on packed rows: prefix sums into the plan's scratch and the launch, in pieces that fit
+// direct plans on packed rows: prefix sums into the plan's scratch and the launch, in pieces that
+// fit (DD_ERR_OOM, with nothing launched: no scratch to be had)
 dd_status launch_dedisperse_pk(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                                int64_t nsamp, void* out, int64_t out_ld, cudaStream_t s);
 // the plan's sums read prefix sums instead of samples

@@ -991,12 +991,16 @@ dd_status cuda_status(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? DD_ERR_OOM : DD_ERR_CUDA;
 }
 
-static void free_dev(dd_plan_s* p) {
+// Frees the device tables, for new ones on device `to` (-1: none).
+static void free_dev(dd_plan_s* p, int to) {
     if (p->dev.device < 0) return;
     int cur = -1;
     cudaGetDevice(&cur);
     if (cur != p->dev.device) cudaSetDevice(p->dev.device);
-    if (!p->prefix_own) {  // in the slab
+    for (uint32_t* q : p->prefix_old) cudaFree(q);  // (what was captured reads tables that go now)
+    p->prefix_old.clear();
+    if (to != p->dev.device) {
+        cudaFree(p->d_prefix);
         p->d_prefix = nullptr;
         p->prefix_elems = 0;
     }
@@ -1045,12 +1049,11 @@ void destroy_plan(dd_plan_s* p) {
     if (p->adj) destroy_plan(p->adj);
     if (p->d_gpad) cudaFree(p->d_gpad);
     if (p->d_gsplit) cudaFree(p->d_gsplit);
-    if (p->prefix_own) cudaFree(p->d_prefix);
     if (p->d_fkey) cudaFree(p->d_fkey);
     if (p->d_fcarry) cudaFree(p->d_fcarry);
     if (p->d_fseam) cudaFree(p->d_fseam);
     if (p->d_fstarts) cudaFree(p->d_fstarts);
-    free_dev(p);
+    free_dev(p, -1);
     delete p;
 }
 
@@ -1060,7 +1063,7 @@ dd_status upload_tables(dd_plan_s* p) {
     if (e != cudaSuccess) return cuda_status(e);
     if (!p->dev_dirty && p->dev.device == dev) return DD_OK;
     if (p->rec_host != p->rec_bytes && !p->w_follows) build_records(p);  // with the host's weights
-    free_dev(p);
+    free_dev(p, dev);
     p->dev.device = dev;
     // one allocation for all tables
     const size_t n = (size_t)p->ndm * p->nchan;
@@ -1075,16 +1078,6 @@ dd_status upload_tables(dd_plan_s* p) {
     const size_t at_delay = room(n * 4), at_taps = room(n * 4), at_lo = room(p->blk_lo.size() * 4),
                  at_rec = room(nrec * p->rec_bytes), at_w = room(wlen * sizeof(float)), at_status = room(4),
                  at_off = room((size_t)p->ndm * sizeof(double));
-    // direct plans' prefix sums: room for the band's block (or 64 Ki outputs), within 2 GiB or what
-    // the longest delay needs; longer calls go in pieces (launch_dedisperse_pk)
-    int64_t pre = 0;
-    if (p->rk == kRowsPk && !p->rl) {
-        const int64_t want = std::max<int64_t>(p->band.nsamp, (int64_t)p->dmax + 65536);
-        const int64_t least = (int64_t)p->dmax + 2 * row_tile_t(kRowsPk, p->nch);
-        pre = ((std::max(least, std::min(want, ((int64_t)1 << 29) / p->nchan)) + 1 + 3) & ~(int64_t)3) * p->nchan;
-        if (pre <= p->prefix_elems) pre = 0;  // there is as much
-    }
-    const size_t at_pre = room((size_t)pre * 4);
     e = cudaMalloc((void**)&p->dev.slab, total);
     if (e != cudaSuccess) return cuda_status(e);
     unsigned char* slab = p->dev.slab;
@@ -1095,15 +1088,13 @@ dd_status upload_tables(dd_plan_s* p) {
     p->dev.w = p->unit ? nullptr : (float*)(slab + at_w);
     p->dev.status = (int32_t*)(slab + at_status);
     p->dev.off = (double*)(slab + at_off);
-    if (pre) {
-        if (p->prefix_own) cudaFree(p->d_prefix);
-        p->prefix_own = false;
-        p->d_prefix = (uint32_t*)(slab + at_pre);
-        p->prefix_elems = pre;
-    }
     const int32_t zero = 0;
+    // small tables as one copy (a copy takes some 16 us whatever its size)
+    std::vector<unsigned char> all(total <= ((size_t)1 << 20) && p->rec_host == p->rec_bytes ? total : 0);
     auto up = [&](void* dst, const void* src, size_t bytes) {
-        if (e == cudaSuccess && bytes) e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess || !bytes) return;
+        if (!all.empty()) std::memcpy(all.data() + ((unsigned char*)dst - slab), src, bytes);
+        else e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
     };
     up(p->dev.delay, p->delay.data(), n * 4);
     up(p->dev.taps, p->taps.data(), n * 4);
@@ -1114,6 +1105,7 @@ dd_status upload_tables(dd_plan_s* p) {
         up(p->dev.rec, p->rec.data(), p->rec.size());
     else if (e == cudaSuccess)
         e = cudaMemcpy2D(p->dev.rec, p->rec_bytes, p->rec.data(), p->rec_host, p->rec_host, nrec, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !all.empty()) e = cudaMemcpy(slab, all.data(), total, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_status(e);
     dd_status st;
     // place dd_boxcar_snr_noalloc's scratch array and kernels on this device now, so
@@ -1585,6 +1577,12 @@ dd_status dd_test_set_wait(dd_plan_t p, int32_t skip_stage, int64_t wait_ns) {
     if (!p || wait_ns < 0) return DD_ERR_ARG;
     p->debug_skip_stage = skip_stage;
     p->wait_ns = wait_ns > 0 ? wait_ns : dd::kWaitNs;
+    return DD_OK;
+}
+
+dd_status dd_test_set_scratch_limit(dd_plan_t p, int64_t bytes) {
+    if (!p || bytes < 0) return DD_ERR_ARG;
+    p->scratch_limit = bytes;
     return DD_OK;
 }
 

@@ -101,3 +101,79 @@ def test_graph_of_a_plan_outlives_batches_of_it(dd):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, want[0])
+
+
+def _u8_plan(dd, C=24, D=60, T=6000, nsamp=None):
+    import torch
+    rng = np.random.default_rng(7)
+    delay = np.cumsum(rng.integers(0, 3, size=(D, C)), axis=0).astype(np.int32)
+    plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, nsamp or T, "u8"), np.zeros(D))
+    plan.set_profiles(delay=delay, taps=np.full((D, C), 2, np.int32))
+    plan.set_method("direct")
+    return plan, torch.from_numpy(rng.integers(0, 256, size=(C, (T + 15) // 16 * 16)).astype(np.uint8)).cuda()
+
+
+def _want(plan, x, T):
+    import oracle
+    delay, taps = plan.tables()
+    return oracle.c_dedisperse(x.cpu().numpy(), delay, taps, nsamp=T).astype(np.int32)
+
+
+def test_plans_for_detection_take_no_prefix_scratch(dd):
+    """Prefix sums get their scratch from the call that reads them: a plan whose series come from
+    elsewhere, or whose sums a batch forms, has none."""
+    import torch
+    C, T, D = 336, 60000, 300
+    x = torch.zeros((C, T), dtype=torch.uint8, device="cuda")
+    plans = [dd.Plan(dd.Band(C, 1130.0, 1.0, 1.0, T, "u8"), np.linspace(0, 600, D)) for _ in range(9)]
+    assert all(p.method == "direct" for p in plans)
+    plans[0].channel_stats(x, nsamp=T)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for p in plans[1:]:
+        p.channel_stats(x, nsamp=T)
+    torch.cuda.synchronize()
+    # tables of some 4 MB a plan; the prefix sums of a block are 81 MB
+    assert before - torch.cuda.mem_get_info()[0] < 8 * 20e6
+
+
+def test_first_dedispersion_of_a_direct_plan_in_a_capture(dd):
+    """With its tables on the device, a direct plan's first dedispersion may be a captured one."""
+    import torch
+    plan, x = _u8_plan(dd)
+    T = x.shape[1]
+    plan.channel_stats(x)
+    out = torch.zeros((plan.ndm, T - plan.d_max), dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan.dedisperse(x, out=out)
+    graph.replay()
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(out.cpu().numpy(), _want(plan, x, T))
+
+
+@pytest.mark.parametrize("limit_cols", [0, 4000])
+def test_direct_calls_of_growing_length(dd, limit_cols):
+    """Calls longer than any before get more scratch, or go in pieces where there is no more; a
+    graph of a short one replays as it was."""
+    import torch
+    T = 30000
+    plan, x = _u8_plan(dd, T=T, nsamp=1000)
+    assert plan.d_max + 2 * 1088 < 4000
+    plan.test_set_scratch_limit(limit_cols * plan.band.nchan * 4)
+    want = _want(plan, x, T)
+    out = torch.zeros((plan.ndm, 600), dtype=torch.int32, device="cuda")
+    short = plan.dedisperse(x, nsamp=plan.d_max + 600)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan.dedisperse(x, nsamp=plan.d_max + 600, out=out)
+    for t_out in (700, 3000, 3300, 9000, T - plan.d_max):
+        got = plan.dedisperse(x, nsamp=plan.d_max + t_out)
+        np.testing.assert_array_equal(got.cpu().numpy(), want[:, :t_out])
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, short)
+    np.testing.assert_array_equal(short.cpu().numpy(), want[:, :600])
+    assert plan.device_status() == 0
