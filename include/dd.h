@@ -36,7 +36,7 @@
  *     grows (normaliser workspace), dd_dedisperse when nsamp grows, on a run-length plan or an
  *     integer plan whose direct sums read prefix sums (prefix scratch, 4 bytes per channel and
  *     sample; the latter's at most 2 GiB unless the longest delay needs more, and less, with
- *     the call in pieces, where that is not to be had; its smaller ones of earlier calls are kept
+ *     the call in pieces or tap by tap, where that is not to be had; its smaller ones of earlier calls are kept
  *     until the tables change, for captured calls that read them), dd_dedisperse_boxcar when its scratch
  *     grows (on those plans prefix sums of all its samples, too), dd_batch_bind, and the first
  *     dd_backward (adjoint workspace).
@@ -230,7 +230,7 @@ dd_status dd_boxcar_snr_noalloc(dd_plan_t plan, const void* d_series, int64_t ld
  * plan-owned device scratch when the sizes grow: the merged maxima (8 bytes per trial
  * and width), per part its carried outputs and seams (12 C bytes per trial of a
  * CTA's block) and, on plans that read prefix sums, those of all samples (4 bytes per channel
- * and sample).  A call with a new width list or a new launch geometry copies small
+ * and sample; direct plans do without where there is no room).  A call with a new width list or a new launch geometry copies small
  * host tables to the device synchronously, so make one such call before capturing the
  * stream in a CUDA graph.  Calls on one plan share its scratch: order them on one
  * stream. */
@@ -327,9 +327,9 @@ dd_status dd_plan_autotune(dd_plan_t plan, const void* d_in, int64_t in_ld, void
  * own launch (dd_dedisperse).  For plans whose own launch leaves SMs idle the batch may take
  * another of their schedules (never where one was set or tuned), with the same results; its tables
  * are the batch's, the plans and what was captured from them stay as they are.
- * Run-length beams first get their per-channel prefix sums (one small launch per beam,
- * into device memory the batch owns: 4 bytes per channel and sample, allocated by
- * dd_batch_bind), then the batched launch sums them. */
+ * Beams whose sums read prefix sums (run-length, and direct integer ones with shared runs, which
+ * do without where there is no room) first get them, one small launch per beam, into device
+ * memory the batch owns: 4 bytes per channel and sample, allocated by dd_batch_bind. */
 typedef struct dd_batch_s* dd_batch_t;
 dd_status dd_batch_create(dd_batch_t* batch, const dd_plan_t* plans, int32_t nbeams);
 /* Binds each beam's device input [nchan][in_ld] and output [ndm][out_ld] (host arrays of
@@ -337,8 +337,8 @@ dd_status dd_batch_create(dd_batch_t* batch, const dd_plan_t* plans, int32_t nbe
  * (allocates; synchronous).  Rebinding invalidates a captured graph. */
 dd_status dd_batch_bind(dd_batch_t batch, const void* const* d_in, const int64_t* in_ld,
                         void* const* d_out, const int64_t* out_ld);
-/* The batched dedispersion launch for all bound beams (on run-length beams the prefix
- * passes before it). */
+/* The batched dedispersion launch for all bound beams (and the prefix passes before
+ * it). */
 dd_status dd_batch_dedisperse(dd_batch_t batch, void* stream);
 /* Binds, per beam, the outputs of the detection stage (boxcar widths shared by all beams;
  * device channel mean/std [nchan], peak S/N and peak time [ndm][nw]). */

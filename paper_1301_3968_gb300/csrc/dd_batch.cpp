@@ -149,7 +149,7 @@ void choose_schedules(dd_batch_s* b) {
         const bool want = ctas > 152 && small(p);
         if (b->twin_id[i] != p->sched_id || !want) {
             if (b->twin[i]) dd::destroy_plan(b->twin[i]);
-            b->twin[i] = want ? dd::twin_of(p) : nullptr;
+            b->twin[i] = want ? dd::twin_of(p, dd::Twin::kSharesSm) : nullptr;
             b->twin_id[i] = want ? p->sched_id : 0;
         }
         b->sched[i] = b->twin[i] ? b->twin[i] : p;
@@ -218,28 +218,35 @@ dd_status dd_batch_bind(dd_batch_t b, const void* const* d_in, const int64_t* in
             const dd_status st = dd::upload_tables(b->twin[i]);
             if (st != DD_OK) return st;
         }
-    build_items(b);
     for (int i = 0; i < nb; ++i) {
         dd_plan_s* p = b->sched[i];
-        const int64_t t_out = plan_t_out(p);
-        if (!dd::reads_prefix(p)) {
-            dd::fill_dedisp_args(p, d_in[i], in_ld[i], 0, t_out, d_out[i], out_ld[i], &args[i]);
-            b->d_prefix.push_back(nullptr);
-            b->ldp.push_back(0);
-            continue;
-        }
         // beams that read prefix sums have their own, which the batch owns
         const int64_t ldp = (p->band.nsamp + 1 + 3) & ~(int64_t)3;
+        const size_t bytes = (size_t)ldp * p->nchan * sizeof(uint32_t);
         uint32_t* q = nullptr;
-        const cudaError_t e = cudaMalloc((void**)&q, (size_t)ldp * p->nchan * sizeof(uint32_t));
-        if (e != cudaSuccess) {
-            free_batch_dev(b);
-            return dd::cuda_status(e);
+        if (dd::reads_prefix(p)) {
+            const int64_t limit = b->plans[i]->scratch_limit;
+            cudaError_t e = limit > 0 && (int64_t)bytes > limit ? cudaErrorMemoryAllocation : cudaMalloc((void**)&q, bytes);
+            if (e == cudaErrorMemoryAllocation && !p->rl) {  // direct sums do without, tap by tap
+                cudaGetLastError();
+                q = nullptr;
+                if (b->twin[i]) dd::destroy_plan(b->twin[i]);
+                b->twin[i] = dd::twin_of(b->plans[i], dd::Twin::kTaps);
+                b->twin_id[i] = 0;  // (chosen anew at the next bind)
+                b->sched[i] = b->twin[i] ? b->twin[i] : b->plans[i];
+                if (b->twin[i] && dd::upload_tables(b->twin[i]) == DD_OK) e = cudaSuccess;
+            }
+            if (e != cudaSuccess) {
+                free_batch_dev(b);
+                return dd::cuda_status(e);
+            }
         }
         b->d_prefix.push_back(q);
         b->ldp.push_back(ldp);
-        dd::fill_dedisp_args(p, q, ldp, 0, t_out, d_out[i], out_ld[i], &args[i]);
+        p = b->sched[i];
+        dd::fill_dedisp_args(p, q ? q : d_in[i], q ? ldp : in_ld[i], 0, plan_t_out(p), d_out[i], out_ld[i], &args[i]);
     }
+    build_items(b);
     int dev = -1, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -408,9 +408,10 @@ cudaError_t PrefixUse::mark(cudaStream_t q) {
     return e == cudaSuccess ? cudaEventRecord(p->prefix_done, q) : e;
 }
 
-PrefixUse::~PrefixUse() {
-    if (id == 0 || err != cudaSuccess) return;
-    if (id == 1 || mark(s) == cudaSuccess) p->prefix_stream = id;
+void PrefixUse::release() {
+    if (id != 0 && err == cudaSuccess && (id == 1 || mark(s) == cudaSuccess)) p->prefix_stream = id;
+    id = 0;
+    if (lock.owns_lock()) lock.unlock();
 }
 
 // Room for `need` words of prefix sums (or DD_ERR_OOM, which leaves a direct plan what it has).  A

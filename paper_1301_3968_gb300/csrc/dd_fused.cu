@@ -426,7 +426,15 @@ extern "C" dd_status dd_dedisperse_boxcar(dd_plan_t p, const void* in, int64_t i
     if (use.err != cudaSuccess) return cuda_status(use.err);
     if (reads_prefix(p)) {
         int64_t ldp = 0;
-        if ((st = launch_prefix(p, in, in_ld, t_offset, nsamp, &ldp, s)) != DD_OK) return st;
+        st = launch_prefix(p, in, in_ld, t_offset, nsamp, &ldp, s);
+        if (st == DD_ERR_OOM && !p->rl) {  // no room for the sums of all samples: the tap kernels need none
+            use.release();
+            dd_plan_s* t = tap_twin(p);
+            if (t)
+                return dd_dedisperse_boxcar(t, in, in_ld, t_offset, nsamp, widths, nw, mean, sd, peak, arg, thresh, cands,
+                                            cap, ncands, stream);
+        }
+        if (st != DD_OK) return st;
         fill_dedisp_args(p, p->d_prefix, ldp, 0, t_out, nullptr, 0, &a);
     } else {
         fill_dedisp_args(p, in, in_ld, t_offset, t_out, nullptr, 0, &a);
@@ -562,5 +570,6 @@ extern "C" dd_status dd_test_fused_smem(int32_t kind, int32_t warps, int32_t nch
 extern "C" dd_status dd_test_set_fused_parts(dd_plan_t p, int32_t nparts) {
     if (!p || nparts < 0) return DD_ERR_ARG;
     p->debug_fused_parts = nparts;
+    if (p->tap) p->tap->debug_fused_parts = nparts;
     return DD_OK;
 }

@@ -330,6 +330,9 @@ struct dd_plan_s {
     bool shares_sm = false;            // rows leave room for two CTAs even where the plan has one wave
     uint64_t sched_id = 0;             // the profiles and schedule as they were last built
     dd_plan_s* owner = nullptr;        // a twin's plan (twin_of): its status word and test hooks count
+    bool no_rows = false;              // tap kernels only
+    dd_plan_s* tap = nullptr;          // direct plans without prefix scratch to be had: the tap kernels'
+    uint64_t tap_id = 0;               // twin, of the profiles and schedule sched_id
     bool w_dev = false;                // weights come from the device (host copy is not theirs)
     bool w_follows = false;            // a device copy of the weights follows every upload
     uint64_t w_id = 0;                 // the upload or copy that the device's weights come from
@@ -362,15 +365,20 @@ dd_status launch_dedisperse_batched(bool u8, bool pair, bool short_taps, const D
                                     bool rl = false);
 int dedisp_batched_blocks_per_sm(bool u8, bool pair, bool short_taps, size_t smem, bool rl = false);
 // A plan with p's profiles and another of its schedules, which leaves p, its tables and what was
-// captured from it as they are: the stages for a launch with other plans' CTAs (shares_sm).  For p's
-// lifetime, until p->sched_id changes; null where its sums would differ from p's.
-dd_plan_s* twin_of(dd_plan_s* p);
+// captured from it as they are: the stages for a launch with other plans' CTAs, or the tap kernels.
+// For p's lifetime, until p->sched_id changes; null where there is none or its sums would differ
+// from p's.
+enum class Twin { kSharesSm, kTaps };
+dd_plan_s* twin_of(dd_plan_s* p, Twin kind);
+// The tap kernels' twin of a direct plan whose prefix scratch is not to be had (kept by the plan).
+dd_plan_s* tap_twin(dd_plan_s* p);
 
 // A call's use of its plan's prefix scratch (p null: none), from the prefix pass to the last launch
 // that reads it: on a direct plan it waits for the last use on another stream.
 struct PrefixUse {
     PrefixUse(dd_plan_s* p, cudaStream_t s);
-    ~PrefixUse();
+    ~PrefixUse() { release(); }
+    void release();  // the last launch has been made
     PrefixUse(const PrefixUse&) = delete;
     PrefixUse& operator=(const PrefixUse&) = delete;
     cudaError_t err = cudaSuccess;

@@ -362,6 +362,7 @@ struct Pattern {
 // The plan's row kind, if its sums can be formed that way: fp32 sums with weights that the
 // host knows, integer sums of runs that fit a half word.
 int row_kind_of(const dd_plan_s* p) {
+    if (p->no_rows) return dd::kRowsNone;
     if (p->pair) return p->w_dev || p->kmax > 0xffff ? dd::kRowsNone : dd::kRowsFir;
     if (p->kmax > dd::kPkMaxTaps) return dd::kRowsNone;
     // (the prefix sums of a direct plan live in a scratch that holds its longest delay)
@@ -1017,7 +1018,7 @@ static void free_dev(dd_plan_s* p, int to) {
     p->widths_on_dev.clear();
 }
 
-dd_plan_s* twin_of(dd_plan_s* p) {
+dd_plan_s* twin_of(dd_plan_s* p, Twin kind) {
     dd_plan_s* t = new (std::nothrow) dd_plan_s;
     if (!t) return nullptr;
     t->band = p->band;
@@ -1038,15 +1039,37 @@ dd_plan_s* twin_of(dd_plan_s* p) {
     t->method = p->method;
     t->w_dev = p->w_dev;
     t->owner = p;
-    t->shares_sm = true;
+    t->shares_sm = kind == Twin::kSharesSm;
+    t->no_rows = kind == Twin::kTaps;
+    t->debug_fused_parts = p->debug_fused_parts;
     // (integer sums are the same from the tap kernels, which such a schedule may be; fp32 ones are not)
-    if (build_schedule(t) == DD_OK && (!t->pair || t->rk == p->rk)) return t;
+    if (build_schedule(t) == DD_OK && (!t->pair || t->rk == p->rk)) {
+        // (the caller's shape, where the tap kernels have it)
+        if (t->no_rows && !p->own_schedule) build_schedule_fixed(t, p->nch, p->cs);
+        return t;
+    }
     delete t;
     return nullptr;
 }
 
+dd_plan_s* tap_twin(dd_plan_s* p) {
+    if (p->rl || p->rk != kRowsPk) return nullptr;
+    std::lock_guard<std::mutex> lock(p->prefix_mu);
+    if (p->tap && p->tap_id != p->sched_id) {
+        destroy_plan(p->tap);
+        p->tap = nullptr;
+    }
+    if (!p->tap) {
+        log_msg(1, "plan %d trials x %d channels: no room for prefix sums, tap by tap", p->ndm, p->nchan);
+        p->tap = twin_of(p, Twin::kTaps);
+        p->tap_id = p->sched_id;
+    }
+    return p->tap;
+}
+
 void destroy_plan(dd_plan_s* p) {
     if (p->adj) destroy_plan(p->adj);
+    if (p->tap) destroy_plan(p->tap);
     if (p->d_gpad) cudaFree(p->d_gpad);
     if (p->d_gsplit) cudaFree(p->d_gsplit);
     if (p->d_fkey) cudaFree(p->d_fkey);
@@ -1356,7 +1379,11 @@ dd_status dd_dedisperse(dd_plan_t p, const void* in, int64_t in_ld, int64_t t_of
     dd_status st = dd::upload_tables(p);
     if (st != DD_OK) return st;
     if (p->rl) return dd::launch_dedisperse_rl(p, in, in_ld, t_offset, nsamp, out, out_ld, (cudaStream_t)stream);
-    if (p->rk == dd::kRowsPk) return dd::launch_dedisperse_pk(p, in, in_ld, t_offset, nsamp, out, out_ld, (cudaStream_t)stream);
+    if (p->rk == dd::kRowsPk) {
+        st = dd::launch_dedisperse_pk(p, in, in_ld, t_offset, nsamp, out, out_ld, (cudaStream_t)stream);
+        dd_plan_s* t = st == DD_ERR_OOM ? dd::tap_twin(p) : nullptr;
+        return t ? dd_dedisperse(t, in, in_ld, t_offset, nsamp, out, out_ld, stream) : st;
+    }
     return dd::launch_dedisperse(p, in, in_ld, t_offset, t_out, out, out_ld, (cudaStream_t)stream);
 }
 
@@ -1575,7 +1602,7 @@ dd_status dd_get_device_status(dd_plan_t p, int32_t* code, void* stream) {
 
 dd_status dd_test_set_wait(dd_plan_t p, int32_t skip_stage, int64_t wait_ns) {
     if (!p || wait_ns < 0) return DD_ERR_ARG;
-    p->debug_skip_stage = skip_stage;
+    p->debug_skip_stage = skip_stage;  // (a twin reads its owner's)
     p->wait_ns = wait_ns > 0 ? wait_ns : dd::kWaitNs;
     return DD_OK;
 }

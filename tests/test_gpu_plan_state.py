@@ -177,3 +177,39 @@ def test_direct_calls_of_growing_length(dd, limit_cols):
     assert torch.equal(out, short)
     np.testing.assert_array_equal(short.cpu().numpy(), want[:, :600])
     assert plan.device_status() == 0
+
+
+@pytest.mark.parametrize("nch", [0, 2])
+def test_direct_plan_without_room_for_prefix_sums(dd, nch):
+    """Where the device has no room for a direct plan's prefix sums, its taps are summed one by one:
+    the same sums and maxima, from the plan, the fused call and a batch, and with the next profiles;
+    with room again, the shared rows."""
+    import torch
+    T = 6000
+    plan, x = _u8_plan(dd, T=T)
+    if nch:
+        plan.set_schedule(nch, 4)
+    want = _want(plan, x, T)
+    mean, sd = plan.channel_stats(x, nsamp=T)
+    wl = np.arange(1, 20, dtype=np.int32)
+    peak, arg, _ = plan.boxcar_snr(torch.from_numpy(want).cuda(), wl, mean, sd)
+    for limit in (1, 0):
+        plan.test_set_scratch_limit(limit)
+        np.testing.assert_array_equal(plan.dedisperse(x, nsamp=T).cpu().numpy(), want)
+        plan.test_set_fused_parts(3)
+        p1, a1, _ = plan.dedisperse_boxcar(x, wl, mean, sd, nsamp=T)
+        assert torch.equal(p1.view(torch.int32), peak.view(torch.int32)) and torch.equal(a1, arg)
+        plan.set_method("direct" if limit else "auto")      # new tables
+        out = torch.zeros((plan.ndm, want.shape[1]), dtype=torch.int32, device="cuda")
+        batch = dd.Batch([plan])
+        batch.bind([x], [out])
+        batch.dedisperse()
+        np.testing.assert_array_equal(out.cpu().numpy(), want)
+        batch.close()
+        assert plan.device_status() == 0
+    plan, x = _u8_plan(dd, T=T)
+    plan.test_set_scratch_limit(1)
+    plan.dedisperse(x, nsamp=T)
+    delay, taps = plan.tables()
+    plan.set_profiles(delay=delay[::-1], taps=taps[::-1] + 1)
+    np.testing.assert_array_equal(plan.dedisperse(x, nsamp=T).cpu().numpy(), _want(plan, x, T))
