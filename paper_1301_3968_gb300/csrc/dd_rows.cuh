@@ -309,11 +309,12 @@ __device__ __forceinline__ void issue_rows(const DedispArgs& a, const RowSmem& s
     int bytes = nin * (int)sizeof(TIN);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) bytes += __shfl_xor_sync(0xffffffffu, bytes, o);
+    if (tail) __syncwarp();  // the lanes' zeros are written before lane 0 arrives on the barrier for them all
     if (lane == 0) {
         mbar_expect_tx(sm.full, (uint32_t)(bytes + rg.rec_bytes));
         *sm.issued += 1;
     }
-    __syncwarp();
+    __syncwarp();  // and the barrier expects the copies before any lane issues one
     if (nin > 0)
         bulk_g2s(sm.raw + (int64_t)lane * a.lcap * sizeof(TIN), (const TIN*)a.in + (int64_t)(c0 + lane) * a.ld + a0,
                  (uint32_t)(nin * sizeof(TIN)), sm.full);

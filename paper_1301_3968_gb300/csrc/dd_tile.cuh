@@ -245,11 +245,12 @@ __device__ void issue_stage_warp(const DedispArgs& a, const StageGeom& g, const 
     int bytes = nin * (int)sizeof(TIN);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) bytes += __shfl_xor_sync(0xffffffffu, bytes, o);
+    __syncwarp();  // the lanes' zeros are written before lane 0 arrives on the barrier for them all
     if (lane == 0) {
         mbar_expect_tx(&sm.full[b], (uint32_t)(bytes + g.rec_bytes));
         sm.issued[b] += 1;
     }
-    __syncwarp();
+    __syncwarp();  // and the barrier expects the copies before any lane issues one
     if (nin > 0)
         bulk_g2s(buf + (int64_t)lane * a.lcap * sizeof(TIN), (const TIN*)a.in + (int64_t)(c0 + lane) * a.ld + a0,
                  (uint32_t)(nin * sizeof(TIN)), &sm.full[b]);
@@ -681,9 +682,10 @@ __device__ __forceinline__ bool dedisp_tile(const DedispArgs a, unsigned char* s
                 __threadfence_block();
                 old = atomicAdd(&sm.cnt[b], 1);
                 if (old == kWarps - 1) sm.cnt[b] = 0;
+                __threadfence_block();
             }
             if (__shfl_sync(0xffffffffu, old, 0) == kWarps - 1 && i + NBUF < nloc) {  // last warp out
-                __threadfence_block();
+                __syncwarp();  // (a shuffle orders no memory: lane 0 has seen the other warps leave)
                 issue_stage_warp<TIN, NBUF>(a, g, sm, blk, s + NBUF, b, base, lane);
             }
         } else if (lane == 0) {
