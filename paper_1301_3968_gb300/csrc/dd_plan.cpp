@@ -848,9 +848,12 @@ dd_status build_schedule(dd_plan_s* p) {
 // autotuner's, which may be a row schedule that the tap kernels have no shared memory for.
 dd_status build_schedule_fixed(dd_plan_s* p, int nch, int cs, bool tuned = false) {
     if (nch < 1 || nch > dd::kWarps || (dd::kWarps % nch) != 0 || cs < 1 || cs > 32) return DD_ERR_ARG;
-    p->sched_id = ++g_gen;
-    p->own_schedule = false;
-    if (tuned && build_rows(p, nch, cs)) return DD_OK;
+    auto done = [&] {
+        p->sched_id = ++g_gen;
+        p->own_schedule = false;
+        return DD_OK;
+    };
+    if (tuned && build_rows(p, nch, cs)) return done();
     const int esz = stage_esz(p);
     const int nu = dd::kWarps / nch * units_per_warp(p);
     const int db = trials_per_unit(p) * nu;
@@ -867,7 +870,7 @@ dd_status build_schedule_fixed(dd_plan_s* p, int nch, int cs, bool tuned = false
         return DD_ERR_UNSUPPORTED;
     p->rk = dd::kRowsNone;
     p->rl_b = rl_b;
-    if (build_rows(p, nch, cs)) return DD_OK;
+    if (build_rows(p, nch, cs)) return done();
     p->blen = blen;
     p->nch = nch;
     p->cs = cs;
@@ -877,7 +880,7 @@ dd_status build_schedule_fixed(dd_plan_s* p, int nch, int cs, bool tuned = false
     block_span(p, db, &p->blk_lo);
     build_records(p);
     p->dev_dirty = true;
-    return DD_OK;
+    return done();
 }
 
 dd_status finish_profiles(dd_plan_s* p) {
@@ -1517,6 +1520,10 @@ dd_status dd_plan_autotune(dd_plan_t p, const void* d_in, int64_t in_ld, void* d
     auto cache = read_cache(cache_path);
     auto hit = cache.find(key);
     if (hit != cache.end() && p->rk && hit->second.second == 0) {  // the plan's own schedule
+        if (!p->own_schedule) {
+            const dd_status st = build_schedule(p);
+            if (st != DD_OK) return st;
+        }
         if (best_ms) *best_ms = -1.0f;
         dd::log_msg(1, "autotune %s: cached: the plan's own schedule", key.c_str());
         return DD_OK;
@@ -1528,6 +1535,7 @@ dd_status dd_plan_autotune(dd_plan_t p, const void* d_in, int64_t in_ld, void* d
         return DD_OK;
     }
     const int orig_nch = p->nch, orig_cs = p->cs, orig_rk = p->rk;
+    const bool orig_own = p->own_schedule;
     std::vector<std::pair<int, int>> cand;  // (time chunks, channels per stage)
     if (orig_rk) cand.push_back({orig_nch, orig_cs});
     for (int nch = 1; nch <= 2; nch *= 2)
@@ -1535,7 +1543,7 @@ dd_status dd_plan_autotune(dd_plan_t p, const void* d_in, int64_t in_ld, void* d
                               : stage_esz(p) == 1 ? std::vector<int>{4, 8, 12, 16} : std::vector<int>{2, 3, 4, 6, 8})
             cand.push_back({nch, cs});
     int best_nch = orig_nch, best_cs = orig_cs;
-    bool own = false;  // the first candidate of a row plan
+    bool own = orig_own;  // the best is the plan's own schedule
     float best = 1e30f;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t ce = cudaEventCreate(&e0);
@@ -1568,14 +1576,15 @@ dd_status dd_plan_autotune(dd_plan_t p, const void* d_in, int64_t in_ld, void* d
         // get too, has to be clearly faster (any lead: 36 small beams 13.6 ms, their own 12.4)
         if (t < (orig_rk && i > 0 ? 0.97f : 1.0f) * best) {
             best = t;
-            own = orig_rk && i == 0;
+            own = orig_own && orig_rk && i == 0;
             best_nch = cand[i].first;
             best_cs = cand[i].second;
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (build_schedule_fixed(p, best_nch, best_cs, true) != DD_OK) build_schedule_fixed(p, orig_nch, orig_cs, true);
+    if (own) build_schedule(p);
+    else if (build_schedule_fixed(p, best_nch, best_cs, true) != DD_OK) build_schedule_fixed(p, orig_nch, orig_cs, true);
     if (st != DD_OK) return st;
     if (best_ms) *best_ms = best;
     dd::log_msg(1, "autotune %s: %d time chunks, %d channels per stage, %.3f ms (default %d, %d)", key.c_str(),

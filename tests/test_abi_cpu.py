@@ -365,3 +365,22 @@ def test_batch_leaves_its_plans_as_they_are(lib):
     assert [p.schedule() for p in plans] == before
     batch.close()
     assert [p.schedule() for p in plans] == before
+
+
+def test_cached_own_schedule_replaces_a_set_one(lib, tmp_path):
+    """An autotuner cache that names a row plan's own schedule (0 channels) gives the plan that,
+    also where a caller had set another."""
+    import paper_1301_3968_gb300 as dd
+    plan = dd.Plan(dd.Band(64, 1200.0, 4.6875, 1.0, 4096, "u8"), np.linspace(0.0, 500.0, 128))
+    own = plan.schedule()
+    delay, taps = plan.tables()
+    d8, e8 = delay.reshape(16, 8, 64), (delay + taps).reshape(16, 8, 64)
+    span = int((e8.max(axis=1) - d8.min(axis=1)).max())
+    key = f"C64_u8_rowsint_s{int(math.log2(span + 1))}_k{int(math.log2(int(taps.max()) + 1))}"
+    cache = tmp_path / "tune.txt"
+    cache.write_text(f"{key} 1 0 0.5\n")
+    plan.set_schedule(1, 4)
+    assert plan.schedule() != own
+    fake, best = ctypes.c_void_p(1 << 20), ctypes.c_float(0.0)
+    assert lib.dd_plan_autotune(plan._h, fake, 4096, fake, 4096, str(cache).encode(), ctypes.addressof(best), None) == 0
+    assert best.value == -1.0 and plan.schedule() == own
