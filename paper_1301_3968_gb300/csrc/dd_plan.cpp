@@ -476,7 +476,7 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
                 double single = 2.0 * (d1 - d0) * span, both = (double)(d1 - d0) * span;
                 for (int k = c; k < c + 2; ++k)
                     for (int r = first[b][k]; r < first[b][k + 1]; ++r) {
-                        const double L = rows[b][r].end - rows[b][r].beg + span;
+                        const double L = (double)rows[b][r].end - rows[b][r].beg + span;
                         single += 3.0 * L;
                         (k == c ? n0 : n1) = std::max(k == c ? n0 : n1, rows[b][r].n);
                     }
@@ -495,7 +495,7 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
                     ps[i].end = std::max(ps[i].end, at);
                     id[d - d0] = (uint8_t)i;
                 }
-                for (const Pattern& q : ps) both += 5.0 * (q.end - q.beg + span);
+                for (const Pattern& q : ps) both += 5.0 * ((double)q.end - q.beg + span);
                 pair = pair && both < single;
             }
             const int32_t i0 = (int32_t)pats[b].size();
@@ -508,9 +508,10 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
         }
     });
     // Words of a row: fp32, a run's whole staged window (its start is aligned to the raw buffer's
-    // quads); packed, what its own trials read.
-    auto whole_len = [&](const Row& r) { return (int64_t)((Q - 1 + r.end + span + 3) & ~3); };
-    auto own_len = [&](int32_t beg, int32_t end) { return (int64_t)((end - beg + span + 3) & ~3); };
+    // quads); packed, what its own trials read.  (In 64 bits: a block's trials may start up to 2^31
+    // samples apart.)
+    auto whole_len = [&](const Row& r) { return ((int64_t)Q - 1 + r.end + span + 3) & ~(int64_t)3; };
+    auto own_len = [&](int32_t beg, int32_t end) { return ((int64_t)end - beg + span + 3) & ~(int64_t)3; };
     auto low_bits = [&](int b, int c) { return lo[(size_t)b * C + c] & (Q - 1); };
     size_t total = 0;
     int64_t need = 0;
@@ -561,7 +562,7 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
                 // samples that building the row reads (dd_rows.cuh)
                 const Row& r = rows[b][i];
                 need = std::max(need, fir ? whole_len(r) + (r.n & ~3) + 4
-                                          : low_bits(b, c) + r.end + (int64_t)((span + 3) & ~3) + 3 + r.n);
+                                          : (int64_t)low_bits(b, c) + r.end + ((span + 3) & ~3) + 3 + r.n);
             }
         for (size_t v = 0; v < items[b].size(); v += grain) {
             const Need k = count_grain(b, v);

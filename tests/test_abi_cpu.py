@@ -384,3 +384,17 @@ def test_cached_own_schedule_replaces_a_set_one(lib, tmp_path):
     fake, best = ctypes.c_void_p(1 << 20), ctypes.c_float(0.0)
     assert lib.dd_plan_autotune(plan._h, fake, 4096, fake, 4096, str(cache).encode(), ctypes.addressof(best), None) == 0
     assert best.value == -1.0 and plan.schedule() == own
+
+
+@pytest.mark.parametrize("kind,group", [("f32", 16), ("u8", 8)])
+@pytest.mark.parametrize("far", [70000, 2 ** 30, 2 ** 31 - 2000, 2 ** 31 - 600, 2 ** 31 - 2])
+def test_trials_up_to_2_31_samples_apart_leave_the_rows(lib, kind, group, far):
+    """Trials that the tap kernels put in blocks of their own and a row kernel's CTA would share, too
+    far apart for its shared memory, up to the last start a table may hold: the tap kernels keep
+    them (their 16 or 8 trials per CTA)."""
+    import paper_1301_3968_gb300 as dd
+    D, C = 64, 2
+    delay = np.where(np.arange(D) // group % 2, far, 0).astype(np.int32)[:, None].repeat(C, axis=1)
+    plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, 4096, kind), np.zeros(D))
+    plan.set_profiles(delay=delay, taps=np.ones((D, C), np.int32))
+    assert plan.schedule()["trials_per_cta"] == group and plan.d_max == far
