@@ -1319,8 +1319,9 @@ dd_status dd_set_weights_device(dd_plan_t p, const float* d_w, int32_t kmax, voi
         st = finish_profiles(p);
     } else if (p->rk == dd::kRowsFir) {
         // the rows shared weights that the host knew: back to a record of every trial's own
+        // (in the shape that a caller set, where there is one)
         p->w_dev = true;
-        st = build_schedule(p);
+        if (p->own_schedule || build_schedule_fixed(p, p->nch, p->cs) != DD_OK) st = build_schedule(p);
     }
     p->w_dev = true;
     if (st == DD_OK) st = dd::upload_tables(p);

@@ -213,3 +213,15 @@ def test_direct_plan_without_room_for_prefix_sums(dd, nch):
     delay, taps = plan.tables()
     plan.set_profiles(delay=delay[::-1], taps=taps[::-1] + 1)
     np.testing.assert_array_equal(plan.dedisperse(x, nsamp=T).cpu().numpy(), _want(plan, x, T))
+
+
+def test_weights_from_the_device_keep_a_set_schedule(dd):
+    """A schedule that a caller set stays when weights from the device replace the host's."""
+    plan, x, w, w2, g = _weighted_plan(dd, D=60)
+    assert plan.schedule()["trials_per_cta"] in (24, 48)      # rows: all trials have one weight
+    plan.set_schedule(2, 3)
+    plan.dedisperse(x)
+    plan.set_weights(w)
+    s = plan.schedule()
+    assert (s["nch"], s["cs"], s["trials_per_cta"]) == (2, 3, 8)
+    assert plan.device_status() == 0
