@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <fstream>
 #include <map>
 #include <mutex>
@@ -60,28 +61,35 @@ void build_trials(const dd_band& b, double dm0, double eps, int n, double extra2
 }
 
 // Runs fn(b) for the blocks 0 .. n - 1 on a few threads when there is enough work
-// (entries: table entries touched); on this thread alone where threads cannot be had.
+// (entries: table entries touched); on this thread alone where threads cannot be had.  What fn
+// throws (no memory for its tables) is thrown here, once all have returned.
 template <typename F>
 void for_blocks(int n, size_t entries, F fn) {
     // (a thread costs about what 6 x 10^4 entries do)
     const int nt = (int)std::min<size_t>(std::min<size_t>(8, std::max(1u, std::thread::hardware_concurrency())),
                                          std::max<size_t>(1, entries >> 16));
     std::vector<std::thread> th;
+    std::vector<std::exception_ptr> thrown((size_t)nt);
+    auto share = [&fn, &thrown, n, nt](int k) {
+        try {
+            for (int b = k; b < n; b += nt) fn(b);
+        } catch (...) {
+            thrown[k] = std::current_exception();
+        }
+    };
     int started = 1;
     if (nt > 1) {
         th.reserve(nt);
         try {
-            for (; started < nt; ++started)
-                th.emplace_back([&fn, n, nt, started] {
-                    for (int b = started; b < n; b += nt) fn(b);
-                });
-        } catch (const std::system_error&) {
+            for (; started < nt; ++started) th.emplace_back(share, started);
+        } catch (const std::exception&) {  // (no thread, or no memory for its state)
         }
     }
-    for (int b = 0; b < n; b += nt) fn(b);
-    for (int k = started; k < nt; ++k)
-        for (int b = k; b < n; b += nt) fn(b);
+    share(0);
+    for (int k = started; k < nt; ++k) share(k);
     for (auto& t : th) t.join();
+    for (auto& e : thrown)
+        if (e) std::rethrow_exception(e);
 }
 
 // The largest fn(b) over the blocks (at least 0).
@@ -1196,13 +1204,8 @@ dd_status dd_trial_dms(const dd_band* band, double dm0, double dm_max, int32_t n
     return DD_OK;
 }
 
-dd_status dd_plan_create(dd_plan_t* out, const dd_band* band, const double* dms, int32_t ndm) {
-    if (!out || !band_ok(band) || !dms || ndm < 1) return DD_ERR_ARG;
-    *out = nullptr;
-    for (int d = 0; d < ndm; ++d)
-        if (!(dms[d] >= 0.0) || !std::isfinite(dms[d])) return DD_ERR_ARG;
-    dd_plan_s* p = new (std::nothrow) dd_plan_s;
-    if (!p) return DD_ERR_OOM;
+// The tables and schedule of a new plan.
+static dd_status fill_plan(dd_plan_s* p, const dd_band* band, const double* dms, int32_t ndm) {
     p->band = *band;
     p->nchan = band->nchan;
     p->ndm = ndm;
@@ -1235,17 +1238,24 @@ dd_status dd_plan_create(dd_plan_t* out, const dd_band* band, const double* dms,
         }
         return 0;
     });
-    if (far) {
-        delete p;
-        return DD_ERR_OVERFLOW;
+    return far ? DD_ERR_OVERFLOW : finish_profiles(p);
+}
+
+dd_status dd_plan_create(dd_plan_t* out, const dd_band* band, const double* dms, int32_t ndm) {
+    if (!out || !band_ok(band) || !dms || ndm < 1) return DD_ERR_ARG;
+    *out = nullptr;
+    for (int d = 0; d < ndm; ++d)
+        if (!(dms[d] >= 0.0) || !std::isfinite(dms[d])) return DD_ERR_ARG;
+    dd_plan_s* p = new (std::nothrow) dd_plan_s;
+    if (!p) return DD_ERR_OOM;
+    dd_status st = DD_ERR_OOM;
+    try {
+        st = fill_plan(p, band, dms, ndm);
+    } catch (const std::bad_alloc&) {
     }
-    dd_status st = finish_profiles(p);
-    if (st != DD_OK) {
-        delete p;
-        return st;
-    }
-    *out = p;
-    return DD_OK;
+    if (st == DD_OK) *out = p;
+    else delete p;
+    return st;
 }
 
 dd_status dd_set_profiles(dd_plan_t p, const int32_t* delay, const int32_t* ntaps,

@@ -398,3 +398,25 @@ def test_trials_up_to_2_31_samples_apart_leave_the_rows(lib, kind, group, far):
     plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, 4096, kind), np.zeros(D))
     plan.set_profiles(delay=delay, taps=np.ones((D, C), np.int32))
     assert plan.schedule()["trials_per_cta"] == group and plan.d_max == far
+
+
+def test_plan_create_without_host_memory(lib):
+    """A plan whose tables do not fit the host's memory is refused with DD_ERR_OOM."""
+    import subprocess
+    import sys
+    code = ("import sys, resource; sys.path.insert(0, %r)\n"
+            "import ctypes, numpy as np, paper_1301_3968_gb300 as dd\n"
+            "from paper_1301_3968_gb300 import _lib\n"
+            "lib = _lib.load()\n"
+            "b = dd.Band(1024, 700.0, 300.0 / 1024, 0.064, 1 << 16, 'u8').c_struct()\n"
+            "dms = np.linspace(0.0, 800.0, 8192)\n"
+            "for mb in (8, 24, 40, 56):\n"
+            "    used = int(open('/proc/self/statm').read().split()[0]) * resource.getpagesize()\n"
+            "    h = ctypes.c_void_p()\n"
+            "    old = resource.getrlimit(resource.RLIMIT_AS)\n"
+            "    resource.setrlimit(resource.RLIMIT_AS, (used + (mb << 20), old[1]))\n"
+            "    st = lib.dd_plan_create(ctypes.byref(h), ctypes.byref(b), dms.ctypes.data, len(dms))\n"
+            "    resource.setrlimit(resource.RLIMIT_AS, old)\n"
+            "    assert st == 3 and not h.value, st\n" % ROOT)
+    res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, (res.returncode, res.stdout, res.stderr[-2000:])
