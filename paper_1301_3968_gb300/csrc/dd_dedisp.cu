@@ -85,12 +85,23 @@ dd_status run(DedispArgs a, cudaStream_t s) {
     return cuda_status(cudaGetLastError());
 }
 
-// A tap launch of at most kUnitCtas CTAs: one CTA per pair unit and 768 outputs instead of per
-// eight units and 864.  A trial's outputs then run on eight warps of one SM, and the blocks'
-// units on SMs of their own; each CTA stages the rows for itself, which costs more copies than
-// it saves once the SMs are full.  One trial x 64 channels x 841 outputs x 32 taps: 36 us
-// against 119.
-constexpr int64_t kUnitCtas = 76;  // half the SMs
+// Small tap launches: one CTA per pair unit and 768 outputs instead of per eight units and 864.  A
+// trial's outputs then run on eight warps of one SM, and the blocks' units on SMs of their own; each
+// CTA stages the rows for itself.  One trial x 64 channels x 841 outputs x 32 taps: 36 us against 119.
+// Up to a CTA per SM that pays whatever the taps are; long runs, which hide the staging, pay to four
+// per SM.  64 and 336 channels, 1-600 trials, 300-9000 outputs, time of the full launch over this
+// one's: up to 152 CTAs 0.96-2.2 with 2 taps, 1.06-2.5 with 6, 2.0-5.2 with 16, 2.6-5.1 with 32 and 48;
+// 153-304 0.61-1.2, 0.87-1.4, 2.1-3.3, 2.4-3.0; 305-608 0.31-0.97, 0.45-1.2, 1.3-2.8, 1.4-2.8; 609-900
+// 0.27-0.38, 0.38-0.46, 1.04-1.10, 0.97-1.11.
+constexpr int64_t kUnitCtas = 152, kUnitCtasLong = 608;
+constexpr double kUnitLongTaps = 16.0;  // mean taps of a run
+struct UnitGrid {
+    int64_t tiles, blocks, units;  // (the last block's units past the trial list have only copies to wait for)
+};
+UnitGrid unit_grid(int64_t t_out, int32_t ndm, int32_t nch) {
+    const int nu = kWarps / nch, tile = kWarps * 32 * kRSmall;
+    return {(t_out + tile - 1) / tile, (ndm + 2 * nu - 1) / (2 * nu), std::min(nu, (ndm + 1) / 2)};
+}
 
 template <typename TIN, int NBUF>
 dd_status run_unit(DedispArgs a, cudaStream_t s) {
@@ -99,10 +110,8 @@ dd_status run_unit(DedispArgs a, cudaStream_t s) {
     auto kern = k_dedisp_unit<TIN, NBUF>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e);
-    const int nu = kWarps / a.nch, tile = kWarps * 32 * kRSmall;
-    const int nblk = (a.ndm + 2 * nu - 1) / (2 * nu);
-    // (the last block's units past the trial list leave at once)
-    dim3 grid((unsigned)((a.t_out + tile - 1) / tile), (unsigned)nblk, (unsigned)std::min(nu, (a.ndm + 1) / 2));
+    const UnitGrid g = unit_grid(a.t_out, a.ndm, a.nch);
+    dim3 grid((unsigned)g.tiles, (unsigned)g.blocks, (unsigned)g.units);
     kern<<<grid, kWarps * 32, smem, s>>>(a);
     return cuda_status(cudaGetLastError());
 }
@@ -355,8 +364,9 @@ dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_
     const bool u8 = p->band.in_type == DD_U8;
     if (!p->pair)
         return p->kmax <= kRInt ? run<uint8_t, false, kStagesInt, 1>(a, s) : run<uint8_t, false, kStagesInt>(a, s);
-    const int64_t tile = (int64_t)chunk_t(true) * a.nch, db = 2 * (kWarps / a.nch);
-    if (nsplit == 1 && (t_out + tile - 1) / tile * ((p->ndm + db - 1) / db) <= kUnitCtas)
+    const UnitGrid ug = unit_grid(t_out, p->ndm, a.nch);
+    const bool long_taps = (double)p->ns_total >= kUnitLongTaps * p->ndm * p->nchan;
+    if (nsplit == 1 && ug.tiles * ug.blocks * ug.units <= (long_taps ? kUnitCtasLong : kUnitCtas))
         return u8 ? run_unit<uint8_t, kStagesPair>(a, s) : run_unit<float, kStagesPair>(a, s);
     // union windows of at most R taps: one unrolled pass; at most 2R: two; longer: a loop
     const int passes = p->umax <= kRPair ? 1 : (p->umax <= 2 * kRPair ? 2 : 0);
