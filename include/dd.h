@@ -273,7 +273,9 @@ dd_status dd_backward(dd_plan_t plan, const float* d_in, int64_t in_ld, int64_t 
  * up to 257 taps; fp32 sums with unit weights, or with weights given from the host that many
  * trials have in common) use kernels that form each shared run's sums once: there a CTA sums
  * 24/nch or 48/nch trials (fp32), 16/nch or 32/nch (integer), by the size of the plan's block,
- * and cs is the most channels of a stage.
+ * and cs is the most channels of a stage.  fp32 lists take them where they are expected to be
+ * faster over the band's nsamp: fine lists always, coarse ones by the size of the plan's block, so
+ * that two plans of one coarse list may round fp32 sums differently.
  * dd_plan_create and dd_set_profiles pick a default; dd_plan_set_schedule overrides it
  * (DD_ERR_UNSUPPORTED if it does not fit in shared memory, the old one is then kept). */
 dd_status dd_plan_set_schedule(dd_plan_t plan, int32_t nch, int32_t cs);

@@ -353,6 +353,12 @@ size_t dedisp_smem_for(const dd_plan_s* p) {
     return smem_for<float, true, kStagesPair>(p->lcap, kp, p->cs, p->nch, p->nchan);
 }
 
+bool takes_units(const dd_plan_s* p, int64_t t_out, int nch) {
+    const UnitGrid g = unit_grid(t_out, p->ndm, nch);
+    const bool long_taps = (double)p->ns_total >= kUnitLongTaps * p->ndm * p->nchan;
+    return g.tiles * g.blocks * g.units <= (long_taps ? kUnitCtasLong : kUnitCtas);
+}
+
 dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                             int64_t t_out, void* out, int64_t out_ld, cudaStream_t s, int nsplit,
                             int64_t split_ld) {
@@ -364,9 +370,7 @@ dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_
     const bool u8 = p->band.in_type == DD_U8;
     if (!p->pair)
         return p->kmax <= kRInt ? run<uint8_t, false, kStagesInt, 1>(a, s) : run<uint8_t, false, kStagesInt>(a, s);
-    const UnitGrid ug = unit_grid(t_out, p->ndm, a.nch);
-    const bool long_taps = (double)p->ns_total >= kUnitLongTaps * p->ndm * p->nchan;
-    if (nsplit == 1 && ug.tiles * ug.blocks * ug.units <= (long_taps ? kUnitCtasLong : kUnitCtas))
+    if (nsplit == 1 && takes_units(p, t_out, a.nch))
         return u8 ? run_unit<uint8_t, kStagesPair>(a, s) : run_unit<float, kStagesPair>(a, s);
     // union windows of at most R taps: one unrolled pass; at most 2R: two; longer: a loop
     const int passes = p->umax <= kRPair ? 1 : (p->umax <= 2 * kRPair ? 2 : 0);

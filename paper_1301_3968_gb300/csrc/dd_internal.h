@@ -416,6 +416,9 @@ int rows_batched_blocks_per_sm(int kind, bool in8, int nw, size_t smem);
 dd_status launch_rows_fused(const dd_plan_s* p, DedispArgs a, const FusedArgs& f, size_t smem, cudaStream_t s);
 int rows_fused_blocks_per_sm(const dd_plan_s* p, size_t smem);
 
+// fp32 tap launches that give each pair unit a CTA (dd_dedisp.cu)
+bool takes_units(const dd_plan_s* p, int64_t t_out, int nch);
+
 // launchers (stream = cudaStream_t)
 dd_status launch_dedisperse(dd_plan_s* p, const void* in, int64_t ld, int64_t t_offset,
                             int64_t t_out, void* out, int64_t out_ld, cudaStream_t s,

@@ -384,8 +384,38 @@ constexpr double kRowsMaxShare = 0.5;
 // samples later.  Elsewhere a trial reads a word per channel and output, which costs what seven or
 // eight packed multiply-adds of the tap kernel do, and a block's spread of starts makes long rows:
 // 92 trials over DM 0-1945 (0.16 of the pairs near) x 336 channels x 4433 samples took 542 us, with
-// taps 178; 400 low-band trials over DM 0-60 (0.36) 2.66 ms, with taps 3.24.
-constexpr double kRowsMinNear = 0.3;
+// taps 178.  Lists with fewer near pairs than kRowsMinNear take the taps, fine lists (kRowsFine) the
+// rows whatever their size, so that a list and its parts take one kernel; between, the plan's block
+// decides by the estimate below.
+constexpr double kRowsMinNear = 0.3, kRowsFine = 0.9;
+
+// Estimated time (us) of a fp32 launch over the plan's block with rows and with taps, fitted to 779
+// launches of either kernel: 64, 336 and 1024 channels, 40-2000 trials with 0.2-0.9 of their pairs
+// near and 1-35 taps, 800-60000 outputs.  A CTA's time per channel, times the rounds of CTAs that an
+// SM works through; two at once take 1.6 (rows) and 1.2 (taps) times one.  Median errors 6 and 13 %.
+// Rows are taken where taps would cost kRowsMargin times as much: of those launches with at least
+// kRowsMinNear 10 are then more than 3 % slower than with taps (0.80 the worst; without the estimate
+// 128, down to 0.19), and 1.33 times as fast in the mean (1.27).
+constexpr double kRowsMargin = 1.1;
+double sm_rounds(int64_t ctas, double pair) {  // two CTAs per SM
+    const int64_t rest = ctas % 304;
+    return (double)(ctas / 304) * pair + (rest > 152 ? pair : rest > 0 ? 1.0 : 0.0);
+}
+// Per (trial block, channel): loads, words that a trial's lane reads; words and work, the rows' words
+// and multiply-adds in units of a tile.
+double rows_us(int nchan, int nw, int64_t ctas, bool one_wave, double loads, double words, double work) {
+    if (nw == dd::kRowWarps)
+        return 18.5 + nchan * (double)((ctas + 151) / 152) * (0.0143 * nw * loads + 0.006 * work + 0.2453 * words + 0.1438);
+    return 18.5 + nchan * (one_wave ? 1.0 : sm_rounds(ctas, 1.6)) * (0.008 * nw * loads + 0.0204 * work + 0.2432 * words + 0.1323);
+}
+// taps: mean of the longer run of a pair.
+double taps_us(const dd_plan_s* p, int nch, double taps) {
+    const int64_t t_out = std::max<int64_t>(1, p->band.nsamp - p->dmax);
+    if (dd::takes_units(p, t_out, nch)) return 11.4 + p->nchan * (0.0157 * taps + 0.508);
+    const int64_t tile = (int64_t)dd::chunk_t(true) * nch, db = 2 * (dd::kWarps / nch);
+    const int64_t ctas = (t_out + tile - 1) / tile * ((p->ndm + db - 1) / db);
+    return 43.1 + p->nchan * sm_rounds(ctas, 1.2) * (0.1034 * taps + 0.382);
+}
 
 // Warps per CTA of the row kernels.  16 (one CTA per SM) form a stage's rows for twice the
 // trials of 8 (two CTAs per SM), which measured 12 % faster on a long launch (CRAFT-like,
@@ -428,11 +458,13 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
         if (p->taps[a] != p->taps[b]) return false;
         return p->unit || std::memcmp(&p->w[a * p->kpad], &p->w[b * p->kpad], (size_t)p->taps[a] * sizeof(float)) == 0;
     };
+    bool fine = true;
     if (fir && p->ndm > 1) {  // (over the list's own neighbours: no matter how blocks fall)
         int64_t near = 0;
         for (size_t i = (size_t)C; i < (size_t)p->ndm * C; ++i)
             near += p->taps[i] == p->taps[i - C] && (uint32_t)(p->delay[i] - p->delay[i - C]) <= 2u;
         if ((double)near < kRowsMinNear * (units - C)) return false;
+        fine = (double)near >= kRowsFine * (units - C);
     }
     // the distinct runs of every (block, channel), and each trial's
     std::vector<std::vector<Row>> rows(nblk);
@@ -579,6 +611,36 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
         }
     }
     if ((double)total > kRowsMaxShare * units) return false;
+    if (fir && !fine) {
+        double words = 0, work = 0, loads = 0, taps = 0;
+        for (int b = 0; b < nblk; ++b)
+            for (const Row& r : rows[b]) {
+                words += (double)whole_len(r);
+                work += (double)whole_len(r) * r.n;
+            }
+        auto step = [&](size_t i) {  // a trial's start after that of the one before, in the same row (else far)
+            return p->taps[i] == p->taps[i - C] ? (uint32_t)(p->delay[i] - p->delay[i - C]) : UINT32_MAX;
+        };
+        const int R = dd::kRFir;  // (fir_channel: all three trials from one window, the first two, or none)
+        for (int d = 0; d < p->ndm; d += nt)
+            for (int c = 0; c < C; ++c) {
+                const size_t i = (size_t)d * C + c;
+                const bool one = d + 1 < p->ndm && step(i + C) <= 2u && d + 2 < p->ndm && step(i + 2 * C) <= 2u;
+                loads += one ? R + 2 : d + 1 < p->ndm && step(i + C) <= 3u ? 2 * R + 2 : 3 * R;
+            }
+        for (int d = 0; d < p->ndm; d += 2)
+            for (int c = 0; c < C; ++c) {
+                const size_t i = (size_t)d * C + c;
+                taps += std::max(p->taps[i], d + 1 < p->ndm ? p->taps[i + C] : 0);
+            }
+        const double per = (double)nblk * C, tile = dd::row_warp_t(kind);
+        const int64_t t = dd::row_tile_t(kind, nch), t_out = std::max<int64_t>(1, p->band.nsamp - p->dmax);
+        const double ru = rows_us(C, nw, (t_out + t - 1) / t * nblk, one_wave,
+                                  loads / ((double)((p->ndm + nt - 1) / nt) * C * 3 * R), words / per / tile, work / per / tile);
+        const double tu = taps_us(p, nch, taps / ((double)((p->ndm + 1) / 2) * C));
+        dd::log_msg(1, "plan %d trials x %d channels: estimated %.0f us with shared rows, %.0f tap by tap", p->ndm, C, ru, tu);
+        if (tu < kRowsMargin * ru) return false;
+    }
     const int64_t lcap = (need + Q - 1) / Q * Q;
     if (lcap > 0xffff || one.w > 0xffff) return false;
     const int64_t zero = dd::row_zero_words(kind, nch);  // the area begins with a row of zeros

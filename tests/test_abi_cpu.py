@@ -420,3 +420,24 @@ def test_plan_create_without_host_memory(lib):
             "    assert st == 3 and not h.value, st\n" % ROOT)
     res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
     assert res.returncode == 0, (res.returncode, res.stdout, res.stderr[-2000:])
+
+
+def _rule_dms(D, top):
+    nu = (1130.0 + np.arange(336) + 1) / 1000.0
+    b = math.sqrt(2.0) / (2 * 4.15 / 1000.0) / float(np.mean(nu ** -3))
+    return b * np.sinh(np.linspace(0.0, math.asinh(top / b), D))
+
+
+@pytest.mark.parametrize("D,top,t_out,rows", [
+    (436, 3540.0, 2075, False),     # a coarse list (0.45 of its pairs near) on a few tiles: 425 us, with rows 465
+    (273, 2288.0, 1842, False),     # 0.38: 489 us with its boxcar scan, with rows 514
+    (1000, 3540.0, 20000, True),
+    (1000, 400.0, 800, True),       # a fine list, rows at any size
+    (1000, 400.0, 60000, True),
+])
+def test_coarse_fp32_lists_take_the_faster_kernel(lib, D, top, t_out, rows):
+    import paper_1301_3968_gb300 as dd
+    dms = _rule_dms(D, top)
+    probe = dd.Plan(dd.Band(336, 1130.0, 1.0, 1.0, 4096, "f32"), dms)
+    plan = dd.Plan(dd.Band(336, 1130.0, 1.0, 1.0, t_out + probe.d_max, "f32"), dms)
+    assert (plan.schedule()["trials_per_cta"] in (24, 48)) == rows
