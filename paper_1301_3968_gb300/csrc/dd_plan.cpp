@@ -391,12 +391,15 @@ constexpr double kRowsMinNear = 0.3, kRowsFine = 0.9;
 
 // Estimated time (us) of a fp32 launch over the plan's block with rows and with taps, fitted to 779
 // launches of either kernel: 64, 336 and 1024 channels, 40-2000 trials with 0.2-0.9 of their pairs
-// near and 1-35 taps, 800-60000 outputs.  A CTA's time per channel, times the rounds of CTAs that an
-// SM works through; two at once take 1.6 (rows) and 1.2 (taps) times one.  Median errors 6 and 13 %.
-// Rows are taken where taps would cost kRowsMargin times as much: of those launches with at least
-// kRowsMinNear 10 are then more than 3 % slower than with taps (0.80 the worst; without the estimate
-// 128, down to 0.19), and 1.33 times as fast in the mean (1.27).
-constexpr double kRowsMargin = 1.1;
+// near and 1-35 taps, 800-60000 outputs (and 531 with uint8 input, whose conversion makes the rows'
+// building a quarter dearer).  A CTA's time per channel, times the rounds of CTAs that an
+// SM works through; two at once take 1.6 (rows) and 1.2 (taps) times one.  Median errors 6 and 13 %,
+// the larger ones where rows are long.  Rows are taken where taps would cost kRowsMargin times as much,
+// and kRowsMarginWords more for each tile's length that a channel's rows are longer than one.  Of 747
+// fp32 launches with at least kRowsMinNear five are then more than 3 % slower than with taps, four of
+// them fine lists (0.82 the worst; without the estimate 128, down to 0.19), and they are 1.35 times as
+// fast as with taps in the mean; uint8 input one of 531 (0.90) and 1.41.
+constexpr double kRowsMargin = 1.05, kRowsMarginWords = 0.1;
 double sm_rounds(int64_t ctas, double pair) {  // two CTAs per SM
     const int64_t rest = ctas % 304;
     return (double)(ctas / 304) * pair + (rest > 152 ? pair : rest > 0 ? 1.0 : 0.0);
@@ -635,11 +638,12 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
             }
         const double per = (double)nblk * C, tile = dd::row_warp_t(kind);
         const int64_t t = dd::row_tile_t(kind, nch), t_out = std::max<int64_t>(1, p->band.nsamp - p->dmax);
+        if (esz == 1) work *= 1.25;
         const double ru = rows_us(C, nw, (t_out + t - 1) / t * nblk, one_wave,
                                   loads / ((double)((p->ndm + nt - 1) / nt) * C * 3 * R), words / per / tile, work / per / tile);
         const double tu = taps_us(p, nch, taps / ((double)((p->ndm + 1) / 2) * C));
         dd::log_msg(1, "plan %d trials x %d channels: estimated %.0f us with shared rows, %.0f tap by tap", p->ndm, C, ru, tu);
-        if (tu < kRowsMargin * ru) return false;
+        if (tu < (kRowsMargin + kRowsMarginWords * (words / per / tile - 1)) * ru) return false;
     }
     const int64_t lcap = (need + Q - 1) / Q * Q;
     if (lcap > 0xffff || one.w > 0xffff) return false;
