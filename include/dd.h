@@ -21,7 +21,11 @@
  *     tables and workspace.  `stream` is a cudaStream_t (NULL = legacy default stream).
  *   - Device calls are asynchronous and stream-ordered.  Argument and plan errors are
  *     reported synchronously by the return value; CUDA launch errors as DD_ERR_CUDA.
- *   - A plan may be used from one stream at a time (its workspace is shared).
+ *   - A plan may be used from one stream at a time (its workspace is shared): order its calls on
+ *     different streams, and the replays of graphs that hold some, by events of your own.  Only
+ *     dd_dedisperse on a direct plan needs none: plans without prefix sums share nothing, and on
+ *     the others a call waits for the last one's reads on another stream (calls that are being
+ *     captured, and their replays, excepted).
  *   - Input rows are `in_ld` elements apart; in_ld * element size must be a multiple of
  *     16 bytes and the input base pointer 16-byte aligned (rows are staged in 16-byte
  *     chunks).  Violations return DD_ERR_ARG.

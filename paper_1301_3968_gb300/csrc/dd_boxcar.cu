@@ -806,7 +806,9 @@ __global__ void __launch_bounds__(256, std::is_same<TB, float>::value ? 3 : 2) k
 // consecutive starts in registers, and B_w(t) = P[t + w] - P[t] costs one load (odd stride: no
 // conflicts), one subtraction and half a three-input maximum whatever the widths are.  Maxima are
 // kept per segment and chunk as in k_boxcar_run; a warp per width finds the earliest start of the
-// winning segment.  Bound by instruction issue (2.6 per start and width) and the shared loads.
+// winning segment.  Bound by the latency of the shared loads with 24 warps on an SM, and the prefix
+// pass's barriers (1500 x 21364, ten octaves: data pipe 56 %, LSU 54 %, issue 48 %; stalls per issue
+// short_scoreboard 3.5, wait 2.2, barrier 1.3).
 // k_boxcar's running sums cost two loads, an addition, a comparison and two selects each: octave
 // widths 1-512 on 1500 x 21364 (normaliser included) 291 us with it, 129 with this.
 __host__ __device__ inline int list_buf(int wmax) { return (256 * kBoxS + wmax + 12) & ~3; }

@@ -395,7 +395,8 @@ dd_status launch_prefix_into(const dd_plan_s* p, const void* in, int64_t ld, int
     return cuda_status(cudaGetLastError());
 }
 
-// A stream that is being captured is not ordered here (its events cannot leave the capture).
+// A stream that is being captured is not ordered here (its events cannot leave the capture; the
+// caller orders the replays).
 // The legacy stream, which outlives every call, is recorded when another stream follows it.
 PrefixUse::PrefixUse(dd_plan_s* plan, cudaStream_t stream) : p(plan), s(stream) {
     if (!p || p->rl) return;

@@ -19,10 +19,6 @@ __device__ __forceinline__ uint64_t pk2(float lo, float hi) {
 __device__ __forceinline__ void fma2(uint64_t& acc, uint64_t w, uint64_t x) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(w), "l"(x));
 }
-// acc += x, both halves (add.rn.f32x2: two independent fp32 additions).
-__device__ __forceinline__ void add2(uint64_t& acc, uint64_t x) {
-    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(x));
-}
 __device__ __forceinline__ void unpk(uint64_t v, float& lo, float& hi) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
