@@ -225,3 +225,24 @@ def test_weights_from_the_device_keep_a_set_schedule(dd):
     s = plan.schedule()
     assert (s["nch"], s["cs"], s["trials_per_cta"]) == (2, 3, 8)
     assert plan.device_status() == 0
+
+
+@pytest.mark.parametrize("K", [1, 5, 16, 40])
+@pytest.mark.parametrize("D", [1, 7, 33, 130])
+def test_small_tap_launches_equal_the_full_one(dd, K, D):
+    """A call that gives each pair unit a CTA returns the bits of a longer call of the same plan,
+    which does not, at the edges of its tiles and of the trial blocks."""
+    import torch
+    rng = np.random.default_rng(K * 1000 + D)
+    C, long = 5, 768 * (620 // ((D + 1) // 2) + 2)
+    plan = dd.Plan(dd.Band(C, 1200.0, 1.0, 1.0, 4096, "f32"), np.zeros(D))
+    delay = rng.integers(0, 60, size=(D, C)).astype(np.int32)
+    plan.set_profiles(delay=delay, taps=np.full((D, C), K, np.int32), weights=np.ones((D, C, K), np.float32))
+    plan.set_weights(torch.from_numpy(rng.standard_normal((D, C, K)).astype(np.float32)).cuda())
+    n = long + plan.d_max
+    x = torch.from_numpy(rng.standard_normal((C, (n + 3) // 4 * 4)).astype(np.float32)).cuda()
+    want = plan.dedisperse(x, nsamp=n)
+    for t in (1, 767, 768, 769, 2305):
+        if t < long:
+            assert torch.equal(plan.dedisperse(x, nsamp=t + plan.d_max), want[:, :t])
+    assert plan.device_status() == 0
