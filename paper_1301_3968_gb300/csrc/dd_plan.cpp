@@ -463,9 +463,16 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
     };
     bool fine = true;
     if (fir && p->ndm > 1) {  // (over the list's own neighbours: no matter how blocks fall)
+        constexpr int kPart = 96;
+        std::vector<int64_t> nr((size_t)(p->ndm + kPart - 1) / kPart, 0);
+        for_blocks((int)nr.size(), (size_t)p->ndm * C, [&](int k) {
+            int64_t n = 0;
+            for (size_t i = (size_t)std::max(1, k * kPart) * C; i < (size_t)std::min(p->ndm, (k + 1) * kPart) * C; ++i)
+                n += p->taps[i] == p->taps[i - C] && (uint32_t)(p->delay[i] - p->delay[i - C]) <= 2u;
+            nr[k] = n;
+        });
         int64_t near = 0;
-        for (size_t i = (size_t)C; i < (size_t)p->ndm * C; ++i)
-            near += p->taps[i] == p->taps[i - C] && (uint32_t)(p->delay[i] - p->delay[i - C]) <= 2u;
+        for (int64_t n : nr) near += n;
         if ((double)near < kRowsMinNear * (units - C)) return false;
         fine = (double)near >= kRowsFine * (units - C);
     }
@@ -625,17 +632,27 @@ bool build_rows(dd_plan_s* p, int nch, int cs_fixed) {
             return p->taps[i] == p->taps[i - C] ? (uint32_t)(p->delay[i] - p->delay[i - C]) : UINT32_MAX;
         };
         const int R = dd::kRFir;  // (fir_channel: all three trials from one window, the first two, or none)
-        for (int d = 0; d < p->ndm; d += nt)
-            for (int c = 0; c < C; ++c) {
-                const size_t i = (size_t)d * C + c;
-                const bool one = d + 1 < p->ndm && step(i + C) <= 2u && d + 2 < p->ndm && step(i + 2 * C) <= 2u;
-                loads += one ? R + 2 : d + 1 < p->ndm && step(i + C) <= 3u ? 2 * R + 2 : 3 * R;
-            }
-        for (int d = 0; d < p->ndm; d += 2)
-            for (int c = 0; c < C; ++c) {
-                const size_t i = (size_t)d * C + c;
-                taps += std::max(p->taps[i], d + 1 < p->ndm ? p->taps[i + C] : 0);
-            }
+        constexpr int kPart = 96;  // trials, whole units and pairs of them
+        const int parts = (p->ndm + kPart - 1) / kPart;
+        std::vector<int64_t> ld((size_t)parts, 0), tp((size_t)parts, 0);
+        for_blocks(parts, (size_t)p->ndm * C, [&](int k) {
+            const int end = std::min(p->ndm, (k + 1) * kPart);
+            for (int d = k * kPart; d < end; d += nt)
+                for (int c = 0; c < C; ++c) {
+                    const size_t i = (size_t)d * C + c;
+                    const uint32_t s1 = d + 1 < end ? step(i + C) : UINT32_MAX;
+                    ld[k] += s1 <= 2u && d + 2 < end && step(i + 2 * C) <= 2u ? R + 2 : s1 <= 3u ? 2 * R + 2 : 3 * R;
+                }
+            for (int d = k * kPart; d < end; d += 2)
+                for (int c = 0; c < C; ++c) {
+                    const size_t i = (size_t)d * C + c;
+                    tp[k] += std::max(p->taps[i], d + 1 < end ? p->taps[i + C] : 0);
+                }
+        });
+        for (int k = 0; k < parts; ++k) {
+            loads += (double)ld[k];
+            taps += (double)tp[k];
+        }
         const double per = (double)nblk * C, tile = dd::row_warp_t(kind);
         const int64_t t = dd::row_tile_t(kind, nch), t_out = std::max<int64_t>(1, p->band.nsamp - p->dmax);
         if (esz == 1) work *= 1.25;
